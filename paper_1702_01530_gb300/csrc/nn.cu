@@ -41,23 +41,24 @@
 //   Every mbarrier wait has an iteration bound; on expiry the kernel sets the
 //   error word, waits (bounded) for what it has in flight and frees its TMEM.
 //
-// Layouts in HBM: the 16-channel maps (network input features, the BCE
-// gradient) are interleaved [P][16]; the 32-channel activations and data
+// Layouts in HBM: the network input features are interleaved [P][16]; the BCE
+// gradient is one chunk per pixel [P][8]; the 32-channel activations and data
 // gradients are chunk-planar [4][P][8] BF16 or [2][P][16] E4M3 (plane k
 // holds one 16-byte chunk of channels of every pixel), so a halo row of one
 // chunk is one contiguous run and each warp's epilogue store a contiguous
 // 512-byte run per plane.
 //
 // Backward pass: data gradients are convolutions with the 3x3 taps flipped
-// and Cin/Cout swapped (same tensor-core kernel); weight gradients are an
-// FP32 CUDA-core reduction over pixels; BCE on the sigmoid output; Adam on
-// FP32 master weights.
+// and Cin/Cout swapped (same tensor-core kernel); weight gradients are
+// contractions over the pixels on the tensor cores (k_wgrad_tc); BCE on the
+// sigmoid output; Adam on FP32 master weights.
 #include <cuda.h>
 #include <cuda_bf16.h>
 #include <cuda_fp8.h>
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <algorithm>
 #include <cstdlib>
 
 #include "rt_internal.cuh"
@@ -220,6 +221,16 @@ __device__ __forceinline__ void tma_load_4d(void* dst, const CUtensorMap* map, i
       "cp.async.bulk.tensor.4d.shared::cluster.global.tile.mbarrier::complete_tx::bytes"
       " [%0], [%1, {%2, %3, %4, %5}], [%6];" ::"r"(smem_u32(dst)),
       "l"(reinterpret_cast<uint64_t>(map)), "r"(c0), "r"(c1), "r"(c2), "r"(c3), "r"(smem_u32(bar))
+      : "memory");
+}
+
+// 3-D tiled TMA load (the same)
+__device__ __forceinline__ void tma_load_3d(void* dst, const CUtensorMap* map, int c0, int c1, int c2,
+                                            uint64_t* bar) {
+  asm volatile(
+      "cp.async.bulk.tensor.3d.shared::cluster.global.tile.mbarrier::complete_tx::bytes"
+      " [%0], [%1, {%2, %3, %4}], [%5];" ::"r"(smem_u32(dst)),
+      "l"(reinterpret_cast<uint64_t>(map)), "r"(c0), "r"(c1), "r"(c2), "r"(smem_u32(bar))
       : "memory");
 }
 
@@ -666,23 +677,22 @@ __global__ void k_amax(const __nv_bfloat16* __restrict__ a, size_t n, unsigned* 
 }
 
 // ------------------------------------------------------- BCE + d(logit)
-// loss = mean(-(y log p + (1-y) log(1-p))), dlogit = p - y (the 1/P factor is
-// applied in the weight-gradient kernel); dlogit goes to channel 0 of a
-// 16-channel BF16 map (the input of the layer-4 data-gradient conv) and to an
-// FP32 copy
+// loss = mean(-(y log p + (1-y) log(1-p))), dlogit g = p - y (the 1/P factor
+// is applied in the weight-gradient reduction). g goes out as one 16-byte
+// channel chunk per pixel, [P][8] BF16: channel 0 = bf16(g), the input of the
+// layer-4 data-gradient conv, and channels 1, 2 = the two BF16 remainders, so
+// that the three add up to the FP32 g exactly and the layer-4 weight gradient
+// keeps all its bits on the tensor cores.
 __global__ void k_bce(const float* __restrict__ prob, const float* __restrict__ label, uint32_t P,
-                      __nv_bfloat16* __restrict__ g16, float* __restrict__ g32,
-                      float* __restrict__ loss_sum) {
+                      uint4* __restrict__ g8, float* __restrict__ loss_sum) {
   float acc = 0.f;
   for (uint32_t p = blockIdx.x * blockDim.x + threadIdx.x; p < P; p += gridDim.x * blockDim.x) {
     const float q = fminf(fmaxf(prob[p], 1e-7f), 1.f - 1e-7f), y = label[p];
     acc += -(y * __logf(q) + (1.f - y) * __logf(1.f - q));
     const float g = prob[p] - y;
-    g32[p] = g;
-    __nv_bfloat16* o = g16 + 16 * (size_t)p;
-    o[0] = __float2bfloat16_rn(g);
-#pragma unroll
-    for (int c = 1; c < 16; ++c) o[c] = __float2bfloat16_rn(0.f);
+    const float hi = __bfloat162float(__float2bfloat16_rn(g));
+    const float mid = __bfloat162float(__float2bfloat16_rn(g - hi));
+    g8[p] = make_uint4(pack_bf16(hi, mid), pack_bf16(g - hi - mid, 0.f), 0u, 0u);
   }
   for (int off = 16; off > 0; off >>= 1) acc += __shfl_down_sync(0xFFFFFFFFu, acc, off);
   if ((threadIdx.x & 31) == 0) atomicAdd(loss_sum, acc);
@@ -690,105 +700,341 @@ __global__ void k_bce(const float* __restrict__ prob, const float* __restrict__ 
 
 // ------------------------------------------------------ weight gradients
 // dW[co][ci][ky][kx] = scale * sum_x dZ[y][x][co] * A[y+ky-1][x+kx-1][ci],
-// db[co] = scale * sum_x dZ[y][x][co]; each CTA takes every gridDim.x-th image
-// row, a 64-pixel chunk at a time through shared memory, FP32 accumulation,
-// and writes its unscaled partial sums (canonical layout: the layer's weights
-// then its biases) to its own row of `part`; k_wgrad_reduce then adds the
-// rows in a fixed order, so the gradient -- and training -- is the same bit
-// for bit from run to run (atomics would add the CTAs in arrival order).
-// A is interleaved [P][16] when CIN_PAD = 16 (the input features) and planar
-// [4][P][8] when CIN_PAD = 32 (activations); dZ comes as FP32 (layer 4, one
-// channel) or as a planar 32-channel BF16 map.
-template <int CIN_PAD, int COUT>
-__global__ void __launch_bounds__(256) k_wgrad(const __nv_bfloat16* __restrict__ A, int cin,
-                                               const __nv_bfloat16* __restrict__ dz16,
-                                               const float* __restrict__ dz32, uint32_t W,
-                                               uint32_t H, float* __restrict__ part) {
-  const size_t P = (size_t)W * H;
-  constexpr int kChunk = 64;
-  constexpr int kOut = COUT * CIN_PAD * 9;
-  constexpr int kPer = (kOut + 255) / 256;
-  __shared__ float sA[3][kChunk + 2][CIN_PAD];
-  __shared__ float sZ[kChunk][COUT];
-  float acc[kPer];
-  float bacc = 0.f;
-#pragma unroll
-  for (int i = 0; i < kPer; ++i) acc[i] = 0.f;
-  const int tid = threadIdx.x;
-  for (uint32_t y = blockIdx.x; y < H; y += gridDim.x) {
-    for (uint32_t x0 = 0; x0 < W; x0 += kChunk) {
-      __syncthreads();
-      for (int k = tid; k < 3 * (kChunk + 2) * CIN_PAD; k += 256) {
-        const int c = k % CIN_PAD, r = k / CIN_PAD;
-        const int dy = r / (kChunk + 2), xx = r % (kChunk + 2);
-        const int gy = (int)y + dy - 1, gx = (int)x0 + xx - 1;
-        float v = 0.f;
-        if (c < cin && gy >= 0 && gy < (int)H && gx >= 0 && gx < (int)W)
-          v = __bfloat162float(CIN_PAD == 32
-                                   ? A[((size_t)(c >> 3) * P + (size_t)gy * W + gx) * 8 + (c & 7)]
-                                   : A[((size_t)gy * W + gx) * CIN_PAD + c]);
-        sA[dy][xx][c] = v;
-      }
-      for (int k = tid; k < kChunk * COUT; k += 256) {
-        const int co = k % COUT, xx = k / COUT;
-        const uint32_t gx = x0 + xx;
-        float v = 0.f;
-        if (gx < W) {
-          const size_t p = (size_t)y * W + gx;
-          v = dz32 ? dz32[p] : __bfloat162float(dz16[((size_t)(co >> 3) * P + p) * 8 + (co & 7)]);
-        }
-        sZ[xx][co] = v;
-      }
-      __syncthreads();
-      const int nx = (int)(W - x0 < (uint32_t)kChunk ? W - x0 : (uint32_t)kChunk);
-#pragma unroll
-      for (int i = 0; i < kPer; ++i) {
-        const int o = tid + i * 256;
-        if (o < kOut) {
-          const int tap = o % 9, rest = o / 9;
-          const int ci = rest % CIN_PAD, co = rest / CIN_PAD;
-          const int dy = tap / 3, dx = tap % 3;
-          float s = 0.f;
-          for (int xx = 0; xx < nx; ++xx) s = fmaf(sZ[xx][co], sA[dy][xx + dx][ci], s);
-          acc[i] += s;
-        }
-      }
-      if (tid < COUT)
-        for (int xx = 0; xx < nx; ++xx) bacc += sZ[xx][tid];
-    }
-  }
-  const size_t n_w = (size_t)COUT * cin * 9;
-  float* row = part + (size_t)blockIdx.x * (n_w + COUT);
-#pragma unroll
-  for (int i = 0; i < kPer; ++i) {
-    const int o = tid + i * 256;
-    if (o < kOut) {
-      const int tap = o % 9, rest = o / 9;
-      const int ci = rest % CIN_PAD, co = rest / CIN_PAD;
-      if (ci < cin) row[((size_t)co * cin + ci) * 9 + tap] = acc[i];
-    }
-  }
-  if (tid < COUT) row[n_w + tid] = bacc;
+// db[co] = scale * sum_x dZ[y][x][co]: a contraction over the pixels, on the
+// tensor cores (tcgen05, BF16 operands whose products are exact in FP32).
+// A is the layer's input (AC 16-byte channel chunks per pixel: 4 planar, or 2
+// interleaved for the features), dZ its data gradient (ZC planar chunks: 4,
+// or the single chunk of k_bce whose three parts are added at the end).
+//
+// A persistent CTA takes tiles of 4 rows x 112 pixels. TMA boxes bring the
+// halo of A (6 rows x 114 pixels) and dZ into shared memory as [row][chunk]
+// [pixel][8 channels]: with the pixel as K that is the MN-major, non-swizzled
+// operand layout (core matrices of 8 pixels x 8 channels, 128 B apart along
+// K), and (row, chunk) is one uniform stride along M and N. So an MMA of
+// M = 128 multiplies 4 halo rows (8 of the 16-channel features) at once with
+// N = two rows of dZ: block (h, r) of D is the tap ky = h - r of dZ row r.
+// Three accumulators, one per kx (the A start moves by kx pixels), 7 K steps
+// of 16 pixels and 2 row pairs: 42 MMAs for the 448 pixels of a tile.
+// The tensor core truncates when it adds a product to its accumulator, the
+// more the longer the sum. So after every CHAIN K steps 8 epilogue warps add
+// the useful blocks to FP32 registers, rounding to nearest (warp w: TMEM lanes
+// 32 (w % 4), dZ row r = w / 4 of a pair), from one of two accumulator sets
+// while the next group's MMAs fill the other; they also add up dZ for the
+// bias. Every CTA writes two rows of unscaled partial sums (one per r), which
+// k_wgrad_reduce adds in a fixed order: the gradient, and training, is the
+// same bit for bit from run to run.
+// Measured (32 x 32 layer with its reduction, hot L2): 0.078 ms at 1920x1080
+// and 0.033 ms at 960x540, bound by the epilogue's TMEM reads (0.065 / 0.026
+// with CHAIN 7); the FP32 loop through shared memory took 24.0 and 5.94 ms,
+// and 14.46 of a 960x540 training step that now takes 0.33 ms.
+// CHAIN = 4 (groups of 4 and 3), or 2 where a CTA has at most kWgFewTiles
+// tiles. Error of a 32 x 32 layer's dW against 64 bits, 2-norm, for dZ of
+// random sign / of one sign, against the earlier FP32 fused-multiply-add loop:
+//   1920x1080 (27 tiles a CTA): loop 2.2e-7 / 6.7e-8; CHAIN 4 2.0e-7 / 4.4e-8;
+//                               2 2.8e-7 / 3.0e-8 (its register sums are long)
+//   960x540 (8): loop 1.9e-7 / 6.3e-8; 4 1.2e-7 / 4.3e-8; 7 1.1e-7 / 8.2e-8
+//   113x5 (1):   loop 5.9e-8 / 4.3e-8; 4 6.0e-8 / 5.2e-8; 2 6.0e-8 / 4.2e-8
+constexpr int kWgRows = 4, kWgW = 112;                // dZ rows and pixels of a tile
+constexpr uint32_t kWgFewTiles = 2;
+constexpr int kWgEpiWarps = 8, kWgThreads = 32 * (kWgEpiWarps + 2);
+static_assert(kWgRows % 2 == 0 && kWgW % 16 == 0, "row pairs, K steps of 16 pixels");
+
+template <int AC, int ZC>
+struct WgradLayout {
+  static constexpr uint32_t kPitchA = (kWgW + 2) * 16u, kPitchZ = kWgW * 16u;   // one row of one chunk
+  static constexpr uint32_t kRowA = AC * kPitchA, kRowZ = ZC * kPitchZ;
+  static constexpr uint32_t kBoxA = (kWgRows + 2) * kRowA, kBoxZ = kWgRows * kRowZ;
+  static constexpr uint32_t kOffZ = (kBoxA + 127u) & ~127u;
+  static constexpr uint32_t kSpanA = (16u / AC) * kRowA;                // bytes an MMA's M = 128 rows span
+  // a stage also covers what the last row pair's MMAs read past the halo
+  // (AC = 2: M rows that no tap uses)
+  static constexpr uint32_t kEndA = (kWgRows - 2) * kRowA + kSpanA + 32u, kEndZ = kOffZ + kBoxZ;
+  static constexpr uint32_t kStage = ((kEndA > kEndZ ? kEndA : kEndZ) + 1023u) & ~1023u;
+  static constexpr uint32_t kFit = (kSmemBudget - 2048u) / kStage;
+  static constexpr int kSt = kFit > 4u ? 4 : (int)kFit;
+  static constexpr int kN = 2 * 8 * ZC;                                 // MMA N: two dZ rows
+  static constexpr uint32_t kSet = 3 * kN;                              // TMEM columns of one accumulator set
+  static constexpr uint32_t kTmemCols = 2 * kSet <= 128 ? 128 : 512;
+  static constexpr size_t kSmem = kSt * (size_t)kStage + kWgEpiWarps * 8 * 4 + 20 * 8 + 16;
+  static constexpr int kCo = ZC == 4 ? 32 : 1;                          // output channels
+  static constexpr int kOuts = 9 * kCo * 8 * AC;                        // partial sums of a row, without the biases
+};
+
+// instruction descriptor: kind::f16, D = F32, A = B = BF16, both MN-major
+__host__ __device__ constexpr uint32_t make_idesc_mn(int M, int N) {
+  return make_idesc(M, N) | (1u << 15) | (1u << 16);
 }
 
-// out[j] = scale * sum over b = 0 .. nblk-1 of part[b][j], in a fixed order:
-// warp w of a block adds rows w, w + 8, w + 16, ... of 32 consecutive
-// columns, then thread 0..31 adds the 8 warp sums in warp order.
-__global__ void __launch_bounds__(256) k_wgrad_reduce(const float* __restrict__ part, uint32_t nblk,
-                                                      uint32_t n, float scale, float* __restrict__ out) {
-  __shared__ float s[8][32];
+// 8 consecutive TMEM columns of this warp's 32 lanes, without the wait
+__device__ __forceinline__ void tmem_ld8_nowait(uint32_t taddr, uint32_t r[8]) {
+  asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
+               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]),
+                 "=r"(r[7])
+               : "r"(taddr));
+}
+
+// (a0, a1) += (b0, b1) in one instruction, each sum rounded to nearest
+__device__ __forceinline__ void add2(float& a0, float& a1, uint32_t b0, uint32_t b1) {
+  asm("{\n\t.reg .b64 x, y;\n\t"
+      "mov.b64 x, {%0, %1};\n\t"
+      "mov.b64 y, {%2, %3};\n\t"
+      "add.rn.f32x2 x, x, y;\n\t"
+      "mov.b64 {%0, %1}, x;\n\t}"
+      : "+f"(a0), "+f"(a1)
+      : "r"(b0), "r"(b1));
+}
+
+// barriers: full[b] TMA bytes of stage b; empty[b] its MMAs (commit) and the
+// 8 epilogue warps' bias sums are done; acc_full[s] / acc_empty[s] as in
+// k_conv_tma. part: 2 gridDim.x rows of kOuts + kCo floats, [tap][co][ci]
+// then [co].
+template <int AC, int ZC, int CHAIN>
+__global__ void __launch_bounds__(kWgThreads, 1)
+    k_wgrad_tc(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ CUtensorMap map_z,
+               uint32_t W, uint32_t H, float* __restrict__ part, uint32_t* err) {
+  using Lt = WgradLayout<AC, ZC>;
+  constexpr int kGroupsRow = (kWgW / 16 + CHAIN - 1) / CHAIN;   // accumulator groups of a row pair
+  constexpr int kGroups = kWgRows / 2 * kGroupsRow;             // ... of a tile
+  extern __shared__ __align__(1024) unsigned char smem[];
+  float* bias_s = reinterpret_cast<float*>(smem + Lt::kSt * (size_t)Lt::kStage);   // [8 warps][8]
+  uint64_t* bars = reinterpret_cast<uint64_t*>(bias_s + kWgEpiWarps * 8);
+  uint64_t* full = bars;            // [kSt]
+  uint64_t* empty = bars + 8;       // [kSt]
+  uint64_t* acc_full = bars + 16;   // [2]
+  uint64_t* acc_empty = bars + 18;  // [2]
+  uint32_t* tslot = reinterpret_cast<uint32_t*>(bars + 20);
+
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const uint32_t tiles_x = (W + kWgW - 1) / kWgW;
+  const uint32_t n_tiles = tiles_x * ((H + kWgRows - 1) / kWgRows);
+  if (tid == 0) {
+    for (int b = 0; b < Lt::kSt; ++b) {
+      mbar_init(full + b, 1);
+      mbar_init(empty + b, 1 + kWgEpiWarps);
+    }
+    for (int b = 0; b < 2; ++b) {
+      mbar_init(acc_full + b, 1);
+      mbar_init(acc_empty + b, 32 * kWgEpiWarps);
+    }
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  }
+  if (warp == 0) tmem_alloc(tslot, Lt::kTmemCols);
+  fence_before();
+  __syncthreads();
+  fence_after();
+  const uint32_t tmem = *tslot;
+  const uint32_t my_tiles = blockIdx.x < n_tiles ? (n_tiles - 1 - blockIdx.x) / gridDim.x + 1 : 0;
+
+  if (warp == kWgEpiWarps) {
+    // ---- MMA issue
+    if (lane == 0) {
+      constexpr uint32_t idesc = make_idesc_mn(128, Lt::kN);
+      // LBO: from one group of 8 pixels (K) to the next; SBO: from one
+      // (row, chunk) group of 8 channels (M or N) to the next
+      constexpr uint32_t hi_a = desc_hi(Lt::kPitchA), hi_z = desc_hi(Lt::kPitchZ);
+      uint32_t n_mma = 0, grp = 0;       // tiles and accumulator groups issued
+      bool ok = true;
+      for (uint32_t it = 0; it < my_tiles && ok; ++it) {
+        const int b = (int)(it % Lt::kSt);
+        if (!mbar_wait(full + b, (it / Lt::kSt) & 1u)) { ok = false; break; }
+        const uint32_t base = smem_u32(smem + (size_t)b * Lt::kStage);
+        const uint32_t a_lo = desc_lo(base, 128u), z_lo = desc_lo(base + Lt::kOffZ, 128u);
+#pragma unroll
+        for (int g = 0; g < kGroups; ++g) {
+          const uint32_t sa = grp & 1u;
+          if (grp >= 2 && !mbar_wait(acc_empty + sa, ((grp >> 1) - 1) & 1u)) { ok = false; break; }
+          fence_after();
+          const int rp = g / kGroupsRow, ks0 = (g % kGroupsRow) * CHAIN;
+#pragma unroll
+          for (int ks = ks0; ks < ks0 + CHAIN && ks < kWgW / 16; ++ks)
+#pragma unroll
+            for (int dx = 0; dx < 3; ++dx) {
+              const uint32_t a_off = (2u * rp) * Lt::kRowA + (uint32_t)(16 * ks + dx) * 16u;
+              const uint32_t z_off = (2u * rp) * Lt::kRowZ + (uint32_t)(16 * ks) * 16u;
+              mma_bf16(tmem + sa * Lt::kSet + (uint32_t)(dx * Lt::kN),
+                       desc_join(a_lo + (a_off >> 4), hi_a), desc_join(z_lo + (z_off >> 4), hi_z), idesc,
+                       ks == ks0 ? 0u : 1u);
+            }
+          mma_commit(acc_full + sa);
+          ++grp;
+        }
+        if (!ok) break;
+        mma_commit(empty + b);
+        n_mma = it + 1;
+      }
+      if (!ok) atomicOr(err, ERR_ITER);
+      // drain: the MMAs issued here complete (and signal) before TMEM is freed
+      for (uint32_t k = grp > 2 ? grp - 2 : 0; k < grp; ++k) mbar_wait(acc_full + (k & 1u), (k >> 1) & 1u);
+      for (uint32_t it = n_mma > (uint32_t)Lt::kSt ? n_mma - Lt::kSt : 0; it < n_mma; ++it)
+        mbar_wait(empty + (it % Lt::kSt), (it / Lt::kSt) & 1u);
+    }
+    __syncwarp();
+  } else if (warp == kWgEpiWarps + 1) {
+    // ---- TMA loads
+    if (lane == 0) {
+      bool ok = true;
+      uint32_t n_loaded = 0;
+      for (uint32_t j = 0; j < my_tiles; ++j) {
+        const int b = (int)(j % Lt::kSt);
+        if (j >= (uint32_t)Lt::kSt && !mbar_wait(empty + b, ((j / Lt::kSt) - 1) & 1u)) { ok = false; break; }
+        const uint32_t tile = blockIdx.x + j * gridDim.x;
+        const int ty = (int)(tile / tiles_x);
+        const int y = ty * kWgRows, x0 = (int)(tile - (uint32_t)ty * tiles_x) * kWgW;
+        unsigned char* st = smem + (size_t)b * Lt::kStage;
+        mbar_arrive_expect_tx(full + b, Lt::kBoxA + Lt::kBoxZ);
+        if (AC == 2) tma_load_4d(st, &map_a, 0, x0 - 1, 0, y - 1, full + b);   // {8 channels, W, chunks, H}
+        else tma_load_3d(st, &map_a, 2 * (x0 - 1), 0, y - 1, full + b);        // {8-byte halves (2 W), chunks, H}
+        tma_load_3d(st + Lt::kOffZ, &map_z, 2 * x0, 0, y, full + b);
+        n_loaded = j + 1;
+      }
+      if (!ok) atomicOr(err, ERR_ITER);
+      // drain: the last copy into each stage has landed before the CTA exits
+      for (uint32_t j = n_loaded > (uint32_t)Lt::kSt ? n_loaded - Lt::kSt : 0; j < n_loaded; ++j)
+        mbar_wait(full + (j % Lt::kSt), (j / Lt::kSt) & 1u);
+    }
+    __syncwarp();
+  } else {
+    // ---- epilogue warps
+    constexpr int kCo = Lt::kCo;                        // output channels a thread accumulates
+    const int q = warp & 3, r = warp >> 2;
+    const int m = q * 32 + lane, h = m / (8 * AC), ci = m % (8 * AC), dy = h - r;
+    const bool useful = dy >= 0 && dy <= 2;
+    const bool warp_useful = __any_sync(0xFFFFFFFFu, useful);
+    constexpr int kPerChunk = 32 * kWgEpiWarps / ZC;    // threads that add up one chunk of dZ
+    const int zc = tid / kPerChunk, zt = tid % kPerChunk;
+    float acc[3][kCo], bacc[8];
+#pragma unroll
+    for (int dx = 0; dx < 3; ++dx)
+#pragma unroll
+      for (int c = 0; c < kCo; ++c) acc[dx][c] = 0.f;
+#pragma unroll
+    for (int c = 0; c < 8; ++c) bacc[c] = 0.f;
+    uint32_t grp = 0;
+    bool ok = true;
+    for (uint32_t it = 0; it < my_tiles && ok; ++it) {
+      const int b = (int)(it % Lt::kSt);
+      // warp-uniform outcome: tcgen05.ld below is a warp-collective instruction
+      if (!__all_sync(0xFFFFFFFFu, mbar_wait(full + b, (it / Lt::kSt) & 1u))) { ok = false; break; }
+      const unsigned char* z = smem + (size_t)b * Lt::kStage + Lt::kOffZ + (uint32_t)zc * Lt::kPitchZ;
+      for (int k = zt; k < kWgRows * kWgW; k += kPerChunk) {
+        const int row = k / kWgW, px = k - row * kWgW;
+        const uint4 v = *reinterpret_cast<const uint4*>(z + (uint32_t)row * Lt::kRowZ + (uint32_t)px * 16u);
+        const uint32_t w4[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+          const __nv_bfloat162 two = *reinterpret_cast<const __nv_bfloat162*>(&w4[i]);
+          bacc[2 * i] += __bfloat162float(two.x);
+          bacc[2 * i + 1] += __bfloat162float(two.y);
+        }
+      }
+      __syncwarp();
+      if (lane == 0) mbar_arrive(empty + b);
+#pragma unroll 1
+      for (int g = 0; g < kGroups; ++g, ++grp) {
+        const uint32_t s = grp & 1u;
+        if (!__all_sync(0xFFFFFFFFu, mbar_wait(acc_full + s, (grp >> 1) & 1u))) { ok = false; break; }
+        fence_after();
+        if (warp_useful) {
+          const uint32_t at = tmem + ((uint32_t)(q * 32) << 16) + s * Lt::kSet + (uint32_t)(r * 8 * ZC);
+          if (ZC == 4) {
+#pragma unroll
+            for (int dx = 0; dx < 3; ++dx) {
+              uint32_t v[2][16];
+              tmem_ld16_nowait(at + (uint32_t)(dx * Lt::kN), v[0]);
+              tmem_ld16_nowait(at + (uint32_t)(dx * Lt::kN + 16), v[1]);
+              tmem_wait_ld();
+#pragma unroll
+              for (int c = 0; c < kCo; c += 2)
+                add2(acc[dx][c], acc[dx][c + 1], v[c / 16][c % 16], v[c / 16][c % 16 + 1]);
+            }
+          } else {
+            uint32_t v[3][8];
+#pragma unroll
+            for (int dx = 0; dx < 3; ++dx) tmem_ld8_nowait(at + (uint32_t)(dx * Lt::kN), v[dx]);
+            tmem_wait_ld();
+#pragma unroll
+            for (int dx = 0; dx < 3; ++dx)
+              acc[dx][0] += (__uint_as_float(v[dx][2]) + __uint_as_float(v[dx][1])) + __uint_as_float(v[dx][0]);
+          }
+        }
+        fence_before();
+        mbar_arrive(acc_empty + s);
+      }
+    }
+    if (!ok && lane == 0) atomicOr(err, ERR_ITER);
+    // partial sums of this CTA: row 2 blockIdx.x + r, [tap][co][ci]
+    float* row = part + (2 * (size_t)blockIdx.x + r) * (Lt::kOuts + kCo);
+    if (useful)
+#pragma unroll
+      for (int dx = 0; dx < 3; ++dx)
+#pragma unroll
+        for (int c = 0; c < kCo; ++c)
+          row[(size_t)((dy * 3 + dx) * kCo + c) * (8 * AC) + ci] = acc[dx][c];
+    // biases: lanes, then the warps of a chunk, in a fixed order
+#pragma unroll
+    for (int c = 0; c < 8; ++c)
+      for (int off = 16; off > 0; off >>= 1) bacc[c] += __shfl_xor_sync(0xFFFFFFFFu, bacc[c], off);
+    if (lane == 0)
+#pragma unroll
+      for (int c = 0; c < 8; ++c) bias_s[warp * 8 + c] = bacc[c];
+  }
+  fence_before();
+  __syncthreads();
+  fence_after();
+  constexpr int kCo = Lt::kCo, kBiasAt = Lt::kOuts, kWarpsPer = kWgEpiWarps / ZC;
+  if (tid < kCo) {
+    float t = 0.f;
+    for (int w = 0; w < kWarpsPer; ++w) {
+      const float* p = bias_s + ((tid / 8) * kWarpsPer + w) * 8;
+      t += ZC == 4 ? p[tid % 8] : (p[2] + p[1]) + p[0];
+    }
+    float* row = part + 2 * (size_t)blockIdx.x * (kBiasAt + kCo);
+    row[kBiasAt + tid] = t;
+    row[kBiasAt + kCo + kBiasAt + tid] = 0.f;
+  }
+  if (warp == 0) tmem_dealloc(tmem, Lt::kTmemCols);
+}
+
+// (s, c) += x with the rounding error of the sum kept in c (Knuth's TwoSum)
+__device__ __forceinline__ void two_sum(float& s, float& c, float x) {
+  const float t = s + x, b = t - s;
+  c += (s - (t - b)) + (x - b);
+  s = t;
+}
+
+// out = scale * the partial rows' sum, in a fixed order and compensated (the
+// FP32 rounding of some hundred rows would cost more precision than the tensor
+// cores do): warp w of a block adds rows w, w + 8, w + 16, ... of 32
+// consecutive columns, then threads 0..31 add the 8 warp sums in warp order.
+// Column j is [tap][co][cin_p] (or, from n_w on, a bias); out is the
+// canonical W[co][cin][9] then b[co].
+__global__ void __launch_bounds__(256) k_wgrad_reduce(const float* __restrict__ part, uint32_t nrow,
+                                                      uint32_t cout, uint32_t cin, uint32_t cin_p,
+                                                      float scale, float* __restrict__ out) {
+  __shared__ float s[8][32], sc[8][32];
   const uint32_t lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const uint32_t n_w = 9 * cout * cin_p, n = n_w + cout;
   const uint32_t j = blockIdx.x * 32 + lane;
-  float a = 0.f;
+  float a = 0.f, c = 0.f;
   if (j < n)
-    for (uint32_t b = warp; b < nblk; b += 8) a += part[(size_t)b * n + j];
+#pragma unroll 8
+    for (uint32_t b = warp; b < nrow; b += 8) two_sum(a, c, part[(size_t)b * n + j]);
   s[warp][lane] = a;
+  sc[warp][lane] = c;
   __syncthreads();
   if (warp == 0 && j < n) {
-    float t = 0.f;
 #pragma unroll
-    for (int w = 0; w < 8; ++w) t += s[w][lane];
-    out[j] = t * scale;
+    for (int w = 1; w < 8; ++w) {
+      c += sc[w][lane];
+      two_sum(a, c, s[w][lane]);
+    }
+    const float t = (a + c) * scale;
+    if (j >= n_w) {
+      out[9 * cout * cin + (j - n_w)] = t;
+    } else {
+      const uint32_t ci = j % cin_p, co = (j / cin_p) % cout, tap = j / (cin_p * cout);
+      if (ci < cin) out[(co * cin + ci) * 9 + tap] = t;
+    }
   }
 }
 
@@ -856,8 +1102,11 @@ EncodeTiledFn encode_tiled() {
 // images} with one box {chunk elements, 1, 130, R+2, 1} per chunk; planar
 // [chunks][images][H][W][16 bytes] as 8-byte elements {2 W, H, images,
 // chunks} with one box {256 (128 pixels), R+2, 1, 1} per chunk.
+// A planar map may hold fewer chunks than the kernel's CIN (`chunks` > 0): the
+// boxes of the others lie outside the tensor and read zeros.
 template <int CIN, bool PLANAR, bool FP8>
-cudaError_t make_halo_map(CUtensorMap* map, const void* in, uint32_t W, uint32_t H, uint32_t n_img) {
+cudaError_t make_halo_map(CUtensorMap* map, const void* in, uint32_t W, uint32_t H, uint32_t n_img,
+                          uint32_t chunks) {
   const EncodeTiledFn fn = encode_tiled();
   if (!fn) return cudaErrorNotSupported;
   if (reinterpret_cast<uintptr_t>(in) & 15u) return cudaErrorInvalidValue;
@@ -866,7 +1115,7 @@ cudaError_t make_halo_map(CUtensorMap* map, const void* in, uint32_t W, uint32_t
   const cuuint32_t estr[5] = {1, 1, 1, 1, 1};
   CUresult r;
   if (PLANAR) {
-    const cuuint64_t d[4] = {2ull * W, H, n_img, kChunks};
+    const cuuint64_t d[4] = {2ull * W, H, n_img, chunks ? chunks : (cuuint64_t)kChunks};
     const cuuint64_t st[3] = {(cuuint64_t)W * 16, P * 16, P * n_img * 16};
     const cuuint32_t bx[4] = {2u * kHaloWPlanar, (cuuint32_t)(kRows + 2), 1, 1};
     r = fn(map, CU_TENSOR_MAP_DATA_TYPE_UINT64, 4, const_cast<void*>(in), d, st, bx, estr,
@@ -885,13 +1134,79 @@ cudaError_t make_halo_map(CUtensorMap* map, const void* in, uint32_t W, uint32_t
   return r == CUDA_SUCCESS ? cudaSuccess : cudaErrorInvalidValue;
 }
 
+// One map of W x H pixels for k_wgrad_tc: `chunks` 16-byte channel chunks per
+// pixel, interleaved ([P][16], 2 chunks) as {8 channels, W, chunks, H} or
+// planar ([chunks][P][8]) as 8-byte elements {2 W, chunks, H}; the box is
+// `px` pixels of every chunk in `rows` rows, in shared memory [row][chunk][px].
+cudaError_t make_wgrad_map(CUtensorMap* map, const void* in, uint32_t W, uint32_t H, uint32_t chunks,
+                           bool interleaved, uint32_t px, uint32_t rows) {
+  const EncodeTiledFn fn = encode_tiled();
+  if (!fn) return cudaErrorNotSupported;
+  if (reinterpret_cast<uintptr_t>(in) & 15u) return cudaErrorInvalidValue;
+  const cuuint64_t P = (cuuint64_t)W * H;
+  const cuuint32_t estr[4] = {1, 1, 1, 1};
+  CUresult r;
+  if (interleaved) {
+    const cuuint64_t d[4] = {8, W, chunks, H}, st[3] = {16ull * chunks, 16, 16ull * chunks * W};
+    const cuuint32_t bx[4] = {8, px, chunks, rows};
+    r = fn(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, const_cast<void*>(in), d, st, bx, estr,
+           CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
+           CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+  } else {
+    const cuuint64_t d[3] = {2ull * W, chunks, H}, st[2] = {P * 16, 16ull * W};
+    const cuuint32_t bx[3] = {2 * px, chunks, rows};
+    r = fn(map, CU_TENSOR_MAP_DATA_TYPE_UINT64, 3, const_cast<void*>(in), d, st, bx, estr,
+           CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+           CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+  }
+  return r == CUDA_SUCCESS ? cudaSuccess : cudaErrorInvalidValue;
+}
+
+uint64_t wgrad_tiles(uint32_t W, uint32_t H) {
+  return (uint64_t)((W + kWgW - 1) / kWgW) * ((H + kWgRows - 1) / kWgRows);
+}
+
+// Weight and bias gradients of one layer: k_wgrad_tc over all pixels, then
+// the reduction of its partial rows into out (canonical layout).
+template <int AC, int ZC>
+cudaError_t launch_wgrad(const void* a, const void* dz, uint32_t W, uint32_t H, uint32_t cin,
+                         float scale, float* part, float* out, uint32_t* err, cudaStream_t st) {
+  using Lt = WgradLayout<AC, ZC>;
+  // more than half of an SM's shared memory: one CTA (and its TMEM) per SM
+  constexpr size_t smem = Lt::kSmem < 116u * 1024u ? 116u * 1024u : Lt::kSmem;
+  static bool configured = false;
+  if (!configured) {
+    cudaError_t e = cudaFuncSetAttribute(k_wgrad_tc<AC, ZC, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         (int)smem);
+    if (e == cudaSuccess)
+      e = cudaFuncSetAttribute(k_wgrad_tc<AC, ZC, 4>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e != cudaSuccess) return e;
+    configured = true;
+  }
+  CUtensorMap ma, mz;
+  cudaError_t e = make_wgrad_map(&ma, a, W, H, AC, AC == 2, kWgW + 2, kWgRows + 2);
+  if (e == cudaSuccess) e = make_wgrad_map(&mz, dz, W, H, ZC, false, kWgW, kWgRows);
+  if (e != cudaSuccess) return e;
+  const uint64_t tiles = wgrad_tiles(W, H);
+  const int grid = (int)std::min<uint64_t>(tiles, (uint64_t)num_sms());   // one CTA per SM
+  if (tiles <= (uint64_t)kWgFewTiles * (uint64_t)grid)
+    k_wgrad_tc<AC, ZC, 2><<<grid, kWgThreads, smem, st>>>(ma, mz, W, H, part, err);
+  else
+    k_wgrad_tc<AC, ZC, 4><<<grid, kWgThreads, smem, st>>>(ma, mz, W, H, part, err);
+  const uint32_t n = (uint32_t)(Lt::kOuts + Lt::kCo);
+  k_wgrad_reduce<<<(n + 31) / 32, 256, 0, st>>>(part, 2u * (uint32_t)grid, (uint32_t)Lt::kCo, cin,
+                                                8u * AC, scale, out);
+  return cudaGetLastError();
+}
+
 // in: BF16 interleaved [P][16] when CIN = 16, BF16 planar [4][P][8] when
-// CIN = 32, E4M3 planar [2][P][16] with IN_FP8
-template <int CIN, int COUT, int EPI, bool IN_FP8 = false>
+// CIN = 32 (or with PLANAR_IN), E4M3 planar [2][P][16] with IN_FP8
+template <int CIN, int COUT, int EPI, bool IN_FP8 = false, bool PLANAR_IN = IN_FP8 || CIN == 32>
 cudaError_t launch_conv(const void* in, const void* wpk, const float* bias, const float* inv,
                         float out_scale, const __nv_bfloat16* mask16, void* out, float* out32,
-                        uint32_t W, uint32_t H, uint32_t* err, cudaStream_t st, uint32_t n_img = 1) {
-  constexpr bool kPlanarIn = IN_FP8 || CIN == 32;
+                        uint32_t W, uint32_t H, uint32_t* err, cudaStream_t st, uint32_t n_img = 1,
+                        uint32_t chunks = 0) {
+  constexpr bool kPlanarIn = PLANAR_IN;
   using Lt = ConvTmaLayout<CIN, COUT, IN_FP8, kPlanarIn>;
   const uint32_t tiles = ((W + Lt::kOutW - 1) / Lt::kOutW) * ((H + kRows - 1) / kRows) * n_img;
   size_t smem = Lt::kSmem + (size_t)(g_conv_smem_pad + conv_smem_pad());
@@ -906,7 +1221,7 @@ cudaError_t launch_conv(const void* in, const void* wpk, const float* bias, cons
     configured = smem;
   }
   CUtensorMap map;
-  cudaError_t e = make_halo_map<CIN, kPlanarIn, IN_FP8>(&map, in, W, H, n_img);
+  cudaError_t e = make_halo_map<CIN, kPlanarIn, IN_FP8>(&map, in, W, H, n_img, chunks);
   if (e != cudaSuccess) return e;
   // resident CTAs per SM from the shared-memory footprint (227 KB usable,
   // 1 KB reserved per CTA) and the TMEM columns (512 per SM) each CTA takes
@@ -1003,46 +1318,36 @@ cudaError_t activation_amax(const __nv_bfloat16* const act[3], uint64_t P, unsig
 // forward activations must be those of the same features and params
 cudaError_t backward(const __nv_bfloat16* feat16, const float* label, __nv_bfloat16* const wb[4],
                      const __nv_bfloat16* act1, const __nv_bfloat16* act2,
-                     const __nv_bfloat16* act3, const float* prob, __nv_bfloat16* g16, float* g32,
+                     const __nv_bfloat16* act3, const float* prob, __nv_bfloat16* g8,
                      __nv_bfloat16* dz_a, __nv_bfloat16* dz_b, float* wpart, float* grads,
                      float* loss_sum, uint32_t W, uint32_t H, uint32_t* err, cudaStream_t st) {
   const uint32_t P = W * H;
   const float scale = 1.f / (float)P;
-  const int rows_grid = wgrad_blocks(H);
-  // weight gradient of layer l from its per-CTA partial sums (fixed order)
-  auto reduce = [&](int l) {
-    const uint32_t n = (uint32_t)kCout[l] * (uint32_t)kCin[l] * 9u + (uint32_t)kCout[l];
-    k_wgrad_reduce<<<(n + 31) / 32, 256, 0, st>>>(wpart, (uint32_t)rows_grid, n, scale, grads + kOffW[l]);
-  };
   cudaMemsetAsync(loss_sum, 0, sizeof(float), st);
-  k_bce<<<num_sms() * 8, 256, 0, st>>>(prob, label, P, g16, g32, loss_sum);
-  // layer 4: dW from g32 (one channel), data gradient into dz_a (masked by act3 > 0)
-  k_wgrad<32, 1><<<rows_grid, 256, 0, st>>>(act3, 32, nullptr, g32, W, H, wpart);
-  reduce(3);
-  cudaError_t e = launch_conv<16, 32, EPI_BWD_MASK_BF16>(g16, wb[3], nullptr, nullptr, 1.f, act3, dz_a,
-                                                         nullptr, W, H, err, st);
+  k_bce<<<num_sms() * 8, 256, 0, st>>>(prob, label, P, reinterpret_cast<uint4*>(g8), loss_sum);
+  // layer 4: dW from the three parts of g, data gradient into dz_a (masked by act3 > 0)
+  cudaError_t e = launch_wgrad<4, 1>(act3, g8, W, H, kCin[3], scale, wpart, grads + kOffW[3], err, st);
+  if (e != cudaSuccess) return e;
+  e = launch_conv<16, 32, EPI_BWD_MASK_BF16, false, true>(g8, wb[3], nullptr, nullptr, 1.f, act3, dz_a,
+                                                          nullptr, W, H, err, st, 1, 1);
   if (e != cudaSuccess) return e;
   // layer 3
-  k_wgrad<32, 32><<<rows_grid, 256, 0, st>>>(act2, 32, dz_a, nullptr, W, H, wpart);
-  reduce(2);
+  e = launch_wgrad<4, 4>(act2, dz_a, W, H, kCin[2], scale, wpart, grads + kOffW[2], err, st);
+  if (e != cudaSuccess) return e;
   e = launch_conv<32, 32, EPI_BWD_MASK_BF16>(dz_a, wb[2], nullptr, nullptr, 1.f, act2, dz_b, nullptr,
                                              W, H, err, st);
   if (e != cudaSuccess) return e;
   // layer 2
-  k_wgrad<32, 32><<<rows_grid, 256, 0, st>>>(act1, 32, dz_b, nullptr, W, H, wpart);
-  reduce(1);
+  e = launch_wgrad<4, 4>(act1, dz_b, W, H, kCin[1], scale, wpart, grads + kOffW[1], err, st);
+  if (e != cudaSuccess) return e;
   e = launch_conv<32, 32, EPI_BWD_MASK_BF16>(dz_b, wb[1], nullptr, nullptr, 1.f, act1, dz_a, nullptr,
                                              W, H, err, st);
   if (e != cudaSuccess) return e;
   // layer 1 (no data gradient for the input features)
-  k_wgrad<16, 32><<<rows_grid, 256, 0, st>>>(feat16, kCin[0], dz_a, nullptr, W, H, wpart);
-  reduce(0);
-  return cudaGetLastError();
+  return launch_wgrad<2, 4>(feat16, dz_a, W, H, kCin[0], scale, wpart, grads + kOffW[0], err, st);
 }
 
-int wgrad_blocks(uint32_t H) { return (int)(H < (uint32_t)(num_sms() * 4) ? H : (uint32_t)(num_sms() * 4)); }
-
-size_t wgrad_part_floats(uint32_t H) { return (size_t)wgrad_blocks(H) * (32u * 32u * 9u + 32u); }
+size_t wgrad_part_floats() { return 2u * (size_t)num_sms() * (32u * 32u * 9u + 32u); }
 
 cudaError_t adam(float* params, const float* grads, float* m, float* v, uint32_t n, float lr,
                  uint32_t step, cudaStream_t st) {

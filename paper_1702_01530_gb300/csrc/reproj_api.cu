@@ -35,8 +35,7 @@ struct rt_net {
   uint64_t tcap = 0;
   __nv_bfloat16* act[3] = {};
   float* prob = nullptr;
-  __nv_bfloat16* g16 = nullptr;
-  float* g32 = nullptr;
+  __nv_bfloat16* g8 = nullptr;  // BCE gradient, 8 channels
   __nv_bfloat16* dz[2] = {};
   float* wpart = nullptr;       // per-CTA partial sums of the weight gradients
   // FP8 inference (rt_net_set_fp8): E4M3 weights of layers 2-4, their
@@ -67,10 +66,10 @@ cudaError_t net_forward(rt_net* net, const __nv_bfloat16* feat16, __nv_bfloat16*
 
 int net_buffers(rt_net* net, uint64_t P) {
   if (net->tb && net->tcap >= P) return RT_OK;
-  const size_t b_act = a256(P * 32 * 2), b_prob = a256(P * 4), b_g16 = a256(P * 16 * 2),
-               b_g32 = a256(P * 4), b_part = a256(rt::nn::wgrad_part_floats(0xFFFFFFFFu) * 4);
+  const size_t b_act = a256(P * 32 * 2), b_prob = a256(P * 4), b_g8 = a256(P * 8 * 2),
+               b_part = a256(rt::nn::wgrad_part_floats() * 4);
   void* base = nullptr;
-  cudaError_t e = cudaMalloc(&base, 3 * b_act + b_prob + b_g16 + b_g32 + 2 * b_act + b_part);
+  cudaError_t e = cudaMalloc(&base, 3 * b_act + b_prob + b_g8 + 2 * b_act + b_part);
   if (e != cudaSuccess) { cudaGetLastError(); return cuda_fail(e, "network activations"); }
   if (net->tb) cudaFree(net->tb);
   net->tb = base;
@@ -78,8 +77,7 @@ int net_buffers(rt_net* net, uint64_t P) {
   char* p = static_cast<char*>(base);
   for (int i = 0; i < 3; ++i) { net->act[i] = reinterpret_cast<__nv_bfloat16*>(p); p += b_act; }
   net->prob = reinterpret_cast<float*>(p); p += b_prob;
-  net->g16 = reinterpret_cast<__nv_bfloat16*>(p); p += b_g16;
-  net->g32 = reinterpret_cast<float*>(p); p += b_g32;
+  net->g8 = reinterpret_cast<__nv_bfloat16*>(p); p += b_g8;
   for (int i = 0; i < 2; ++i) { net->dz[i] = reinterpret_cast<__nv_bfloat16*>(p); p += b_act; }
   net->wpart = reinterpret_cast<float*>(p);
   return RT_OK;
@@ -425,7 +423,7 @@ int rt_net_train_step(rt_net* net, const uint16_t* d_feat16, const float* d_labe
                                   net->prob, W, H, net->err, st);
   if (e == cudaSuccess)
     e = rt::nn::backward(f16, d_label, net->wb, net->act[0], net->act[1], net->act[2], net->prob,
-                         net->g16, net->g32, net->dz[0], net->dz[1], net->wpart, net->grads,
+                         net->g8, net->dz[0], net->dz[1], net->wpart, net->grads,
                          net->loss, W, H, net->err, st);
   if (e == cudaSuccess && d_grads)
     e = cudaMemcpyAsync(d_grads, net->grads, (size_t)rt::nn::kParams * 4, cudaMemcpyDeviceToDevice, st);
