@@ -3,19 +3,25 @@
 // (E4M3 for layers 2-4 in FP8 inference) and FP32 accumulation on the
 // 5th-generation tensor cores (sm_103a).
 //
+// Forward pass: k_net_fused, all four layers in one kernel; activations are
+// written only where training or calibration asks for them.
+//
+// Backward pass: data gradients are convolutions with the 3x3 taps flipped and
+// Cin/Cout swapped (k_conv_tma, below); weight gradients are contractions over
+// the pixels (k_wgrad_tc); BCE on the sigmoid output; Adam on FP32 master
+// weights.
+//
 // Convolution as implicit GEMM on tcgen05 (k_conv_tma):
-//   a persistent CTA computes tiles of R rows x W_t consecutive pixels:
-//   output row ry is D_ry[128 pixels, Cout] = sum over the 9 taps (dy, dx) of
-//   A(ry+dy, dx)[128, Cin] x B(dy, dx)[Cin, Cout], where A(h, dx) is halo row h
+//   a persistent CTA computes tiles of R rows x 126 consecutive pixels:
+//   output row ry is D_ry[128 pixels, 32] = sum over the 9 taps (dy, dx) of
+//   A(ry+dy, dx)[128, Cin] x B(dy, dx)[Cin, 32], where A(h, dx) is halo row h
 //   shifted by dx pixels. The input halo (R+2 rows of Cin channels) sits in
 //   shared memory as 16-byte channel chunks ordered [chunk][halo pixel], so
-//   every A(h, dx) is the same matrix shifted by h*pitch + dx rows: the
+//   every A(h, dx) is the same matrix shifted by h*128 + dx rows: the
 //   K-major, non-swizzled operand layout with 8-row core matrices 128 B apart
-//   (SBO) and chunk planes (R+2)*pitch*16 B (rounded up to 128 B) apart (LBO).
-//   Interleaved inputs (the 16-channel features) have 130-pixel halo rows and
-//   W_t = 128; chunk-planar inputs (activations) are loaded as 2 KB box rows
-//   of 128 pixels, W_t = 126 (the MMA lanes 126 and 127 read the next row and
-//   are not stored).
+//   (SBO) and chunk planes (R+2)*128*16 B apart (LBO). The chunk planes are
+//   loaded as 2 KB box rows of 128 pixels (the MMA lanes 126 and 127 read the
+//   next row and are not stored).
 //   Stacked taps: an MMA of N = Cout costs the tensor core as much as one of
 //   N = 64 (about 45 cycles on GB300, measured; N = 96 about 56, N = 256 about
 //   128, the full rate), so the three vertical taps of a kernel column are
@@ -32,26 +38,18 @@
 //   layout, [dx][chunk][3 Cout][chunk elements].
 //   The CTA is warp-specialised: a TMA warp loads each tile's halo
 //   (cp.async.bulk.tensor, zeros outside the image) into a ring of halo
-//   buffers; an MMA warp issues the tile's MMAs (kind::f16 with BF16 inputs,
-//   kind::f8f6f4 with E4M3) into one of two TMEM accumulator sets; the
-//   epilogue warps read their TMEM lanes (tcgen05.ld 32x32b), hand the set
-//   back and apply the fused epilogue (bias + ReLU -> BF16 or E4M3, bias +
-//   sigmoid -> FP32, or the backward ReLU mask), so loads, MMAs and
+//   buffers; an MMA warp issues the tile's MMAs into one of two TMEM
+//   accumulator sets; the epilogue warps read their TMEM lanes (tcgen05.ld
+//   32x32b), hand the set back and apply the ReLU mask, so loads, MMAs and
 //   epilogues of consecutive tiles overlap.
 //   Every mbarrier wait has an iteration bound; on expiry the kernel sets the
 //   error word, waits (bounded) for what it has in flight and frees its TMEM.
 //
 // Layouts in HBM: the network input features are interleaved [P][16]; the BCE
 // gradient is one chunk per pixel [P][8]; the 32-channel activations and data
-// gradients are chunk-planar [4][P][8] BF16 or [2][P][16] E4M3 (plane k
-// holds one 16-byte chunk of channels of every pixel), so a halo row of one
-// chunk is one contiguous run and each warp's epilogue store a contiguous
-// 512-byte run per plane.
-//
-// Backward pass: data gradients are convolutions with the 3x3 taps flipped
-// and Cin/Cout swapped (same tensor-core kernel); weight gradients are
-// contractions over the pixels on the tensor cores (k_wgrad_tc); BCE on the
-// sigmoid output; Adam on FP32 master weights.
+// gradients are chunk-planar [4][P][8] BF16 (plane k holds one 16-byte chunk of
+// channels of every pixel), so a halo row of one chunk is one contiguous run
+// and each warp's epilogue store a contiguous 512-byte run per plane.
 #include <cuda.h>
 #include <cuda_bf16.h>
 #include <cuda_fp8.h>
@@ -66,18 +64,14 @@
 namespace rt {
 namespace nn {
 
-// Tuning knobs: RT_CONV_ROWS = image rows per tile (R accumulators of 128
-// pixels share one halo of R+2 rows; with the stacked taps each accumulator
-// set takes (R+4) * Cout TMEM columns, so R <= 4); RT_CONV_STAGES = the most
-// halo buffers a CTA keeps (each layer takes as many as fit in ~220 KB of
-// shared memory, up to this; the loads run that many tiles ahead of the MMAs).
-// A halo load took ~5600 cycles to land at 1080p, two to three tiles' MMAs,
-// yet deeper rings were slower: 3 / 4 / 5 / 6 / 8 stages, FP8 network at
-// 1920x1080: 0.145 / 0.147 / 0.155 / 0.163 / 0.172 ms (3840x2160, 8 images:
-// 0.398 / 0.397 / 0.426 / 0.434 ms per image for 3-6);
-// RT_CONV_EPI_WG = epilogue warpgroups (4 warps each; group g takes the rows
-// ry with ry % RT_CONV_EPI_WG == g of every tile; 4 groups were slower than 2:
-// 0.197 against 0.147 ms, FP8 at 1920x1080).
+// Tuning knobs of k_conv_tma: RT_CONV_ROWS = image rows per tile (R accumulators
+// of 128 pixels share one halo of R+2 rows; with the stacked taps each
+// accumulator set takes (R+4) * 32 TMEM columns, so R <= 4); RT_CONV_STAGES =
+// the most halo buffers a CTA keeps (as many as fit in ~220 KB of shared
+// memory, up to this; the loads run that many tiles ahead of the MMAs; deeper
+// rings were slower); RT_CONV_EPI_WG = epilogue warpgroups (4 warps each; group
+// g takes the rows ry with ry % RT_CONV_EPI_WG == g of every tile; 4 groups were
+// slower than 2).
 #ifndef RT_CONV_ROWS
 #define RT_CONV_ROWS 4
 #endif
@@ -94,22 +88,12 @@ constexpr int kEpiWarps = 4 * RT_CONV_EPI_WG;
 constexpr int kConvTmaThreads = 32 * (kEpiWarps + 2);   // + the MMA warp and the TMA warp
 constexpr int kRows = RT_CONV_ROWS;
 constexpr int kTileM = 128;          // pixels per row tile (one MMA M block)
-// The operand layout does not limit the MMAs: a 128-byte-swizzled operand
-// costs what the non-swizzled one does (measured), and neither a halo whose odd
-// chunks start a few pixels early (other shared-memory banks) nor swizzled
-// weights changed the layered network's time.
-constexpr int kHaloW = kTileM + 2;           // halo pixels per row of an interleaved input
-// A planar (chunk-plane) input is loaded as one TMA box per chunk whose rows
-// are 128 pixels x 16 bytes (256 8-byte elements, the largest box row), so
-// its tiles are 126 output pixels wide (the MMA lanes 126 and 127 read the
-// next halo row and are not stored). Boxes with rows of one 16-byte chunk
-// make one 16-byte request per pixel that moves a whole 32-byte sector from
-// L2: ~1500 requests per tile, whose transfer took longer than the tile's
-// MMAs (measured).
-constexpr int kHaloWPlanar = kTileM;
+// An input is loaded as one TMA box per chunk whose rows are 128 pixels x 16
+// bytes (256 8-byte elements, the largest box row), so tiles are 126 output
+// pixels wide. Boxes with rows of one 16-byte chunk make one 16-byte request
+// per pixel that moves a whole 32-byte sector from L2 (measured slower).
+constexpr int kHaloW = kTileM;
 constexpr uint32_t kWaitBound = 1u << 26;
-
-enum Epi : int { EPI_RELU_BF16 = 0, EPI_SIGMOID_F32 = 1, EPI_BWD_MASK_BF16 = 2, EPI_RELU_FP8 = 3 };
 
 // ------------------------------------------------------------ PTX helpers
 __device__ __forceinline__ uint32_t smem_u32(const void* p) {
@@ -142,6 +126,7 @@ __device__ __forceinline__ void mbar_init(uint64_t* bar, uint32_t count) {
 
 __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t phase) {
   const uint32_t a = smem_u32(bar);
+#pragma unroll 1
   for (uint32_t i = 0; i < kWaitBound; ++i) {
     uint32_t done;
     asm volatile(
@@ -154,6 +139,30 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t phase) {
     if (done) return true;
   }
   return false;
+}
+
+// true in one lane of the (converged) warp
+__device__ __forceinline__ bool elect_one() {
+  uint32_t p;
+  asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xFFFFFFFF;\n\tselp.u32 %0, 1, 0, p;\n\t}" : "=r"(p));
+  return p != 0;
+}
+
+// waits for two barriers' phases; with OVERLAP their first polls overlap
+template <bool OVERLAP>
+__device__ __forceinline__ bool mbar_wait2(uint64_t* bar0, uint32_t phase0, uint64_t* bar1, uint32_t phase1) {
+  if (!OVERLAP) return mbar_wait(bar0, phase0) && mbar_wait(bar1, phase1);
+  uint32_t d0, d1;
+  asm volatile(
+      "{\n\t.reg .pred p, q;\n\t"
+      "mbarrier.try_wait.parity.shared::cta.b64 p, [%2], %3;\n\t"
+      "mbarrier.try_wait.parity.shared::cta.b64 q, [%4], %5;\n\t"
+      "selp.u32 %0, 1, 0, p;\n\t"
+      "selp.u32 %1, 1, 0, q;\n\t}"
+      : "=r"(d0), "=r"(d1)
+      : "r"(smem_u32(bar0)), "r"(phase0), "r"(smem_u32(bar1)), "r"(phase1)
+      : "memory");
+  return (d0 || mbar_wait(bar0, phase0)) && (d1 || mbar_wait(bar1, phase1));
 }
 
 __device__ __forceinline__ void tmem_alloc(uint32_t* slot, uint32_t ncols) {
@@ -262,17 +271,58 @@ __device__ __forceinline__ uint32_t pack_bf16(float a, float b) {
   return *reinterpret_cast<uint32_t*>(&h);
 }
 
+// (a0, a1) += (b0, b1) in one instruction, each sum rounded to nearest
+__device__ __forceinline__ void add2(float& a0, float& a1, float b0, float b1) {
+  asm("{\n\t.reg .b64 x, y;\n\t"
+      "mov.b64 x, {%0, %1};\n\t"
+      "mov.b64 y, {%2, %3};\n\t"
+      "add.rn.f32x2 x, x, y;\n\t"
+      "mov.b64 {%0, %1}, x;\n\t}"
+      : "+f"(a0), "+f"(a1)
+      : "f"(b0), "f"(b1));
+}
+
+// (a0, a1) = fma((a0, a1), (m0, m1), (b0, b1))
+__device__ __forceinline__ void fma2(float& a0, float& a1, float m0, float m1, float b0, float b1) {
+  asm("{\n\t.reg .b64 x, m, y;\n\t"
+      "mov.b64 x, {%0, %1};\n\t"
+      "mov.b64 m, {%2, %3};\n\t"
+      "mov.b64 y, {%4, %5};\n\t"
+      "fma.rn.f32x2 x, x, m, y;\n\t"
+      "mov.b64 {%0, %1}, x;\n\t}"
+      : "+f"(a0), "+f"(a1)
+      : "f"(m0), "f"(m1), "f"(b0), "f"(b1));
+}
+// max(x, 0) of two BF16 (0 for a NaN, as fmaxf gives)
+__device__ __forceinline__ uint32_t relu_bf16(uint32_t x) {
+  uint32_t y;
+  asm("max.bf16x2 %0, %1, %2;" : "=r"(y) : "r"(x), "r"(0u));
+  return y;
+}
+
+// e4m3(max(x, 0)) of four values, round to nearest even, saturating (a NaN
+// stays a NaN)
+__device__ __forceinline__ uint32_t relu_e4m3x4(float x0, float x1, float x2, float x3) {
+  uint32_t d;
+  asm("{\n\t.reg .b16 lo, hi;\n\t"
+      "cvt.rn.satfinite.relu.e4m3x2.f32 lo, %2, %1;\n\t"
+      "cvt.rn.satfinite.relu.e4m3x2.f32 hi, %4, %3;\n\t"
+      "mov.b32 %0, {lo, hi};\n\t}"
+      : "=r"(d)
+      : "f"(x0), "f"(x1), "f"(x2), "f"(x3));
+  return d;
+}
+
 // All MMAs of one tile: for halo row h, kernel column dx and 32-byte K step
-// ks (16 BF16 or 32 E4M3 channels), the halo shifted by h*130 + dx pixels
-// times the stacked weights B(dx) (N = 3*COUT) accumulate into TMEM columns
-// dtmem + h*COUT .. + 3*COUT - 1 (output rows h-2 .. h). kChunks = 16-byte
-// channel chunks per pixel, kPlaneBytes = the distance between chunk planes
-// of the halo, kPitch = pixels from one halo row to the next. The
+// ks (16 channels), the halo shifted by h*128 + dx pixels times the stacked
+// weights B(dx) (N = 96) accumulate into TMEM columns dtmem + h*32 .. + 95
+// (output rows h-2 .. h). kChunks = 16-byte channel chunks per pixel,
+// kPlaneBytes = the distance between chunk planes of the halo. The
 // accumulators start at zero (cleared by the epilogue).
-template <int kChunks, int COUT, uint32_t kPlaneBytes, int kPitch, bool FP8>
-__device__ __forceinline__ void issue_tile_mmas(uint32_t hbase, uint32_t wbase, uint32_t dtmem,
-                                                uint32_t idesc) {
-  constexpr int kN = 3 * COUT;
+template <int kChunks, uint32_t kPlaneBytes>
+__device__ __forceinline__ void issue_tile_mmas(uint32_t hbase, uint32_t wbase, uint32_t dtmem) {
+  constexpr int kN = 96;
+  constexpr uint32_t idesc = make_idesc(kTileM, kN);
   // A: LBO = the distance from an even chunk's core matrix to the odd one's;
   // B: chunk c + 1 of a weight row sits kN * 16 bytes after chunk c
   const uint32_t a_lo = desc_lo(hbase, kPlaneBytes), b_lo = desc_lo(wbase, kN * 16);
@@ -283,11 +333,10 @@ __device__ __forceinline__ void issue_tile_mmas(uint32_t hbase, uint32_t wbase, 
     for (int dx = 0; dx < 3; ++dx) {
 #pragma unroll
       for (int ks = 0; ks < kChunks / 2; ++ks) {
-        const uint32_t a_off = (2u * ks) * kPlaneBytes + (uint32_t)(h * kPitch + dx) * 16u;
+        const uint32_t a_off = (2u * ks) * kPlaneBytes + (uint32_t)(h * kHaloW + dx) * 16u;
         const uint32_t b_off = (uint32_t)((dx * kChunks + 2 * ks) * kN) * 16u;
-        const uint64_t da = desc_join(a_lo + (a_off >> 4), hi), db = desc_join(b_lo + (b_off >> 4), hi);
-        if (FP8) mma_e4m3(dtmem + (uint32_t)(h * COUT), da, db, idesc, 1u);
-        else mma_bf16(dtmem + (uint32_t)(h * COUT), da, db, idesc, 1u);
+        mma_bf16(dtmem + (uint32_t)(h * 32), desc_join(a_lo + (a_off >> 4), hi),
+                 desc_join(b_lo + (b_off >> 4), hi), idesc, 1u);
       }
     }
   }
@@ -303,30 +352,21 @@ __device__ __forceinline__ void tmem_zero16(uint32_t taddr) {
 }
 __device__ __forceinline__ void tmem_wait_st() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
 
-// ------------------------------------------------------------ conv kernel
-// in:  BF16 [P][16] interleaved (CIN = 16) or [4][P][8] planar (CIN = 32);
-//      with IN_FP8, E4M3 [2][P][16] planar (CIN = 32)
-// wpk: packed weights, [dx][16-byte chunk][3 COUT: dy = 2, 1, 0][chunk elements]
-//      (BF16 or E4M3)
-// With IN_FP8 the accumulator of channel co is first multiplied by inv[co]
-// (the product of the input's activation scale and the channel's weight
-// scale, inverted: a power of two).
-// EPI_RELU_BF16:     out (BF16 planar [4][P][8]) = relu(acc + bias)
-// EPI_SIGMOID_F32:   out32[P] = sigmoid(acc[0] + bias[0])
-// EPI_BWD_MASK_BF16: out (BF16 planar) = acc * (mask16 (planar) > 0)
-// EPI_RELU_FP8:      out (E4M3 planar [2][P][16]) = e4m3(relu(acc + bias) * out_scale),
-//                    round to nearest even, saturating at +-448
+// ------------------------------------------------------- data gradients
+// in:  CIN / 8 chunk planes of BF16 ([P][8] each); a map with fewer planes (the
+//      BCE gradient's one) reads zeros for the others
+// wpk: packed weights, [dx][16-byte chunk][96: dy = 2, 1, 0][8]
+// out: BF16 planar [4][P][8] = acc where the layer's activation (mask16, same
+//      layout) is positive, else 0
 //
-// Three roles. The last warp's first lane loads each tile's halo (one TMA box
-// per 16-byte channel chunk, zeros outside the image) into a ring of
-// RT_CONV_STAGES halo buffers, as far ahead as the ring allows; the warp
-// before it issues the tile's MMAs into one of two TMEM accumulator sets as
-// soon as its halo has landed and the epilogue has drained that set; the
-// epilogue warps (RT_CONV_EPI_WG warpgroups; warp w reads TMEM lanes
-// 32 (w % 4) .. +31) run the epilogue of tile i while the tensor cores work on
-// tile i+1 and the TMA engine fetches the next tiles. Loads, MMAs and
-// epilogues each wait only on their own barriers (in one thread, the loads'
-// issue and the waits for their buffers held up the MMAs, measured).
+// Three roles. The last warp loads each tile's halo (one TMA box per 16-byte
+// channel chunk, zeros outside the image) into a ring of RT_CONV_STAGES halo
+// buffers, as far ahead as the ring allows; the warp before it issues the
+// tile's MMAs into one of two TMEM accumulator sets as soon as its halo has
+// landed and the epilogue has drained that set; the epilogue warps
+// (RT_CONV_EPI_WG warpgroups; warp w reads TMEM lanes 32 (w % 4) .. +31) run
+// the epilogue of tile i while the tensor cores work on tile i+1 and the TMA
+// engine fetches the next tiles.
 //   halo_full[b]:  TMA bytes of halo buffer b arrived (expect_tx by the loader)
 //   halo_empty[b]: the MMAs that read buffer b completed (tcgen05.commit)
 //   acc_full[s]:   MMAs of accumulator set s done (tcgen05.commit)
@@ -334,60 +374,46 @@ __device__ __forceinline__ void tmem_wait_st() { asm volatile("tcgen05.wait::st.
 // Every wait is bounded; a wait that gives up sets the error word, and before
 // the CTA frees TMEM and exits, the TMA warp waits (bounded) for the last copy
 // into each buffer and the MMA warp for the MMAs it has issued.
-template <int CIN, int COUT, bool IN_FP8, bool PLANAR>
+template <int CIN>
 struct ConvTmaLayout {
-  static constexpr int kElem = IN_FP8 ? 1 : 2;                           // bytes per channel
-  static constexpr int kChunks = CIN * kElem / 16;                       // 16-byte chunks per pixel
-  static constexpr int kPitch = PLANAR ? kHaloWPlanar : kHaloW;          // halo pixels per row
-  static constexpr int kOutW = kPitch - 2;                               // output pixels per row
-  static constexpr uint32_t kBox = (uint32_t)(kRows + 2) * kPitch * 16u; // bytes of one TMA box
-  static constexpr uint32_t kPlane = (kBox + 127u) & ~127u;            // chunk plane stride
-  static constexpr uint32_t kHalo = ((kChunks * kPlane) + 1023u) & ~1023u;
-  static constexpr uint32_t kWBytes = 9u * COUT * CIN * kElem;
-  static constexpr uint32_t kW = (kWBytes + 127u) & ~127u;
-  static constexpr uint32_t kAcc = (uint32_t)(kRows + 4) * COUT;       // rows -2 .. R+1
-  static constexpr uint32_t kSet = kAcc <= 32 ? 32 : (kAcc <= 64 ? 64 : (kAcc <= 128 ? 128 : 256));
-  static constexpr uint32_t kTmemCols = 2 * kSet;
+  static constexpr int kChunks = CIN / 8;                                // 16-byte chunks per pixel
+  static constexpr int kOutW = kHaloW - 2;                               // output pixels per row
+  static constexpr uint32_t kPlane = (uint32_t)(kRows + 2) * kHaloW * 16u;   // one TMA box
+  static constexpr uint32_t kHalo = kChunks * kPlane;
+  static constexpr uint32_t kW = 9u * 32 * CIN * 2;
+  static constexpr uint32_t kSet = (kRows + 4) * 32;                     // rows -2 .. R+1
+  static constexpr uint32_t kTmemCols = 512;
   static constexpr uint32_t kFit = (kSmemBudget - kW - 1024u) / kHalo;   // halo buffers that fit
   static constexpr int kSt = kFit < 2u ? 2 : (kFit > (uint32_t)kMaxStages ? kMaxStages : (int)kFit);
-  static constexpr size_t kSmem = kSt * (size_t)kHalo + kW + 64 * 4 + 20 * 8 + 16;
+  static constexpr size_t kSmem = kSt * (size_t)kHalo + kW + 20 * 8 + 16;
+  static_assert(2 * kSet <= kTmemCols, "two accumulator sets must fit in TMEM");
 };
 
-template <int CIN, int COUT, int EPI, bool PLANAR_IN, bool IN_FP8>
+template <int CIN>
 __global__ void __launch_bounds__(kConvTmaThreads, 1)
     k_conv_tma(const __grid_constant__ CUtensorMap tmap, const void* __restrict__ wpk,
-               const float* __restrict__ bias, const float* __restrict__ inv,
-               float out_scale, const __nv_bfloat16* __restrict__ mask16, void* __restrict__ out,
-               float* __restrict__ out32, uint32_t W, uint32_t H, uint32_t n_img, uint32_t* err) {
-  using Lt = ConvTmaLayout<CIN, COUT, IN_FP8, PLANAR_IN>;
-  static_assert(CIN % 16 == 0 && (COUT == 16 || COUT == 32), "shape");
-  static_assert(Lt::kTmemCols <= 512, "two accumulator sets must fit in TMEM");
+               const __nv_bfloat16* __restrict__ mask16, __nv_bfloat16* __restrict__ out, uint32_t W,
+               uint32_t H, uint32_t* err) {
+  using Lt = ConvTmaLayout<CIN>;
+  static_assert(CIN % 16 == 0, "shape");
   extern __shared__ __align__(1024) unsigned char smem[];
   unsigned char* halo0 = smem;
   unsigned char* wsm = smem + Lt::kSt * Lt::kHalo;
-  float* bsm = reinterpret_cast<float*>(wsm + Lt::kW);    // bias[32], then inv[32]
-  float* ism = bsm + 32;
-  uint64_t* bars = reinterpret_cast<uint64_t*>(bsm + 64);
+  uint64_t* bars = reinterpret_cast<uint64_t*>(wsm + Lt::kW);
   uint64_t* halo_full = bars;        // [kSt]
   uint64_t* halo_empty = bars + 8;   // [kSt]
   uint64_t* acc_full = bars + 16;    // [2]
   uint64_t* acc_empty = bars + 18;   // [2]
   uint32_t* tslot = reinterpret_cast<uint32_t*>(bars + 20);
 
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  // n_img images of W x H pixels stacked in memory (image-major); a tile
-  // never spans two images, and the halo rows outside its image read zeros
+  const int tid = threadIdx.x, lane = tid & 31;
+  const int warp = __shfl_sync(0xFFFFFFFFu, tid >> 5, 0);   // known to be uniform
   const uint32_t tiles_x = (W + Lt::kOutW - 1) / Lt::kOutW;
-  const uint32_t tiles_img = tiles_x * ((H + kRows - 1) / kRows);
-  const uint32_t n_tiles = tiles_img * n_img;
+  const uint32_t n_tiles = tiles_x * ((H + kRows - 1) / kRows);
   {
     const uint4* src = reinterpret_cast<const uint4*>(wpk);
     uint4* dst = reinterpret_cast<uint4*>(wsm);
-    for (uint32_t i = tid; i < Lt::kWBytes / 16u; i += blockDim.x) dst[i] = src[i];
-    if (tid < COUT) {
-      bsm[tid] = bias ? bias[tid] : 0.f;
-      ism[tid] = inv ? inv[tid] : 1.f;
-    }
+    for (uint32_t i = tid; i < Lt::kW / 16u; i += blockDim.x) dst[i] = src[i];
   }
   if (tid == 0) {
     for (int b = 0; b < Lt::kSt; ++b) {
@@ -406,7 +432,7 @@ __global__ void __launch_bounds__(kConvTmaThreads, 1)
   fence_before();
   __syncthreads();
   fence_after();
-  const uint32_t tmem = *tslot;
+  const uint32_t tmem = __shfl_sync(0xFFFFFFFFu, *tslot, 0);
   // the MMAs only accumulate: clear both accumulator sets once (warp w % 4
   // may address TMEM lanes 32 (w % 4) .. +31)
   if (warp < 4) {
@@ -419,37 +445,34 @@ __global__ void __launch_bounds__(kConvTmaThreads, 1)
 
   const uint32_t my_tiles = blockIdx.x < n_tiles ? (n_tiles - 1 - blockIdx.x) / gridDim.x + 1 : 0;
   if (warp == kEpiWarps) {
-    // ---- MMA issue: tile it of this CTA's sequence reads halo buffer it % kSt
-    if (lane == 0) {
-      const uint32_t idesc = IN_FP8 ? make_idesc_e4m3(kTileM, 3 * COUT) : make_idesc(kTileM, 3 * COUT);
-      const uint32_t wbase = smem_u32(wsm);
-      bool issued_acc[2] = {false, false}, issued_he[Lt::kSt];
-      uint32_t acc_par[2] = {0, 0}, he_par[Lt::kSt];     // parity of the last commit
-#pragma unroll
-      for (int b = 0; b < Lt::kSt; ++b) { issued_he[b] = false; he_par[b] = 0; }
-      bool ok = true;
-      for (uint32_t it = 0; it < my_tiles; ++it) {
-        const int b = (int)(it % Lt::kSt), sa = (int)(it & 1u);
-        if (!mbar_wait(halo_full + b, (it / Lt::kSt) & 1u)) { ok = false; break; }
-        if (it >= 2 && !mbar_wait(acc_empty + sa, ((it >> 1) - 1) & 1u)) { ok = false; break; }
-        fence_after();
-        issue_tile_mmas<Lt::kChunks, COUT, Lt::kPlane, Lt::kPitch, IN_FP8>(
-            smem_u32(halo0 + (size_t)b * Lt::kHalo), wbase, tmem + (uint32_t)sa * Lt::kSet, idesc);
+    // ---- MMA issue: tile it of this CTA's sequence reads halo buffer it % kSt.
+    // The whole warp walks the loop and one elected lane issues, so that the
+    // compiler keeps the descriptors in uniform registers (in a loop of one
+    // lane every MMA paid for moving them there).
+    const uint32_t wbase = smem_u32(wsm);
+    uint32_t n_mma = 0;
+    bool ok = true;
+    for (uint32_t it = 0; it < my_tiles; ++it) {
+      const uint32_t b = it % Lt::kSt, sa = it & 1u;
+      ok = mbar_wait(halo_full + b, (it / Lt::kSt) & 1u) &&
+           (it < 2 || mbar_wait(acc_empty + sa, ((it >> 1) - 1) & 1u));
+      ok = __all_sync(0xFFFFFFFFu, ok);
+      if (!ok) break;
+      fence_after();
+      if (elect_one()) {
+        issue_tile_mmas<Lt::kChunks, Lt::kPlane>(smem_u32(halo0) + b * Lt::kHalo, wbase, tmem + sa * Lt::kSet);
         mma_commit(halo_empty + b);   // the buffer may be reloaded once these MMAs completed
         mma_commit(acc_full + sa);
-        issued_he[b] = true;
-        he_par[b] = (it / Lt::kSt) & 1u;
-        issued_acc[sa] = true;
-        acc_par[sa] = (it >> 1) & 1u;
       }
-      if (!ok) atomicOr(err, ERR_ITER);
-      // drain: the MMAs issued here complete (and signal) before TMEM is freed
-      for (int b = 0; b < 2; ++b)
-        if (issued_acc[b]) mbar_wait(acc_full + b, acc_par[b]);
-      for (int b = 0; b < Lt::kSt; ++b)
-        if (issued_he[b]) mbar_wait(halo_empty + b, he_par[b]);
+      __syncwarp();
+      n_mma = it + 1;
     }
-    __syncwarp();
+    if (!ok && lane == 0) atomicOr(err, ERR_ITER);
+    // drain: the MMAs issued here complete (and signal) before TMEM is freed
+    for (uint32_t it = n_mma > 2 ? n_mma - 2 : 0; it < n_mma; ++it)
+      mbar_wait(acc_full + (it & 1u), (it >> 1) & 1u);
+    for (uint32_t it = n_mma > (uint32_t)Lt::kSt ? n_mma - Lt::kSt : 0; it < n_mma; ++it)
+      mbar_wait(halo_empty + it % Lt::kSt, (it / Lt::kSt) & 1u);
   } else if (warp == kEpiWarps + 1) {
     // ---- TMA loads: tile j into buffer j % kSt once the MMAs of tile
     // j - kSt (the buffer's previous tile) completed
@@ -460,19 +483,13 @@ __global__ void __launch_bounds__(kConvTmaThreads, 1)
         const int b = (int)(j % Lt::kSt);
         if (j >= (uint32_t)Lt::kSt && !mbar_wait(halo_empty + b, ((j / Lt::kSt) - 1) & 1u)) { ok = false; break; }
         const uint32_t tile = blockIdx.x + j * gridDim.x;
-        const int img = (int)(tile / tiles_img);
-        const uint32_t it_img = tile - (uint32_t)img * tiles_img;
-        const int ty = (int)(it_img / tiles_x);
-        const int y = ty * kRows, x0 = (int)(it_img - (uint32_t)ty * tiles_x) * Lt::kOutW;
-        mbar_arrive_expect_tx(halo_full + b, (uint32_t)Lt::kChunks * Lt::kBox);
+        const int ty = (int)(tile / tiles_x);
+        const int y = ty * kRows, x0 = (int)(tile - (uint32_t)ty * tiles_x) * Lt::kOutW;
+        mbar_arrive_expect_tx(halo_full + b, (uint32_t)Lt::kChunks * Lt::kPlane);
 #pragma unroll
-        for (int c = 0; c < Lt::kChunks; ++c) {
-          unsigned char* plane = halo0 + (size_t)b * Lt::kHalo + (size_t)c * Lt::kPlane;
-          if (PLANAR_IN)   // tensor {8-byte halves of pixels (2 W), H, images, chunks}
-            tma_load_4d(plane, &tmap, 2 * (x0 - 1), y - 1, img, c, halo_full + b);
-          else             // tensor {16 B of channels, chunks, W, H, images}
-            tma_load_5d(plane, &tmap, 0, c, x0 - 1, y - 1, img, halo_full + b);
-        }
+        for (int c = 0; c < Lt::kChunks; ++c)   // tensor {8-byte halves of pixels (2 W), H, chunks}
+          tma_load_3d(halo0 + (size_t)b * Lt::kHalo + (size_t)c * Lt::kPlane, &tmap, 2 * (x0 - 1), y - 1, c,
+                      halo_full + b);
         n_loaded = j + 1;
       }
       if (!ok) atomicOr(err, ERR_ITER);
@@ -488,21 +505,9 @@ __global__ void __launch_bounds__(kConvTmaThreads, 1)
     // stores: the tensor core then waits only for the TMEM reads, not for the
     // whole epilogue.
     constexpr int kMine = kRows / RT_CONV_EPI_WG;   // rows per epilogue warp
-    constexpr int kHalves = COUT / 16;
     static_assert(kRows % RT_CONV_EPI_WG == 0, "rows per tile must split evenly over the epilogue groups");
     const int quarter = warp & 3, group = warp >> 2;   // TMEM lanes 32*quarter .. +31
-    const size_t P = (size_t)W * H * n_img;            // pixels of a channel plane
-    // per output channel c: out = max(fma(acc, sc[c], bi[c]), 0) (or the
-    // sigmoid of it), with the input's inverse scale (E4M3 inputs) and the
-    // output scale (E4M3 outputs) folded in: all are powers of two, so the
-    // folded form rounds exactly like scaling the rounded sum
-    float sc[COUT], bi[COUT];
-#pragma unroll
-    for (int c = 0; c < COUT; ++c) {
-      const float os = EPI == EPI_RELU_FP8 ? out_scale : 1.f;
-      sc[c] = (IN_FP8 ? ism[c] : 1.f) * os;
-      bi[c] = bsm[c] * os;
-    }
+    const size_t P = (size_t)W * H;                    // pixels of a channel plane
     uint32_t it = 0;
     for (uint32_t tile = blockIdx.x; tile < n_tiles; tile += gridDim.x, ++it) {
       const int s = (int)(it & 1u);
@@ -512,93 +517,58 @@ __global__ void __launch_bounds__(kConvTmaThreads, 1)
         break;
       }
       fence_after();
-      // output row ry's sums sit in columns (ry + 2) * COUT of the set
+      // output row ry's sums sit in columns (ry + 2) * 32 of the set
       const uint32_t set_addr = tmem + ((uint32_t)(quarter * 32) << 16) + (uint32_t)s * Lt::kSet;
-      uint32_t r[kMine][kHalves][16];
+      uint32_t r[kMine][2][16];
 #pragma unroll
       for (int k = 0; k < kMine; ++k)
 #pragma unroll
-        for (int half = 0; half < kHalves; ++half)
-          tmem_ld16_nowait(set_addr + (uint32_t)((group + k * RT_CONV_EPI_WG + 2) * COUT + half * 16), r[k][half]);
+        for (int half = 0; half < 2; ++half)
+          tmem_ld16_nowait(set_addr + (uint32_t)((group + k * RT_CONV_EPI_WG + 2) * 32 + half * 16), r[k][half]);
       tmem_wait_ld();
 #pragma unroll
       for (int k = 0; k < kMine; ++k)
 #pragma unroll
-        for (int half = 0; half < kHalves; ++half)
-          tmem_zero16(set_addr + (uint32_t)((group + k * RT_CONV_EPI_WG + 2) * COUT + half * 16));
+        for (int half = 0; half < 2; ++half)
+          tmem_zero16(set_addr + (uint32_t)((group + k * RT_CONV_EPI_WG + 2) * 32 + half * 16));
       if (group == 0) {   // rows -2, -1, R, R+1
 #pragma unroll
-        for (int c = 0; c < 2 * COUT; c += 16) {
+        for (int c = 0; c < 64; c += 16) {
           tmem_zero16(set_addr + (uint32_t)c);
-          tmem_zero16(set_addr + (uint32_t)((kRows + 2) * COUT + c));
+          tmem_zero16(set_addr + (uint32_t)((kRows + 2) * 32 + c));
         }
       }
       tmem_wait_st();
       fence_before();
       mbar_arrive(acc_empty + s);
 
-      const uint32_t img = tile / tiles_img;
-      const uint32_t it_img = tile - img * tiles_img;
-      const int ty = (int)(it_img / tiles_x);
+      const int ty = (int)(tile / tiles_x);
       const int y = ty * kRows;
-      const int x0 = (int)(it_img - (uint32_t)ty * tiles_x) * Lt::kOutW;
+      const int x0 = (int)(tile - (uint32_t)ty * tiles_x) * Lt::kOutW;
       const int x = x0 + quarter * 32 + lane;
       const bool lane_ok = quarter * 32 + lane < Lt::kOutW;
 #pragma unroll
       for (int k = 0; k < kMine; ++k) {
         const int yy = y + group + k * RT_CONV_EPI_WG;
         if (!(lane_ok && x < (int)W && yy < (int)H)) continue;
-        const size_t p = ((size_t)img * H + yy) * W + x;
-        if (EPI == EPI_SIGMOID_F32) {
-          const float z = fmaf(__uint_as_float(r[k][0][0]), sc[0], bi[0]);
-          out32[p] = 1.f / (1.f + __expf(-z));
-        } else if (EPI == EPI_RELU_FP8) {
+        const size_t p = (size_t)yy * W + x;
 #pragma unroll
-          for (int half = 0; half < kHalves; ++half) {
-            uint32_t packed[4];
+        for (int half = 0; half < 2; ++half) {
+          // channels 16 half + 0..7 and + 8..15 sit in planes 2 half, 2 half + 1
+          const uint4 ma = *reinterpret_cast<const uint4*>(mask16 + ((2 * half) * P + p) * 8);
+          const uint4 mb = *reinterpret_cast<const uint4*>(mask16 + ((2 * half + 1) * P + p) * 8);
+          const uint32_t mw[8] = {ma.x, ma.y, ma.z, ma.w, mb.x, mb.y, mb.z, mb.w};
+          uint32_t packed[8];
 #pragma unroll
-            for (int i = 0; i < 8; ++i) {
-              const int c0 = half * 16 + 2 * i, c1 = c0 + 1;
-              const float a0 = __uint_as_float(r[k][half][2 * i]), a1 = __uint_as_float(r[k][half][2 * i + 1]);
-              const float y0 = fmaxf(fmaf(a0, sc[c0], bi[c0]), 0.f);
-              const float y1 = fmaxf(fmaf(a1, sc[c1], bi[c1]), 0.f);
-              const uint32_t q = __nv_cvt_float2_to_fp8x2(make_float2(y0, y1), __NV_SATFINITE, __NV_E4M3);
-              if (i & 1) packed[i >> 1] |= q << 16; else packed[i >> 1] = q;
-            }
-            // E4M3 planar: plane `half` holds channels 16 half .. 16 half + 15
-            *reinterpret_cast<uint4*>(static_cast<uint8_t*>(out) + (half * P + p) * 16) =
-                make_uint4(packed[0], packed[1], packed[2], packed[3]);
+          for (int i = 0; i < 8; ++i) {
+            const __nv_bfloat162 mm = *reinterpret_cast<const __nv_bfloat162*>(&mw[i]);
+            packed[i] = pack_bf16(__bfloat162float(mm.x) > 0.f ? __uint_as_float(r[k][half][2 * i]) : 0.f,
+                                  __bfloat162float(mm.y) > 0.f ? __uint_as_float(r[k][half][2 * i + 1]) : 0.f);
           }
-        } else {
-          __nv_bfloat16* out16 = static_cast<__nv_bfloat16*>(out);
-#pragma unroll
-          for (int half = 0; half < kHalves; ++half) {
-            float v[16];
-#pragma unroll
-            for (int i = 0; i < 16; ++i) v[i] = __uint_as_float(r[k][half][i]);
-            uint32_t packed[8];
-            if (EPI == EPI_RELU_BF16) {
-#pragma unroll
-              for (int i = 0; i < 8; ++i)
-                packed[i] = pack_bf16(fmaxf(v[2 * i] + bi[half * 16 + 2 * i], 0.f),
-                                      fmaxf(v[2 * i + 1] + bi[half * 16 + 2 * i + 1], 0.f));
-            } else {
-              // planar: channels 16 half + 0..7 and + 8..15 sit in planes 2 half, 2 half + 1
-              const uint4 ma = *reinterpret_cast<const uint4*>(mask16 + ((2 * half) * P + p) * 8);
-              const uint4 mb = *reinterpret_cast<const uint4*>(mask16 + ((2 * half + 1) * P + p) * 8);
-              const uint32_t mw[8] = {ma.x, ma.y, ma.z, ma.w, mb.x, mb.y, mb.z, mb.w};
-#pragma unroll
-              for (int i = 0; i < 8; ++i) {
-                const __nv_bfloat162 mm = *reinterpret_cast<const __nv_bfloat162*>(&mw[i]);
-                const float m0 = __bfloat162float(mm.x), m1 = __bfloat162float(mm.y);
-                packed[i] = pack_bf16(m0 > 0.f ? v[2 * i] : 0.f, m1 > 0.f ? v[2 * i + 1] : 0.f);
-              }
-            }
-            *reinterpret_cast<uint4*>(out16 + ((2 * half) * P + p) * 8) =
-                make_uint4(packed[0], packed[1], packed[2], packed[3]);
-            *reinterpret_cast<uint4*>(out16 + ((2 * half + 1) * P + p) * 8) =
-                make_uint4(packed[4], packed[5], packed[6], packed[7]);
-          }
+          *reinterpret_cast<uint4*>(out + ((2 * half) * P + p) * 8) =
+              make_uint4(packed[0], packed[1], packed[2], packed[3]);
+          *reinterpret_cast<uint4*>(out + ((2 * half + 1) * P + p) * 8) =
+              make_uint4(packed[4], packed[5], packed[6], packed[7]);
         }
       }
     }
@@ -609,6 +579,471 @@ __global__ void __launch_bounds__(kConvTmaThreads, 1)
   if (warp == 0) tmem_dealloc(tmem, Lt::kTmemCols);
 }
 
+// ------------------------------------------------------------ fused forward
+// The whole network in one kernel: a strip of 122 output pixels streams down
+// the image, one input row at a time, through the four layers; the
+// activations between them never leave the SM (32 bytes of features in and 4
+// of probability out per pixel, against 420 when each layer wrote its output).
+//
+// Streaming and stacked taps: input row h of a layer adds tap dy = 2 to output
+// row h - 2, dy = 1 to h - 1 and dy = 0 to h. The three rows' accumulators are
+// three 32-column TMEM slots, row r in slot r % 3, so one MMA of N = 96 per
+// kernel column and K step serves all three vertical taps, every input row is
+// read once, and no product falls outside the tile. Which tap a slot takes
+// rotates with the row: the weights of a (dx, chunk) lie in shared memory as
+// five blocks [dy 2 | 1 | 0 | 2 | 1], and the window of three blocks that
+// starts at block 2 - row % 3 has the right order. After input row h the epilogue
+// reads the finished row h - 2 and zeroes its slot, which becomes row h + 1's.
+// An MMA of N = 96 takes ~56 cycles, one of N <= 32 ~45 (measured): a row of
+// 122 pixels takes 3 (layer 1) + 6 + 6 (layers 2, 3, BF16) MMAs of N = 96.
+// Layer 4 (one output channel) puts its 9 taps along N = 16 instead: 2 MMAs a
+// row, no shift of A; its epilogue adds the three vertical taps of each kernel
+// column in registers while the rows pass and exchanges two values with the
+// neighbouring pixels: 930 cycles a row in all (BF16), 548 (E4M3 layers 2-4).
+//
+// Pixels: lane m of layer k's accumulators (k = 0 .. 3) is the image column
+// x_strip - 3 + min(k, 2) + m; each layer's output row is stored at pixel m of
+// the next one's input row (16-byte channel chunks [chunk][130 pixels]), so
+// kernel column dx is the A operand moved by dx pixels. Lanes past the strip
+// (126, 127 of layer 2, ...) hold what they hold and are never used. Outputs
+// outside the image are stored as zeros, the next layer's padding.
+//
+// Roles: per layer one thread issues the MMAs (layer 1's also loads the feature
+// rows, kFuF - 1 ahead) and one warpgroup runs the epilogue, so rows of all
+// four layers are in flight. One thread for the MMAs of all layers spent more
+// time waiting for their barriers in turn than the tensor core needs: 3490
+// cycles a row.
+// The warp of an issuing thread walks its loop as a whole and elects the thread,
+// which keeps the descriptors in uniform registers (107 -> 71 us, BF16 1080p).
+//
+// Measured: 1920x1080 0.206 -> 0.074 ms (BF16), 8 images of 3840x2160 3.185 ->
+// 1.83 ms (FP8), against one launch per layer. A BF16 row takes ~960 cycles,
+// 890 of shared-memory reads by the MMAs (4 KB of A and 3 KB of weights each,
+// at 128 bytes a cycle) and 930 of tensor issue: both are nearly full. An FP8
+// row takes as long: half the MMAs, but each layer's next row waits for the
+// epilogue's read of its accumulators (~700 cycles from MMA to MMA).
+//   full[k][d]      input row in slot d of layer k's ring has arrived (TMA
+//                   bytes for k = 0, the 4 epilogue warps of layer k - 1 else)
+//   done[k][d]      the MMAs that read it completed (commit): its slot may be
+//                   refilled, and the accumulators are up to date
+//   acc_empty[k]    layer k's epilogue has read and zeroed its slot (k < 3)
+//   acc4_empty[b]   layer 4's epilogue has read TMEM buffer b
+// Every wait is bounded, as in k_conv_tma.
+constexpr int kFuW = 122;                     // output pixels of a strip
+constexpr int kFuPx = 130;                    // pixels of a row buffer
+constexpr uint32_t kFuPitch = kFuPx * 16u;    // one chunk of a row buffer
+constexpr int kFuF = 6, kFuD = 3;             // ring depths: feature rows, activation rows
+constexpr int kFuThreads = 32 * (16 + 4);
+
+template <bool FP8>
+struct FusedLayout {
+  static constexpr int kCh = FP8 ? 2 : 4;                                  // chunks of an activation pixel
+  static constexpr uint32_t kRowF = (2 * kFuPitch + 127u) & ~127u, kRowA = kCh * kFuPitch;
+  static constexpr uint32_t kW1 = 3u * 2 * 160 * 16, kWk = 3u * kCh * 160 * 16, kW4 = kCh * 16u * 16;
+  static constexpr uint32_t kOffA = kFuF * kRowF;                          // 3 rings of kFuD rows
+  static constexpr uint32_t kOffW = kOffA + 3 * kFuD * kRowA;              // W1, W2, W3, W4
+  static constexpr uint32_t kOffC = kOffW + kW1 + 2 * kWk + kW4;           // scale[4][32], bias[4][32]
+  static constexpr uint32_t kOffX = kOffC + 2 * 4 * 32 * 4;                // layer 4's exchange, [2][2][128] floats
+  static constexpr uint32_t kOffB = kOffX + 2 * 2 * 128 * 4;               // barriers
+  static constexpr uint32_t kBars = 2 * 4 * kFuF + 3 + 3 + 1;
+  static constexpr uint32_t kSmem = kOffB + kBars * 8 + 16;
+};
+
+struct FusedArgs {
+  const void* w[4];              // packed weights (pack_weights, pack_weights_fp8)
+  const float* bias[4];
+  const float* inv[4];           // E4M3 inputs: inverse scale per output channel (null: 1)
+  float out_scale[4];            // E4M3 outputs (1 otherwise)
+  __nv_bfloat16* act[3];         // hidden activations to keep, BF16 planar [4][P][8] (null: none)
+  float* prob;
+  uint32_t W, H, n_img, strips, segs, rows;   // rows: output rows of a segment
+  uint32_t* err;
+};
+
+// a unit of work: `rows` output rows (fewer at the bottom) of one strip
+struct FusedItem {
+  int img, x0, y0, rows;         // x0: image column of layer 1's lane 0
+};
+__device__ __forceinline__ FusedItem fused_item(const FusedArgs& a, uint32_t item) {
+  const uint32_t strip = item % a.strips, q = item / a.strips, seg = q % a.segs;
+  FusedItem it;
+  it.img = (int)(q / a.segs);
+  it.x0 = (int)strip * kFuW - 3;
+  it.y0 = (int)(seg * a.rows);
+  it.rows = (int)min(a.rows, a.H - seg * a.rows);
+  return it;
+}
+
+// One row of a stacked layer: for kernel column dx and 32-byte K step, the
+// input row moved by dx pixels times the window of weight blocks at wbase.
+template <int CH, bool E4M3>
+__device__ __forceinline__ void issue_row_mmas(uint32_t abase, uint32_t wbase, uint32_t dtmem) {
+  constexpr uint32_t idesc = E4M3 ? make_idesc_e4m3(128, 96) : make_idesc(128, 96);
+  const uint32_t a_lo = desc_lo(abase, kFuPitch), b_lo = desc_lo(wbase, 160u * 16u);
+  constexpr uint32_t hi = desc_hi(128u);
+#pragma unroll
+  for (int dx = 0; dx < 3; ++dx)
+#pragma unroll
+    for (int ks = 0; ks < CH / 2; ++ks) {
+      const uint32_t a_off = 2u * ks * kFuPitch + dx * 16u, b_off = (uint32_t)(dx * CH + 2 * ks) * 160u * 16u;
+      const uint64_t da = desc_join(a_lo + (a_off >> 4), hi), db = desc_join(b_lo + (b_off >> 4), hi);
+      if (E4M3) mma_e4m3(dtmem, da, db, idesc, 1u);
+      else mma_bf16(dtmem, da, db, idesc, 1u);
+    }
+}
+
+// ring position of a layer's rows: slot and the parity of its current use
+struct Ring {
+  uint32_t slot = 0, par = 0;
+  __device__ __forceinline__ void next(uint32_t depth) {
+    if (++slot == depth) { slot = 0; par ^= 1u; }
+  }
+};
+
+// The feature rows of a CTA's items in order: one TMA box per row into the
+// ring, zeros outside the image.
+struct FeatureLoader {
+  uint32_t item, n_loaded;
+  int i;
+  FusedItem it;
+  __device__ __forceinline__ void load(const FusedArgs& a, const CUtensorMap* map, unsigned char* smem,
+                                       uint32_t row_bytes, uint64_t* full, uint32_t n_items) {
+    if (item >= n_items) return;
+    if (i == 0) it = fused_item(a, item);
+    const uint32_t d = n_loaded % kFuF;
+    if (elect_one()) {
+      mbar_arrive_expect_tx(full + d, 2 * kFuPitch);
+      tma_load_5d(smem + d * row_bytes, map, 0, it.x0 - 1, 0, it.y0 - 4 + i, it.img, full + d);
+    }
+    ++n_loaded;
+    if (++i == it.rows + 8) { i = 0; item += gridDim.x; }
+  }
+};
+
+// MMAs of layer K's rows (one thread): a row is issued once it has arrived and
+// the epilogue has read and zeroed the slot it will finish. Layer 1's thread
+// also loads the feature rows: when the epilogue has read row r - 1's sums,
+// that row's MMAs are done and its slot takes row r - 1 + kFuF.
+// KIND: 0 layer 1, 1 layers 2 and 3 (K = 1, 2), 2 layer 4.
+template <int KIND, bool FP8>
+__device__ __forceinline__ bool fused_mmas(const int K, const FusedArgs& a, const CUtensorMap* map,
+                                           unsigned char* smem, uint64_t* full, uint64_t* done,
+                                           uint64_t* empty, uint32_t tmem) {
+  using Lt = FusedLayout<FP8>;
+  const uint32_t sbase = smem_u32(smem);
+  constexpr uint32_t kDepth = KIND == 0 ? kFuF : kFuD;
+  constexpr uint32_t kRow = KIND == 0 ? Lt::kRowF : Lt::kRowA;
+  const uint32_t rows0 = sbase + (KIND == 0 ? 0u : Lt::kOffA + (uint32_t)(K - 1) * kFuD * Lt::kRowA);
+  const uint32_t w0 = sbase + Lt::kOffW + (K > 0 ? Lt::kW1 : 0u) + (K > 1 ? (uint32_t)(K - 1) * Lt::kWk : 0u);
+  const uint32_t n_items = a.strips * a.segs * a.n_img;
+  uint64_t* full_k = full + K * kFuF;
+  uint64_t* done_k = done + K * kFuF;
+  Ring ring;
+  uint32_t row3 = 0, n_row = 0;
+  bool ok = true;
+  FeatureLoader ld = {blockIdx.x, 0u, 0, {}};
+  if (KIND == 0)
+    for (int i = 0; i < kFuF - 1; ++i) ld.load(a, map, smem, Lt::kRowF, full, n_items);
+  for (uint32_t item = blockIdx.x; ok && item < n_items; item += gridDim.x) {
+    const int n = fused_item(a, item).rows + 8 - 2 * K;
+    for (int i = 0; i < n; ++i) {
+      if (KIND < 2)
+        ok = n_row == 0 ? mbar_wait(full_k + ring.slot, ring.par)
+                        : mbar_wait2<FP8>(full_k + ring.slot, ring.par, empty + K, (n_row - 1) & 1u);
+      else
+        ok = n_row < 3 ? mbar_wait(full_k + ring.slot, ring.par)
+                       : mbar_wait2<FP8>(full_k + ring.slot, ring.par, empty + row3, (n_row / 3 - 1) & 1u);
+      ok = __all_sync(0xFFFFFFFFu, ok);
+      if (!ok) break;
+      fence_after();
+      if (elect_one()) {
+        const uint32_t abase = rows0 + ring.slot * kRow;
+        if (KIND < 2) {
+          issue_row_mmas<KIND == 0 ? 2 : Lt::kCh, (KIND > 0 && FP8)>(abase, w0 + (2u - row3) * 512u, tmem + 96u * K);
+        } else {
+          constexpr uint32_t idesc = FP8 ? make_idesc_e4m3(128, 16) : make_idesc(128, 16);
+          constexpr uint32_t hi = desc_hi(128u);
+          const uint32_t a_lo = desc_lo(abase, kFuPitch), b_lo = desc_lo(w0, 256u);
+#pragma unroll
+          for (int ks = 0; ks < Lt::kCh / 2; ++ks) {
+            const uint64_t da = desc_join(a_lo + ((2u * ks * kFuPitch) >> 4), hi);
+            const uint64_t db = desc_join(b_lo + ((2u * ks * 256u) >> 4), hi);
+            if (FP8) mma_e4m3(tmem + 288u + 16u * row3, da, db, idesc, ks > 0);
+            else mma_bf16(tmem + 288u + 16u * row3, da, db, idesc, ks > 0);
+          }
+        }
+        mma_commit(done_k + ring.slot);
+      }
+      if (KIND == 0) ld.load(a, map, smem, Lt::kRowF, full, n_items);
+      __syncwarp();
+      ring.next(kDepth);
+      row3 = row3 == 2u ? 0u : row3 + 1u;
+      ++n_row;
+    }
+  }
+  // drain: the last copy into each slot has landed before the CTA exits
+  if (KIND == 0)
+    for (uint32_t j = ld.n_loaded > (uint32_t)kFuF ? ld.n_loaded - kFuF : 0; j < ld.n_loaded; ++j)
+      mbar_wait(full + j % kFuF, (j / kFuF) & 1u);
+  // drain: the last MMAs complete (and signal) before TMEM is freed
+  for (uint32_t r = n_row > kDepth ? n_row - kDepth : 0; r < n_row; ++r)
+    mbar_wait(done_k + r % kDepth, (r / kDepth) & 1u);
+  return ok;
+}
+
+// Epilogue of layers 1-3 (K = 0 .. 2): one warpgroup, lane = pixel. K is no
+// template argument: three copies of the loop, each run by one warp per
+// scheduler, kept missing the instruction cache.
+template <int KT, bool FP8, bool STORE>
+__device__ __forceinline__ bool fused_epilogue(const int KR, const FusedArgs& a, unsigned char* smem, uint64_t* full,
+                                               uint64_t* done, uint64_t* acc_empty, uint32_t tmem) {
+  using Lt = FusedLayout<FP8>;
+  const int K = KT < 0 ? KR : KT;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int quarter = warp & 3, m = quarter * 32 + lane;
+  // Biases and (E4M3 output) scales stay in registers: shared memory is what
+  // bounds this kernel, and reading them there for every pixel took 190 (BF16)
+  // to 640 (FP8) of its cycles a row.
+  const float* cst = reinterpret_cast<const float*>(smem + Lt::kOffC) + K * 32;
+  float bi[32];
+  float sc[FP8 ? 32 : 1];
+#pragma unroll
+  for (int c = 0; c < 32; ++c) bi[c] = cst[4 * 32 + c];
+  if (FP8)
+#pragma unroll
+    for (int c = 0; c < 32; ++c) sc[c % (FP8 ? 32 : 1)] = cst[c];
+  const uint32_t slots = tmem + ((uint32_t)(quarter * 32) << 16) + 96u * K;
+  unsigned char* ring = smem + Lt::kOffA + (uint32_t)K * kFuD * Lt::kRowA + (uint32_t)m * 16u;
+  const uint32_t n_items = a.strips * a.segs * a.n_img;
+  const uint32_t depth = K == 0 ? kFuF : kFuD;
+  uint64_t* full_n = full + (K + 1) * kFuF;
+  uint64_t* done_k = done + K * kFuF;
+  uint64_t* done_n = done + (K + 1) * kFuF;
+  Ring in, out;                       // rows read from this layer's ring / written to the next one's
+  bool out_wrapped = false;
+  uint32_t fin = 1;                   // slot of the finished row: (row - 2) % 3
+  for (uint32_t item = blockIdx.x; item < n_items; item += gridDim.x) {
+    const FusedItem it = fused_item(a, item);
+    const int n = it.rows + 8 - 2 * K;
+    const int x = it.x0 + K + m;
+    const bool col_in = x >= 0 && x < (int)a.W;
+    for (int i = 0; i < n; ++i) {
+      // the sums, and (from the first reuse on) the output row's slot
+      const bool ok = i >= 2 && out_wrapped ? mbar_wait2<FP8>(done_n + out.slot, out.par ^ 1u, done_k + in.slot, in.par)
+                                            : mbar_wait(done_k + in.slot, in.par);
+      if (!__all_sync(0xFFFFFFFFu, ok)) return false;
+      in.next(depth);
+      fence_after();
+      uint32_t r[2][16];
+      const uint32_t at = slots + fin * 32u;
+      tmem_ld16_nowait(at, r[0]);
+      tmem_ld16_nowait(at + 16u, r[1]);
+      tmem_wait_ld();
+      tmem_zero16(at);
+      tmem_zero16(at + 16u);
+      tmem_wait_st();
+      fence_before();
+      __syncwarp();
+      if (lane == 0) mbar_arrive(acc_empty + K);
+      fin = fin == 2u ? 0u : fin + 1u;
+      if (i < 2) continue;            // rows above the segment: never read
+      const int y = it.y0 - 3 + K + (i - 2);
+      const bool inside = col_in && y >= 0 && y < (int)a.H;
+      unsigned char* dst = ring + out.slot * Lt::kRowA;
+      uint4 v[Lt::kCh];
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+        uint32_t packed[8];
+#pragma unroll
+        for (int j = 0; j < 8; j += 2) {
+          const int c0 = h * 16 + 2 * j;
+          float y0 = __uint_as_float(r[h][2 * j]), y1 = __uint_as_float(r[h][2 * j + 1]);
+          float y2 = __uint_as_float(r[h][2 * j + 2]), y3 = __uint_as_float(r[h][2 * j + 3]);
+          if (FP8) {
+            constexpr int kS = FP8 ? 32 : 1;
+            fma2(y0, y1, sc[c0 % kS], sc[(c0 + 1) % kS], bi[c0], bi[c0 + 1]);
+            fma2(y2, y3, sc[(c0 + 2) % kS], sc[(c0 + 3) % kS], bi[c0 + 2], bi[c0 + 3]);
+            if (K == 0) { y0 = fmaxf(y0, 0.f); y1 = fmaxf(y1, 0.f); y2 = fmaxf(y2, 0.f); y3 = fmaxf(y3, 0.f); }
+            packed[j >> 1] = relu_e4m3x4(y0, y1, y2, y3);
+          } else {
+            add2(y0, y1, bi[c0], bi[c0 + 1]);
+            add2(y2, y3, bi[c0 + 2], bi[c0 + 3]);
+            packed[j] = relu_bf16(pack_bf16(y0, y1));
+            packed[j + 1] = relu_bf16(pack_bf16(y2, y3));
+          }
+        }
+        if (FP8) {
+          v[h] = make_uint4(packed[0], packed[1], packed[2], packed[3]);
+        } else {
+          v[(2 * h) % Lt::kCh] = make_uint4(packed[0], packed[1], packed[2], packed[3]);
+          v[(2 * h + 1) % Lt::kCh] = make_uint4(packed[4], packed[5], packed[6], packed[7]);
+        }
+      }
+      if (!__all_sync(0xFFFFFFFFu, inside)) {
+        if (!inside)
+#pragma unroll
+          for (int c = 0; c < Lt::kCh; ++c) v[c] = make_uint4(0u, 0u, 0u, 0u);
+      }
+#pragma unroll
+      for (int c = 0; c < Lt::kCh; ++c) *reinterpret_cast<uint4*>(dst + (uint32_t)c * kFuPitch) = v[c];
+      fence_async_smem();
+      __syncwarp();
+      if (lane == 0) mbar_arrive(full_n + out.slot);
+      out.next(kFuD);
+      if (out.slot == 0) out_wrapped = true;
+      if (STORE && !FP8) {            // the segment's own pixels: image columns x0 + 3 .. x0 + 3 + 121
+        const int own = m + K - 3;
+        if (inside && own >= 0 && own < kFuW && y >= it.y0 && y < it.y0 + it.rows) {
+          const size_t P = (size_t)a.W * a.H * a.n_img, p = ((size_t)it.img * a.H + y) * a.W + x;
+#pragma unroll
+          for (int c = 0; c < Lt::kCh; ++c) *reinterpret_cast<uint4*>(a.act[K] + ((size_t)c * P + p) * 8) = v[c];
+        }
+      }
+    }
+  }
+  return true;
+}
+
+template <bool FP8, bool STORE>
+__global__ void __launch_bounds__(kFuThreads, 1)
+    k_net_fused(const __grid_constant__ CUtensorMap tmap, const __grid_constant__ FusedArgs a) {
+  using Lt = FusedLayout<FP8>;
+  extern __shared__ __align__(1024) unsigned char smem[];
+  uint64_t* bars = reinterpret_cast<uint64_t*>(smem + Lt::kOffB);
+  uint64_t* full = bars;                         // [4][kFuF]
+  uint64_t* done = bars + 4 * kFuF;              // [4][kFuF]
+  uint64_t* acc_empty = bars + 8 * kFuF;         // [3]
+  uint64_t* acc4_empty = acc_empty + 3;          // [3]
+  uint64_t* xbar = acc4_empty + 3;               // layer 4's exchange
+  uint32_t* tslot = reinterpret_cast<uint32_t*>(xbar + 1);
+  const int tid = threadIdx.x, lane = tid & 31;
+  const int warp = __shfl_sync(0xFFFFFFFFu, tid >> 5, 0);   // known to be uniform
+  const uint32_t n_items = a.strips * a.segs * a.n_img;
+
+  // weights: three stacked blocks per (dx, chunk) become five
+  uint32_t off_w[4] = {Lt::kOffW, Lt::kOffW + Lt::kW1, Lt::kOffW + Lt::kW1 + Lt::kWk,
+                       Lt::kOffW + Lt::kW1 + 2 * Lt::kWk};
+#pragma unroll
+  for (int k = 0; k < 3; ++k) {
+    const uint32_t groups = 3u * (k == 0 ? 2u : (uint32_t)Lt::kCh);
+    const uint4* src = static_cast<const uint4*>(a.w[k]);
+    uint4* dst = reinterpret_cast<uint4*>(smem + off_w[k]);
+    for (uint32_t i = tid; i < groups * 160u; i += kFuThreads) {
+      const uint32_t g = i / 160u, r = i - g * 160u;
+      dst[i] = src[g * 96u + (r >= 96u ? r - 96u : r)];
+    }
+  }
+  for (uint32_t i = tid; i < Lt::kW4 / 16u; i += kFuThreads)
+    reinterpret_cast<uint4*>(smem + off_w[3])[i] = static_cast<const uint4*>(a.w[3])[i];
+  float* cst = reinterpret_cast<float*>(smem + Lt::kOffC);
+  for (uint32_t i = tid; i < 4u * 32u; i += kFuThreads) {
+    const uint32_t k = i / 32u, c = i % 32u;
+    const bool real = k < 3u || c == 0u;
+    // powers of two: the folded form rounds like scaling the rounded sum
+    cst[i] = real ? (a.inv[k] ? a.inv[k][c] : 1.f) * a.out_scale[k] : 0.f;
+    cst[4 * 32 + i] = real ? a.bias[k][c] * a.out_scale[k] : 0.f;
+  }
+  // the two pixels past every activation row feed unused lanes only: finite
+  for (uint32_t i = tid; i < 3u * kFuD * Lt::kRowA / 16u; i += kFuThreads)
+    reinterpret_cast<uint4*>(smem + Lt::kOffA)[i] = make_uint4(0u, 0u, 0u, 0u);
+  if (tid == 0) {
+    for (int k = 0; k < 4; ++k)
+      for (int d = 0; d < kFuF; ++d) {
+        mbar_init(full + k * kFuF + d, k == 0 ? 1 : 4);
+        mbar_init(done + k * kFuF + d, 1);
+      }
+    for (int k = 0; k < 3; ++k) {
+      mbar_init(acc_empty + k, 4);
+      mbar_init(acc4_empty + k, 4);
+    }
+    mbar_init(xbar, 4);
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&tmap)) : "memory");
+  }
+  if (warp == 0) tmem_alloc(tslot, 512);
+  fence_async_smem();
+  fence_before();
+  __syncthreads();
+  fence_after();
+  const uint32_t tmem = __shfl_sync(0xFFFFFFFFu, *tslot, 0);
+  if (warp < 4) {
+    for (uint32_t c = 0; c < 288u; c += 16) tmem_zero16(tmem + ((uint32_t)(warp * 32) << 16) + c);
+    tmem_wait_st();
+  }
+  fence_before();
+  __syncthreads();
+  fence_after();
+
+  // registers by role: 128 x (3 x 120 + 64 + 40) of the 640 x 96 launched with
+  if (warp >= 16) {
+    // ---- MMA issue, one thread per layer
+    asm volatile("setmaxnreg.dec.sync.aligned.u32 40;");
+    const bool ok = warp == 16  ? fused_mmas<0, FP8>(0, a, &tmap, smem, full, done, acc_empty, tmem)
+                    : warp < 19 ? fused_mmas<1, FP8>(warp - 16, a, &tmap, smem, full, done, acc_empty, tmem)
+                                : fused_mmas<2, FP8>(3, a, &tmap, smem, full, done, acc4_empty, tmem);
+    if (!ok && lane == 0) atomicOr(a.err, ERR_ITER);
+  } else if (warp < 12) {
+    asm volatile("setmaxnreg.inc.sync.aligned.u32 120;");
+    bool ok;
+    if (FP8)
+      ok = warp < 4   ? fused_epilogue<0, FP8, STORE>(0, a, smem, full, done, acc_empty, tmem)
+           : warp < 8 ? fused_epilogue<1, FP8, STORE>(1, a, smem, full, done, acc_empty, tmem)
+                      : fused_epilogue<2, FP8, STORE>(2, a, smem, full, done, acc_empty, tmem);
+    else
+      ok = fused_epilogue<-1, FP8, STORE>(warp >> 2, a, smem, full, done, acc_empty, tmem);
+    if (!ok && lane == 0) atomicOr(a.err, ERR_ITER);
+  } else {
+    // ---- layer 4: sums[dx] of the three vertical taps, then the neighbours'
+    asm volatile("setmaxnreg.dec.sync.aligned.u32 64;");
+    const int quarter = warp & 3, m = quarter * 32 + lane;
+    float* xs = reinterpret_cast<float*>(smem + Lt::kOffX);      // [parity][dx 0 or 2][pixel]
+    const float sc = cst[3 * 32], bi = cst[7 * 32];
+    Ring in;
+    uint32_t buf = 0, n_row = 0;
+    float s1[3] = {0.f, 0.f, 0.f}, s2[3] = {0.f, 0.f, 0.f};      // rows with one and with two taps added
+    bool ok = true;
+    for (uint32_t item = blockIdx.x; ok && item < n_items; item += gridDim.x) {
+      const FusedItem it = fused_item(a, item);
+      const int x = it.x0 + 2 + m;
+      for (int i = 0; i < it.rows + 2; ++i, ++n_row) {
+        if (!__all_sync(0xFFFFFFFFu, mbar_wait(done + 3 * kFuF + in.slot, in.par))) { ok = false; break; }
+        in.next(kFuD);
+        fence_after();
+        uint32_t r[16];
+        tmem_ld16_nowait(tmem + ((uint32_t)(quarter * 32) << 16) + 288u + 16u * buf, r);
+        tmem_wait_ld();
+        fence_before();
+        __syncwarp();
+        if (lane == 0) mbar_arrive(acc4_empty + buf);
+        buf = buf == 2u ? 0u : buf + 1u;
+        float z[3];
+#pragma unroll
+        for (int dx = 0; dx < 3; ++dx) {
+          z[dx] = s2[dx] + __uint_as_float(r[6 + dx]);
+          s2[dx] = s1[dx] + __uint_as_float(r[3 + dx]);
+          s1[dx] = __uint_as_float(r[dx]);
+        }
+        float* px = xs + (n_row & 1u) * 256u;
+        px[m] = z[0];
+        px[128 + m] = z[2];
+        __syncwarp();
+        if (lane == 0) mbar_arrive(xbar);
+        if (!__all_sync(0xFFFFFFFFu, mbar_wait(xbar, n_row & 1u))) { ok = false; break; }
+        if (i < 2) continue;
+        const int y = it.y0 + i - 2;
+        if (m >= 1 && m <= kFuW && x < (int)a.W) {
+          const float v = fmaf((px[m - 1] + z[1]) + px[128 + m + 1], sc, bi);
+          a.prob[((size_t)it.img * a.H + y) * a.W + x] = 1.f / (1.f + __expf(-v));
+        }
+      }
+    }
+    if (!ok && lane == 0) atomicOr(a.err, ERR_ITER);
+  }
+  fence_before();
+  __syncthreads();
+  fence_after();
+  if (warp == 0) tmem_dealloc(tmem, 512);
+}
 
 // ------------------------------------------------ weight packing (FP32 -> BF16)
 // Canonical parameter layout of a layer: W[Cout][Cin][3][3] then b[Cout].
@@ -662,6 +1097,24 @@ __global__ void k_pack_fwd_fp8(const float* __restrict__ Wt, int cout, int cin, 
     const StackedIndex x = stacked_index(i, 16, cout_pad, cin_pad);
     float v = 0.f;
     if (x.co < cout && x.ci < cin) v = Wt[((size_t)x.co * cin + x.ci) * 9 + x.tap] * scale[x.co];
+    out[i] = (uint8_t)__nv_cvt_float_to_fp8(v, __NV_SATFINITE, __NV_E4M3);
+  }
+}
+
+// Layer 4 of the fused forward pass: its 9 taps along N, [chunk][16][chunk
+// elements] with W[0][ci][tap] at n = tap < 9 (BF16, or E4M3 scaled like the
+// other layers), zero fill
+__global__ void k_pack_taps(const float* __restrict__ Wt, int cin, __nv_bfloat16* __restrict__ out) {
+  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < 16 * cin; i += gridDim.x * blockDim.x) {
+    const int ci = i / (16 * 8) * 8 + i % 8, n = i / 8 % 16;
+    out[i] = __float2bfloat16_rn(n < 9 ? Wt[ci * 9 + n] : 0.f);
+  }
+}
+__global__ void k_pack_taps_fp8(const float* __restrict__ Wt, int cin, const float* __restrict__ scale,
+                                uint8_t* __restrict__ out) {
+  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < 16 * cin; i += gridDim.x * blockDim.x) {
+    const int ci = i / (16 * 16) * 16 + i % 16, n = i / 16 % 16;
+    const float v = n < 9 ? Wt[ci * 9 + n] * scale[0] : 0.f;
     out[i] = (uint8_t)__nv_cvt_float_to_fp8(v, __NV_SATFINITE, __NV_E4M3);
   }
 }
@@ -773,17 +1226,6 @@ __device__ __forceinline__ void tmem_ld8_nowait(uint32_t taddr, uint32_t r[8]) {
                : "r"(taddr));
 }
 
-// (a0, a1) += (b0, b1) in one instruction, each sum rounded to nearest
-__device__ __forceinline__ void add2(float& a0, float& a1, uint32_t b0, uint32_t b1) {
-  asm("{\n\t.reg .b64 x, y;\n\t"
-      "mov.b64 x, {%0, %1};\n\t"
-      "mov.b64 y, {%2, %3};\n\t"
-      "add.rn.f32x2 x, x, y;\n\t"
-      "mov.b64 {%0, %1}, x;\n\t}"
-      : "+f"(a0), "+f"(a1)
-      : "r"(b0), "r"(b1));
-}
-
 // barriers: full[b] TMA bytes of stage b; empty[b] its MMAs (commit) and the
 // 8 epilogue warps' bias sums are done; acc_full[s] / acc_empty[s] as in
 // k_conv_tma. part: 2 gridDim.x rows of kOuts + kCo floats, [tap][co][ci]
@@ -804,7 +1246,8 @@ __global__ void __launch_bounds__(kWgThreads, 1)
   uint64_t* acc_empty = bars + 18;  // [2]
   uint32_t* tslot = reinterpret_cast<uint32_t*>(bars + 20);
 
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int tid = threadIdx.x, lane = tid & 31;
+  const int warp = __shfl_sync(0xFFFFFFFFu, tid >> 5, 0);   // known to be uniform
   const uint32_t tiles_x = (W + kWgW - 1) / kWgW;
   const uint32_t n_tiles = tiles_x * ((H + kWgRows - 1) / kWgRows);
   if (tid == 0) {
@@ -822,28 +1265,30 @@ __global__ void __launch_bounds__(kWgThreads, 1)
   fence_before();
   __syncthreads();
   fence_after();
-  const uint32_t tmem = *tslot;
+  const uint32_t tmem = __shfl_sync(0xFFFFFFFFu, *tslot, 0);
   const uint32_t my_tiles = blockIdx.x < n_tiles ? (n_tiles - 1 - blockIdx.x) / gridDim.x + 1 : 0;
 
   if (warp == kWgEpiWarps) {
-    // ---- MMA issue
-    if (lane == 0) {
-      constexpr uint32_t idesc = make_idesc_mn(128, Lt::kN);
-      // LBO: from one group of 8 pixels (K) to the next; SBO: from one
-      // (row, chunk) group of 8 channels (M or N) to the next
-      constexpr uint32_t hi_a = desc_hi(Lt::kPitchA), hi_z = desc_hi(Lt::kPitchZ);
-      uint32_t n_mma = 0, grp = 0;       // tiles and accumulator groups issued
-      bool ok = true;
-      for (uint32_t it = 0; it < my_tiles && ok; ++it) {
-        const int b = (int)(it % Lt::kSt);
-        if (!mbar_wait(full + b, (it / Lt::kSt) & 1u)) { ok = false; break; }
-        const uint32_t base = smem_u32(smem + (size_t)b * Lt::kStage);
-        const uint32_t a_lo = desc_lo(base, 128u), z_lo = desc_lo(base + Lt::kOffZ, 128u);
+    // ---- MMA issue (the whole warp walks the loop, an elected lane issues)
+    constexpr uint32_t idesc = make_idesc_mn(128, Lt::kN);
+    // LBO: from one group of 8 pixels (K) to the next; SBO: from one
+    // (row, chunk) group of 8 channels (M or N) to the next
+    constexpr uint32_t hi_a = desc_hi(Lt::kPitchA), hi_z = desc_hi(Lt::kPitchZ);
+    uint32_t n_mma = 0, grp = 0;       // tiles and accumulator groups issued
+    bool ok = true;
+    for (uint32_t it = 0; it < my_tiles && ok; ++it) {
+      const uint32_t b = it % Lt::kSt;
+      ok = __all_sync(0xFFFFFFFFu, mbar_wait(full + b, (it / Lt::kSt) & 1u));
+      if (!ok) break;
+      const uint32_t base = smem_u32(smem) + b * Lt::kStage;
+      const uint32_t a_lo = desc_lo(base, 128u), z_lo = desc_lo(base + Lt::kOffZ, 128u);
 #pragma unroll
-        for (int g = 0; g < kGroups; ++g) {
-          const uint32_t sa = grp & 1u;
-          if (grp >= 2 && !mbar_wait(acc_empty + sa, ((grp >> 1) - 1) & 1u)) { ok = false; break; }
-          fence_after();
+      for (int g = 0; g < kGroups; ++g) {
+        const uint32_t sa = grp & 1u;
+        if (grp >= 2) ok = __all_sync(0xFFFFFFFFu, mbar_wait(acc_empty + sa, ((grp >> 1) - 1) & 1u));
+        if (!ok) break;
+        fence_after();
+        if (elect_one()) {
           const int rp = g / kGroupsRow, ks0 = (g % kGroupsRow) * CHAIN;
 #pragma unroll
           for (int ks = ks0; ks < ks0 + CHAIN && ks < kWgW / 16; ++ks)
@@ -856,19 +1301,18 @@ __global__ void __launch_bounds__(kWgThreads, 1)
                        ks == ks0 ? 0u : 1u);
             }
           mma_commit(acc_full + sa);
-          ++grp;
+          if (g == kGroups - 1) mma_commit(empty + b);
         }
-        if (!ok) break;
-        mma_commit(empty + b);
-        n_mma = it + 1;
+        __syncwarp();
+        ++grp;
       }
-      if (!ok) atomicOr(err, ERR_ITER);
-      // drain: the MMAs issued here complete (and signal) before TMEM is freed
-      for (uint32_t k = grp > 2 ? grp - 2 : 0; k < grp; ++k) mbar_wait(acc_full + (k & 1u), (k >> 1) & 1u);
-      for (uint32_t it = n_mma > (uint32_t)Lt::kSt ? n_mma - Lt::kSt : 0; it < n_mma; ++it)
-        mbar_wait(empty + (it % Lt::kSt), (it / Lt::kSt) & 1u);
+      if (ok) n_mma = it + 1;
     }
-    __syncwarp();
+    if (!ok && lane == 0) atomicOr(err, ERR_ITER);
+    // drain: the MMAs issued here complete (and signal) before TMEM is freed
+    for (uint32_t k = grp > 2 ? grp - 2 : 0; k < grp; ++k) mbar_wait(acc_full + (k & 1u), (k >> 1) & 1u);
+    for (uint32_t it = n_mma > (uint32_t)Lt::kSt ? n_mma - Lt::kSt : 0; it < n_mma; ++it)
+      mbar_wait(empty + (it % Lt::kSt), (it / Lt::kSt) & 1u);
   } else if (warp == kWgEpiWarps + 1) {
     // ---- TMA loads
     if (lane == 0) {
@@ -945,7 +1389,8 @@ __global__ void __launch_bounds__(kWgThreads, 1)
               tmem_wait_ld();
 #pragma unroll
               for (int c = 0; c < kCo; c += 2)
-                add2(acc[dx][c], acc[dx][c + 1], v[c / 16][c % 16], v[c / 16][c % 16 + 1]);
+                add2(acc[dx][c], acc[dx][c + 1], __uint_as_float(v[c / 16][c % 16]),
+                     __uint_as_float(v[c / 16][c % 16 + 1]));
             }
           } else {
             uint32_t v[3][8];
@@ -1060,20 +1505,6 @@ namespace rt {
 namespace nn {
 
 namespace {
-// extra dynamic shared memory per conv CTA (bytes), from RT_CONV_SMEM_PAD:
-// lets a first run on new hardware keep every descriptor-addressed byte
-// inside the CTA's allocation even under another reading of the layout
-int conv_smem_pad() {
-  static int pad = -1;
-  if (pad < 0) {
-    const char* v = getenv("RT_CONV_SMEM_PAD");
-    pad = v ? atoi(v) : 0;
-    if (pad < 0 || pad > 160 * 1024) pad = 0;
-  }
-  return pad;
-}
-int g_conv_smem_pad = 0;
-
 // cuTensorMapEncodeTiled from the driver, looked up once through the runtime
 // (no link-time dependency on libcuda)
 using EncodeTiledFn = CUresult (*)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*,
@@ -1097,40 +1528,20 @@ EncodeTiledFn encode_tiled() {
   return fn;
 }
 
-// Tensor map of a BF16 or E4M3 map for the halo boxes of k_conv_tma.
-// Interleaved [images][H][W][C] is viewed as {chunk elements, chunks, W, H,
-// images} with one box {chunk elements, 1, 130, R+2, 1} per chunk; planar
-// [chunks][images][H][W][16 bytes] as 8-byte elements {2 W, H, images,
-// chunks} with one box {256 (128 pixels), R+2, 1, 1} per chunk.
-// A planar map may hold fewer chunks than the kernel's CIN (`chunks` > 0): the
-// boxes of the others lie outside the tensor and read zeros.
-template <int CIN, bool PLANAR, bool FP8>
-cudaError_t make_halo_map(CUtensorMap* map, const void* in, uint32_t W, uint32_t H, uint32_t n_img,
-                          uint32_t chunks) {
+// Tensor map of `chunks` BF16 chunk planes for the halo boxes of k_conv_tma:
+// 8-byte elements {2 W, H, chunks}, one box {256 (128 pixels), R+2, 1} per
+// chunk. A map may hold fewer chunks than the kernel's CIN: the boxes of the
+// others lie outside the tensor and read zeros.
+cudaError_t make_halo_map(CUtensorMap* map, const void* in, uint32_t W, uint32_t H, uint32_t chunks) {
   const EncodeTiledFn fn = encode_tiled();
   if (!fn) return cudaErrorNotSupported;
   if (reinterpret_cast<uintptr_t>(in) & 15u) return cudaErrorInvalidValue;
-  constexpr int kElem = FP8 ? 1 : 2, kPer = 16 / kElem, kChunks = CIN / kPer;
-  const cuuint64_t P = (cuuint64_t)W * H;
-  const cuuint32_t estr[5] = {1, 1, 1, 1, 1};
-  CUresult r;
-  if (PLANAR) {
-    const cuuint64_t d[4] = {2ull * W, H, n_img, chunks ? chunks : (cuuint64_t)kChunks};
-    const cuuint64_t st[3] = {(cuuint64_t)W * 16, P * 16, P * n_img * 16};
-    const cuuint32_t bx[4] = {2u * kHaloWPlanar, (cuuint32_t)(kRows + 2), 1, 1};
-    r = fn(map, CU_TENSOR_MAP_DATA_TYPE_UINT64, 4, const_cast<void*>(in), d, st, bx, estr,
-           CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
-           CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
-  } else {
-    const cuuint64_t d[5] = {kPer, kChunks, W, H, n_img};
-    const cuuint64_t st[4] = {16, (cuuint64_t)CIN * kElem, (cuuint64_t)W * CIN * kElem,
-                              P * CIN * kElem};
-    const cuuint32_t bx[5] = {kPer, 1, (cuuint32_t)kHaloW, (cuuint32_t)(kRows + 2), 1};
-    r = fn(map, FP8 ? CU_TENSOR_MAP_DATA_TYPE_UINT8 : CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 5,
-           const_cast<void*>(in), d, st, bx, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
-           CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
-           CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
-  }
+  const cuuint32_t estr[3] = {1, 1, 1};
+  const cuuint64_t d[3] = {2ull * W, H, chunks}, st[2] = {16ull * W, 16ull * W * H};
+  const cuuint32_t bx[3] = {2u * kHaloW, (cuuint32_t)(kRows + 2), 1};
+  const CUresult r = fn(map, CU_TENSOR_MAP_DATA_TYPE_UINT64, 3, const_cast<void*>(in), d, st, bx, estr,
+                        CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE,
+                        CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
   return r == CUDA_SUCCESS ? cudaSuccess : cudaErrorInvalidValue;
 }
 
@@ -1199,44 +1610,30 @@ cudaError_t launch_wgrad(const void* a, const void* dz, uint32_t W, uint32_t H, 
   return cudaGetLastError();
 }
 
-// in: BF16 interleaved [P][16] when CIN = 16, BF16 planar [4][P][8] when
-// CIN = 32 (or with PLANAR_IN), E4M3 planar [2][P][16] with IN_FP8
-template <int CIN, int COUT, int EPI, bool IN_FP8 = false, bool PLANAR_IN = IN_FP8 || CIN == 32>
-cudaError_t launch_conv(const void* in, const void* wpk, const float* bias, const float* inv,
-                        float out_scale, const __nv_bfloat16* mask16, void* out, float* out32,
-                        uint32_t W, uint32_t H, uint32_t* err, cudaStream_t st, uint32_t n_img = 1,
-                        uint32_t chunks = 0) {
-  constexpr bool kPlanarIn = PLANAR_IN;
-  using Lt = ConvTmaLayout<CIN, COUT, IN_FP8, kPlanarIn>;
-  const uint32_t tiles = ((W + Lt::kOutW - 1) / Lt::kOutW) * ((H + kRows - 1) / kRows) * n_img;
-  size_t smem = Lt::kSmem + (size_t)(g_conv_smem_pad + conv_smem_pad());
+// data gradient of a layer: `in` holds `chunks` planes (CIN / 8 at most)
+template <int CIN>
+cudaError_t launch_conv(const void* in, uint32_t chunks, const void* wpk, const __nv_bfloat16* mask16,
+                        __nv_bfloat16* out, uint32_t W, uint32_t H, uint32_t* err, cudaStream_t st) {
+  using Lt = ConvTmaLayout<CIN>;
+  const uint32_t tiles = ((W + Lt::kOutW - 1) / Lt::kOutW) * ((H + kRows - 1) / kRows);
   // a CTA that takes all 512 TMEM columns must be alone on its SM: ask for
   // more than half of the SM's shared memory so a second one cannot be placed
-  if (Lt::kTmemCols == 512 && smem < 116u * 1024u) smem = 116u * 1024u;
-  static size_t configured = 0;
-  if (configured < smem) {
-    cudaError_t e = cudaFuncSetAttribute(k_conv_tma<CIN, COUT, EPI, kPlanarIn, IN_FP8>,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  constexpr size_t smem = Lt::kSmem < 116u * 1024u ? 116u * 1024u : Lt::kSmem;
+  static bool configured = false;
+  if (!configured) {
+    const cudaError_t e = cudaFuncSetAttribute(k_conv_tma<CIN>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                               (int)smem);
     if (e != cudaSuccess) return e;
-    configured = smem;
+    configured = true;
   }
   CUtensorMap map;
-  cudaError_t e = make_halo_map<CIN, kPlanarIn, IN_FP8>(&map, in, W, H, n_img, chunks);
+  const cudaError_t e = make_halo_map(&map, in, W, H, chunks);
   if (e != cudaSuccess) return e;
-  // resident CTAs per SM from the shared-memory footprint (227 KB usable,
-  // 1 KB reserved per CTA) and the TMEM columns (512 per SM) each CTA takes
-  int per_sm = (int)((227u * 1024u) / (smem + 1024u));
-  if (per_sm > (int)(512 / Lt::kTmemCols)) per_sm = (int)(512 / Lt::kTmemCols);
-  if (per_sm < 1) per_sm = 1;
-  uint32_t grid = (uint32_t)(num_sms() * per_sm);
-  if (grid > tiles) grid = tiles;
-  k_conv_tma<CIN, COUT, EPI, kPlanarIn, IN_FP8><<<grid, kConvTmaThreads, smem, st>>>(
-      map, wpk, bias, inv, out_scale, mask16, out, out32, W, H, n_img, err);
+  const uint32_t grid = std::min<uint32_t>((uint32_t)num_sms(), tiles);
+  k_conv_tma<CIN><<<grid, kConvTmaThreads, smem, st>>>(map, wpk, mask16, out, W, H, err);
   return cudaGetLastError();
 }
 }  // namespace
-
-void set_conv_smem_pad(int bytes) { g_conv_smem_pad = bytes; }
 
 // parameter offsets (canonical layout W[Cout][Cin][3][3], b[Cout] per layer)
 constexpr uint32_t kOffW[4] = {0, 2912, 12160, 21408};
@@ -1246,64 +1643,119 @@ constexpr int kCin[4] = {10, 32, 32, 32};
 constexpr int kCinPad[4] = {16, 32, 32, 32};
 constexpr int kCoutPad[4] = {32, 32, 32, 16};
 
-size_t packed_fwd_elems(int l) { return 9ull * kCinPad[l] * kCoutPad[l]; }
+// layers 1-3 stacked for the fused forward pass, layer 4 taps along N
+size_t packed_fwd_elems(int l) { return l == 3 ? 16ull * kCinPad[l] : 9ull * kCinPad[l] * kCoutPad[l]; }
 size_t packed_bwd_elems(int l) { return 9ull * kCoutPad[l] * kCinPad[l]; }
 
 cudaError_t pack_weights(const float* params, __nv_bfloat16* const wf[4], __nv_bfloat16* const wb[4],
                          cudaStream_t st) {
   for (int l = 0; l < 4; ++l) {
-    k_pack_fwd<<<64, 256, 0, st>>>(params + kOffW[l], kCout[l], kCin[l], kCoutPad[l], kCinPad[l], wf[l]);
+    if (l < 3)
+      k_pack_fwd<<<64, 256, 0, st>>>(params + kOffW[l], kCout[l], kCin[l], kCoutPad[l], kCinPad[l], wf[l]);
+    else
+      k_pack_taps<<<2, 256, 0, st>>>(params + kOffW[l], kCin[l], wf[l]);
     if (l > 0 && wb[l])
       k_pack_bwd<<<64, 256, 0, st>>>(params + kOffW[l], kCout[l], kCin[l], kCoutPad[l], kCinPad[l], wb[l]);
   }
   return cudaGetLastError();
 }
 
+namespace {
+// feature maps [n_img][H][W][16] BF16 as {8 channels, W, chunks, H, images}:
+// one box is one row of a strip, in shared memory [chunk][130 pixels]
+cudaError_t make_feature_map(CUtensorMap* map, const void* in, uint32_t W, uint32_t H, uint32_t n_img) {
+  const EncodeTiledFn fn = encode_tiled();
+  if (!fn) return cudaErrorNotSupported;
+  if (reinterpret_cast<uintptr_t>(in) & 15u) return cudaErrorInvalidValue;
+  const cuuint32_t estr[5] = {1, 1, 1, 1, 1};
+  const cuuint64_t d[5] = {8, W, 2, H, n_img}, st[4] = {32, 16, 32ull * W, 32ull * W * H};
+  const cuuint32_t bx[5] = {8, (cuuint32_t)kFuPx, 2, 1, 1};
+  const CUresult r = fn(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 5, const_cast<void*>(in), d, st, bx, estr,
+                        CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE,
+                        CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+  return r == CUDA_SUCCESS ? cudaSuccess : cudaErrorInvalidValue;
+}
+
+template <bool FP8, bool STORE>
+cudaError_t launch_fused(const __nv_bfloat16* feat16, FusedArgs& a, uint32_t W, uint32_t H,
+                         uint32_t n_img, cudaStream_t st) {
+  using Lt = FusedLayout<FP8>;
+  // a CTA takes all TMEM columns: more than half of an SM's shared memory, so
+  // that no second one can be placed beside it
+  constexpr uint32_t smem = Lt::kSmem < 116u * 1024u ? 116u * 1024u : Lt::kSmem;
+  static bool configured = false;
+  if (!configured) {
+    const cudaError_t e = cudaFuncSetAttribute(k_net_fused<FP8, STORE>,
+                                               cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e != cudaSuccess) return e;
+    configured = true;
+  }
+  CUtensorMap map;
+  const cudaError_t e = make_feature_map(&map, feat16, W, H, n_img);
+  if (e != cudaSuccess) return e;
+  // Segments per strip: a segment of R rows costs R + 8 steps (the rows above
+  // and below it that its first layers recompute), and the CTAs take the
+  // segments in whole rounds, so the fewest steps over all rounds.
+  a.W = W; a.H = H; a.n_img = n_img;
+  a.strips = (W + kFuW - 1) / kFuW;
+  uint64_t best = ~0ull;
+  const uint64_t strips = (uint64_t)a.strips * n_img, sms = (uint64_t)num_sms();
+  for (uint32_t rows = H;;) {
+    const uint32_t segs = (H + rows - 1) / rows;
+    const uint64_t cost = (strips * segs + sms - 1) / sms * (rows + 8u);
+    if (cost < best) { best = cost; a.segs = segs; a.rows = rows; }
+    if (rows == 1) break;
+    rows = std::min(rows - 1, (H + segs) / (segs + 1));   // one more segment, shorter by a row at least
+  }
+  const uint64_t items = strips * a.segs;
+  k_net_fused<FP8, STORE><<<(int)std::min(items, sms), kFuThreads, smem, st>>>(map, a);
+  return cudaGetLastError();
+}
+}  // namespace
+
 cudaError_t forward(const __nv_bfloat16* feat16, const float* params, __nv_bfloat16* const wf[4],
-                    __nv_bfloat16* act1, __nv_bfloat16* act2, __nv_bfloat16* act3, float* prob,
-                    uint32_t W, uint32_t H, uint32_t* err, cudaStream_t st, uint32_t n_img) {
-  cudaError_t e;
-  e = launch_conv<16, 32, EPI_RELU_BF16>(feat16, wf[0], params + kOffB[0], nullptr, 1.f, nullptr, act1,
-                                         nullptr, W, H, err, st, n_img);
-  if (e != cudaSuccess) return e;
-  e = launch_conv<32, 32, EPI_RELU_BF16>(act1, wf[1], params + kOffB[1], nullptr, 1.f, nullptr, act2,
-                                         nullptr, W, H, err, st, n_img);
-  if (e != cudaSuccess) return e;
-  e = launch_conv<32, 32, EPI_RELU_BF16>(act2, wf[2], params + kOffB[2], nullptr, 1.f, nullptr, act3,
-                                         nullptr, W, H, err, st, n_img);
-  if (e != cudaSuccess) return e;
-  return launch_conv<32, 16, EPI_SIGMOID_F32>(act3, wf[3], params + kOffB[3], nullptr, 1.f, nullptr,
-                                             nullptr, prob, W, H, err, st, n_img);
+                    __nv_bfloat16* const act[3], float* prob, uint32_t W, uint32_t H, uint32_t* err,
+                    cudaStream_t st, uint32_t n_img) {
+  FusedArgs a = {};
+  for (int l = 0; l < 4; ++l) {
+    a.w[l] = wf[l];
+    a.bias[l] = params + kOffB[l];
+    a.out_scale[l] = 1.f;
+  }
+  a.prob = prob;
+  a.err = err;
+  if (!act) return launch_fused<false, false>(feat16, a, W, H, n_img, st);
+  for (int l = 0; l < 3; ++l) a.act[l] = act[l];
+  return launch_fused<false, true>(feat16, a, W, H, n_img, st);
 }
 
 cudaError_t pack_weights_fp8(const float* params, const float* const scale[3], uint8_t* const w8[3],
                              cudaStream_t st) {
-  for (int l = 1; l < 4; ++l)
+  for (int l = 1; l < 3; ++l)
     k_pack_fwd_fp8<<<64, 256, 0, st>>>(params + kOffW[l], kCout[l], kCin[l], kCoutPad[l], kCinPad[l],
                                        scale[l - 1], w8[l - 1]);
+  k_pack_taps_fp8<<<2, 256, 0, st>>>(params + kOffW[3], kCin[3], scale[2], w8[2]);
   return cudaGetLastError();
 }
 
-size_t packed_fp8_bytes(int l) { return 9ull * kCinPad[l] * kCoutPad[l]; }
+size_t packed_fp8_bytes(int l) { return packed_fwd_elems(l); }
 
 // the FP8 network: layer 1 in BF16 with E4M3 output, layers 2-4 on E4M3
-// operands (kind::f8f6f4); act8 buffers hold E4M3 planar [2][P][16]
+// operands (kind::f8f6f4)
 cudaError_t forward_fp8(const __nv_bfloat16* feat16, const float* params, __nv_bfloat16* const wf[4],
                         uint8_t* const w8[3], const float* const inv[3], const float act_scale[3],
-                        uint8_t* act8_1, uint8_t* act8_2, uint8_t* act8_3, float* prob, uint32_t W,
-                        uint32_t H, uint32_t* err, cudaStream_t st, uint32_t n_img) {
-  cudaError_t e;
-  e = launch_conv<16, 32, EPI_RELU_FP8>(feat16, wf[0], params + kOffB[0], nullptr, act_scale[0], nullptr,
-                                        act8_1, nullptr, W, H, err, st, n_img);
-  if (e != cudaSuccess) return e;
-  e = launch_conv<32, 32, EPI_RELU_FP8, true>(act8_1, w8[0], params + kOffB[1], inv[0], act_scale[1],
-                                              nullptr, act8_2, nullptr, W, H, err, st, n_img);
-  if (e != cudaSuccess) return e;
-  e = launch_conv<32, 32, EPI_RELU_FP8, true>(act8_2, w8[1], params + kOffB[2], inv[1], act_scale[2],
-                                              nullptr, act8_3, nullptr, W, H, err, st, n_img);
-  if (e != cudaSuccess) return e;
-  return launch_conv<32, 16, EPI_SIGMOID_F32, true>(act8_3, w8[2], params + kOffB[3], inv[2], 1.f, nullptr,
-                                                    nullptr, prob, W, H, err, st, n_img);
+                        float* prob, uint32_t W, uint32_t H, uint32_t* err, cudaStream_t st,
+                        uint32_t n_img) {
+  FusedArgs a = {};
+  for (int l = 0; l < 4; ++l) {
+    a.w[l] = l == 0 ? static_cast<const void*>(wf[0]) : w8[l - 1];
+    a.bias[l] = params + kOffB[l];
+    a.inv[l] = l == 0 ? nullptr : inv[l - 1];
+    a.out_scale[l] = l < 3 ? act_scale[l] : 1.f;
+  }
+  a.prob = prob;
+  a.err = err;
+  return launch_fused<true, false>(feat16, a, W, H, n_img, st);
 }
 
 // raises amax3[l] to the largest value of hidden activation l (the caller
@@ -1328,20 +1780,17 @@ cudaError_t backward(const __nv_bfloat16* feat16, const float* label, __nv_bfloa
   // layer 4: dW from the three parts of g, data gradient into dz_a (masked by act3 > 0)
   cudaError_t e = launch_wgrad<4, 1>(act3, g8, W, H, kCin[3], scale, wpart, grads + kOffW[3], err, st);
   if (e != cudaSuccess) return e;
-  e = launch_conv<16, 32, EPI_BWD_MASK_BF16, false, true>(g8, wb[3], nullptr, nullptr, 1.f, act3, dz_a,
-                                                          nullptr, W, H, err, st, 1, 1);
+  e = launch_conv<16>(g8, 1, wb[3], act3, dz_a, W, H, err, st);
   if (e != cudaSuccess) return e;
   // layer 3
   e = launch_wgrad<4, 4>(act2, dz_a, W, H, kCin[2], scale, wpart, grads + kOffW[2], err, st);
   if (e != cudaSuccess) return e;
-  e = launch_conv<32, 32, EPI_BWD_MASK_BF16>(dz_a, wb[2], nullptr, nullptr, 1.f, act2, dz_b, nullptr,
-                                             W, H, err, st);
+  e = launch_conv<32>(dz_a, 4, wb[2], act2, dz_b, W, H, err, st);
   if (e != cudaSuccess) return e;
   // layer 2
   e = launch_wgrad<4, 4>(act1, dz_b, W, H, kCin[1], scale, wpart, grads + kOffW[1], err, st);
   if (e != cudaSuccess) return e;
-  e = launch_conv<32, 32, EPI_BWD_MASK_BF16>(dz_b, wb[1], nullptr, nullptr, 1.f, act1, dz_a, nullptr,
-                                             W, H, err, st);
+  e = launch_conv<32>(dz_b, 4, wb[1], act1, dz_a, W, H, err, st);
   if (e != cudaSuccess) return e;
   // layer 1 (no data gradient for the input features)
   return launch_wgrad<2, 4>(feat16, dz_a, W, H, kCin[0], scale, wpart, grads + kOffW[0], err, st);

@@ -53,17 +53,16 @@ namespace {
 size_t a256(size_t b) { return (b + 255) & ~size_t(255); }
 
 // the network's forward pass in the precision it is set to (BF16, or FP8
-// after rt_net_set_fp8); act: three scratch maps of W*H*32 BF16 each
-cudaError_t net_forward(rt_net* net, const __nv_bfloat16* feat16, __nv_bfloat16* const act[3],
-                        float* prob, uint32_t W, uint32_t H, cudaStream_t st, uint32_t n_img = 1) {
+// after rt_net_set_fp8); it needs no buffers of its own
+cudaError_t net_forward(rt_net* net, const __nv_bfloat16* feat16, float* prob, uint32_t W, uint32_t H,
+                        cudaStream_t st, uint32_t n_img = 1) {
   if (!net->fp8)
-    return rt::nn::forward(feat16, net->params, net->wf, act[0], act[1], act[2], prob, W, H, net->err, st,
-                           n_img);
-  return rt::nn::forward_fp8(feat16, net->params, net->wf, net->w8, net->inv, net->act_scale,
-                             reinterpret_cast<uint8_t*>(act[0]), reinterpret_cast<uint8_t*>(act[1]),
-                             reinterpret_cast<uint8_t*>(act[2]), prob, W, H, net->err, st, n_img);
+    return rt::nn::forward(feat16, net->params, net->wf, nullptr, prob, W, H, net->err, st, n_img);
+  return rt::nn::forward_fp8(feat16, net->params, net->wf, net->w8, net->inv, net->act_scale, prob, W, H,
+                             net->err, st, n_img);
 }
 
+// training and calibration scratch for maps of P pixels
 int net_buffers(rt_net* net, uint64_t P) {
   if (net->tb && net->tcap >= P) return RT_OK;
   const size_t b_act = a256(P * 32 * 2), b_prob = a256(P * 4), b_g8 = a256(P * 8 * 2),
@@ -88,8 +87,8 @@ int reproj_buffers(const rt_scene* sc_c, uint64_t P) {
   rt::ReprojBuffers& rp = sc->ws.rp;
   if (rp.base && rp.cap >= P) return RT_OK;
   const size_t b4 = a256(P * 4), b12 = a256(P * 12), b8 = a256(P * 8), b1 = a256(P),
-               bf = a256(P * 16 * 2), bact = a256(P * 32 * 2);
-  const size_t total = b4 + b12 + b4 + b4 + b8 + bf + b1 + b12 + b1 + b4 + 256 + b4 + 3 * bact;
+               bf = a256(P * 16 * 2);
+  const size_t total = b4 + b12 + b4 + b4 + b8 + bf + b1 + b12 + b1 + b4 + 256 + b4;
   void* base = nullptr;
   cudaError_t e = cudaMalloc(&base, total);
   if (e != cudaSuccess) { cudaGetLastError(); return cuda_fail(e, "reprojection buffers"); }
@@ -108,8 +107,7 @@ int reproj_buffers(const rt_scene* sc_c, uint64_t P) {
   rp.mask = reinterpret_cast<uint8_t*>(p); p += b1;
   rp.plist = reinterpret_cast<uint32_t*>(p); p += b4;
   rp.count = reinterpret_cast<uint32_t*>(p); p += 256;
-  rp.prob = reinterpret_cast<float*>(p); p += b4;
-  for (int i = 0; i < 3; ++i) { rp.act[i] = reinterpret_cast<__nv_bfloat16*>(p); p += bact; }
+  rp.prob = reinterpret_cast<float*>(p);
   return RT_OK;
 }
 
@@ -279,7 +277,7 @@ int rt_net_activation_amax(rt_net* net, const uint16_t* d_feat16, uint32_t W, ui
   cudaError_t e = cudaMemsetAsync(net->amax, 0, 3 * sizeof(unsigned), st);
   if (e == cudaSuccess)
     e = rt::nn::forward(reinterpret_cast<const __nv_bfloat16*>(d_feat16), net->params, net->wf,
-                        net->act[0], net->act[1], net->act[2], net->prob, W, H, net->err, st);
+                        net->act, net->prob, W, H, net->err, st);
   if (e == cudaSuccess) e = rt::nn::activation_amax(net->act, (uint64_t)W * H, net->amax, st);
   unsigned bits[3] = {0, 0, 0};
   if (e == cudaSuccess) e = cudaMemcpyAsync(bits, net->amax, sizeof bits, cudaMemcpyDeviceToHost, st);
@@ -302,7 +300,7 @@ int rt_net_calibrate_fp8(rt_net* net, const uint16_t* const* d_feats, uint32_t n
   cudaError_t e = cudaMemsetAsync(net->amax, 0, 3 * sizeof(unsigned), st);
   for (uint32_t i = 0; i < n_maps && e == cudaSuccess; ++i) {
     e = rt::nn::forward(reinterpret_cast<const __nv_bfloat16*>(d_feats[i]), net->params, net->wf,
-                        net->act[0], net->act[1], net->act[2], net->prob, W, H, net->err, st);
+                        net->act, net->prob, W, H, net->err, st);
     if (e == cudaSuccess) e = rt::nn::activation_amax(net->act, (uint64_t)W * H, net->amax, st);
   }
   unsigned bits[3] = {0, 0, 0};
@@ -389,10 +387,8 @@ int rt_net_forward(rt_net* net, const uint16_t* d_feat16, uint32_t W, uint32_t H
                    void* cuda_stream) {
   if (!net || !d_feat16 || !d_prob || W < 1 || H < 1) return fail(RT_ERR_INVALID_ARG, "bad argument");
   if ((uint64_t)W * H > (1ull << 30)) return fail(RT_ERR_INVALID_ARG, "image too large");
-  int rc = net_buffers(net, (uint64_t)W * H);
-  if (rc) return rc;
-  cudaError_t e = net_forward(net, reinterpret_cast<const __nv_bfloat16*>(d_feat16), net->act, d_prob,
-                              W, H, static_cast<cudaStream_t>(cuda_stream));
+  cudaError_t e = net_forward(net, reinterpret_cast<const __nv_bfloat16*>(d_feat16), d_prob, W, H,
+                              static_cast<cudaStream_t>(cuda_stream));
   if (e != cudaSuccess) return cuda_fail(e, "network forward");
   return RT_OK;
 }
@@ -401,10 +397,8 @@ int rt_net_forward_images(rt_net* net, const uint16_t* d_feat16, uint32_t n_img,
                           float* d_prob, void* cuda_stream) {
   if (!net || !d_feat16 || !d_prob || n_img < 1 || W < 1 || H < 1) return fail(RT_ERR_INVALID_ARG, "bad argument");
   if ((uint64_t)W * H * n_img > (1ull << 30)) return fail(RT_ERR_INVALID_ARG, "images too large");
-  int rc = net_buffers(net, (uint64_t)W * H * n_img);
-  if (rc) return rc;
-  cudaError_t e = net_forward(net, reinterpret_cast<const __nv_bfloat16*>(d_feat16), net->act, d_prob,
-                              W, H, static_cast<cudaStream_t>(cuda_stream), n_img);
+  cudaError_t e = net_forward(net, reinterpret_cast<const __nv_bfloat16*>(d_feat16), d_prob, W, H,
+                              static_cast<cudaStream_t>(cuda_stream), n_img);
   if (e != cudaSuccess) return cuda_fail(e, "network forward (images)");
   return RT_OK;
 }
@@ -419,8 +413,8 @@ int rt_net_train_step(rt_net* net, const uint16_t* d_feat16, const float* d_labe
   if (rc) return rc;
   cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
   const __nv_bfloat16* f16 = reinterpret_cast<const __nv_bfloat16*>(d_feat16);
-  cudaError_t e = rt::nn::forward(f16, net->params, net->wf, net->act[0], net->act[1], net->act[2],
-                                  net->prob, W, H, net->err, st);
+  cudaError_t e = rt::nn::forward(f16, net->params, net->wf, net->act, net->prob, W, H, net->err,
+                                  st);
   if (e == cudaSuccess)
     e = rt::nn::backward(f16, d_label, net->wb, net->act[0], net->act[1], net->act[2], net->prob,
                          net->g8, net->dz[0], net->dz[1], net->wpart, net->grads,
@@ -499,7 +493,6 @@ int rt_render_stereo_reproj(const rt_scene* scene, const rt_camera* cam, float e
   const uint64_t P = (uint64_t)W * H;
   rc = rt::ensure_workspace(scene, W, H);
   if (!rc) rc = reproj_buffers(scene, P);
-  if (!rc && net) rc = net_buffers(net, P);
   if (rc) return rc;
   rt_scene* sc = const_cast<rt_scene*>(scene);
   rt::ReprojBuffers& rp = sc->ws.rp;
@@ -518,7 +511,7 @@ int rt_render_stereo_reproj(const rt_scene* scene, const rt_camera* cam, float e
   rt::profile_mark(sc->ws, rt::ST_WARP, st);
   // 3. retrace probability
   if (e == cudaSuccess && net) {
-    e = net_forward(net, rp.feat16, rp.act, rp.prob, W, H, st);
+    e = net_forward(net, rp.feat16, rp.prob, W, H, st);
     rt::profile_mark(sc->ws, rt::ST_NET, st);
   }
   // 4. mask = hole, reflective source, or p > threshold, compacted
@@ -575,7 +568,6 @@ int rt_render_stereo_reproj_frames(const rt_scene* scene, const rt_camera* cams,
   }
   rc = rt::ensure_workspace(scene, W, H * n_frames);
   if (!rc) rc = reproj_buffers(scene, FP);
-  if (!rc && net) rc = net_buffers(net, FP);
   if (rc) return rc;
   rt_scene* sc = const_cast<rt_scene*>(scene);
   rt::ReprojBuffers& rp = sc->ws.rp;
@@ -598,7 +590,7 @@ int rt_render_stereo_reproj_frames(const rt_scene* scene, const rt_camera* cams,
   // 3. the network over all frames, one launch per layer (a 3x3 window never
   //    crosses from one frame into the next)
   if (e == cudaSuccess && net) {
-    e = net_forward(net, rp.feat16, rp.act, rp.prob, W, H, st, n_frames);
+    e = net_forward(net, rp.feat16, rp.prob, W, H, st, n_frames);
     rt::profile_mark(sc->ws, rt::ST_NET, st);
   }
   // 4. mask over every right pixel of every frame, compacted into one list

@@ -91,7 +91,6 @@ struct ReprojBuffers {
   uint32_t* plist = nullptr;     // masked pixels (global indices)
   uint32_t* count = nullptr;     // number of masked pixels
   float* prob = nullptr;         // network output
-  __nv_bfloat16* act[3] = {nullptr, nullptr, nullptr};  // hidden activations (32 channels)
 };
 
 // scratch of one render (scene-owned, grown on demand)
@@ -215,16 +214,16 @@ cudaError_t reproj_compose(const uint8_t* mask, const uint32_t* accum_R, const f
 // retrace network (nn.cu)
 namespace nn {
 constexpr uint32_t kParams = 21697;
-void set_conv_smem_pad(int bytes);
 size_t packed_fwd_elems(int l);
 size_t packed_bwd_elems(int l);
 cudaError_t pack_weights(const float* params, __nv_bfloat16* const wf[4], __nv_bfloat16* const wb[4],
                          cudaStream_t st);
 // forward / forward_fp8: n_img feature maps of W x H pixels each, stacked
-// image after image (one launch per layer for all of them)
+// image after image, in one launch; act (or null): BF16 planar maps that
+// receive the three hidden activations
 cudaError_t forward(const __nv_bfloat16* feat16, const float* params, __nv_bfloat16* const wf[4],
-                    __nv_bfloat16* act1, __nv_bfloat16* act2, __nv_bfloat16* act3, float* prob,
-                    uint32_t W, uint32_t H, uint32_t* err, cudaStream_t st, uint32_t n_img = 1);
+                    __nv_bfloat16* const act[3], float* prob, uint32_t W, uint32_t H, uint32_t* err,
+                    cudaStream_t st, uint32_t n_img = 1);
 cudaError_t backward(const __nv_bfloat16* feat16, const float* label, __nv_bfloat16* const wb[4],
                      const __nv_bfloat16* act1, const __nv_bfloat16* act2,
                      const __nv_bfloat16* act3, const float* prob, __nv_bfloat16* g8,
@@ -240,8 +239,8 @@ cudaError_t pack_weights_fp8(const float* params, const float* const scale[3], u
                              cudaStream_t st);
 cudaError_t forward_fp8(const __nv_bfloat16* feat16, const float* params, __nv_bfloat16* const wf[4],
                         uint8_t* const w8[3], const float* const inv[3], const float act_scale[3],
-                        uint8_t* act8_1, uint8_t* act8_2, uint8_t* act8_3, float* prob, uint32_t W,
-                        uint32_t H, uint32_t* err, cudaStream_t st, uint32_t n_img = 1);
+                        float* prob, uint32_t W, uint32_t H, uint32_t* err, cudaStream_t st,
+                        uint32_t n_img = 1);
 cudaError_t activation_amax(const __nv_bfloat16* const act[3], uint64_t P, unsigned* amax3,
                             cudaStream_t st);
 }  // namespace nn
