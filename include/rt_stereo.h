@@ -306,8 +306,9 @@ int rt_debug_set_pool_capacity(rt_scene* scene, uint32_t entries);
  * tree in use (the SAH tree for RT_TREE_WIDE). The 4-wide tree is built the
  * first time it is chosen (synchronous: the device is synchronised and a
  * scratch buffer of ~21 bytes per primitive is allocated and freed; errors
- * RT_ERR_CUDA); choosing a tree is otherwise host-only and takes effect with
- * the next render. Other values: RT_ERR_INVALID_ARG.
+ * RT_ERR_CUDA); choosing the LBVH for the first time converts its nodes to the
+ * form renders walk (synchronous too, no allocation); choosing a tree is
+ * otherwise host-only and takes effect with the next render. Other values: RT_ERR_INVALID_ARG.
  */
 #define RT_TREE_SAH 0
 #define RT_TREE_WIDE 1

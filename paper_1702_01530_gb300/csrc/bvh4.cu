@@ -9,10 +9,12 @@
 // memory; the rest follow in binary-tree index order. The binary tree's root
 // is node 0 and `parent` gives the parent of each inner node.
 //
-// Node layout (7 x float4 = 112 B): lo.x[4], hi.x[4], lo.y[4], hi.y[4],
-// lo.z[4], hi.z[4], child[4] (int bits: >= 0 4-wide node, < 0 leaf ~k).
+// The binary tree is given by its render nodes: boxes as centre and half extent,
+// which the 4-wide nodes keep, so that both walks take the same leaves.
+// Node layout (7 x float4 = 112 B): c.x[4], e.x[4], c.y[4], e.y[4], c.z[4],
+// e.z[4], child[4] (int bits: >= 0 4-wide node, < 0 leaf ~k).
 // An unused slot holds child kEmptyChild (never visited: the traversal masks
-// it) and the point box (+inf, +inf, +inf).
+// it) and an empty box (extent -inf).
 #include <cuda_runtime.h>
 #include <stdint.h>
 
@@ -35,13 +37,13 @@ __global__ void k_depth_flags(const int32_t* __restrict__ parent, uint32_t n_inn
   depth_out[i] = (uint8_t)(d < 255 ? d : 255);
 }
 
-__device__ __forceinline__ void child_box(const float4* nodes, int32_t node, int slot, float lo[3],
-                                          float hi[3]) {
+__device__ __forceinline__ void child_box(const float4* nodes, int32_t node, int slot, float ctr[3],
+                                          float ext[3]) {
   const float4 a = nodes[4 * (size_t)node + (slot ? 1 : 0)];
   const float4 c = nodes[4 * (size_t)node + 2];
-  lo[0] = a.x; hi[0] = a.y; lo[1] = a.z; hi[1] = a.w;
-  lo[2] = slot ? c.z : c.x;
-  hi[2] = slot ? c.w : c.y;
+  ctr[0] = a.x; ext[0] = a.z; ctr[1] = a.y; ext[1] = a.w;
+  ctr[2] = slot ? c.z : c.x;
+  ext[2] = slot ? c.w : c.y;
 }
 
 __global__ void k_build4(const float4* __restrict__ nodes, uint32_t n_inner,
@@ -59,7 +61,7 @@ __global__ void k_build4(const float4* __restrict__ nodes, uint32_t n_inner,
   auto idx4 = [&](int32_t g) -> int32_t {
     return (int32_t)(flag_top[g] ? scan_top[g] : n_top + scan_rest[g]);
   };
-  float lo[3][4], hi[3][4];
+  float ctr[3][4], ext[3][4];
   int32_t ch[4] = {0, 0, 0, 0};
   int slot = 0;
   const float4 ci = nodes[4 * (size_t)i + 3];
@@ -69,29 +71,29 @@ __global__ void k_build4(const float4* __restrict__ nodes, uint32_t n_inner,
     float l[3], h[3];
     if (c < 0) {
       child_box(nodes, (int32_t)i, s, l, h);
-      for (int a = 0; a < 3; ++a) { lo[a][slot] = l[a]; hi[a][slot] = h[a]; }
+      for (int a = 0; a < 3; ++a) { ctr[a][slot] = l[a]; ext[a][slot] = h[a]; }
       ch[slot++] = c;
     } else {
       const float4 cc = nodes[4 * (size_t)c + 3];
       const int32_t gk[2] = {__float_as_int(cc.x), __float_as_int(cc.y)};
       for (int s2 = 0; s2 < 2; ++s2) {
         child_box(nodes, c, s2, l, h);
-        for (int a = 0; a < 3; ++a) { lo[a][slot] = l[a]; hi[a][slot] = h[a]; }
+        for (int a = 0; a < 3; ++a) { ctr[a][slot] = l[a]; ext[a][slot] = h[a]; }
         ch[slot++] = gk[s2] < 0 ? gk[s2] : idx4(gk[s2]);
       }
     }
   }
   for (; slot < 4; ++slot) {
-    for (int a = 0; a < 3; ++a) { lo[a][slot] = INFINITY; hi[a][slot] = INFINITY; }
+    for (int a = 0; a < 3; ++a) { ctr[a][slot] = 0.f; ext[a][slot] = -INFINITY; }
     ch[slot] = kEmptyChild;
   }
   float4* o = nodes4 + 7 * (size_t)idx4((int32_t)i);
-  o[0] = make_float4(lo[0][0], lo[0][1], lo[0][2], lo[0][3]);
-  o[1] = make_float4(hi[0][0], hi[0][1], hi[0][2], hi[0][3]);
-  o[2] = make_float4(lo[1][0], lo[1][1], lo[1][2], lo[1][3]);
-  o[3] = make_float4(hi[1][0], hi[1][1], hi[1][2], hi[1][3]);
-  o[4] = make_float4(lo[2][0], lo[2][1], lo[2][2], lo[2][3]);
-  o[5] = make_float4(hi[2][0], hi[2][1], hi[2][2], hi[2][3]);
+  o[0] = make_float4(ctr[0][0], ctr[0][1], ctr[0][2], ctr[0][3]);
+  o[1] = make_float4(ext[0][0], ext[0][1], ext[0][2], ext[0][3]);
+  o[2] = make_float4(ctr[1][0], ctr[1][1], ctr[1][2], ctr[1][3]);
+  o[3] = make_float4(ext[1][0], ext[1][1], ext[1][2], ext[1][3]);
+  o[4] = make_float4(ctr[2][0], ctr[2][1], ctr[2][2], ctr[2][3]);
+  o[5] = make_float4(ext[2][0], ext[2][1], ext[2][2], ext[2][3]);
   o[6] = make_float4(__int_as_float(ch[0]), __int_as_float(ch[1]), __int_as_float(ch[2]),
                      __int_as_float(ch[3]));
 }

@@ -154,7 +154,7 @@ int make_render_args(const rt_scene* scene, const rt_camera* cam, float eye_sep,
   // binary renders walk the SAH tree unless the LBVH is asked for; the
   // 4-wide tree (and the work counts of a 4-wide scene) derive from the SAH
   // tree
-  a.sc.nodes = scene->tree == RT_TREE_LBVH ? scene->nodes : scene->nodes_sah;
+  a.sc.nodes = scene->tree == RT_TREE_LBVH ? scene->render_lbvh : scene->render_sah;
   a.sc.nodes4 = scene->nodes4;
   a.sc.n4 = scene->n4;
   a.sc.n_top = scene->n_top;
@@ -245,7 +245,7 @@ int rt_scene_create(const rt_sphere* spheres, uint32_t n_spheres, const rt_trian
   const size_t b_parent = align256((2 * n - 1) * sizeof(int32_t));
   const size_t b_nodes4 = align256((n > 1 ? n - 1 : 1) * 7 * sizeof(float4));
   const size_t b_err = 256;
-  const size_t total = 2 * b_nodes + b_prims + b_mats + b_lights + b_keys + b_parent + b_nodes4 + b_err;
+  const size_t total = 4 * b_nodes + b_prims + b_mats + b_lights + b_keys + b_parent + b_nodes4 + b_err;
   cudaError_t e = cudaMalloc(&sc->block, total);
   if (e != cudaSuccess) { cudaGetLastError(); delete sc; return cuda_fail(e, "scene allocation"); }
   char* p = static_cast<char*>(sc->block);
@@ -257,6 +257,8 @@ int rt_scene_create(const rt_sphere* spheres, uint32_t n_spheres, const rt_trian
   sc->parent = reinterpret_cast<int32_t*>(p); p += b_parent;
   sc->nodes4 = reinterpret_cast<float4*>(p); p += b_nodes4;
   sc->nodes_sah = reinterpret_cast<float4*>(p); p += b_nodes;
+  sc->render_sah = reinterpret_cast<float4*>(p); p += b_nodes;
+  sc->render_lbvh = reinterpret_cast<float4*>(p); p += b_nodes;
   sc->err = reinterpret_cast<uint32_t*>(p);
   e = cudaMallocHost(&sc->h_err, sizeof(uint32_t));
   if (e != cudaSuccess) { cudaGetLastError(); cudaFree(sc->block); delete sc; return cuda_fail(e, "pinned allocation"); }
@@ -283,6 +285,7 @@ int rt_scene_create(const rt_sphere* spheres, uint32_t n_spheres, const rt_trian
   // the render tree: SAH splits over the LBVH's leaves
   if (e == cudaSuccess)
     e = rt::build_sah_tree(sc->nodes, sc->parent, (uint32_t)n, sc->nodes_sah, d_lbvh, sc->err, st);
+  if (e == cudaSuccess) e = rt::render_nodes(sc->nodes_sah, (uint32_t)n, sc->render_sah, st);
   // (the 4-wide tree is built when a render first asks for it:
   // rt_scene_set_traversal)
   if (e == cudaSuccess) e = cudaMemcpyAsync(sc->h_err, sc->err, sizeof(uint32_t), cudaMemcpyDeviceToHost, st);
@@ -556,6 +559,10 @@ int rt_debug_set_node(rt_scene* scene, uint32_t node, int32_t left, int32_t righ
     nd[2].w = -1.f;
   }
   e = cudaMemcpy(scene->nodes + 4 * (size_t)node, nd, sizeof nd, cudaMemcpyHostToDevice);
+  if (e == cudaSuccess && scene->lbvh_ready) {
+    e = rt::render_nodes(scene->nodes, scene->n, scene->render_lbvh, 0);
+    if (e == cudaSuccess) e = cudaDeviceSynchronize();
+  }
   if (e != cudaSuccess) return cuda_fail(e, "node upload");
   return RT_OK;
 }
@@ -604,7 +611,7 @@ int rt_scene_set_traversal(rt_scene* scene, int tree) {
     e = cudaMemset(d_counts, 0, 2 * sizeof(uint32_t));
     if (e == cudaSuccess) e = rt::inner_parents(scene->nodes_sah, n, sah_parent, 0);
     if (e == cudaSuccess)
-      e = rt::build_bvh4(scene->nodes_sah, sah_parent, n, rt::treelet_depth(), scene->nodes4, d_counts,
+      e = rt::build_bvh4(scene->render_sah, sah_parent, n, rt::treelet_depth(), scene->nodes4, d_counts,
                          tmp, 0);
     if (e == cudaSuccess) e = cudaMemcpy(counts, d_counts, sizeof counts, cudaMemcpyDeviceToHost);
     cudaFree(tmp);
@@ -612,6 +619,14 @@ int rt_scene_set_traversal(rt_scene* scene, int tree) {
     scene->n_top = counts[0];
     scene->n4 = counts[1];
     scene->wide_built = true;
+  }
+  if (tree == RT_TREE_LBVH && !scene->lbvh_ready) {
+    // the render nodes of the LBVH (the SAH tree's are made with the scene)
+    cudaError_t e = cudaSetDevice(scene->device);
+    if (e == cudaSuccess) e = rt::render_nodes(scene->nodes, scene->n, scene->render_lbvh, 0);
+    if (e == cudaSuccess) e = cudaDeviceSynchronize();
+    if (e != cudaSuccess) return cuda_fail(e, "LBVH render nodes");
+    scene->lbvh_ready = true;
   }
   scene->tree = tree;
   return RT_OK;

@@ -7,6 +7,12 @@
 //              [1] = (c1.lo.x, c1.hi.x, c1.lo.y, c1.hi.y)
 //              [2] = (c0.lo.z, c0.hi.z, c1.lo.z, c1.hi.z)
 //              [3] = (left, right, -, -) as int bits; >= 0 internal, < 0 leaf ~k
+//   render nodes (the copy of a tree that renders walk, same numbering): each
+//            child box as centre c and half extent e:
+//              [0] = (c0.c.x, c0.c.y, c0.e.x, c0.e.y)
+//              [1] = (c1.c.x, c1.c.y, c1.e.x, c1.e.y)
+//              [2] = (c0.c.z, c0.e.z, c1.c.z, c1.e.z)
+//              [3] = (left, right, -, -)
 //   prims  : n leaf records of 48 B = 3 x float4 in leaf (sorted key) order:
 //            triangle: (v0.xyz, id) (e1.xyz, material) (e2.xyz, 0)
 //            sphere  : (c.xyz, id)  (r, 0, 0, material)  (0, 0, 0, 0)
@@ -42,7 +48,7 @@ constexpr float kAmbient = 0.1f;
 constexpr float kBgR = 0.2f, kBgG = 0.3f, kBgB = 0.5f;
 
 struct DeviceScene {
-  const float4* nodes;
+  const float4* nodes;    // render nodes
   const float4* nodes4;   // 4-wide nodes (7 float4 each), the top n_top first
   const float4* prims;
   const float4* mats;
@@ -185,6 +191,8 @@ size_t sah_tmp_bytes(uint32_t n);
 // node layout and leaf slots, root 0; synchronises st once per tree level
 cudaError_t build_sah_tree(const float4* lbvh_nodes, const int32_t* parent, uint32_t n,
                            float4* out, void* tmp, uint32_t* err, cudaStream_t st);
+// the render nodes of a binary tree over n primitives
+cudaError_t render_nodes(const float4* nodes, uint32_t n, float4* out, cudaStream_t st);
 size_t bvh4_tmp_bytes(uint32_t n);
 void set_sah_slicing(bool on);   // slice the top levels of the SAH build (default on)
 cudaError_t inner_parents(const float4* nodes, uint32_t n, int32_t* parent, cudaStream_t st);
@@ -255,6 +263,9 @@ struct rt_scene {
   float4* nodes = nullptr;
   float4* nodes4 = nullptr;
   float4* nodes_sah = nullptr; // binary tree rebuilt with the SAH over the same leaves (sah.cu)
+  float4* render_sah = nullptr;   // render nodes of the SAH tree
+  float4* render_lbvh = nullptr;  // render nodes of the LBVH (made on first use)
+  bool lbvh_ready = false;     // render_lbvh holds them
   uint32_t n4 = 0, n_top = 0;
   bool wide_built = false;     // nodes4 holds the 4-wide tree (built on first use)
   int tree = RT_TREE_SAH;      // the tree renders walk (rt_scene_set_traversal)

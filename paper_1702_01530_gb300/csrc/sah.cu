@@ -861,7 +861,42 @@ k_sah_small(const float4* __restrict__ leaf_lo, const float4* __restrict__ leaf_
 
 namespace {
 bool g_sah_slicing = true;
+
+// Centre and half extent of [lo, hi], so that [c - e, c + e] contains it: e is
+// rounded up, and widened by 2^-22 of the box's distance from the origin for
+// the rounding of the two products the walk forms from it. An empty box
+// (lo > hi) gets e = -inf, which no ray hits.
+__device__ __forceinline__ void centre_extent(float lo, float hi, float& c, float& e) {
+  if (!(lo <= hi)) { c = 0.f; e = -INFINITY; return; }
+  c = (float)(0.5 * ((double)lo + (double)hi));
+  const double half = fmax((double)hi - (double)c, (double)c - (double)lo);
+  e = __double2float_ru(half + 0x1p-22 * fmax(fabs((double)lo), fabs((double)hi)));
+}
+
+__global__ void k_render_nodes(const float4* __restrict__ nodes, uint32_t n_inner, float4* __restrict__ out) {
+  const uint32_t i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (i >= n_inner) return;
+  const float4 a = nodes[4 * (size_t)i], b = nodes[4 * (size_t)i + 1], c = nodes[4 * (size_t)i + 2];
+  float4 u, v, w;
+  centre_extent(a.x, a.y, u.x, u.z);
+  centre_extent(a.z, a.w, u.y, u.w);
+  centre_extent(b.x, b.y, v.x, v.z);
+  centre_extent(b.z, b.w, v.y, v.w);
+  centre_extent(c.x, c.y, w.x, w.y);
+  centre_extent(c.z, c.w, w.z, w.w);
+  float4* o = out + 4 * (size_t)i;
+  o[0] = u;
+  o[1] = v;
+  o[2] = w;
+  o[3] = nodes[4 * (size_t)i + 3];
+}
 }  // namespace
+
+cudaError_t render_nodes(const float4* nodes, uint32_t n, float4* out, cudaStream_t st) {
+  if (n < 2) return cudaSuccess;      // no inner node
+  k_render_nodes<<<(n - 1 + 255) / 256, 256, 0, st>>>(nodes, n - 1, out);
+  return cudaGetLastError();
+}
 
 void set_sah_slicing(bool on) { g_sah_slicing = on; }
 

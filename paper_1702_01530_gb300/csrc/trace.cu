@@ -36,8 +36,9 @@
 // bitwise identical.
 //
 // Traversal (Table 1 of the paper: BVH trees): BVH2 nodes of 64 B with both
-// child boxes, read as four 16-byte vector loads through the read-only path;
-// slab tests in FP32 with fused multiply-adds and three-input min/max; the
+// child boxes as centre and half extent, read as four vector loads through the
+// read-only path; slab tests in FP32 with (two-wide) fused multiply-adds and
+// three-input min/max; the
 // far child is pushed on a per-thread stack of 64 entries, the near child is
 // visited first. The tree is the SAH rebuild of the scene's LBVH (sah.cu,
 // depth <= 60 by its depth budget) or the LBVH itself (depth <= 64: a radix

@@ -18,20 +18,13 @@ namespace {
 // default, 0.221 ms for a 10-primitive scene):
 // RT_MIN_BLOCKS = minimum resident blocks per SM requested from the register
 // allocator (0 = no request; 9 measured best: the default walk fits 56
-// registers without spills, 36 warps per SM; against 8 blocks (64 registers,
+// registers with 8 bytes spilled outside its loop, 36 warps per SM; against 8 blocks (64 registers,
 // 32 warps) 1.005 against 1.014 ms per 1080p blob pair and 13.94 against
 // 14.05 ms per 4K terrain frame; 6 blocks: 1.051 / 0.216 ms; 7 blocks: 1.048
 // ms; 10 blocks (48 registers, spills in the shading code): 1.047 / 0.242 ms
-// in earlier builds); RT_WHILE_WHILE = 1 postpones the first leaf a ray
-// meets and keeps descending until every active lane of the warp holds a
-// leaf, so the leaf tests of a warp run together instead of interleaving
-// with node visits (the "while-while" loop of Aila & Laine, HPG 2009) --
-// 1.247 ms with one primitive per leaf, hence off by default.
+// in earlier builds).
 #ifndef RT_MIN_BLOCKS
 #define RT_MIN_BLOCKS 9
-#endif
-#ifndef RT_WHILE_WHILE
-#define RT_WHILE_WHILE 0
 #endif
 constexpr int kStack4 = 100;   // 3 pushes per 4-wide level, <= 33 levels
 // shared-memory treelet: 4-wide levels staged per block (RT_TREELET_DEPTH
@@ -40,37 +33,6 @@ constexpr int kStack4 = 100;   // 3 pushes per 4-wide level, <= 33 levels
 #define RT_TREELET_DEPTH 2
 #endif
 constexpr int kMaxTopBytes = 85 * 7 * 16;
-// binary traversal keeps the top of its stack in a register: a pop hands
-// the register over at once and reloads it from local memory in the
-// background, so the pop and the next node fetch do not wait in series;
-// 1.093 ms: off by default
-#ifndef RT_STACK_TOP_REG
-#define RT_STACK_TOP_REG 0
-#endif
-// binary traversal prefetches both children of every visited node into L1
-// (prefetch.global.L1) as soon as their indices are known, so a child's
-// fetch that misses L1 overlaps the current node's slab tests; 1.583
-// against 1.299 ms (LBVH, one eye per warp): off
-#ifndef RT_PREFETCH
-#define RT_PREFETCH 0
-#endif
-// binary traversal defers leaf tests: a lane keeps up to two leaves pending
-// and walks on; the warp tests the pending leaves together once
-// RT_DEFER_LEAVES lanes hold one, or as soon as any lane can go no further
-// (both slots full and the next node a leaf, or nothing left to visit).
-// Same images; 1.302 ms at 16 lanes against 1.042 (1.399 / 1.417 / 1.442 at
-// 16 / 8 / 4 against 1.149 with one eye per warp), so 0 = off by default
-#ifndef RT_DEFER_LEAVES
-#define RT_DEFER_LEAVES 0
-#endif
-// binary traversal reads a 64-byte node with two 32-byte loads
-// (ld.global.nc.v8.f32, sm_100 and later) instead of four 16-byte ones:
-// half the load instructions and L1 requests per node visit; 1 = plain,
-// 2 = with an L1 evict-last hint. 1.149 / 1.150 ms against 1.146 (SAH
-// tree, one eye per warp): off by default
-#ifndef RT_LD256
-#define RT_LD256 0
-#endif
 // 4-wide closest-hit traversal pushes the other hit children farthest first
 #ifndef RT_ORDERED_PUSH
 #define RT_ORDERED_PUSH 0
@@ -138,16 +100,20 @@ __device__ __forceinline__ float safe_rcp(float x) {
 
 struct WorkCount { uint32_t inner, sphere, tri; };
 
-// Two float4 of one 32-byte aligned block through the read-only path in one
-// 256-bit load.
-__device__ __forceinline__ void ldg2x16(const float4* p, float4& u, float4& v) {
-#if RT_LD256 == 2
-  asm("ld.global.nc.L1::evict_last.v8.f32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
-#else
-  asm("ld.global.nc.v8.f32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
-#endif
-      : "=f"(u.x), "=f"(u.y), "=f"(u.z), "=f"(u.w), "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w)
-      : "l"(p));
+// two FP32 values in one 64-bit register, and fma on both in one instruction
+typedef unsigned long long f32x2;
+__device__ __forceinline__ f32x2 pack2(float a, float b) {
+  f32x2 r;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
+  return r;
+}
+__device__ __forceinline__ void unpack2(f32x2 r, float& a, float& b) {
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(r));
+}
+__device__ __forceinline__ f32x2 fma2(f32x2 a, f32x2 b, f32x2 c) {
+  f32x2 r;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+  return r;
 }
 
 // Ray-sphere (d unit length). Stable form: disc = r^2 - |oc - b d|^2 keeps
@@ -189,16 +155,29 @@ __device__ __forceinline__ bool hit_tri(float4 p0, float4 p1, float4 p2, V3 o, V
 // BVH traversal. ANY = any-hit with t < tmax (returns true if blocked);
 // otherwise closest hit with t <= t_best (equal t -> lower id), returns
 // whether anything was hit.
+//
+// Nodes hold each child box as centre c and half extent e (render_nodes): per
+// axis t_c = (c - o) / d, and the ray is inside the slab from t_c - e |1/d| to
+// t_c + e |1/d|, which needs no minimum and maximum to order the two planes;
+// x and y of a child share one two-wide fma. A child takes 6 fma instructions
+// (3 of them two-wide) and 4 three-input minima and maxima, against 6 fma and
+// 10 minima and maxima with the box as two corners: 721 -> 656 M warp
+// instructions for the 1080p blob pair, 0.987 -> 0.946 ms; 4K frame of a
+// 2.1 M-triangle terrain 12.34 -> 11.25 ms. What bounds it now is the latency of
+// the node loads (5.0 of 13 stalled warps per issue) and the L1 (72 % of its
+// throughput): a node as two 32-byte loads (11.48 ms), 10 blocks of 48 registers
+// (0.966 / 11.46 ms) and leaving the triangle test after its first failed bound
+// (0.956 / 11.29 ms) were slower.
 template <bool ANY, bool COUNT>
 __device__ __forceinline__ bool traverse(const DeviceScene& sc, V3 o, V3 d, float tmax,
                                          float& t_best, uint32_t& id_best, uint32_t& k_best,
                                          WorkCount& wc, uint32_t* err) {
-  constexpr int32_t kNone = 0x7FFFFFFF;        // no node: empty stack
   const V3 idir = v3(safe_rcp(d.x), safe_rcp(d.y), safe_rcp(d.z));
-  const V3 ood = v3(o.x * idir.x, o.y * idir.y, o.z * idir.z);
+  const f32x2 id_xy = pack2(idir.x, idir.y), od_xy = pack2(-o.x * idir.x, -o.y * idir.y);
+  const f32x2 ai_xy = pack2(fabsf(idir.x), fabsf(idir.y)), na_xy = pack2(-fabsf(idir.x), -fabsf(idir.y));
+  const float od_z = -o.z * idir.z, ai_z = fabsf(idir.z);
   int32_t stack[kStackSize];
   int sp = 0;
-  int32_t stop = kNone;                         // top of the stack (register copy)
   const uint32_t n = sc.n_prims;
   int32_t node = n == 1 ? ~0 : 0;
   const uint32_t it_max = 2u * n + 64u;
@@ -213,54 +192,33 @@ __device__ __forceinline__ bool traverse(const DeviceScene& sc, V3 o, V3 d, floa
         break;
       }
       const float4* np = sc.nodes + 4 * (size_t)node;
-      float4 a, b, c, e;
-      if (RT_LD256) {                  // nodes are 64-byte aligned
-        ldg2x16(np, a, b);
-        ldg2x16(np + 2, c, e);
-      } else {
-        a = __ldg(np); b = __ldg(np + 1); c = __ldg(np + 2); e = __ldg(np + 3);
-      }
+      const ulonglong2 a = __ldg(reinterpret_cast<const ulonglong2*>(np));       // (c.xy, e.xy) of child 0
+      const ulonglong2 b = __ldg(reinterpret_cast<const ulonglong2*>(np + 1));   // ... of child 1
+      const float4 c = __ldg(np + 2);                                            // c.z, e.z of both
+      const int2 e = __ldg(reinterpret_cast<const int2*>(np + 3));               // the children
       if (COUNT) wc.inner++;
-      if (RT_PREFETCH) {
-        const int32_t pl = __float_as_int(e.x), pr = __float_as_int(e.y);
-        // only in-range children are prefetched (the traversal checks them again)
-        if (pl >= 0 ? (uint32_t)pl < n - 1 : (uint32_t)~pl < n)
-          asm volatile("prefetch.global.L1 [%0];" ::"l"(pl >= 0 ? sc.nodes + 4 * (size_t)pl
-                                                                 : sc.prims + 3 * (size_t)~pl));
-        if (pr >= 0 ? (uint32_t)pr < n - 1 : (uint32_t)~pr < n)
-          asm volatile("prefetch.global.L1 [%0];" ::"l"(pr >= 0 ? sc.nodes + 4 * (size_t)pr
-                                                                 : sc.prims + 3 * (size_t)~pr));
-      }
-      const float l0x = fmaf(a.x, idir.x, -ood.x), h0x = fmaf(a.y, idir.x, -ood.x);
-      const float l0y = fmaf(a.z, idir.y, -ood.y), h0y = fmaf(a.w, idir.y, -ood.y);
-      const float l0z = fmaf(c.x, idir.z, -ood.z), h0z = fmaf(c.y, idir.z, -ood.z);
-      const float l1x = fmaf(b.x, idir.x, -ood.x), h1x = fmaf(b.y, idir.x, -ood.x);
-      const float l1y = fmaf(b.z, idir.y, -ood.y), h1y = fmaf(b.w, idir.y, -ood.y);
-      const float l1z = fmaf(c.z, idir.z, -ood.z), h1z = fmaf(c.w, idir.z, -ood.z);
-      const float in0 = fmax3(fminf(l0x, h0x), fminf(l0y, h0y), fmaxf(fminf(l0z, h0z), 0.f));
-      const float out0 = fmin3(fmaxf(l0x, h0x), fmaxf(l0y, h0y), fminf(fmaxf(l0z, h0z), tcur));
-      const float in1 = fmax3(fminf(l1x, h1x), fminf(l1y, h1y), fmaxf(fminf(l1z, h1z), 0.f));
-      const float out1 = fmin3(fmaxf(l1x, h1x), fmaxf(l1y, h1y), fminf(fmaxf(l1z, h1z), tcur));
+      const f32x2 t0 = fma2(a.x, id_xy, od_xy), t1 = fma2(b.x, id_xy, od_xy);
+      const float z0 = fmaf(c.x, idir.z, od_z), z1 = fmaf(c.z, idir.z, od_z);
+      float i0x, i0y, o0x, o0y, i1x, i1y, o1x, o1y;
+      unpack2(fma2(a.y, na_xy, t0), i0x, i0y);
+      unpack2(fma2(a.y, ai_xy, t0), o0x, o0y);
+      unpack2(fma2(b.y, na_xy, t1), i1x, i1y);
+      unpack2(fma2(b.y, ai_xy, t1), o1x, o1y);
+      const float in0 = fmax3(i0x, i0y, fmaxf(fmaf(-c.y, ai_z, z0), 0.f));
+      const float out0 = fmin3(o0x, o0y, fminf(fmaf(c.y, ai_z, z0), tcur));
+      const float in1 = fmax3(i1x, i1y, fmaxf(fmaf(-c.w, ai_z, z1), 0.f));
+      const float out1 = fmin3(o1x, o1y, fminf(fmaf(c.w, ai_z, z1), tcur));
       const bool hit0 = in0 <= out0 * kRobust;
       const bool hit1 = in1 <= out1 * kRobust;
-      const int32_t cl = __float_as_int(e.x), cr = __float_as_int(e.y);
-      if (hit0 && hit1) {
-        const bool swap = in1 < in0;
-        const int32_t far = swap ? cl : cr;
-        if (RT_STACK_TOP_REG) {
-          if (stop != kNone) {
-            if (sp >= kStackSize) { atomicOr(err, ERR_STACK); break; }
-            stack[sp++] = stop;
-          }
-          stop = far;
-        } else {
+      if (hit0 | hit1) {
+        const bool second = hit1 && (!hit0 || in1 < in0);
+        node = second ? e.y : e.x;
+        if (hit0 & hit1) {
           if (sp >= kStackSize) { atomicOr(err, ERR_STACK); break; }
-          stack[sp++] = far;
+          stack[sp++] = second ? e.x : e.y;
         }
-        node = swap ? cr : cl;
         continue;
       }
-      if (hit0 | hit1) { node = hit0 ? cl : cr; continue; }
     } else {
       const uint32_t k = (uint32_t)~node;
       if (k >= n) { atomicOr(err, ERR_INDEX); break; }
@@ -285,14 +243,8 @@ __device__ __forceinline__ bool traverse(const DeviceScene& sc, V3 o, V3 d, floa
         any = true;
       }
     }
-    if (RT_STACK_TOP_REG) {
-      if (stop == kNone) break;
-      node = stop;
-      stop = sp ? stack[--sp] : kNone;
-    } else {
-      if (sp == 0) break;
-      node = stack[--sp];
-    }
+    if (sp == 0) break;
+    node = stack[--sp];
   }
   if (!ANY) t_best = tcur;
   return any;
@@ -306,7 +258,8 @@ __device__ __forceinline__ bool traverse4(const DeviceScene& sc, const float4* t
                                           float tmax, float& t_best, uint32_t& id_best,
                                           uint32_t& k_best, uint32_t* err) {
   const V3 idir = v3(safe_rcp(d.x), safe_rcp(d.y), safe_rcp(d.z));
-  const V3 ood = v3(o.x * idir.x, o.y * idir.y, o.z * idir.z);
+  const V3 od = v3(-o.x * idir.x, -o.y * idir.y, -o.z * idir.z);
+  const V3 ai = v3(fabsf(idir.x), fabsf(idir.y), fabsf(idir.z));
   int32_t stack[kStack4];
   int sp = 0;
   const uint32_t n = sc.n_prims;
@@ -318,30 +271,32 @@ __device__ __forceinline__ bool traverse4(const DeviceScene& sc, const float4* t
     if (it >= it_max) { atomicOr(err, ERR_ITER); break; }
     if (node >= 0) {
       if ((uint32_t)node >= sc.n4) { atomicOr(err, ERR_INDEX); break; }
-      float4 lx, hx, ly, hy, lz, hz, cc;
+      float4 cx, ex, cy, ey, cz, ez, cc;
       if ((uint32_t)node < sc.n_top) {             // shared-memory treelet
         const float4* np = top + 7 * node;
-        lx = np[0]; hx = np[1]; ly = np[2]; hy = np[3]; lz = np[4]; hz = np[5]; cc = np[6];
+        cx = np[0]; ex = np[1]; cy = np[2]; ey = np[3]; cz = np[4]; ez = np[5]; cc = np[6];
       } else {                                     // read-only global path
         const float4* np = sc.nodes4 + 7 * (size_t)node;
-        lx = __ldg(np); hx = __ldg(np + 1); ly = __ldg(np + 2); hy = __ldg(np + 3);
-        lz = __ldg(np + 4); hz = __ldg(np + 5); cc = __ldg(np + 6);
+        cx = __ldg(np); ex = __ldg(np + 1); cy = __ldg(np + 2); ey = __ldg(np + 3);
+        cz = __ldg(np + 4); ez = __ldg(np + 5); cc = __ldg(np + 6);
       }
       float tin[4];
       bool hit[4];
-#define RT_SLAB(c, LX, HX, LY, HY, LZ, HZ)                                                  \
-      {                                                                                     \
-        const float ax = fmaf(LX, idir.x, -ood.x), bx = fmaf(HX, idir.x, -ood.x);           \
-        const float ay = fmaf(LY, idir.y, -ood.y), by = fmaf(HY, idir.y, -ood.y);           \
-        const float az = fmaf(LZ, idir.z, -ood.z), bz = fmaf(HZ, idir.z, -ood.z);           \
-        tin[c] = fmax3(fminf(ax, bx), fminf(ay, by), fmaxf(fminf(az, bz), 0.f));             \
-        const float tout = fmin3(fmaxf(ax, bx), fmaxf(ay, by), fminf(fmaxf(az, bz), tcur));  \
-        hit[c] = tin[c] <= tout * kRobust;                                                  \
+      // the binary walk's box test, so that every tree takes the same leaves
+#define RT_SLAB(c, F)                                                                         \
+      {                                                                                       \
+        const float tx = fmaf(cx.F, idir.x, od.x), ty = fmaf(cy.F, idir.y, od.y),             \
+                    tz = fmaf(cz.F, idir.z, od.z);                                            \
+        tin[c] = fmax3(fmaf(-ex.F, ai.x, tx), fmaf(-ey.F, ai.y, ty),                          \
+                       fmaxf(fmaf(-ez.F, ai.z, tz), 0.f));                                    \
+        const float tout = fmin3(fmaf(ex.F, ai.x, tx), fmaf(ey.F, ai.y, ty),                  \
+                                 fminf(fmaf(ez.F, ai.z, tz), tcur));                          \
+        hit[c] = tin[c] <= tout * kRobust;                                                    \
       }
-      RT_SLAB(0, lx.x, hx.x, ly.x, hy.x, lz.x, hz.x)
-      RT_SLAB(1, lx.y, hx.y, ly.y, hy.y, lz.y, hz.y)
-      RT_SLAB(2, lx.z, hx.z, ly.z, hy.z, lz.z, hz.z)
-      RT_SLAB(3, lx.w, hx.w, ly.w, hy.w, lz.w, hz.w)
+      RT_SLAB(0, x)
+      RT_SLAB(1, y)
+      RT_SLAB(2, z)
+      RT_SLAB(3, w)
 #undef RT_SLAB
       const int32_t ch[4] = {__float_as_int(cc.x), __float_as_int(cc.y), __float_as_int(cc.z),
                              __float_as_int(cc.w)};
@@ -407,193 +362,6 @@ __device__ __forceinline__ bool traverse4(const DeviceScene& sc, const float4* t
   return any;
 }
 
-#if RT_WHILE_WHILE
-// Same traversal with postponed leaves. Internal nodes are visited until
-// every active lane of the warp holds one pending leaf (or has finished);
-// then the pending leaves (and any leaves that follow directly) are tested.
-template <bool ANY, bool COUNT>
-__device__ __forceinline__ bool traverse_ww(const DeviceScene& sc, V3 o, V3 d, float tmax,
-                                            float& t_best, uint32_t& id_best, uint32_t& k_best,
-                                            WorkCount& wc, uint32_t* err) {
-  constexpr int32_t kDone = 0x7FFFFFFF;   // larger than any internal node index
-  const V3 idir = v3(safe_rcp(d.x), safe_rcp(d.y), safe_rcp(d.z));
-  const V3 ood = v3(o.x * idir.x, o.y * idir.y, o.z * idir.z);
-  int32_t stack[kStackSize];
-  int sp = 0;
-  const uint32_t n = sc.n_prims;
-  int32_t node = n == 1 ? ~0 : 0;
-  int32_t leaf = 0;
-  const uint32_t it_max = 2u * n + 64u;
-  uint32_t it = 0;
-  float tcur = ANY ? tmax : t_best;
-  bool any = false;
-  if (node < 0) { leaf = node; node = kDone; }
-  while (node != kDone || leaf != 0) {
-    while ((uint32_t)node < (uint32_t)kDone) {   // node >= 0 and not done
-      if (++it > it_max) { atomicOr(err, ERR_ITER); node = kDone; leaf = 0; break; }
-      if ((uint32_t)node >= n - 1) { atomicOr(err, ERR_INDEX); node = kDone; leaf = 0; break; }
-      const float4* np = sc.nodes + 4 * (size_t)node;
-      const float4 a = __ldg(np), b = __ldg(np + 1), c = __ldg(np + 2), e = __ldg(np + 3);
-      if (COUNT) wc.inner++;
-      const float l0x = fmaf(a.x, idir.x, -ood.x), h0x = fmaf(a.y, idir.x, -ood.x);
-      const float l0y = fmaf(a.z, idir.y, -ood.y), h0y = fmaf(a.w, idir.y, -ood.y);
-      const float l0z = fmaf(c.x, idir.z, -ood.z), h0z = fmaf(c.y, idir.z, -ood.z);
-      const float l1x = fmaf(b.x, idir.x, -ood.x), h1x = fmaf(b.y, idir.x, -ood.x);
-      const float l1y = fmaf(b.z, idir.y, -ood.y), h1y = fmaf(b.w, idir.y, -ood.y);
-      const float l1z = fmaf(c.z, idir.z, -ood.z), h1z = fmaf(c.w, idir.z, -ood.z);
-      const float in0 = fmax3(fminf(l0x, h0x), fminf(l0y, h0y), fmaxf(fminf(l0z, h0z), 0.f));
-      const float out0 = fmin3(fmaxf(l0x, h0x), fmaxf(l0y, h0y), fminf(fmaxf(l0z, h0z), tcur));
-      const float in1 = fmax3(fminf(l1x, h1x), fminf(l1y, h1y), fmaxf(fminf(l1z, h1z), 0.f));
-      const float out1 = fmin3(fmaxf(l1x, h1x), fmaxf(l1y, h1y), fminf(fmaxf(l1z, h1z), tcur));
-      const bool hit0 = in0 <= out0 * kRobust;
-      const bool hit1 = in1 <= out1 * kRobust;
-      const int32_t cl = __float_as_int(e.x), cr = __float_as_int(e.y);
-      if (hit0 && hit1) {
-        const bool swap = in1 < in0;
-        if (sp >= kStackSize) { atomicOr(err, ERR_STACK); node = kDone; leaf = 0; break; }
-        stack[sp++] = swap ? cl : cr;
-        node = swap ? cr : cl;
-      } else if (hit0 | hit1) {
-        node = hit0 ? cl : cr;
-      } else {
-        node = sp ? stack[--sp] : kDone;
-      }
-      if (node < 0 && leaf == 0) {           // postpone this leaf, keep descending
-        leaf = node;
-        node = sp ? stack[--sp] : kDone;
-      }
-      if (!__any_sync(__activemask(), leaf == 0)) break;
-    }
-    while (leaf < 0) {
-      if (++it > it_max) { atomicOr(err, ERR_ITER); node = kDone; leaf = 0; break; }
-      const uint32_t k = (uint32_t)~leaf;
-      if (k >= n) { atomicOr(err, ERR_INDEX); node = kDone; leaf = 0; break; }
-      const float4* pp = sc.prims + 3 * (size_t)k;
-      const float4 p0 = __ldg(pp), p1 = __ldg(pp + 1);
-      const uint32_t id = __float_as_uint(p0.w);
-      float t;
-      bool h;
-      if (id < sc.n_spheres) {
-        if (COUNT) wc.sphere++;
-        h = hit_sphere(p0, p1.x, o, d, t);
-      } else {
-        if (COUNT) wc.tri++;
-        h = hit_tri(p0, p1, __ldg(pp + 2), o, d, t);
-      }
-      if (ANY) {
-        if (h && t < tmax) { any = true; node = kDone; leaf = 0; break; }
-      } else if (h && (t < tcur || (t == tcur && id < id_best))) {
-        tcur = t;
-        id_best = id;
-        k_best = k;
-        any = true;
-      }
-      leaf = 0;
-      if (node < 0) {                         // the next node is a leaf too
-        leaf = node;
-        node = sp ? stack[--sp] : kDone;
-      }
-    }
-  }
-  if (!ANY) t_best = tcur;
-  return any;
-}
-#endif
-
-#if RT_DEFER_LEAVES
-// Binary traversal with deferred leaves (the speculative "while-while" idea
-// of Aila & Laine, HPG 2009, in one loop): node visits and leaf tests of a
-// warp run in separate passes of the same iteration, so a leaf met by one
-// lane no longer costs every other lane a full primitive test. A deferred
-// leaf can only make the closest-hit bound tcur shrink later, so the set of
-// leaves tested contains the one the eager walk would accept: the hit (t,
-// lower id on ties) and the any-hit answer are the same.
-template <bool ANY>
-__device__ __forceinline__ bool traverse_dl(const DeviceScene& sc, V3 o, V3 d, float tmax,
-                                            float& t_best, uint32_t& id_best, uint32_t& k_best,
-                                            uint32_t* err) {
-  constexpr int32_t kDone = 0x7FFFFFFF;        // larger than any internal node index
-  const V3 idir = v3(safe_rcp(d.x), safe_rcp(d.y), safe_rcp(d.z));
-  const V3 ood = v3(o.x * idir.x, o.y * idir.y, o.z * idir.z);
-  int32_t stack[kStackSize];
-  int sp = 0;
-  const uint32_t n = sc.n_prims;
-  int32_t node = n == 1 ? ~0 : 0;
-  int32_t l0 = 0, l1 = 0;                      // pending leaves (~k), 0 = empty; l1 != 0 => l0 != 0
-  // every iteration visits a node, moves a leaf to a slot or tests the
-  // slots, and a ray visits each node and leaf at most once
-  const uint32_t it_max = 2u * n + 64u;
-  float tcur = ANY ? tmax : t_best;
-  bool any = false;
-  for (uint32_t it = 0;; ++it) {
-    if (it >= it_max) { atomicOr(err, ERR_ITER); break; }
-    if (node >= 0 && node != kDone) {
-      if ((uint32_t)node >= n - 1) { atomicOr(err, ERR_INDEX); break; }
-      const float4* np = sc.nodes + 4 * (size_t)node;
-      const float4 a = __ldg(np), b = __ldg(np + 1), c = __ldg(np + 2), e = __ldg(np + 3);
-      const float l0x = fmaf(a.x, idir.x, -ood.x), h0x = fmaf(a.y, idir.x, -ood.x);
-      const float l0y = fmaf(a.z, idir.y, -ood.y), h0y = fmaf(a.w, idir.y, -ood.y);
-      const float l0z = fmaf(c.x, idir.z, -ood.z), h0z = fmaf(c.y, idir.z, -ood.z);
-      const float l1x = fmaf(b.x, idir.x, -ood.x), h1x = fmaf(b.y, idir.x, -ood.x);
-      const float l1y = fmaf(b.z, idir.y, -ood.y), h1y = fmaf(b.w, idir.y, -ood.y);
-      const float l1z = fmaf(c.z, idir.z, -ood.z), h1z = fmaf(c.w, idir.z, -ood.z);
-      const float in0 = fmax3(fminf(l0x, h0x), fminf(l0y, h0y), fmaxf(fminf(l0z, h0z), 0.f));
-      const float out0 = fmin3(fmaxf(l0x, h0x), fmaxf(l0y, h0y), fminf(fmaxf(l0z, h0z), tcur));
-      const float in1 = fmax3(fminf(l1x, h1x), fminf(l1y, h1y), fmaxf(fminf(l1z, h1z), 0.f));
-      const float out1 = fmin3(fmaxf(l1x, h1x), fmaxf(l1y, h1y), fminf(fmaxf(l1z, h1z), tcur));
-      const bool hit0 = in0 <= out0 * kRobust;
-      const bool hit1 = in1 <= out1 * kRobust;
-      const int32_t cl = __float_as_int(e.x), cr = __float_as_int(e.y);
-      if (hit0 && hit1) {
-        if (sp >= kStackSize) { atomicOr(err, ERR_STACK); break; }
-        const bool swap = in1 < in0;
-        stack[sp++] = swap ? cl : cr;
-        node = swap ? cr : cl;
-      } else if (hit0 | hit1) {
-        node = hit0 ? cl : cr;
-      } else {
-        node = sp ? stack[--sp] : kDone;
-      }
-    }
-    if (node < 0 && l0 == 0) { l0 = node; node = sp ? stack[--sp] : kDone; }
-    if (node < 0 && l1 == 0) { l1 = node; node = sp ? stack[--sp] : kDone; }
-    const bool pend = l0 != 0;
-    const bool stuck = pend && (node < 0 || node == kDone);
-    const unsigned m = __activemask();
-    const bool flush = __any_sync(m, stuck) || __popc(__ballot_sync(m, pend)) >= RT_DEFER_LEAVES;
-    if (flush && pend) {
-      bool bad = false;
-#pragma unroll 1
-      for (int s = 0; s < 2; ++s) {
-        const int32_t lf = s ? l1 : l0;
-        if (lf == 0) break;
-        const uint32_t k = (uint32_t)~lf;
-        if (k >= n) { bad = true; break; }
-        const float4* pp = sc.prims + 3 * (size_t)k;
-        const float4 p0 = __ldg(pp), p1 = __ldg(pp + 1);
-        const uint32_t id = __float_as_uint(p0.w);
-        float t;
-        const bool h = id < sc.n_spheres ? hit_sphere(p0, p1.x, o, d, t)
-                                         : hit_tri(p0, p1, __ldg(pp + 2), o, d, t);
-        if (ANY) {
-          if (h && t < tmax) { any = true; node = kDone; break; }
-        } else if (h && (t < tcur || (t == tcur && id < id_best))) {
-          tcur = t;
-          id_best = id;
-          k_best = k;
-          any = true;
-        }
-      }
-      if (bad) { atomicOr(err, ERR_INDEX); break; }
-      l0 = l1 = 0;
-    }
-    if (node == kDone && l0 == 0) break;
-  }
-  if (!ANY) t_best = tcur;
-  return any;
-}
-#endif
-
 // The instrumented (COUNT) walk and the binary renders use the binary tree
 // in sc.nodes (the SAH tree, or the LBVH whose node visits define the
 // algorithmic work); a 4-wide render walks the 4-wide tree (the same leaves,
@@ -604,14 +372,7 @@ __device__ __forceinline__ bool trace_ray(const DeviceScene& sc, const float4* t
                                           float tmax, float& t_best, uint32_t& id_best,
                                           uint32_t& k_best, WorkCount& wc, uint32_t* err) {
   if (TREE == kTreeWide4 && !COUNT) return traverse4<ANY>(sc, top, o, d, tmax, t_best, id_best, k_best, err);
-#if RT_DEFER_LEAVES
-  if (!COUNT) return traverse_dl<ANY>(sc, o, d, tmax, t_best, id_best, k_best, err);
-#endif
-#if RT_WHILE_WHILE
-  return traverse_ww<ANY, COUNT>(sc, o, d, tmax, t_best, id_best, k_best, wc, err);
-#else
   return traverse<ANY, COUNT>(sc, o, d, tmax, t_best, id_best, k_best, wc, err);
-#endif
 }
 
 __device__ __forceinline__ uint32_t lane_id() { return threadIdx.x & 31; }
