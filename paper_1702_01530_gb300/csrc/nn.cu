@@ -8,7 +8,7 @@
 //
 // Backward pass: data gradients are convolutions with the 3x3 taps flipped and
 // Cin/Cout swapped (k_conv_tma, below); weight gradients are contractions over
-// the pixels (k_wgrad_tc); BCE on the sigmoid output; Adam on FP32 master
+// the pixels (k_wgrad); BCE on the sigmoid output; Adam on FP32 master
 // weights.
 //
 // Convolution as implicit GEMM on tcgen05 (k_conv_tma):
@@ -655,7 +655,12 @@ struct FusedArgs {
   const float* inv[4];           // E4M3 inputs: inverse scale per output channel (null: 1)
   float out_scale[4];            // E4M3 outputs (1 otherwise)
   __nv_bfloat16* act[3];         // hidden activations to keep, BF16 planar [4][P][8] (null: none)
-  float* prob;
+  float* prob;                   // output (null: none)
+  // training: labels in, the BCE's gradient out and the loss' partial sums,
+  // one per warp of layer 4's epilogue (see "BCE and d(logit)")
+  const float* label;
+  uint4* g8;
+  float* loss_part;
   uint32_t W, H, n_img, strips, segs, rows;   // rows: output rows of a segment
   uint32_t* err;
 };
@@ -904,6 +909,22 @@ __device__ __forceinline__ bool fused_epilogue(const int KR, const FusedArgs& a,
   return true;
 }
 
+// ------------------------------------------------------- BCE and d(logit)
+// loss = mean(-(y log p + (1-y) log(1-p))), dlogit g = p - y (the 1/P factor
+// is applied in the weight-gradient reduction). g goes out as one 16-byte
+// channel chunk per pixel, [P][8] BF16: channel 0 = bf16(g), the input of the
+// layer-4 data-gradient conv, and channels 1, 2 = the two BF16 remainders, so
+// that the three add up to the FP32 g exactly and the layer-4 weight gradient
+// keeps all its bits on the tensor cores. Returns the pixel's loss.
+__device__ __forceinline__ float bce_gradient(float p, float y, uint4& g8) {
+  const float q = fminf(fmaxf(p, 1e-7f), 1.f - 1e-7f);
+  const float g = p - y;
+  const float hi = __bfloat162float(__float2bfloat16_rn(g));
+  const float mid = __bfloat162float(__float2bfloat16_rn(g - hi));
+  g8 = make_uint4(pack_bf16(hi, mid), pack_bf16(g - hi - mid, 0.f), 0u, 0u);
+  return -(y * __logf(q) + (1.f - y) * __logf(1.f - q));
+}
+
 template <bool FP8, bool STORE>
 __global__ void __launch_bounds__(kFuThreads, 1)
     k_net_fused(const __grid_constant__ CUtensorMap tmap, const __grid_constant__ FusedArgs a) {
@@ -1000,6 +1021,7 @@ __global__ void __launch_bounds__(kFuThreads, 1)
     const float sc = cst[3 * 32], bi = cst[7 * 32];
     Ring in;
     uint32_t buf = 0, n_row = 0;
+    float loss = 0.f;
     float s1[3] = {0.f, 0.f, 0.f}, s2[3] = {0.f, 0.f, 0.f};      // rows with one and with two taps added
     bool ok = true;
     for (uint32_t item = blockIdx.x; ok && item < n_items; item += gridDim.x) {
@@ -1033,9 +1055,16 @@ __global__ void __launch_bounds__(kFuThreads, 1)
         const int y = it.y0 + i - 2;
         if (m >= 1 && m <= kFuW && x < (int)a.W) {
           const float v = fmaf((px[m - 1] + z[1]) + px[128 + m + 1], sc, bi);
-          a.prob[((size_t)it.img * a.H + y) * a.W + x] = 1.f / (1.f + __expf(-v));
+          const float prob = 1.f / (1.f + __expf(-v));
+          const size_t p = ((size_t)it.img * a.H + y) * a.W + x;
+          if (!STORE || a.prob) a.prob[p] = prob;
+          if (STORE && a.label) loss += bce_gradient(prob, a.label[p], a.g8[p]);
         }
       }
+    }
+    if (STORE && a.label) {
+      for (int off = 16; off > 0; off >>= 1) loss += __shfl_xor_sync(0xFFFFFFFFu, loss, off);
+      if (lane == 0) a.loss_part[blockIdx.x * 4 + quarter] = loss;
     }
     if (!ok && lane == 0) atomicOr(a.err, ERR_ITER);
   }
@@ -1129,35 +1158,14 @@ __global__ void k_amax(const __nv_bfloat16* __restrict__ a, size_t n, unsigned* 
   if ((threadIdx.x & 31) == 0) atomicMax(out, __float_as_uint(m));
 }
 
-// ------------------------------------------------------- BCE + d(logit)
-// loss = mean(-(y log p + (1-y) log(1-p))), dlogit g = p - y (the 1/P factor
-// is applied in the weight-gradient reduction). g goes out as one 16-byte
-// channel chunk per pixel, [P][8] BF16: channel 0 = bf16(g), the input of the
-// layer-4 data-gradient conv, and channels 1, 2 = the two BF16 remainders, so
-// that the three add up to the FP32 g exactly and the layer-4 weight gradient
-// keeps all its bits on the tensor cores.
-__global__ void k_bce(const float* __restrict__ prob, const float* __restrict__ label, uint32_t P,
-                      uint4* __restrict__ g8, float* __restrict__ loss_sum) {
-  float acc = 0.f;
-  for (uint32_t p = blockIdx.x * blockDim.x + threadIdx.x; p < P; p += gridDim.x * blockDim.x) {
-    const float q = fminf(fmaxf(prob[p], 1e-7f), 1.f - 1e-7f), y = label[p];
-    acc += -(y * __logf(q) + (1.f - y) * __logf(1.f - q));
-    const float g = prob[p] - y;
-    const float hi = __bfloat162float(__float2bfloat16_rn(g));
-    const float mid = __bfloat162float(__float2bfloat16_rn(g - hi));
-    g8[p] = make_uint4(pack_bf16(hi, mid), pack_bf16(g - hi - mid, 0.f), 0u, 0u);
-  }
-  for (int off = 16; off > 0; off >>= 1) acc += __shfl_down_sync(0xFFFFFFFFu, acc, off);
-  if ((threadIdx.x & 31) == 0) atomicAdd(loss_sum, acc);
-}
-
 // ------------------------------------------------------ weight gradients
 // dW[co][ci][ky][kx] = scale * sum_x dZ[y][x][co] * A[y+ky-1][x+kx-1][ci],
 // db[co] = scale * sum_x dZ[y][x][co]: a contraction over the pixels, on the
 // tensor cores (tcgen05, BF16 operands whose products are exact in FP32).
 // A is the layer's input (AC 16-byte channel chunks per pixel: 4 planar, or 2
 // interleaved for the features), dZ its data gradient (ZC planar chunks: 4,
-// or the single chunk of k_bce whose three parts are added at the end).
+// or the BCE gradient's single chunk, whose three parts are added at the end).
+// All four layers run in one launch, each on its share of the SMs.
 //
 // A persistent CTA takes tiles of 4 rows x 112 pixels. TMA boxes bring the
 // halo of A (6 rows x 114 pixels) and dZ into shared memory as [row][chunk]
@@ -1172,24 +1180,31 @@ __global__ void k_bce(const float* __restrict__ prob, const float* __restrict__ 
 // more the longer the sum. So after every CHAIN K steps 8 epilogue warps add
 // the useful blocks to FP32 registers, rounding to nearest (warp w: TMEM lanes
 // 32 (w % 4), dZ row r = w / 4 of a pair), from one of two accumulator sets
-// while the next group's MMAs fill the other; they also add up dZ for the
-// bias. Every CTA writes two rows of unscaled partial sums (one per r), which
-// k_wgrad_reduce adds in a fixed order: the gradient, and training, is the
-// same bit for bit from run to run.
-// Measured (32 x 32 layer with its reduction, hot L2): 0.078 ms at 1920x1080
-// and 0.033 ms at 960x540, bound by the epilogue's TMEM reads (0.065 / 0.026
-// with CHAIN 7); the FP32 loop through shared memory took 24.0 and 5.94 ms,
-// and 14.46 of a 960x540 training step that now takes 0.33 ms.
+// while the next group's MMAs fill the other; two more warps add up dZ for the
+// bias. After every kWgFlush tiles (more in large images) the registers go out as two rows of unscaled
+// partial sums (one per r) and start again; k_update adds the rows in a fixed
+// order, compensated: the gradient, and training, is the same bit for bit from
+// run to run.
+// Measured (all four layers and the reduction, hot L2): 0.231 ms at 1920x1080,
+// 0.066 at 960x540, 0.017 at 251x143. A tile takes ~2980 cycles, 2190 of them the
+// tensor core's 42 MMAs. The FP32 loop through shared memory took 24 ms for one
+// 32 x 32 layer at 1920x1080, and 14.4 of a 960x540 training step's 14.5 ms.
 // CHAIN = 4 (groups of 4 and 3), or 2 where a CTA has at most kWgFewTiles
-// tiles. Error of a 32 x 32 layer's dW against 64 bits, 2-norm, for dZ of
-// random sign / of one sign, against the earlier FP32 fused-multiply-add loop:
-//   1920x1080 (27 tiles a CTA): loop 2.2e-7 / 6.7e-8; CHAIN 4 2.0e-7 / 4.4e-8;
-//                               2 2.8e-7 / 3.0e-8 (its register sums are long)
-//   960x540 (8): loop 1.9e-7 / 6.3e-8; 4 1.2e-7 / 4.3e-8; 7 1.1e-7 / 8.2e-8
-//   113x5 (1):   loop 5.9e-8 / 4.3e-8; 4 6.0e-8 / 5.2e-8; 2 6.0e-8 / 4.2e-8
+// tiles. Error of a 32 x 32 layer's dW against 64 bits, 2-norm, for dZ of random
+// sign / of one sign, and what that FP32 loop had:
+//   3840x2160  2.8e-7 / 4.4e-8   loop 3.2e-7 / 6.8e-8
+//   1920x1080  1.5e-7 / 4.3e-8        2.2e-7 / 6.7e-8
+//   960x540    1.5e-7 / 4.4e-8        1.9e-7 / 6.3e-8
+//   251x143    7.3e-8 / 4.0e-8        1.1e-7 / 4.8e-8
+//   113x5      6.0e-8 / 4.2e-8        5.9e-8 / 4.3e-8   (CHAIN 2; 4: 6.0e-8 / 5.2e-8)
+// (whole tiles inside the tensor core, CHAIN 7: 2.0e-7 with one sign).
 constexpr int kWgRows = 4, kWgW = 112;                // dZ rows and pixels of a tile
 constexpr uint32_t kWgFewTiles = 2;
-constexpr int kWgEpiWarps = 8, kWgThreads = 32 * (kWgEpiWarps + 2);
+// tiles between flushes of a CTA, and flushes at most (they bound the partial
+// rows: 90 MB for any image)
+constexpr uint32_t kWgFlush = 16, kWgFlushes = 8;
+// 8 epilogue warps, the MMA warp, the TMA warp and two bias warps
+constexpr int kWgEpiWarps = 8, kWgBiasWarps = 2, kWgThreads = 32 * (kWgEpiWarps + 2 + kWgBiasWarps);
 static_assert(kWgRows % 2 == 0 && kWgW % 16 == 0, "row pairs, K steps of 16 pixels");
 
 template <int AC, int ZC>
@@ -1207,8 +1222,7 @@ struct WgradLayout {
   static constexpr int kSt = kFit > 4u ? 4 : (int)kFit;
   static constexpr int kN = 2 * 8 * ZC;                                 // MMA N: two dZ rows
   static constexpr uint32_t kSet = 3 * kN;                              // TMEM columns of one accumulator set
-  static constexpr uint32_t kTmemCols = 2 * kSet <= 128 ? 128 : 512;
-  static constexpr size_t kSmem = kSt * (size_t)kStage + kWgEpiWarps * 8 * 4 + 20 * 8 + 16;
+  static constexpr size_t kSmem = kSt * (size_t)kStage + 4 * 8 * 4 + 20 * 8 + 16;
   static constexpr int kCo = ZC == 4 ? 32 : 1;                          // output channels
   static constexpr int kOuts = 9 * kCo * 8 * AC;                        // partial sums of a row, without the biases
 };
@@ -1226,20 +1240,46 @@ __device__ __forceinline__ void tmem_ld8_nowait(uint32_t taddr, uint32_t r[8]) {
                : "r"(taddr));
 }
 
-// barriers: full[b] TMA bytes of stage b; empty[b] its MMAs (commit) and the
-// 8 epilogue warps' bias sums are done; acc_full[s] / acc_empty[s] as in
-// k_conv_tma. part: 2 gridDim.x rows of kOuts + kCo floats, [tap][co][ci]
-// then [co].
+// (s, c) += x with the rounding error of the sum kept in c (Knuth's TwoSum)
+__device__ __forceinline__ void two_sum(float& s, float& c, float x) {
+  const float t = s + x, b = t - s;
+  c += (s - (t - b)) + (x - b);
+  s = t;
+}
+
+constexpr uint32_t kWgTmemCols = 512;
+
+// a layer's share of the launch: CTAs blk0 .. blk0 + nblk - 1, and the partial
+// rows they write (2 nblk flushes of them, from element part0 on)
+struct WgradShare {
+  uint32_t blk0, nblk, flush_every, flushes;   // a flush every so many tiles of a CTA
+  uint64_t part0;
+};
+struct WgradArgs {
+  CUtensorMap a[4], z[4];        // layers 1 .. 4: input activations, data gradients
+  WgradShare share[4];
+  uint32_t W, H;
+  float* part;
+  uint32_t* err;
+};
+
+// One CTA's tiles of one layer. Barriers: full[b] TMA bytes of stage b;
+// empty[b] its MMAs (commit) and the bias warps' sums are done;
+// acc_full[s] / acc_empty[s] as in k_conv_tma. A partial row is kOuts + kCo
+// floats, [tap][co][ci] then [co].
 template <int AC, int ZC, int CHAIN>
-__global__ void __launch_bounds__(kWgThreads, 1)
-    k_wgrad_tc(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ CUtensorMap map_z,
-               uint32_t W, uint32_t H, float* __restrict__ part, uint32_t* err) {
+__device__ __forceinline__ void wgrad_body(const WgradArgs& args, const int layer, unsigned char* smem) {
   using Lt = WgradLayout<AC, ZC>;
   constexpr int kGroupsRow = (kWgW / 16 + CHAIN - 1) / CHAIN;   // accumulator groups of a row pair
   constexpr int kGroups = kWgRows / 2 * kGroupsRow;             // ... of a tile
-  extern __shared__ __align__(1024) unsigned char smem[];
-  float* bias_s = reinterpret_cast<float*>(smem + Lt::kSt * (size_t)Lt::kStage);   // [8 warps][8]
-  uint64_t* bars = reinterpret_cast<uint64_t*>(bias_s + kWgEpiWarps * 8);
+  const CUtensorMap& map_a = args.a[layer];
+  const CUtensorMap& map_z = args.z[layer];
+  const uint32_t W = args.W, H = args.H, nblk = args.share[layer].nblk;
+  const uint32_t blk = blockIdx.x - args.share[layer].blk0;
+  float* part = args.part + args.share[layer].part0;
+  uint32_t* err = args.err;
+  float* bias_s = reinterpret_cast<float*>(smem + Lt::kSt * (size_t)Lt::kStage);   // [4][8]
+  uint64_t* bars = reinterpret_cast<uint64_t*>(bias_s + 4 * 8);
   uint64_t* full = bars;            // [kSt]
   uint64_t* empty = bars + 8;       // [kSt]
   uint64_t* acc_full = bars + 16;   // [2]
@@ -1253,7 +1293,7 @@ __global__ void __launch_bounds__(kWgThreads, 1)
   if (tid == 0) {
     for (int b = 0; b < Lt::kSt; ++b) {
       mbar_init(full + b, 1);
-      mbar_init(empty + b, 1 + kWgEpiWarps);
+      mbar_init(empty + b, 1 + kWgBiasWarps);
     }
     for (int b = 0; b < 2; ++b) {
       mbar_init(acc_full + b, 1);
@@ -1261,15 +1301,16 @@ __global__ void __launch_bounds__(kWgThreads, 1)
     }
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
-  if (warp == 0) tmem_alloc(tslot, Lt::kTmemCols);
+  if (warp == 0) tmem_alloc(tslot, kWgTmemCols);
   fence_before();
   __syncthreads();
   fence_after();
   const uint32_t tmem = __shfl_sync(0xFFFFFFFFu, *tslot, 0);
-  const uint32_t my_tiles = blockIdx.x < n_tiles ? (n_tiles - 1 - blockIdx.x) / gridDim.x + 1 : 0;
+  const uint32_t my_tiles = blk < n_tiles ? (n_tiles - 1 - blk) / nblk + 1 : 0;
 
   if (warp == kWgEpiWarps) {
     // ---- MMA issue (the whole warp walks the loop, an elected lane issues)
+    asm volatile("setmaxnreg.dec.sync.aligned.u32 80;");
     constexpr uint32_t idesc = make_idesc_mn(128, Lt::kN);
     // LBO: from one group of 8 pixels (K) to the next; SBO: from one
     // (row, chunk) group of 8 channels (M or N) to the next
@@ -1315,13 +1356,14 @@ __global__ void __launch_bounds__(kWgThreads, 1)
       mbar_wait(empty + (it % Lt::kSt), (it / Lt::kSt) & 1u);
   } else if (warp == kWgEpiWarps + 1) {
     // ---- TMA loads
+    asm volatile("setmaxnreg.dec.sync.aligned.u32 80;");
     if (lane == 0) {
       bool ok = true;
       uint32_t n_loaded = 0;
       for (uint32_t j = 0; j < my_tiles; ++j) {
         const int b = (int)(j % Lt::kSt);
         if (j >= (uint32_t)Lt::kSt && !mbar_wait(empty + b, ((j / Lt::kSt) - 1) & 1u)) { ok = false; break; }
-        const uint32_t tile = blockIdx.x + j * gridDim.x;
+        const uint32_t tile = blk + j * nblk;
         const int ty = (int)(tile / tiles_x);
         const int y = ty * kWgRows, x0 = (int)(tile - (uint32_t)ty * tiles_x) * kWgW;
         unsigned char* st = smem + (size_t)b * Lt::kStage;
@@ -1337,163 +1379,230 @@ __global__ void __launch_bounds__(kWgThreads, 1)
         mbar_wait(full + (j % Lt::kSt), (j / Lt::kSt) & 1u);
     }
     __syncwarp();
+  } else if (warp > kWgEpiWarps + 1) {
+    // ---- bias warps: dZ summed over the tile's pixels, tile after tile
+    // compensated (by the epilogue warps it held up the accumulators: 1400 of
+    // 4000 cycles a tile)
+    asm volatile("setmaxnreg.dec.sync.aligned.u32 80;");
+    constexpr int kPer = 32 * kWgBiasWarps / ZC;       // threads that add up one chunk of dZ
+    const int t = tid - 32 * (kWgEpiWarps + 2), zc = t / kPer, zt = t % kPer;
+    float sum[8], comp[8];
+#pragma unroll
+    for (int c = 0; c < 8; ++c) sum[c] = comp[c] = 0.f;
+    bool ok = true;
+    for (uint32_t it = 0; it < my_tiles && ok; ++it) {
+      const int b = (int)(it % Lt::kSt);
+      ok = __all_sync(0xFFFFFFFFu, mbar_wait(full + b, (it / Lt::kSt) & 1u));
+      if (!ok) break;
+      const unsigned char* z = smem + (size_t)b * Lt::kStage + Lt::kOffZ + (uint32_t)zc * Lt::kPitchZ;
+      float part8[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+      constexpr int kLoads = (kWgW + kPer - 1) / kPer;   // of a row
+#pragma unroll 1
+      for (int row = 0; row < kWgRows; ++row) {
+        uint4 v[kLoads];
+#pragma unroll
+        for (int k = 0; k < kLoads; ++k) {
+          const int px = zt + k * kPer;
+          v[k] = px < kWgW ? *reinterpret_cast<const uint4*>(z + (uint32_t)row * Lt::kRowZ + (uint32_t)px * 16u)
+                           : make_uint4(0u, 0u, 0u, 0u);
+        }
+#pragma unroll
+        for (int k = 0; k < kLoads; ++k) {
+          const uint32_t w4[4] = {v[k].x, v[k].y, v[k].z, v[k].w};
+#pragma unroll
+          for (int i = 0; i < 4; ++i)
+            add2(part8[2 * i], part8[2 * i + 1], __uint_as_float(w4[i] << 16), __uint_as_float(w4[i] & 0xFFFF0000u));
+        }
+      }
+      __syncwarp();
+      if (lane == 0) mbar_arrive(empty + b);
+#pragma unroll
+      for (int c = 0; c < 8; ++c) two_sum(sum[c], comp[c], part8[c]);
+    }
+    if (!ok && lane == 0) atomicOr(err, ERR_ITER);
+    // lanes of a chunk (16, or the warp's 32 when there is one chunk), in a fixed order
+    constexpr int kLanes = kPer < 32 ? kPer : 32;
+#pragma unroll
+    for (int c = 0; c < 8; ++c) {
+      sum[c] += comp[c];
+      for (int off = kLanes / 2; off > 0; off >>= 1) sum[c] += __shfl_xor_sync(0xFFFFFFFFu, sum[c], off);
+    }
+    if (lane % kLanes == 0)
+#pragma unroll
+      for (int c = 0; c < 8; ++c) bias_s[(t / kLanes) * 8 + c] = sum[c];
   } else {
-    // ---- epilogue warps
+    // ---- epilogue warps: 256 x 208 + 128 x 80 of the 384 x 168 registers launched with
+    asm volatile("setmaxnreg.inc.sync.aligned.u32 208;");
     constexpr int kCo = Lt::kCo;                        // output channels a thread accumulates
     const int q = warp & 3, r = warp >> 2;
     const int m = q * 32 + lane, h = m / (8 * AC), ci = m % (8 * AC), dy = h - r;
     const bool useful = dy >= 0 && dy <= 2;
     const bool warp_useful = __any_sync(0xFFFFFFFFu, useful);
-    constexpr int kPerChunk = 32 * kWgEpiWarps / ZC;    // threads that add up one chunk of dZ
-    const int zc = tid / kPerChunk, zt = tid % kPerChunk;
-    float acc[3][kCo], bacc[8];
-#pragma unroll
-    for (int dx = 0; dx < 3; ++dx)
-#pragma unroll
-      for (int c = 0; c < kCo; ++c) acc[dx][c] = 0.f;
-#pragma unroll
-    for (int c = 0; c < 8; ++c) bacc[c] = 0.f;
-    uint32_t grp = 0;
+    float acc[3][kCo];
+    uint32_t grp = 0, it = 0;
     bool ok = true;
-    for (uint32_t it = 0; it < my_tiles && ok; ++it) {
-      const int b = (int)(it % Lt::kSt);
-      // warp-uniform outcome: tcgen05.ld below is a warp-collective instruction
-      if (!__all_sync(0xFFFFFFFFu, mbar_wait(full + b, (it / Lt::kSt) & 1u))) { ok = false; break; }
-      const unsigned char* z = smem + (size_t)b * Lt::kStage + Lt::kOffZ + (uint32_t)zc * Lt::kPitchZ;
-      for (int k = zt; k < kWgRows * kWgW; k += kPerChunk) {
-        const int row = k / kWgW, px = k - row * kWgW;
-        const uint4 v = *reinterpret_cast<const uint4*>(z + (uint32_t)row * Lt::kRowZ + (uint32_t)px * 16u);
-        const uint32_t w4[4] = {v.x, v.y, v.z, v.w};
-#pragma unroll
-        for (int i = 0; i < 4; ++i) {
-          const __nv_bfloat162 two = *reinterpret_cast<const __nv_bfloat162*>(&w4[i]);
-          bacc[2 * i] += __bfloat162float(two.x);
-          bacc[2 * i + 1] += __bfloat162float(two.y);
-        }
-      }
-      __syncwarp();
-      if (lane == 0) mbar_arrive(empty + b);
-#pragma unroll 1
-      for (int g = 0; g < kGroups; ++g, ++grp) {
-        const uint32_t s = grp & 1u;
-        if (!__all_sync(0xFFFFFFFFu, mbar_wait(acc_full + s, (grp >> 1) & 1u))) { ok = false; break; }
-        fence_after();
-        if (warp_useful) {
-          const uint32_t at = tmem + ((uint32_t)(q * 32) << 16) + s * Lt::kSet + (uint32_t)(r * 8 * ZC);
-          if (ZC == 4) {
-#pragma unroll
-            for (int dx = 0; dx < 3; ++dx) {
-              uint32_t v[2][16];
-              tmem_ld16_nowait(at + (uint32_t)(dx * Lt::kN), v[0]);
-              tmem_ld16_nowait(at + (uint32_t)(dx * Lt::kN + 16), v[1]);
-              tmem_wait_ld();
-#pragma unroll
-              for (int c = 0; c < kCo; c += 2)
-                add2(acc[dx][c], acc[dx][c + 1], __uint_as_float(v[c / 16][c % 16]),
-                     __uint_as_float(v[c / 16][c % 16 + 1]));
-            }
-          } else {
-            uint32_t v[3][8];
-#pragma unroll
-            for (int dx = 0; dx < 3; ++dx) tmem_ld8_nowait(at + (uint32_t)(dx * Lt::kN), v[dx]);
-            tmem_wait_ld();
-#pragma unroll
-            for (int dx = 0; dx < 3; ++dx)
-              acc[dx][0] += (__uint_as_float(v[dx][2]) + __uint_as_float(v[dx][1])) + __uint_as_float(v[dx][0]);
-          }
-        }
-        fence_before();
-        mbar_arrive(acc_empty + s);
-      }
-    }
-    if (!ok && lane == 0) atomicOr(err, ERR_ITER);
-    // partial sums of this CTA: row 2 blockIdx.x + r, [tap][co][ci]
-    float* row = part + (2 * (size_t)blockIdx.x + r) * (Lt::kOuts + kCo);
-    if (useful)
+    for (uint32_t f = 0; f < args.share[layer].flushes; ++f) {
 #pragma unroll
       for (int dx = 0; dx < 3; ++dx)
 #pragma unroll
-        for (int c = 0; c < kCo; ++c)
-          row[(size_t)((dy * 3 + dx) * kCo + c) * (8 * AC) + ci] = acc[dx][c];
-    // biases: lanes, then the warps of a chunk, in a fixed order
+        for (int c = 0; c < kCo; ++c) acc[dx][c] = 0.f;
+      const uint32_t end = min(my_tiles, (f + 1) * args.share[layer].flush_every);
+      for (; it < end && ok; ++it) {
+        // warp-uniform outcomes: tcgen05.ld below is a warp-collective instruction
+#pragma unroll 1
+        for (int g = 0; g < kGroups; ++g, ++grp) {
+          const uint32_t s = grp & 1u;
+          if (!__all_sync(0xFFFFFFFFu, mbar_wait(acc_full + s, (grp >> 1) & 1u))) { ok = false; break; }
+          fence_after();
+          // every column of the group first, then hand the set back, then add
+          uint32_t v[3][ZC == 4 ? 32 : 8];
+          if (warp_useful) {
+            const uint32_t at = tmem + ((uint32_t)(q * 32) << 16) + s * Lt::kSet + (uint32_t)(r * 8 * ZC);
 #pragma unroll
-    for (int c = 0; c < 8; ++c)
-      for (int off = 16; off > 0; off >>= 1) bacc[c] += __shfl_xor_sync(0xFFFFFFFFu, bacc[c], off);
-    if (lane == 0)
+            for (int dx = 0; dx < 3; ++dx) {
+              if (ZC == 4) {
+                tmem_ld16_nowait(at + (uint32_t)(dx * Lt::kN), v[dx]);
+                tmem_ld16_nowait(at + (uint32_t)(dx * Lt::kN + 16), v[dx] + (ZC == 4 ? 16 : 0));
+              } else {
+                tmem_ld8_nowait(at + (uint32_t)(dx * Lt::kN), v[dx]);
+              }
+            }
+            tmem_wait_ld();
+          }
+          fence_before();
+          mbar_arrive(acc_empty + s);
+          if (warp_useful) {
 #pragma unroll
-      for (int c = 0; c < 8; ++c) bias_s[warp * 8 + c] = bacc[c];
+            for (int dx = 0; dx < 3; ++dx) {
+              if (ZC == 4) {
+#pragma unroll
+                for (int c = 0; c < kCo; c += 2)
+                  add2(acc[dx][c], acc[dx][(c + 1) % kCo], __uint_as_float(v[dx][c]), __uint_as_float(v[dx][c + 1]));
+              } else {
+                acc[dx][0] += (__uint_as_float(v[dx][2]) + __uint_as_float(v[dx][1])) + __uint_as_float(v[dx][0]);
+              }
+            }
+          }
+        }
+      }
+      // partial sums since the last flush (zeros where a CTA has fewer than
+      // others): row 2 (f nblk + blk) + r, [tap][co][ci]
+      if (useful) {
+        float* row = part + (2 * ((size_t)f * nblk + blk) + r) * (Lt::kOuts + kCo) + (size_t)(dy * 3 * kCo) * (8 * AC) + ci;
+#pragma unroll
+        for (int dx = 0; dx < 3; ++dx)
+#pragma unroll
+          for (int c = 0; c < kCo; ++c) row[(dx * kCo + c) * (8 * AC)] = acc[dx][c];
+      }
+    }
+    if (!ok && lane == 0) atomicOr(err, ERR_ITER);
   }
   fence_before();
   __syncthreads();
   fence_after();
-  constexpr int kCo = Lt::kCo, kBiasAt = Lt::kOuts, kWarpsPer = kWgEpiWarps / ZC;
+  constexpr int kCo = Lt::kCo, kBiasAt = Lt::kOuts;
   if (tid < kCo) {
-    float t = 0.f;
-    for (int w = 0; w < kWarpsPer; ++w) {
-      const float* p = bias_s + ((tid / 8) * kWarpsPer + w) * 8;
-      t += ZC == 4 ? p[tid % 8] : (p[2] + p[1]) + p[0];
-    }
-    float* row = part + 2 * (size_t)blockIdx.x * (kBiasAt + kCo);
-    row[kBiasAt + tid] = t;
-    row[kBiasAt + kCo + kBiasAt + tid] = 0.f;
+    // four chunks of 8 channels, or the two halves of the one chunk's pixels
+    const float t = ZC == 4 ? bias_s[tid]
+                            : ((bias_s[2] + bias_s[10]) + (bias_s[1] + bias_s[9])) + (bias_s[0] + bias_s[8]);
+    for (uint32_t f = 0; f < args.share[layer].flushes; ++f)
+      for (uint32_t r = 0; r < 2; ++r)
+        part[(2 * ((size_t)f * nblk + blk) + r) * (kBiasAt + kCo) + kBiasAt + tid] = f + r == 0 ? t : 0.f;
   }
-  if (warp == 0) tmem_dealloc(tmem, Lt::kTmemCols);
+  if (warp == 0) tmem_dealloc(tmem, kWgTmemCols);
 }
 
-// (s, c) += x with the rounding error of the sum kept in c (Knuth's TwoSum)
-__device__ __forceinline__ void two_sum(float& s, float& c, float x) {
-  const float t = s + x, b = t - s;
-  c += (s - (t - b)) + (x - b);
-  s = t;
+template <int CHAIN>
+__global__ void __launch_bounds__(kWgThreads, 1) k_wgrad(const __grid_constant__ WgradArgs args) {
+  extern __shared__ __align__(1024) unsigned char smem[];
+  if (blockIdx.x < args.share[1].blk0) wgrad_body<2, 4, CHAIN>(args, 0, smem);
+  else if (blockIdx.x < args.share[2].blk0) wgrad_body<4, 4, CHAIN>(args, 1, smem);
+  else if (blockIdx.x < args.share[3].blk0) wgrad_body<4, 4, CHAIN>(args, 2, smem);
+  else wgrad_body<4, 1, CHAIN>(args, 3, smem);
 }
 
-// out = scale * the partial rows' sum, in a fixed order and compensated (the
-// FP32 rounding of some hundred rows would cost more precision than the tensor
-// cores do): warp w of a block adds rows w, w + 8, w + 16, ... of 32
-// consecutive columns, then threads 0..31 add the 8 warp sums in warp order.
-// Column j is [tap][co][cin_p] (or, from n_w on, a bias); out is the
-// canonical W[co][cin][9] then b[co].
-__global__ void __launch_bounds__(256) k_wgrad_reduce(const float* __restrict__ part, uint32_t nrow,
-                                                      uint32_t cout, uint32_t cin, uint32_t cin_p,
-                                                      float scale, float* __restrict__ out) {
+// ------------------------------------------ reduction, Adam and packing
+// One launch for everything after the gradients' contractions, all layers:
+// 32 columns of a layer's partial rows per block. grad = scale * the rows' sum,
+// in a fixed order and compensated (the FP32 rounding of some hundred rows
+// would cost more precision than the tensor cores do): warp w adds rows w,
+// w + 8, w + 16, ..., then threads 0..31 add the 8 warp sums in warp order.
+// Column j is [tap][co][cin_p] (or, from n_w on, a bias). With an update, Adam
+// on the parameter, whose new value goes into the packed weights of the forward
+// and the data-gradient kernels (their zero padding never changes). Block 0
+// also adds up the loss.
+struct UpdateLayer {
+  uint32_t block0;               // first block of the layer
+  uint32_t nrow, cout, cin, cin_p, off_w, off_b;
+  uint64_t part0;
+  __nv_bfloat16* wf;
+  __nv_bfloat16* wb;             // null: none (layer 1)
+};
+struct UpdateArgs {
+  UpdateLayer layer[4];
+  const float* part;
+  float scale;                   // 1 / P
+  float* grads;                  // null: not wanted
+  float *w, *m, *v;              // m null: no update
+  float lr, c1, c2;              // step size and Adam's bias corrections
+  const float* loss_part;
+  uint32_t n_loss;
+  float* loss;
+};
+
+__global__ void __launch_bounds__(256) k_update(const __grid_constant__ UpdateArgs a) {
   __shared__ float s[8][32], sc[8][32];
   const uint32_t lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const uint32_t n_w = 9 * cout * cin_p, n = n_w + cout;
-  const uint32_t j = blockIdx.x * 32 + lane;
-  float a = 0.f, c = 0.f;
-  if (j < n)
+  int l = 3;
+  while (l > 0 && blockIdx.x < a.layer[l].block0) --l;
+  const UpdateLayer& y = a.layer[l];
+  const uint32_t n_w = 9 * y.cout * y.cin_p, n = n_w + y.cout;
+  const uint32_t j = (blockIdx.x - y.block0) * 32 + lane;
+  float t = 0.f, c = 0.f;
+  if (j < n) {
+    const float* part = a.part + y.part0 + j;
 #pragma unroll 8
-    for (uint32_t b = warp; b < nrow; b += 8) two_sum(a, c, part[(size_t)b * n + j]);
-  s[warp][lane] = a;
+    for (uint32_t b = warp; b < y.nrow; b += 8) two_sum(t, c, part[(size_t)b * n]);
+  }
+  s[warp][lane] = t;
   sc[warp][lane] = c;
   __syncthreads();
-  if (warp == 0 && j < n) {
-#pragma unroll
-    for (int w = 1; w < 8; ++w) {
-      c += sc[w][lane];
-      two_sum(a, c, s[w][lane]);
-    }
-    const float t = (a + c) * scale;
-    if (j >= n_w) {
-      out[9 * cout * cin + (j - n_w)] = t;
-    } else {
-      const uint32_t ci = j % cin_p, co = (j / cin_p) % cout, tap = j / (cin_p * cout);
-      if (ci < cin) out[(co * cin + ci) * 9 + tap] = t;
-    }
+  if (warp == 1 && blockIdx.x == 0) {
+    float acc = 0.f, e = 0.f;
+    for (uint32_t i = lane; i < a.n_loss; i += 32) two_sum(acc, e, a.loss_part[i]);
+    acc += e;
+    for (int off = 16; off > 0; off >>= 1) acc += __shfl_xor_sync(0xFFFFFFFFu, acc, off);
+    if (lane == 0) *a.loss = acc;
   }
-}
-
-// ---------------------------------------------------------------- Adam
-__global__ void k_adam(float* __restrict__ w, const float* __restrict__ g, float* __restrict__ m,
-                       float* __restrict__ v, uint32_t n, float lr, float b1, float b2, float eps,
-                       float c1, float c2) {
-  for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
-    const float gi = g[i];
-    const float mi = b1 * m[i] + (1.f - b1) * gi;
-    const float vi = b2 * v[i] + (1.f - b2) * gi * gi;
-    m[i] = mi;
-    v[i] = vi;
-    w[i] -= lr * (mi / c1) / (sqrtf(vi / c2) + eps);
+  if (warp != 0 || j >= n) return;
+#pragma unroll
+  for (int w = 1; w < 8; ++w) {
+    c += sc[w][lane];
+    two_sum(t, c, s[w][lane]);
+  }
+  const float g = (t + c) * a.scale;
+  const uint32_t ci = j % y.cin_p, co = j < n_w ? (j / y.cin_p) % y.cout : j - n_w, tap = j / (y.cin_p * y.cout);
+  if (j < n_w && ci >= y.cin) return;                   // a padding channel
+  const uint32_t at = j < n_w ? y.off_w + (co * y.cin + ci) * 9 + tap : y.off_b + co;
+  if (a.grads) a.grads[at] = g;
+  if (!a.m) return;
+  constexpr float b1 = 0.9f, b2 = 0.999f, eps = 1e-8f;
+  const float mi = b1 * a.m[at] + (1.f - b1) * g;
+  const float vi = b2 * a.v[at] + (1.f - b2) * g * g;
+  a.m[at] = mi;
+  a.v[at] = vi;
+  const float w = a.w[at] - a.lr * (mi / a.c1) / (sqrtf(vi / a.c2) + eps);
+  a.w[at] = w;
+  if (j >= n_w) return;
+  const __nv_bfloat16 wb = __float2bfloat16_rn(w);
+  const uint32_t dy = tap / 3, dx = tap - 3 * dy;
+  if (l < 3)   // stacked taps, as k_pack_fwd
+    y.wf[((dx * (y.cin_p / 8) + ci / 8) * (3 * y.cout) + (2 - dy) * y.cout + co) * 8 + ci % 8] = wb;
+  else         // taps along N, as k_pack_taps
+    y.wf[(ci / 8) * 128 + tap * 8 + ci % 8] = wb;
+  if (y.wb) {  // flipped taps, channels swapped, as k_pack_bwd
+    const uint32_t cout_p = l == 3 ? 16u : 32u, fy = 2 - dy, fx = 2 - dx;
+    y.wb[((fx * (cout_p / 8) + co / 8) * (3 * y.cin_p) + (2 - fy) * y.cin_p + ci) * 8 + co % 8] = wb;
   }
 }
 
@@ -1545,7 +1654,7 @@ cudaError_t make_halo_map(CUtensorMap* map, const void* in, uint32_t W, uint32_t
   return r == CUDA_SUCCESS ? cudaSuccess : cudaErrorInvalidValue;
 }
 
-// One map of W x H pixels for k_wgrad_tc: `chunks` 16-byte channel chunks per
+// One map of W x H pixels for k_wgrad: `chunks` 16-byte channel chunks per
 // pixel, interleaved ([P][16], 2 chunks) as {8 channels, W, chunks, H} or
 // planar ([chunks][P][8]) as 8-byte elements {2 W, chunks, H}; the box is
 // `px` pixels of every chunk in `rows` rows, in shared memory [row][chunk][px].
@@ -1577,37 +1686,35 @@ uint64_t wgrad_tiles(uint32_t W, uint32_t H) {
   return (uint64_t)((W + kWgW - 1) / kWgW) * ((H + kWgRows - 1) / kWgRows);
 }
 
-// Weight and bias gradients of one layer: k_wgrad_tc over all pixels, then
-// the reduction of its partial rows into out (canonical layout).
-template <int AC, int ZC>
-cudaError_t launch_wgrad(const void* a, const void* dz, uint32_t W, uint32_t H, uint32_t cin,
-                         float scale, float* part, float* out, uint32_t* err, cudaStream_t st) {
-  using Lt = WgradLayout<AC, ZC>;
-  // more than half of an SM's shared memory: one CTA (and its TMEM) per SM
-  constexpr size_t smem = Lt::kSmem < 116u * 1024u ? 116u * 1024u : Lt::kSmem;
-  static bool configured = false;
-  if (!configured) {
-    cudaError_t e = cudaFuncSetAttribute(k_wgrad_tc<AC, ZC, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)smem);
-    if (e == cudaSuccess)
-      e = cudaFuncSetAttribute(k_wgrad_tc<AC, ZC, 4>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-    configured = true;
-  }
-  CUtensorMap ma, mz;
-  cudaError_t e = make_wgrad_map(&ma, a, W, H, AC, AC == 2, kWgW + 2, kWgRows + 2);
-  if (e == cudaSuccess) e = make_wgrad_map(&mz, dz, W, H, ZC, false, kWgW, kWgRows);
-  if (e != cudaSuccess) return e;
+// Shares of the SMs: the next CTA always goes to the layer that would take
+// longest (tiles a CTA times a tile's cost; at most one CTA per tile)
+void wgrad_shares(uint32_t W, uint32_t H, WgradShare share[4], uint64_t* part_floats) {
+  static const float kCost[4] = {0.8f, 1.f, 1.f, 0.8f};
   const uint64_t tiles = wgrad_tiles(W, H);
-  const int grid = (int)std::min<uint64_t>(tiles, (uint64_t)num_sms());   // one CTA per SM
-  if (tiles <= (uint64_t)kWgFewTiles * (uint64_t)grid)
-    k_wgrad_tc<AC, ZC, 2><<<grid, kWgThreads, smem, st>>>(ma, mz, W, H, part, err);
-  else
-    k_wgrad_tc<AC, ZC, 4><<<grid, kWgThreads, smem, st>>>(ma, mz, W, H, part, err);
-  const uint32_t n = (uint32_t)(Lt::kOuts + Lt::kCo);
-  k_wgrad_reduce<<<(n + 31) / 32, 256, 0, st>>>(part, 2u * (uint32_t)grid, (uint32_t)Lt::kCo, cin,
-                                                8u * AC, scale, out);
-  return cudaGetLastError();
+  uint32_t nb[4] = {1, 1, 1, 1};
+  for (int used = 4; used < num_sms(); ++used) {
+    int at = -1;
+    float most = 0.f;
+    for (int l = 0; l < 4; ++l) {
+      const float t = (float)((tiles + nb[l] - 1) / nb[l]) * kCost[l];
+      if (nb[l] < tiles && t > most) { most = t; at = l; }
+    }
+    if (at < 0) break;
+    ++nb[at];
+  }
+  static const uint32_t kRow[4] = {WgradLayout<2, 4>::kOuts + 32, WgradLayout<4, 4>::kOuts + 32,
+                                   WgradLayout<4, 4>::kOuts + 32, WgradLayout<4, 1>::kOuts + 1};
+  uint32_t blk = 0;
+  uint64_t at = 0;
+  for (int l = 0; l < 4; ++l) {
+    const uint32_t most = (uint32_t)((tiles + nb[l] - 1) / nb[l]);   // tiles of a CTA
+    const uint32_t every = std::max(kWgFlush, (most + kWgFlushes - 1) / kWgFlushes);
+    const uint32_t flushes = (most + every - 1) / every;
+    share[l] = {blk, nb[l], every, flushes, at};
+    blk += nb[l];
+    at += 2ull * nb[l] * flushes * kRow[l];
+  }
+  *part_floats = at;
 }
 
 // data gradient of a layer: `in` holds `chunks` planes (CIN / 8 at most)
@@ -1678,7 +1785,7 @@ cudaError_t make_feature_map(CUtensorMap* map, const void* in, uint32_t W, uint3
 
 template <bool FP8, bool STORE>
 cudaError_t launch_fused(const __nv_bfloat16* feat16, FusedArgs& a, uint32_t W, uint32_t H,
-                         uint32_t n_img, cudaStream_t st) {
+                         uint32_t n_img, cudaStream_t st, int* grid_out = nullptr) {
   using Lt = FusedLayout<FP8>;
   // a CTA takes all TMEM columns: more than half of an SM's shared memory, so
   // that no second one can be placed beside it
@@ -1708,7 +1815,9 @@ cudaError_t launch_fused(const __nv_bfloat16* feat16, FusedArgs& a, uint32_t W, 
     rows = std::min(rows - 1, (H + segs) / (segs + 1));   // one more segment, shorter by a row at least
   }
   const uint64_t items = strips * a.segs;
-  k_net_fused<FP8, STORE><<<(int)std::min(items, sms), kFuThreads, smem, st>>>(map, a);
+  const int grid = (int)std::min(items, sms);
+  if (grid_out) *grid_out = grid;
+  k_net_fused<FP8, STORE><<<grid, kFuThreads, smem, st>>>(map, a);
   return cudaGetLastError();
 }
 }  // namespace
@@ -1766,43 +1875,88 @@ cudaError_t activation_amax(const __nv_bfloat16* const act[3], uint64_t P, unsig
   return cudaGetLastError();
 }
 
-// gradients of the mean BCE loss into grads (same layout as params); the
-// forward activations must be those of the same features and params
-cudaError_t backward(const __nv_bfloat16* feat16, const float* label, __nv_bfloat16* const wb[4],
-                     const __nv_bfloat16* act1, const __nv_bfloat16* act2,
-                     const __nv_bfloat16* act3, const float* prob, __nv_bfloat16* g8,
-                     __nv_bfloat16* dz_a, __nv_bfloat16* dz_b, float* wpart, float* grads,
-                     float* loss_sum, uint32_t W, uint32_t H, uint32_t* err, cudaStream_t st) {
-  const uint32_t P = W * H;
-  const float scale = 1.f / (float)P;
-  cudaMemsetAsync(loss_sum, 0, sizeof(float), st);
-  k_bce<<<num_sms() * 8, 256, 0, st>>>(prob, label, P, reinterpret_cast<uint4*>(g8), loss_sum);
-  // layer 4: dW from the three parts of g, data gradient into dz_a (masked by act3 > 0)
-  cudaError_t e = launch_wgrad<4, 1>(act3, g8, W, H, kCin[3], scale, wpart, grads + kOffW[3], err, st);
-  if (e != cudaSuccess) return e;
-  e = launch_conv<16>(g8, 1, wb[3], act3, dz_a, W, H, err, st);
-  if (e != cudaSuccess) return e;
-  // layer 3
-  e = launch_wgrad<4, 4>(act2, dz_a, W, H, kCin[2], scale, wpart, grads + kOffW[2], err, st);
-  if (e != cudaSuccess) return e;
-  e = launch_conv<32>(dz_a, 4, wb[2], act2, dz_b, W, H, err, st);
-  if (e != cudaSuccess) return e;
-  // layer 2
-  e = launch_wgrad<4, 4>(act1, dz_b, W, H, kCin[1], scale, wpart, grads + kOffW[1], err, st);
-  if (e != cudaSuccess) return e;
-  e = launch_conv<32>(dz_b, 4, wb[1], act1, dz_a, W, H, err, st);
-  if (e != cudaSuccess) return e;
-  // layer 1 (no data gradient for the input features)
-  return launch_wgrad<2, 4>(feat16, dz_a, W, H, kCin[0], scale, wpart, grads + kOffW[0], err, st);
+size_t wgrad_part_floats(uint32_t W, uint32_t H) {
+  WgradShare share[4];
+  uint64_t floats = 0;
+  wgrad_shares(W, H, share, &floats);
+  return (size_t)floats;
 }
 
-size_t wgrad_part_floats() { return 2u * (size_t)num_sms() * (32u * 32u * 9u + 32u); }
+int loss_parts() { return 4 * num_sms(); }
 
-cudaError_t adam(float* params, const float* grads, float* m, float* v, uint32_t n, float lr,
-                 uint32_t step, cudaStream_t st) {
-  const float b1 = 0.9f, b2 = 0.999f, eps = 1e-8f;
-  const float c1 = 1.f - powf(b1, (float)step), c2 = 1.f - powf(b2, (float)step);
-  k_adam<<<(n + 255) / 256, 256, 0, st>>>(params, grads, m, v, n, lr, b1, b2, eps, c1, c2);
+// One training step on the mean BCE: forward with its activations kept, data
+// gradients of layers 4 to 2, weight gradients of all layers, and the update.
+cudaError_t train_step(const __nv_bfloat16* feat16, const float* label, const TrainBuffers& t, uint32_t W,
+                       uint32_t H, float lr, uint32_t step, float* grads, uint32_t* err, cudaStream_t st) {
+  FusedArgs f = {};
+  for (int l = 0; l < 4; ++l) {
+    f.w[l] = t.wf[l];
+    f.bias[l] = t.params + kOffB[l];
+    f.out_scale[l] = 1.f;
+  }
+  for (int l = 0; l < 3; ++l) f.act[l] = t.act[l];
+  f.label = label;
+  f.g8 = reinterpret_cast<uint4*>(t.g8);
+  f.loss_part = t.loss_part;
+  f.err = err;
+  int fwd_grid = 0;
+  cudaError_t e = launch_fused<false, true>(feat16, f, W, H, 1, st, &fwd_grid);
+  if (e == cudaSuccess) e = launch_conv<16>(t.g8, 1, t.wb[3], t.act[2], t.dz[0], W, H, err, st);
+  if (e == cudaSuccess) e = launch_conv<32>(t.dz[0], 4, t.wb[2], t.act[1], t.dz[1], W, H, err, st);
+  if (e == cudaSuccess) e = launch_conv<32>(t.dz[1], 4, t.wb[1], t.act[0], t.dz[2], W, H, err, st);
+  if (e != cudaSuccess) return e;
+
+  // weight gradients: layer l + 1 from its input and its data gradient
+  WgradArgs g;
+  const void* in[4] = {feat16, t.act[0], t.act[1], t.act[2]};
+  const void* dz[4] = {t.dz[2], t.dz[1], t.dz[0], t.g8};
+  for (int l = 0; l < 4 && e == cudaSuccess; ++l) {
+    const uint32_t zc = l == 3 ? 1 : 4;
+    e = make_wgrad_map(&g.a[l], in[l], W, H, l == 0 ? 2 : 4, l == 0, kWgW + 2, kWgRows + 2);
+    if (e == cudaSuccess) e = make_wgrad_map(&g.z[l], dz[l], W, H, zc, false, kWgW, kWgRows);
+  }
+  if (e != cudaSuccess) return e;
+  uint64_t floats = 0;
+  wgrad_shares(W, H, g.share, &floats);
+  g.W = W;
+  g.H = H;
+  g.part = t.wpart;
+  g.err = err;
+  // the largest layer's stages; one CTA (and its TMEM) per SM
+  constexpr size_t smem = std::max(std::max(WgradLayout<2, 4>::kSmem, WgradLayout<4, 4>::kSmem),
+                                   std::max(WgradLayout<4, 1>::kSmem, (size_t)116 * 1024));
+  static bool configured = false;
+  if (!configured) {
+    e = cudaFuncSetAttribute(k_wgrad<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(k_wgrad<4>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e != cudaSuccess) return e;
+    configured = true;
+  }
+  const uint32_t grid = g.share[3].blk0 + g.share[3].nblk;
+  if (wgrad_tiles(W, H) <= (uint64_t)kWgFewTiles * g.share[1].nblk) k_wgrad<2><<<grid, kWgThreads, smem, st>>>(g);
+  else k_wgrad<4><<<grid, kWgThreads, smem, st>>>(g);
+
+  UpdateArgs u = {};
+  uint32_t block = 0;
+  for (int l = 0; l < 4; ++l) {
+    const uint32_t n = 9u * (uint32_t)(kCout[l] * kCinPad[l]) + (uint32_t)kCout[l];
+    u.layer[l] = {block, 2u * g.share[l].nblk * g.share[l].flushes, (uint32_t)kCout[l], (uint32_t)kCin[l],
+                  (uint32_t)kCinPad[l], kOffW[l], kOffB[l], g.share[l].part0, t.wf[l], l ? t.wb[l] : nullptr};
+    block += (n + 31) / 32;
+  }
+  u.part = t.wpart;
+  u.scale = 1.f / (float)(W * H);
+  u.grads = grads;
+  u.w = t.params;
+  u.v = t.v;
+  if (lr > 0.f) u.m = t.m;
+  u.lr = lr;
+  u.c1 = 1.f - powf(0.9f, (float)step);
+  u.c2 = 1.f - powf(0.999f, (float)step);
+  u.loss_part = t.loss_part;
+  u.n_loss = 4u * (uint32_t)fwd_grid;
+  u.loss = t.loss;
+  k_update<<<block, 256, 0, st>>>(u);
   return cudaGetLastError();
 }
 

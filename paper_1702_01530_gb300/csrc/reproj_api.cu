@@ -22,7 +22,6 @@ using rt::fail;
 struct rt_net {
   void* block = nullptr;        // params, grads, Adam m and v, packed weights, scalars
   float* params = nullptr;
-  float* grads = nullptr;
   float* m = nullptr;
   float* v = nullptr;
   __nv_bfloat16* wf[4] = {};
@@ -36,7 +35,9 @@ struct rt_net {
   __nv_bfloat16* act[3] = {};
   float* prob = nullptr;
   __nv_bfloat16* g8 = nullptr;  // BCE gradient, 8 channels
-  __nv_bfloat16* dz[2] = {};
+  __nv_bfloat16* dz[3] = {};
+  float* loss_part = nullptr;   // partial sums of the loss
+  uint64_t part_floats = 0;     // size of wpart
   float* wpart = nullptr;       // per-CTA partial sums of the weight gradients
   // FP8 inference (rt_net_set_fp8): E4M3 weights of layers 2-4, their
   // per-output-channel scales and the inverse scales the epilogues apply
@@ -62,23 +63,27 @@ cudaError_t net_forward(rt_net* net, const __nv_bfloat16* feat16, float* prob, u
                              net->err, st, n_img);
 }
 
-// training and calibration scratch for maps of P pixels
-int net_buffers(rt_net* net, uint64_t P) {
-  if (net->tb && net->tcap >= P) return RT_OK;
-  const size_t b_act = a256(P * 32 * 2), b_prob = a256(P * 4), b_g8 = a256(P * 8 * 2),
-               b_part = a256(rt::nn::wgrad_part_floats() * 4);
+// training and calibration scratch for maps of W x H pixels
+int net_buffers(rt_net* net, uint32_t W, uint32_t H) {
+  const uint64_t P = (uint64_t)W * H, floats = rt::nn::wgrad_part_floats(W, H);
+  if (net->tb && net->tcap >= P && net->part_floats >= floats) return RT_OK;
+  const uint64_t cap = std::max(net->tcap, P), part = std::max(net->part_floats, floats);
+  const size_t b_act = a256(cap * 32 * 2), b_prob = a256(cap * 4), b_g8 = a256(cap * 8 * 2),
+               b_part = a256(part * 4), b_loss = a256((size_t)rt::nn::loss_parts() * 4);
   void* base = nullptr;
-  cudaError_t e = cudaMalloc(&base, 3 * b_act + b_prob + b_g8 + 2 * b_act + b_part);
+  cudaError_t e = cudaMalloc(&base, 6 * b_act + b_prob + b_g8 + b_part + b_loss);
   if (e != cudaSuccess) { cudaGetLastError(); return cuda_fail(e, "network activations"); }
   if (net->tb) cudaFree(net->tb);
   net->tb = base;
-  net->tcap = P;
+  net->tcap = cap;
+  net->part_floats = part;
   char* p = static_cast<char*>(base);
   for (int i = 0; i < 3; ++i) { net->act[i] = reinterpret_cast<__nv_bfloat16*>(p); p += b_act; }
   net->prob = reinterpret_cast<float*>(p); p += b_prob;
   net->g8 = reinterpret_cast<__nv_bfloat16*>(p); p += b_g8;
-  for (int i = 0; i < 2; ++i) { net->dz[i] = reinterpret_cast<__nv_bfloat16*>(p); p += b_act; }
-  net->wpart = reinterpret_cast<float*>(p);
+  for (int i = 0; i < 3; ++i) { net->dz[i] = reinterpret_cast<__nv_bfloat16*>(p); p += b_act; }
+  net->wpart = reinterpret_cast<float*>(p); p += b_part;
+  net->loss_part = reinterpret_cast<float*>(p);
   return RT_OK;
 }
 
@@ -164,11 +169,10 @@ int rt_net_create(const float* host_params, uint32_t n_params, rt_net** out) {
   for (int l = 0; l < 4; ++l) bw += a256(rt::nn::packed_fwd_elems(l) * 2) + a256(rt::nn::packed_bwd_elems(l) * 2);
   size_t b8 = 256;                                          // amax
   for (int l = 1; l < 4; ++l) b8 += a256(rt::nn::packed_fp8_bytes(l)) + 2 * 256;
-  cudaError_t e = cudaMalloc(&net->block, 4 * bp + bw + 512 + b8);
+  cudaError_t e = cudaMalloc(&net->block, 3 * bp + bw + 512 + b8);
   if (e != cudaSuccess) { cudaGetLastError(); delete net; return cuda_fail(e, "network allocation"); }
   char* p = static_cast<char*>(net->block);
   net->params = reinterpret_cast<float*>(p); p += bp;
-  net->grads = reinterpret_cast<float*>(p); p += bp;
   net->m = reinterpret_cast<float*>(p); p += bp;
   net->v = reinterpret_cast<float*>(p); p += bp;
   for (int l = 0; l < 4; ++l) {
@@ -271,7 +275,7 @@ int rt_net_activation_amax(rt_net* net, const uint16_t* d_feat16, uint32_t W, ui
                            float* host_amax, void* cuda_stream) {
   if (!net || !d_feat16 || !host_amax || W < 1 || H < 1) return fail(RT_ERR_INVALID_ARG, "bad argument");
   if ((uint64_t)W * H > (1ull << 30)) return fail(RT_ERR_INVALID_ARG, "image too large");
-  int rc = net_buffers(net, (uint64_t)W * H);
+  int rc = net_buffers(net, W, H);
   if (rc) return rc;
   cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
   cudaError_t e = cudaMemsetAsync(net->amax, 0, 3 * sizeof(unsigned), st);
@@ -293,7 +297,7 @@ int rt_net_calibrate_fp8(rt_net* net, const uint16_t* const* d_feats, uint32_t n
   if ((uint64_t)W * H > (1ull << 30)) return fail(RT_ERR_INVALID_ARG, "image too large");
   for (uint32_t i = 0; i < n_maps; ++i)
     if (!d_feats[i]) return fail(RT_ERR_INVALID_ARG, "feature map " + std::to_string(i) + " is NULL");
-  int rc = net_buffers(net, (uint64_t)W * H);
+  int rc = net_buffers(net, W, H);
   if (rc) return rc;
   cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
   // maxima of the BF16 network's three hidden activations over every map
@@ -409,23 +413,20 @@ int rt_net_train_step(rt_net* net, const uint16_t* d_feat16, const float* d_labe
     return fail(RT_ERR_INVALID_ARG, "bad argument");
   if ((uint64_t)W * H > (1ull << 30)) return fail(RT_ERR_INVALID_ARG, "image too large");
   const uint64_t P = (uint64_t)W * H;
-  int rc = net_buffers(net, P);
+  int rc = net_buffers(net, W, H);
   if (rc) return rc;
   cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
-  const __nv_bfloat16* f16 = reinterpret_cast<const __nv_bfloat16*>(d_feat16);
-  cudaError_t e = rt::nn::forward(f16, net->params, net->wf, net->act, net->prob, W, H, net->err,
-                                  st);
-  if (e == cudaSuccess)
-    e = rt::nn::backward(f16, d_label, net->wb, net->act[0], net->act[1], net->act[2], net->prob,
-                         net->g8, net->dz[0], net->dz[1], net->wpart, net->grads,
-                         net->loss, W, H, net->err, st);
-  if (e == cudaSuccess && d_grads)
-    e = cudaMemcpyAsync(d_grads, net->grads, (size_t)rt::nn::kParams * 4, cudaMemcpyDeviceToDevice, st);
-  if (e == cudaSuccess && lr > 0.f) {
-    net->step += 1;
-    e = rt::nn::adam(net->params, net->grads, net->m, net->v, rt::nn::kParams, lr, net->step, st);
-    if (e == cudaSuccess) e = rt::nn::pack_weights(net->params, net->wf, net->wb, st);
-  }
+  rt::nn::TrainBuffers t = {};
+  t.params = net->params; t.m = net->m; t.v = net->v;
+  for (int l = 0; l < 4; ++l) { t.wf[l] = net->wf[l]; t.wb[l] = net->wb[l]; }
+  for (int i = 0; i < 3; ++i) { t.act[i] = net->act[i]; t.dz[i] = net->dz[i]; }
+  t.g8 = net->g8;
+  t.wpart = net->wpart;
+  t.loss_part = net->loss_part;
+  t.loss = net->loss;
+  cudaError_t e = rt::nn::train_step(reinterpret_cast<const __nv_bfloat16*>(d_feat16), d_label, t, W, H, lr,
+                                     net->step + 1, d_grads, net->err, st);
+  if (e == cudaSuccess && lr > 0.f) net->step += 1;
   if (e == cudaSuccess && host_loss) {
     float sum = 0.f;
     e = cudaMemcpyAsync(&sum, net->loss, 4, cudaMemcpyDeviceToHost, st);

@@ -232,16 +232,24 @@ cudaError_t pack_weights(const float* params, __nv_bfloat16* const wf[4], __nv_b
 cudaError_t forward(const __nv_bfloat16* feat16, const float* params, __nv_bfloat16* const wf[4],
                     __nv_bfloat16* const act[3], float* prob, uint32_t W, uint32_t H, uint32_t* err,
                     cudaStream_t st, uint32_t n_img = 1);
-cudaError_t backward(const __nv_bfloat16* feat16, const float* label, __nv_bfloat16* const wb[4],
-                     const __nv_bfloat16* act1, const __nv_bfloat16* act2,
-                     const __nv_bfloat16* act3, const float* prob, __nv_bfloat16* g8,
-                     __nv_bfloat16* dz_a, __nv_bfloat16* dz_b, float* wpart, float* grads,
-                     float* loss_sum, uint32_t W, uint32_t H, uint32_t* err, cudaStream_t st);
-// floats of the weight gradients' partial-sum buffer (two rows of a layer's
-// gradients per CTA, any image size)
-size_t wgrad_part_floats();
-cudaError_t adam(float* params, const float* grads, float* m, float* v, uint32_t n, float lr,
-                 uint32_t step, cudaStream_t st);
+// buffers of a training step on maps of P pixels
+struct TrainBuffers {
+  float *params, *m, *v;             // kParams each
+  __nv_bfloat16* wf[4];              // packed weights, updated with the parameters
+  __nv_bfloat16* wb[4];
+  __nv_bfloat16* act[3];             // hidden activations, planar
+  __nv_bfloat16* dz[3];              // data gradients of layers 3, 2, 1, planar
+  __nv_bfloat16* g8;                 // BCE gradient, 8 channels per pixel
+  float* wpart;                      // wgrad_part_floats partial sums
+  float* loss_part;                  // loss_parts partial sums of the loss
+  float* loss;                       // sum of the pixels' losses
+};
+size_t wgrad_part_floats(uint32_t W, uint32_t H);
+int loss_parts();
+// forward, backward and (lr > 0) the Adam update number `step`; grads (or
+// null): kParams floats, device
+cudaError_t train_step(const __nv_bfloat16* feat16, const float* label, const TrainBuffers& t, uint32_t W,
+                       uint32_t H, float lr, uint32_t step, float* grads, uint32_t* err, cudaStream_t st);
 size_t packed_fp8_bytes(int l);
 cudaError_t pack_weights_fp8(const float* params, const float* const scale[3], uint8_t* const w8[3],
                              cudaStream_t st);

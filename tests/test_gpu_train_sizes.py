@@ -1,9 +1,10 @@
 """Weight gradients on the tensor cores at the edges of their tiles.
 
-The kernel takes tiles of 112 x 4 pixels, one CTA per SM, and sums 2 K steps of
-16 pixels inside the tensor core where a CTA has at most 2 tiles, else 4. Sizes
-on both sides of a tile edge, a single pixel, and enough tiles for the longer
-sums, against the oracle's backward pass in float64 that rounds to BF16 where
+The kernel takes tiles of 112 x 4 pixels, the SMs shared out among the layers,
+sums 2 K steps of 16 pixels inside the tensor core where a CTA has at most 2
+tiles, else 4, and writes partial sums every 16 tiles. Sizes on both sides of a
+tile edge, a single pixel, enough tiles for the longer sums and for several
+flushes, against the oracle's backward pass in float64 that rounds to BF16 where
 the kernels do. What remains are FP32 sums (1e-6) and activations or data
 gradients that round to BF16 the other way: a relative change of 2^-8 at most
 in one factor, in about one value of a thousand, independently from pixel to
@@ -19,7 +20,8 @@ from paper_1702_01530_gb300 import capi, scenegen as sg
 pytestmark = pytest.mark.gpu
 
 
-@pytest.mark.parametrize("W,H", [(1, 1), (111, 3), (112, 4), (113, 5), (225, 9), (3, 700), (1800, 77)])
+@pytest.mark.parametrize("W,H", [(1, 1), (111, 3), (112, 4), (113, 5), (225, 9), (3, 700), (900, 37),
+                                 (1800, 340)])
 def test_weight_gradients_at_tile_edges(W, H):
     import torch
     params = sg.net_params_he(71)
