@@ -188,7 +188,7 @@ cudaError_t build_lbvh(const float4* d_sph_in, const float* d_tri_in, uint32_t n
 size_t lbvh_tmp_bytes(uint32_t n);
 size_t sah_tmp_bytes(uint32_t n);
 // binned-SAH binary tree over the leaves of the LBVH (nodes, parent): same
-// node layout and leaf slots, root 0; synchronises st once per tree level
+// node layout and leaf slots, root 0; synchronises st about once
 cudaError_t build_sah_tree(const float4* lbvh_nodes, const int32_t* parent, uint32_t n,
                            float4* out, void* tmp, uint32_t* err, cudaStream_t st);
 // the render nodes of a binary tree over n primitives

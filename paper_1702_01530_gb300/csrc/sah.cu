@@ -12,63 +12,105 @@
 // same image 11 % faster. Any binary tree over the same conservative leaf
 // boxes yields the same closest hit and the same any-hit answer.
 //
-// Scene creation with this build (GB300; upload, LBVH, SAH tree): the blob
-// scene's 257k primitives 4.0 ms, the 10M-triangle terrain 77 ms (with the
-// 4-wide tree built too: 4.5 ms and 95 ms; with one block per node on every
-// level: 6.3 ms and 0.18 s; with 256 threads for every level and no bin
-// combining: 12.2 ms and 0.49 s).
-// One level of the tree per launch, one block per node of the level (nodes
-// of at most kSmallLeaves leaves: their whole subtree in one warp):
-//   1. centroid bounds of the node's leaves (block reduction);
-//   2. kBins bins per axis: leaf count and the union of the leaf boxes
-//      (shared-memory atomics on order-preserving integer images of floats,
-//      one set of bins per warp, merged; the lanes of a warp that fall in one
-//      bin combine their values first, as neighbouring leaves in Morton order
-//      usually do);
-//   3. the split of least SAH cost, area(L) n(L) + area(R) n(R), over the
-//      3 (kBins - 1) bin boundaries; an object-median split when the centroids
-//      coincide or the depth budget is low, so that no leaf lies deeper than
-//      kMaxDepth (the traversal stack holds 64 entries);
-//   4. a stable partition of the node's leaf slots (block prefix sums), so
-//      the tree does not depend on thread timing;
-//   5. the node record: both child boxes, leaf children as ~slot, inner
-//      children filled in by the children themselves one level later.
+// Two phases, without a host decision between them:
+//   top   one level per step, every node of more than kMidLeaves leaves cut into
+//         slices of kSlice leaves, one block each: (1) 16 bins per axis of the
+//         slice, added to the node's; (2) the split of least SAH cost, area(L)
+//         n(L) + area(R) n(R), over the 45 bin boundaries, and a stable
+//         partition of the slice (lefts before it from the slices' bin
+//         counts), with the centroid bounds of the two children; (3) the node
+//         record and the children's entries. The kernels read their counts on
+//         the device, so the levels are queued without waiting; the host looks
+//         only after as many as a balanced tree has.
+//   mid   a subtree of at most kMidLeaves leaves in one block, one thread per
+//         leaf: the same steps in shared memory for all its nodes of a level
+//         at once, down to segments of at most 32 leaves; then one warp per
+//         segment, all its nodes of a level at once, each split at the least
+//         SAH cost over every position of its leaves sorted by centroid (a
+//         warp sort by (segment, centroid, position), segmented prefix and
+//         suffix boxes).
+// An object-median split stands in when the centroids coincide or the depth
+// budget is low, so that no leaf lies deeper than kMaxDepth (the traversal stack
+// holds 64 entries). All combined values are minima, maxima and integer sums,
+// and partitions are stable, so the tree does not depend on thread timing or on
+// the slicing.
 // Node numbering: a binary tree over n leaves has n - 1 inner nodes and each
 // owns one split position s (left = [begin, s), right = [s, end)), s in
 // [1, n-1]; node id = s - 1, except that the root is 0 and the node whose
 // split position is 1 takes the root's id. Ids are therefore unique, dense
-// and independent of launch order.
+// and independent of launch order. A node writes its own id into its parent's
+// record, and its leaf children into its own.
+//
+// Bound by the latency of the levels at 257k primitives and by shared-memory
+// atomics and shuffles at 10M. Measured (kernels of the build alone): 257k blob
+// primitives 0.53 ms, 10M terrain triangles 10.4 ms; with one block per node, a
+// host read per level, lane reductions for every bin and one warp per subtree
+// stack in the last 32 leaves: 1.76 ms and 36.5 ms.
 #include <cuda_runtime.h>
 #include <stdint.h>
 
 #include <algorithm>
+#include <utility>
 
 #include "rt_internal.cuh"
 
 namespace rt {
 namespace {
 
-#ifndef RT_SAH_THREADS
-#define RT_SAH_THREADS 256
-#endif
-#ifndef RT_SAH_THREADS_TOP
-#define RT_SAH_THREADS_TOP 1024
-#endif
-// threads per node (block): 256 for the many nodes of the lower levels, 1024 for the levels of
-// fewer than kTopJobs nodes, whose blocks each cover many leaves
-constexpr int kSahThreads = RT_SAH_THREADS;
-// levels with fewer nodes than kTopJobs run kSahThreadsTop threads per node:
-// their few blocks cover many leaves each
-constexpr int kSahThreadsTop = RT_SAH_THREADS_TOP;
-constexpr uint32_t kTopJobs = 1024;
+constexpr int kThreads = 256;
+constexpr int kWarps = kThreads / 32;
 constexpr int kBins = 16;
 constexpr int kMaxDepth = 60;        // median splits keep every leaf at or above this depth
-constexpr int kSmallLeaves = 32;     // subtrees of at most this many leaves: one warp each (k_sah_small)
+constexpr uint32_t kMidLeaves = 256; // subtrees of at most this many leaves: one block each
+constexpr uint32_t kSmallLeaves = 32;
+constexpr uint32_t kSlice = 1024;    // leaves of a slice of a top node
+constexpr uint32_t kRoot = 0xFFFFFFFFu;   // parent_slot of the root
 
 struct Job {
   uint32_t begin, end;               // leaf slots idx[begin, end) of this node (end - begin >= 2)
-  uint32_t parent_slot;              // parent id << 1 | child slot, or 0xFFFFFFFF for the root
-  uint32_t depth;
+  uint32_t parent_slot;              // parent id << 1 | child slot, or kRoot
+  uint32_t depth;                    // top bit (mid jobs): which index buffer holds the leaves
+};
+
+struct Control;
+struct TopNode;
+
+// the scratch of a build over n leaves, and where its results go
+struct Build {
+  uint32_t slice, max_slices, max_nodes, max_mid;   // leaves per slice; entries of a level and of the build
+  float4 *lo, *hi;                                  // leaf boxes
+  uint32_t* idx[2];                                 // leaf order, nodes and the node of each slice:
+  TopNode* nodes[2];                                // [0] this level's, [1] the next one's
+  uint32_t* slice_node[2];
+  int* slice_cnt;                                   // of each slice, the leaves up to each bin of an axis
+  Job* mid;
+  Control* ctl;
+  float4* out;
+  uint32_t* err;
+  uint32_t n;
+};
+
+// order-preserving ints are used for all boxes that atomics combine
+struct Bins {
+  int cnt[3][kBins];
+  int box[3][kBins][6];              // lo xyz, hi xyz
+};
+constexpr int kBinWords = (int)(sizeof(Bins) / sizeof(int));
+
+struct TopNode {
+  Job job;
+  uint32_t slice0, n_slices;
+  int bounds[6];                     // centroid bounds of the leaves
+  Bins bins;
+  int child_bounds[2][6];            // centroid bounds of the two sides
+  int child_box[2][6];               // their boxes (median splits only; else from the bins)
+  uint32_t done;                     // slices partitioned
+};
+
+// per level parity: nodes and slices of that level; and of the whole build
+struct Control {
+  uint32_t n_nodes[2], n_slices[2];
+  uint32_t n_mid, root_split;
 };
 
 __device__ __forceinline__ int f2o(float f) {        // order-preserving int image of a float
@@ -76,6 +118,25 @@ __device__ __forceinline__ int f2o(float f) {        // order-preserving int ima
   return i >= 0 ? i : i ^ 0x7FFFFFFF;
 }
 __device__ __forceinline__ float o2f(int i) { return __int_as_float(i >= 0 ? i : i ^ 0x7FFFFFFF); }
+// value i of an empty box
+__device__ __forceinline__ int empty6(int i) { return i < 3 ? f2o(INFINITY) : f2o(-INFINITY); }
+
+// word i of a set of bins: its empty value, and what it combines by (0 sum, -1 min, 1 max)
+__device__ __forceinline__ int empty_word(int i) { return i < 3 * kBins ? 0 : empty6((i - 3 * kBins) % 6); }
+__device__ __forceinline__ int word_op(int i) { return i < 3 * kBins ? 0 : (i - 3 * kBins) % 6 < 3 ? -1 : 1; }
+__device__ __forceinline__ int* words(Bins& b) { return &b.cnt[0][0]; }
+
+// A leaf's box and centroid as values to combine by minimum (0..2) and maximum
+// (3..5). A centroid that is no number (its box spans all floats) bounds nothing.
+__device__ __forceinline__ void centroid(const float4& lo, const float4& hi, float c[3]) {
+  c[0] = 0.5f * (lo.x + hi.x); c[1] = 0.5f * (lo.y + hi.y); c[2] = 0.5f * (lo.z + hi.z);
+}
+__device__ __forceinline__ void centroid6(const float c[3], int v[6]) {
+  for (int q = 0; q < 3; ++q) { v[q] = f2o(fminf(c[q], INFINITY)); v[3 + q] = f2o(fmaxf(c[q], -INFINITY)); }
+}
+__device__ __forceinline__ void box6(const float4& lo, const float4& hi, int v[6]) {
+  v[0] = f2o(lo.x); v[1] = f2o(lo.y); v[2] = f2o(lo.z); v[3] = f2o(hi.x); v[4] = f2o(hi.y); v[5] = f2o(hi.z);
+}
 
 __device__ __forceinline__ float half_area(const float lo[3], const float hi[3]) {
   const float dx = fmaxf(hi[0] - lo[0], 0.f), dy = fmaxf(hi[1] - lo[1], 0.f),
@@ -83,794 +144,816 @@ __device__ __forceinline__ float half_area(const float lo[3], const float hi[3])
   return dx * dy + dy * dz + dz * dx;
 }
 
-// SAH cost of splitting after bin s on axis a, from merged bins (counts and
-// order-preserving box images); INFINITY when a side is empty
-__device__ __forceinline__ float split_cost(const int (*cnt)[kBins], const int (*box)[kBins][6],
-                                            float cext_a, int a, int s) {
-  float llo[3] = {INFINITY, INFINITY, INFINITY}, lhi[3] = {-INFINITY, -INFINITY, -INFINITY};
-  float rlo[3] = {INFINITY, INFINITY, INFINITY}, rhi[3] = {-INFINITY, -INFINITY, -INFINITY};
-  int nl = 0, nr = 0;
-  for (int q = 0; q < kBins; ++q) {
-    const int c = cnt[a][q];
-    if (!c) continue;
-    float* blo = q <= s ? llo : rlo;
-    float* bhi = q <= s ? lhi : rhi;
-    for (int x = 0; x < 3; ++x) {
-      blo[x] = fminf(blo[x], o2f(box[a][q][x]));
-      bhi[x] = fmaxf(bhi[x], o2f(box[a][q][3 + x]));
+__device__ __forceinline__ int bin_of(float c, float cmin, float cext) {
+  return min(kBins - 1, (int)((c - cmin) * ((float)kBins / cext)));
+}
+
+// centroid frame of a node, and whether it splits at the object median (its
+// centroids coincide, or the depth budget is short)
+__device__ __forceinline__ bool node_frame(const int* bounds, uint32_t m, uint32_t depth, float cmin[3],
+                                           float cext[3]) {
+  bool spread = false;
+  for (int a = 0; a < 3; ++a) {
+    cmin[a] = o2f(bounds[a]);
+    cext[a] = o2f(bounds[3 + a]) - cmin[a];
+    spread |= cext[a] > 0.f;
+  }
+  const uint32_t lg = 32 - __clz(m - 1);
+  return !spread || depth + lg >= (uint32_t)kMaxDepth - 4;
+}
+
+// The split of a node from its bins (one warp): of the 3 x 15 bin boundaries
+// the first of least cost, area(L) n(L) + area(R) n(R); axis -1 if none has
+// leaves on both sides. Lanes 0-15 hold the bins in order and take the boxes
+// and counts of all bins up to theirs, lanes 16-31 hold them in reverse and
+// take those from theirs on.
+__device__ __forceinline__ void choose_split(const Bins& bins, const float cext[3], int& axis, int& bin) {
+  const int lane = threadIdx.x & 31, i = lane & 15, q = lane < 16 ? i : 15 - i;
+  float best = INFINITY;
+  int at = 3 * kBins;
+#pragma unroll
+  for (int a = 0; a < 3; ++a) {
+    int n = bins.cnt[a][q];
+    float v[6];
+    for (int x = 0; x < 6; ++x) v[x] = o2f(bins.box[a][q][x]);
+#pragma unroll
+    for (int o = 1; o < kBins; o <<= 1) {
+      const int m = __shfl_up_sync(0xFFFFFFFFu, n, o, kBins);
+      if (i >= o) n += m;
+#pragma unroll
+      for (int x = 0; x < 6; ++x) {
+        const float u = __shfl_up_sync(0xFFFFFFFFu, v[x], o, kBins);
+        if (i >= o) v[x] = x < 3 ? fminf(v[x], u) : fmaxf(v[x], u);
+      }
     }
-    if (q <= s) nl += c; else nr += c;
+    const float area = half_area(v, v + 3);
+    const float rc = __shfl_sync(0xFFFFFFFFu, __fmul_rn(area, (float)n), 30 - lane);   // of the bins after this one
+    const int rn = __shfl_sync(0xFFFFFFFFu, n, 30 - lane);
+    const float cost = __fmaf_rn(area, (float)n, rc);
+    if (lane < kBins - 1 && cext[a] > 0.f && n > 0 && rn > 0 && cost < best) {
+      best = cost;
+      at = a * kBins + lane;
+    }
   }
-  return (cext_a > 0.f && nl > 0 && nr > 0)
-             ? half_area(llo, lhi) * (float)nl + half_area(rlo, rhi) * (float)nr
-             : INFINITY;
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    const float c = __shfl_xor_sync(0xFFFFFFFFu, best, o);
+    const int i2 = __shfl_xor_sync(0xFFFFFFFFu, at, o);
+    if (c < best || (c == best && i2 < at)) { best = c; at = i2; }
+  }
+  axis = at == 3 * kBins ? -1 : at / kBins;
+  bin = at == 3 * kBins ? 0 : at % kBins;
 }
 
-// the first of equal least costs (deterministic): axis (-1 = none) and bin
-__device__ __forceinline__ void pick_split(const float* cost, int* choice) {
-  int best = -1;
-  float bc = INFINITY;
-  for (int i = 0; i < 3 * (kBins - 1); ++i)
-    if (cost[i] < bc) { bc = cost[i]; best = i; }
-  choice[0] = best < 0 ? -1 : best / (kBins - 1);
-  choice[1] = best < 0 ? 0 : best % (kBins - 1);
+// the id of a node from its split position; it goes into the parent's record
+__device__ __forceinline__ uint32_t place_node(uint32_t split, uint32_t parent_slot, uint32_t root_split,
+                                               float4* __restrict__ out, uint32_t n, uint32_t* __restrict__ err) {
+  if (parent_slot == kRoot) return 0u;
+  uint32_t id = split == 1 ? root_split - 1 : split - 1;
+  if (id >= n - 1) { atomicOr(err, ERR_BUILD); id = n - 2; }   // splits lie in [1, n-1]: cannot happen
+  reinterpret_cast<int32_t*>(out + 4 * (size_t)(parent_slot >> 1) + 3)[parent_slot & 1u] = (int32_t)id;
+  return id;
 }
 
-// Step 5 of a node (one thread): its id from its split position, its record
-// (child boxes cl/ch, leaf children as ~slot) and the jobs of its inner
-// children, next level or small list.
-__device__ void write_node(const Job& job, uint32_t n_left, const float cl[2][3], const float ch[2][3],
-                          const uint32_t* __restrict__ idx_out, Job* __restrict__ next,
-                          uint32_t* __restrict__ next_count, Job* __restrict__ small,
-                          uint32_t* __restrict__ small_count, uint32_t out_buf, float4* __restrict__ out,
-                          uint32_t* __restrict__ root_split, uint32_t n, uint32_t* __restrict__ err) {
-  const uint32_t b = job.begin, e = job.end;
-  const uint32_t split = b + n_left;               // split position in [1, n-1]
-  uint32_t id;
-  if (job.parent_slot == 0xFFFFFFFFu) {
-    id = 0;
-    *root_split = split;
-  } else {
-    const uint32_t rs = *root_split;                // written one level earlier
-    id = split == 1 ? rs - 1 : split - 1;
-    // hand the id to the parent's child slot
-    const uint32_t p = job.parent_slot >> 1, slot = job.parent_slot & 1u;
-    reinterpret_cast<int32_t*>(out + 4 * (size_t)p + 3)[slot] = (int32_t)id;
-  }
-  if (id >= n - 1) { atomicOr(err, ERR_BUILD); return; }
+// a node's boxes, and its leaf children (slots; kRoot: an inner child, which
+// writes itself)
+__device__ __forceinline__ void write_node(float4* __restrict__ out, uint32_t id, const float cl[2][3],
+                                           const float ch[2][3], uint32_t leaf0, uint32_t leaf1) {
   float4* o = out + 4 * (size_t)id;
   o[0] = make_float4(cl[0][0], ch[0][0], cl[0][1], ch[0][1]);
   o[1] = make_float4(cl[1][0], ch[1][0], cl[1][1], ch[1][1]);
   o[2] = make_float4(cl[0][2], ch[0][2], cl[1][2], ch[1][2]);
-  int32_t child[2] = {0, 0};
-  const uint32_t rb[2] = {b, split}, re[2] = {split, e};
-  for (int c = 0; c < 2; ++c) {
-    if (re[c] - rb[c] == 1) {
-      child[c] = ~(int32_t)idx_out[rb[c]];
-    } else {
-      const bool is_small = re[c] - rb[c] <= (uint32_t)kSmallLeaves;
-      const uint32_t at = atomicAdd(is_small ? small_count : next_count, 1u);
-      if (at >= n / 2 + 1) { atomicOr(err, ERR_BUILD); continue; }
-      // a small subtree is built later by one warp from the leaf slots this
-      // level wrote (idx buffer out_buf, kept in the depth field's top bit)
-      (is_small ? small : next)[at] =
-          Job{rb[c], re[c], id << 1 | (uint32_t)c, (job.depth + 1) | (is_small ? out_buf << 31 : 0u)};
-      child[c] = 0;                                 // filled in by the child
+  int32_t* w = reinterpret_cast<int32_t*>(o + 3);
+  if (leaf0 != kRoot) w[0] = ~(int32_t)leaf0;
+  if (leaf1 != kRoot) w[1] = ~(int32_t)leaf1;
+  w[2] = 0;
+  w[3] = 0;
+}
+
+// one leaf into a bin
+__device__ __forceinline__ void add_box(Bins& bins, int a, int bin, const int v[6]) {
+  atomicAdd(&bins.cnt[a][bin], 1);
+  for (int q = 0; q < 3; ++q) {
+    atomicMin(&bins.box[a][bin][q], v[q]);
+    atomicMax(&bins.box[a][bin][3 + q], v[3 + q]);
+  }
+}
+
+__device__ __forceinline__ float at3(const float v[3], int a) { return a == 0 ? v[0] : a == 1 ? v[1] : v[2]; }
+
+// Minima (values 0..2) and maxima (3..5) of the lanes of `grp`, combined into
+// dst by its first lane
+__device__ __forceinline__ void combine6(uint32_t grp, const int v[6], int* dst) {
+  int r[6];
+  for (int q = 0; q < 3; ++q) {
+    r[q] = __reduce_min_sync(grp, v[q]);
+    r[3 + q] = __reduce_max_sync(grp, v[3 + q]);
+  }
+  if ((uint32_t)(__ffs(grp) - 1) == (threadIdx.x & 31))
+    for (int q = 0; q < 3; ++q) {
+      atomicMin(dst + q, r[q]);
+      atomicMax(dst + 3 + q, r[3 + q]);
+    }
+}
+
+// leaf box of slot k: the child box of k's parent that holds leaf ~k; the
+// identity order; and the centroid bounds of all leaves
+__global__ void __launch_bounds__(kThreads)
+k_leaves(const float4* __restrict__ nodes, const int32_t* __restrict__ parent, uint32_t n,
+         float4* __restrict__ lo, float4* __restrict__ hi, uint32_t* __restrict__ idx, TopNode* root) {
+  const uint32_t k = blockIdx.x * blockDim.x + threadIdx.x;
+  __shared__ int s_bounds[6];
+  if (threadIdx.x < 6) s_bounds[threadIdx.x] = empty6(threadIdx.x);
+  __syncthreads();
+  int v[6];
+  for (int q = 0; q < 6; ++q) v[q] = empty6(q);
+  if (k < n) {
+    const int32_t p = parent[n - 1 + k];
+    const float4 a = nodes[4 * (size_t)p], b = nodes[4 * (size_t)p + 1],
+                 c = nodes[4 * (size_t)p + 2], e = nodes[4 * (size_t)p + 3];
+    const bool first = __float_as_int(e.x) == ~(int32_t)k;
+    const float4 l = first ? make_float4(a.x, a.z, c.x, 0.f) : make_float4(b.x, b.z, c.z, 0.f);
+    const float4 h = first ? make_float4(a.y, a.w, c.y, 0.f) : make_float4(b.y, b.w, c.w, 0.f);
+    lo[k] = l;
+    hi[k] = h;
+    idx[k] = k;
+    float m[3];
+    centroid(l, h, m);
+    centroid6(m, v);
+  }
+  if (!root) return;
+  combine6(0xFFFFFFFFu, v, s_bounds);
+  __syncthreads();
+  if (threadIdx.x < 3) atomicMin(&root->bounds[threadIdx.x], s_bounds[threadIdx.x]);
+  else if (threadIdx.x < 6) atomicMax(&root->bounds[threadIdx.x], s_bounds[threadIdx.x]);
+}
+
+// the build's control words and, in a build with a top phase, its root entry;
+// else the whole build is one mid job
+__global__ void k_begin(Control* c, TopNode* root, uint32_t* slice_node, Job* mid, uint32_t n, uint32_t slice) {
+  const uint32_t slices = (uint32_t)(((uint64_t)n + slice - 1) / slice);
+  if (root) {
+    for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < slices; i += gridDim.x * blockDim.x)
+      slice_node[i] = 0;
+    if (blockIdx.x == 0) {
+      for (int i = threadIdx.x; i < kBinWords; i += blockDim.x) words(root->bins)[i] = empty_word(i);
+      if (threadIdx.x < 6) root->bounds[threadIdx.x] = empty6(threadIdx.x);
+      if (threadIdx.x < 12) {
+        root->child_bounds[threadIdx.x / 6][threadIdx.x % 6] = empty6(threadIdx.x % 6);
+        root->child_box[threadIdx.x / 6][threadIdx.x % 6] = empty6(threadIdx.x % 6);
+      }
     }
   }
-  o[3] = make_float4(__int_as_float(child[0]), __int_as_float(child[1]), 0.f, 0.f);
-}
-
-// leaf box of slot k: the child box of k's parent that holds leaf ~k
-__global__ void k_leaf_boxes(const float4* __restrict__ nodes, const int32_t* __restrict__ parent,
-                             uint32_t n, float4* __restrict__ lo, float4* __restrict__ hi) {
-  const uint32_t k = blockIdx.x * blockDim.x + threadIdx.x;
-  if (k >= n) return;
-  const int32_t p = parent[n - 1 + k];
-  const float4 a = nodes[4 * (size_t)p], b = nodes[4 * (size_t)p + 1],
-               c = nodes[4 * (size_t)p + 2], e = nodes[4 * (size_t)p + 3];
-  if (__float_as_int(e.x) == ~(int32_t)k) {
-    lo[k] = make_float4(a.x, a.z, c.x, 0.f);
-    hi[k] = make_float4(a.y, a.w, c.y, 0.f);
-  } else {
-    lo[k] = make_float4(b.x, b.z, c.z, 0.f);
-    hi[k] = make_float4(b.y, b.w, c.w, 0.f);
+  if (blockIdx.x == 0 && threadIdx.x == 0) {
+    *c = Control{{root ? 1u : 0u, 0u}, {root ? slices : 0u, 0u}, root ? 0u : 1u, 0u};
+    if (root) {
+      root->job = Job{0u, n, kRoot, 0u};
+      root->slice0 = 0;
+      root->n_slices = slices;
+      root->done = 0;
+    } else {
+      mid[0] = Job{0u, n, kRoot, 0u};
+    }
   }
 }
 
-__global__ void k_iota(uint32_t* idx, uint32_t n) {
-  const uint32_t k = blockIdx.x * blockDim.x + threadIdx.x;
-  if (k < n) idx[k] = k;
+// ------------------------------------------------------------------ top phase
+// a slice's leaves: [sb, se) of its node's range
+__device__ __forceinline__ void slice_range(const TopNode& t, uint32_t s, uint32_t slice, uint32_t& sb,
+                                            uint32_t& se) {
+  const uint64_t at = (uint64_t)t.job.begin + (uint64_t)(s - t.slice0) * slice;
+  sb = (uint32_t)at;
+  se = (uint32_t)min((uint64_t)t.job.end, at + slice);
 }
 
-template <int kSahThreads>
-__global__ void __launch_bounds__(kSahThreads)
-k_sah_level(const float4* __restrict__ leaf_lo, const float4* __restrict__ leaf_hi,
-            const uint32_t* __restrict__ idx_in, uint32_t* __restrict__ idx_out,
-            const Job* __restrict__ jobs, uint32_t n_jobs, Job* __restrict__ next,
-            uint32_t* __restrict__ next_count, Job* __restrict__ small, uint32_t* __restrict__ small_count,
-            uint32_t out_buf, float4* __restrict__ out, uint32_t* __restrict__ root_split,
-            uint32_t n, uint32_t* __restrict__ err) {
-  constexpr int kSahWarps = kSahThreads / 32;
-  // bins per warp (fewer shared-memory atomics on one address), merged into warp 0's
-  __shared__ int s_cnt[kSahWarps][3][kBins];
-  __shared__ int s_box[kSahWarps][3][kBins][6];   // lo xyz, hi xyz as order-preserving ints
-  __shared__ int s_red[12];                  // centroid bounds, then child boxes of a median split
-  __shared__ uint32_t s_scan[kSahThreads / 32];
-  __shared__ float s_cost[3 * (kBins - 1)];
-  __shared__ int s_choice[2];                // axis (-1: median), bin
-  if (blockIdx.x >= n_jobs) return;
-  const Job job = jobs[blockIdx.x];
-  const uint32_t b = job.begin, e = job.end, m = e - b;
-  const uint32_t tid = threadIdx.x;
+// the boxes (and slots) of leaves base + u kThreads + thread below `end`, all
+// loads in flight at once: a slice is a chain of two dependent loads otherwise
+constexpr int kUnroll = 4;
+__device__ __forceinline__ void load_leaves(const Build& g, uint32_t base, uint32_t end, float4 lo[kUnroll],
+                                            float4 hi[kUnroll], uint32_t* slot) {
+  uint32_t k[kUnroll];
+#pragma unroll
+  for (int u = 0; u < kUnroll; ++u) {
+    const uint32_t i = base + u * kThreads + threadIdx.x;
+    k[u] = i < end ? g.idx[0][i] : 0u;
+  }
+#pragma unroll
+  for (int u = 0; u < kUnroll; ++u) {
+    lo[u] = g.lo[k[u]];
+    hi[u] = g.hi[k[u]];
+    if (slot) slot[u] = k[u];
+  }
+}
 
-  // 1. centroid bounds
-  if (tid < 6) s_red[tid] = tid < 3 ? f2o(INFINITY) : f2o(-INFINITY);
-  for (int i = tid; i < kSahWarps * 3 * kBins; i += kSahThreads) {
-    const int w = i / (3 * kBins), a = (i / kBins) % 3, q = i % kBins;
-    s_cnt[w][a][q] = 0;
-    for (int c = 0; c < 6; ++c) s_box[w][a][q][c] = c < 3 ? f2o(INFINITY) : f2o(-INFINITY);
-  }
-  __syncthreads();
-  float clo[3] = {INFINITY, INFINITY, INFINITY}, chi[3] = {-INFINITY, -INFINITY, -INFINITY};
-  for (uint32_t i = b + tid; i < e; i += kSahThreads) {
-    const uint32_t k = idx_in[i];
-    const float4 lo = leaf_lo[k], hi = leaf_hi[k];
-    const float c[3] = {0.5f * (lo.x + hi.x), 0.5f * (lo.y + hi.y), 0.5f * (lo.z + hi.z)};
-    for (int a = 0; a < 3; ++a) { clo[a] = fminf(clo[a], c[a]); chi[a] = fmaxf(chi[a], c[a]); }
-  }
-  for (int a = 0; a < 3; ++a) { atomicMin(&s_red[a], f2o(clo[a])); atomicMax(&s_red[3 + a], f2o(chi[a])); }
-  __syncthreads();
-  float cmin[3], cext[3];
-  bool spread = false;
-  for (int a = 0; a < 3; ++a) {
-    cmin[a] = o2f(s_red[a]);
-    cext[a] = o2f(s_red[3 + a]) - cmin[a];
-    spread |= cext[a] > 0.f;
-  }
-  // depth budget: a median split keeps the subtree ceil(log2 m) deep
-  const uint32_t lg = 32 - __clz(m - 1);
-  const bool median = !spread || job.depth + lg >= (uint32_t)kMaxDepth - 4;
-
-  // 2-3. bins and the SAH split
-  if (!median) {
-    for (uint32_t i = b + tid; i < e; i += kSahThreads) {
-      const uint32_t k = idx_in[i];
-      const float4 lo = leaf_lo[k], hi = leaf_hi[k];
-      const float c[3] = {0.5f * (lo.x + hi.x), 0.5f * (lo.y + hi.y), 0.5f * (lo.z + hi.z)};
-      const float l3[3] = {lo.x, lo.y, lo.z}, h3[3] = {hi.x, hi.y, hi.z};
-      // neighbouring leaves (Morton order) mostly share a bin: the lanes of a
-      // bin combine their values first and one of them updates the bin
-      const uint32_t active = __activemask();
-      for (int a = 0; a < 3; ++a) {
-        if (!(cext[a] > 0.f)) continue;          // uniform over the block
-        const int bin = min(kBins - 1, (int)((c[a] - cmin[a]) * ((float)kBins / cext[a])));
-        const uint32_t grp = __match_any_sync(active, bin);
+// 1. bins of a slice, added to its node's; the slice's own counts are kept
+__global__ void __launch_bounds__(kThreads)
+k_top_bins(const Build g, int cur) {
+  const uint32_t* __restrict__ slice_node = g.slice_node[0];
+  int* __restrict__ slice_cnt = g.slice_cnt;
+  TopNode* nodes = g.nodes[0];
+  Control* ctl = g.ctl;
+  const uint32_t slice = g.slice;
+  __shared__ Bins s_bins[kWarps];              // one per warp: fewer atomics on one address
+  const uint32_t tid = threadIdx.x, n_slices = ctl->n_slices[cur];
+  if (blockIdx.x == 0 && tid == 0) ctl->n_nodes[cur ^ 1] = ctl->n_slices[cur ^ 1] = 0;   // step 3 fills them
+  for (uint32_t s = blockIdx.x; s < n_slices; s += gridDim.x) {
+    TopNode& t = nodes[slice_node[s]];
+    float cmin[3], cext[3];
+    if (node_frame(t.bounds, t.job.end - t.job.begin, t.job.depth, cmin, cext)) continue;   // block-uniform
+    uint32_t sb, se;
+    slice_range(t, s, slice, sb, se);
+    __syncthreads();
+    for (int i = tid; i < kWarps * kBinWords; i += kThreads) words(s_bins[0])[i] = empty_word(i % kBinWords);
+    __syncthreads();
+    Bins& mine = s_bins[tid >> 5];
+    for (uint32_t base = sb; base < se; base += kUnroll * kThreads) {
+      float4 lo[kUnroll], hi[kUnroll];
+      load_leaves(g, base, se, lo, hi, nullptr);
+#pragma unroll
+      for (int u = 0; u < kUnroll; ++u) {
+        const bool in = base + u * kThreads + tid < se;
+        const uint32_t active = __ballot_sync(0xFFFFFFFFu, in);
+        if (!in) continue;
+        float c[3];
         int v[6];
-        for (int q = 0; q < 3; ++q) {
-          v[q] = __reduce_min_sync(grp, f2o(l3[q]));
-          v[3 + q] = __reduce_max_sync(grp, f2o(h3[q]));
-        }
-        if ((uint32_t)(__ffs(grp) - 1) == (tid & 31)) {
-          const int w = tid >> 5;
-          atomicAdd(&s_cnt[w][a][bin], __popc(grp));
-          for (int q = 0; q < 3; ++q) {
-            atomicMin(&s_box[w][a][bin][q], v[q]);
-            atomicMax(&s_box[w][a][bin][3 + q], v[3 + q]);
+        centroid(lo[u], hi[u], c);
+        box6(lo[u], hi[u], v);
+        // Neighbouring leaves mostly share a bin: where a warp's leaves fall
+        // in at most two bins, their lanes combine first. The reductions of
+        // different lane sets run one after another, so with more bins plain
+        // shared-memory atomics are faster (20 levels of 10M leaves: 4.5 ms
+        // always combining, 8.5 never, 3.2 with this rule; 3.4 from four bins up).
+#pragma unroll
+        for (int a = 0; a < 3; ++a) {
+          if (!(cext[a] > 0.f)) continue;        // uniform over the block
+          const int bin = bin_of(c[a], cmin[a], cext[a]);
+          const uint32_t grp = __match_any_sync(active, bin);
+          const bool leader = (uint32_t)(__ffs(grp) - 1) == (tid & 31);
+          if (__popc(__ballot_sync(active, leader)) <= 2) {
+            if (leader) atomicAdd(&mine.cnt[a][bin], __popc(grp));
+            combine6(grp, v, mine.box[a][bin]);
+          } else {
+            add_box(mine, a, bin, v);
           }
         }
       }
     }
     __syncthreads();
-    // merge the warps' bins into warp 0's
-    for (int i = tid; i < 3 * kBins * 7; i += kSahThreads) {
-      const int a = i / (kBins * 7), q = (i / 7) % kBins, f = i % 7;
-      if (f == 6) {
-        int t = 0;
-        for (int w = 0; w < kSahWarps; ++w) t += s_cnt[w][a][q];
-        s_cnt[0][a][q] = t;
-      } else {
-        int v = s_box[0][a][q][f];
-        for (int w = 1; w < kSahWarps; ++w) v = f < 3 ? min(v, s_box[w][a][q][f]) : max(v, s_box[w][a][q][f]);
-        s_box[0][a][q][f] = v;
+    for (int i = tid; i < kBinWords; i += kThreads) {
+      const int op = word_op(i);                 // the counts are words 0..47
+      int v = words(s_bins[0])[i];
+      for (int w = 1; w < kWarps; ++w) {
+        const int x = words(s_bins[w])[i];
+        v = op == 0 ? v + x : op < 0 ? min(v, x) : max(v, x);
       }
-    }
-    __syncthreads();
-    if (tid < 3 * (kBins - 1)) {
-      const int a = tid / (kBins - 1), s = tid % (kBins - 1);   // split after bin s
-      s_cost[tid] = split_cost(s_cnt[0], s_box[0], cext[a], a, s);
-    }
-    __syncthreads();
-    if (tid == 0) pick_split(s_cost, s_choice);
-  } else if (tid == 0) {
-    s_choice[0] = -1;
-    s_choice[1] = 0;
-  }
-  __syncthreads();
-  const int axis = s_choice[0], split_bin = s_choice[1];
-
-  // 4. stable partition into idx_out[b, e): left leaves first, in their order
-  uint32_t n_left;
-  if (axis < 0) {
-    n_left = m / 2;                                  // object median in the current order
-    for (uint32_t i = b + tid; i < e; i += kSahThreads) idx_out[i] = idx_in[i];
-  } else {
-    const float scale = (float)kBins / cext[axis];
-    uint32_t cnt_left = 0;
-    for (uint32_t base = b; base < e; base += kSahThreads) {
-      const uint32_t i = base + tid;
-      bool left = false;
-      uint32_t k = 0;
-      if (i < e) {
-        k = idx_in[i];
-        const float4 lo = leaf_lo[k], hi = leaf_hi[k];
-        const float c = 0.5f * ((&lo.x)[axis] + (&hi.x)[axis]);
-        left = min(kBins - 1, (int)((c - cmin[axis]) * scale)) <= split_bin;
-      }
-      // block-wide exclusive scan of `left`
-      const uint32_t ball = __ballot_sync(0xFFFFFFFFu, left);
-      const uint32_t lane = tid & 31, warp = tid >> 5;
-      __syncthreads();
-      if (lane == 0) s_scan[warp] = __popc(ball);
-      __syncthreads();
-      uint32_t before = 0, chunk = 0;
-      for (uint32_t w = 0; w < kSahThreads / 32; ++w) {
-        if (w < warp) before += s_scan[w];
-        chunk += s_scan[w];
-      }
-      const uint32_t rank = before + __popc(ball & ((1u << lane) - 1u));
-      if (i < e) {
-        // lefts from the front in order; rights from the back, reversed
-        // (right number r of the range goes to e - 1 - r)
-        if (left) idx_out[b + cnt_left + rank] = k;
-        else idx_out[e - 1 - ((i - b) - (cnt_left + rank))] = k;
-      }
-      cnt_left += chunk;
-    }
-    n_left = cnt_left;
-    // the right side was written from the end backwards (reversed); restore
-    // its original order so the partition is stable
-    __syncthreads();
-    const uint32_t n_right = m - n_left;
-    for (uint32_t i = tid; i < n_right / 2; i += kSahThreads) {
-      const uint32_t x = b + n_left + i, y = e - 1 - i;
-      const uint32_t t = idx_out[x];
-      idx_out[x] = idx_out[y];
-      idx_out[y] = t;
-    }
-  }
-  __syncthreads();
-  bool to_median = false;
-  if (axis >= 0 && (n_left == 0 || n_left == m)) {
-    // cannot happen (the partition repeats the binning arithmetic); an empty
-    // side would break the tree, so fall back to the object median
-    to_median = true;
-    n_left = m / 2;
-    for (uint32_t i = b + tid; i < e; i += kSahThreads) idx_out[i] = idx_in[i];
-    __syncthreads();
-  }
-
-  // child boxes
-  float cl[2][3], ch[2][3];
-  if (axis >= 0 && !to_median) {
-    for (int c = 0; c < 2; ++c)
-      for (int x = 0; x < 3; ++x) { cl[c][x] = INFINITY; ch[c][x] = -INFINITY; }
-    for (int q = 0; q < kBins; ++q) {
-      if (!s_cnt[0][axis][q]) continue;
-      const int c = q <= split_bin ? 0 : 1;
-      for (int x = 0; x < 3; ++x) {
-        cl[c][x] = fminf(cl[c][x], o2f(s_box[0][axis][q][x]));
-        ch[c][x] = fmaxf(ch[c][x], o2f(s_box[0][axis][q][3 + x]));
-      }
-    }
-  } else {
-    if (tid < 12) s_red[tid] = (tid % 6) < 3 ? f2o(INFINITY) : f2o(-INFINITY);
-    __syncthreads();
-    float l[2][3], h[2][3];
-    for (int c = 0; c < 2; ++c)
-      for (int x = 0; x < 3; ++x) { l[c][x] = INFINITY; h[c][x] = -INFINITY; }
-    for (uint32_t i = b + tid; i < e; i += kSahThreads) {
-      const uint32_t k = idx_out[i];
-      const int c = (i - b) < n_left ? 0 : 1;
-      const float4 lo = leaf_lo[k], hi = leaf_hi[k];
-      l[c][0] = fminf(l[c][0], lo.x); l[c][1] = fminf(l[c][1], lo.y); l[c][2] = fminf(l[c][2], lo.z);
-      h[c][0] = fmaxf(h[c][0], hi.x); h[c][1] = fmaxf(h[c][1], hi.y); h[c][2] = fmaxf(h[c][2], hi.z);
-    }
-    for (int c = 0; c < 2; ++c)
-      for (int x = 0; x < 3; ++x) {
-        atomicMin(&s_red[6 * c + x], f2o(l[c][x]));
-        atomicMax(&s_red[6 * c + 3 + x], f2o(h[c][x]));
-      }
-    __syncthreads();
-    for (int c = 0; c < 2; ++c)
-      for (int x = 0; x < 3; ++x) { cl[c][x] = o2f(s_red[6 * c + x]); ch[c][x] = o2f(s_red[6 * c + 3 + x]); }
-  }
-
-  // 5. this node's id, its record, and the jobs of its inner children
-  if (tid == 0)
-    write_node(job, n_left, cl, ch, idx_out, next, next_count, small, small_count, out_buf, out,
-               root_split, n, err);
-}
-
-// ---------------------------------------------------------------------------
-// The top levels, where a level has few nodes of many leaves each: one block
-// per node would leave most SMs idle (level 0 of a 257k-leaf scene is one
-// block over every leaf), so each node's leaves are cut into S slices and the
-// steps above run as five launches over (node, slice) blocks, with the
-// per-node results (centroid bounds, bins, the split, left counts per slice,
-// child boxes) combined in global memory by integer atomics and sums. Every
-// combined value equals the one-block value (min / max / sums of integers),
-// the split is chosen by the same code from the same bins, and the partition
-// is stable (slices in order, each slice's lefts and rights in order), so
-// the tree is the same as the one-block build's.
-constexpr int kWideThreads = 512;
-constexpr uint32_t kWideJobs = 32;       // levels of at most this many nodes may be sliced
-constexpr uint32_t kWideMinLeaves = 16384;   // ... when their nodes average at least this many leaves
-constexpr uint32_t kWideMinSlice = 1024;     // leaves per slice, at least
-constexpr uint32_t kWideMaxSlices = 1024;    // (node, slice) blocks of a level, at most
-
-struct WideNode {                        // per node of a sliced level
-  int bounds[6];                         // centroid bounds (order-preserving images)
-  int cnt[3][kBins];
-  int box[3][kBins][6];
-  int child[2][6];                       // child boxes (order-preserving images)
-  int choice[2];                         // axis (-1: median), bin
-  uint32_t n_left;                       // final left size
-};
-
-__device__ __forceinline__ void slice_range(const Job& job, uint32_t s, uint32_t S, uint32_t& sb,
-                                            uint32_t& se) {
-  const uint64_t m = job.end - job.begin;
-  sb = job.begin + (uint32_t)(m * s / S);
-  se = job.begin + (uint32_t)(m * (s + 1) / S);
-}
-
-__global__ void k_wide_init(WideNode* __restrict__ w, uint32_t count) {
-  const uint32_t j = blockIdx.x;
-  if (j >= count) return;
-  WideNode& v = w[j];
-  for (int i = threadIdx.x; i < 3 * kBins * 7; i += blockDim.x) {
-    const int a = i / (kBins * 7), q = (i / 7) % kBins, f = i % 7;
-    if (f == 6) v.cnt[a][q] = 0;
-    else v.box[a][q][f] = f < 3 ? f2o(INFINITY) : f2o(-INFINITY);
-  }
-  if (threadIdx.x < 6) v.bounds[threadIdx.x] = threadIdx.x < 3 ? f2o(INFINITY) : f2o(-INFINITY);
-  if (threadIdx.x < 12) v.child[threadIdx.x / 6][threadIdx.x % 6] =
-      (threadIdx.x % 6) < 3 ? f2o(INFINITY) : f2o(-INFINITY);
-}
-
-// 1. centroid bounds
-__global__ void __launch_bounds__(kWideThreads)
-k_wide_bounds(const float4* __restrict__ leaf_lo, const float4* __restrict__ leaf_hi,
-              const uint32_t* __restrict__ idx_in, const Job* __restrict__ jobs, uint32_t S,
-              WideNode* __restrict__ w) {
-  __shared__ int s_red[6];
-  const uint32_t j = blockIdx.x / S, sl = blockIdx.x % S, tid = threadIdx.x;
-  const Job job = jobs[j];
-  uint32_t sb, se;
-  slice_range(job, sl, S, sb, se);
-  if (tid < 6) s_red[tid] = tid < 3 ? f2o(INFINITY) : f2o(-INFINITY);
-  __syncthreads();
-  float clo[3] = {INFINITY, INFINITY, INFINITY}, chi[3] = {-INFINITY, -INFINITY, -INFINITY};
-  for (uint32_t i = sb + tid; i < se; i += kWideThreads) {
-    const uint32_t k = idx_in[i];
-    const float4 lo = leaf_lo[k], hi = leaf_hi[k];
-    const float c[3] = {0.5f * (lo.x + hi.x), 0.5f * (lo.y + hi.y), 0.5f * (lo.z + hi.z)};
-    for (int a = 0; a < 3; ++a) { clo[a] = fminf(clo[a], c[a]); chi[a] = fmaxf(chi[a], c[a]); }
-  }
-  for (int a = 0; a < 3; ++a) { atomicMin(&s_red[a], f2o(clo[a])); atomicMax(&s_red[3 + a], f2o(chi[a])); }
-  __syncthreads();
-  if (tid < 3) atomicMin(&w[j].bounds[tid], s_red[tid]);
-  else if (tid < 6) atomicMax(&w[j].bounds[tid], s_red[tid]);
-}
-
-// the node's centroid frame and whether it splits at the object median
-__device__ __forceinline__ bool wide_frame(const WideNode& v, const Job& job, float cmin[3], float cext[3]) {
-  bool spread = false;
-  for (int a = 0; a < 3; ++a) {
-    cmin[a] = o2f(v.bounds[a]);
-    cext[a] = o2f(v.bounds[3 + a]) - cmin[a];
-    spread |= cext[a] > 0.f;
-  }
-  const uint32_t m = job.end - job.begin;
-  const uint32_t lg = 32 - __clz(m - 1);
-  return !spread || job.depth + lg >= (uint32_t)kMaxDepth - 4;
-}
-
-// 2. bins (per-warp bins of the block, merged, added to the node's)
-__global__ void __launch_bounds__(kWideThreads)
-k_wide_bins(const float4* __restrict__ leaf_lo, const float4* __restrict__ leaf_hi,
-            const uint32_t* __restrict__ idx_in, const Job* __restrict__ jobs, uint32_t S,
-            WideNode* __restrict__ w) {
-  constexpr int kWarps = kWideThreads / 32;
-  __shared__ int s_cnt[kWarps][3][kBins];
-  __shared__ int s_box[kWarps][3][kBins][6];
-  const uint32_t j = blockIdx.x / S, sl = blockIdx.x % S, tid = threadIdx.x;
-  const Job job = jobs[j];
-  float cmin[3], cext[3];
-  if (wide_frame(w[j], job, cmin, cext)) return;         // uniform over the block
-  uint32_t sb, se;
-  slice_range(job, sl, S, sb, se);
-  for (int i = tid; i < kWarps * 3 * kBins; i += kWideThreads) {
-    const int wi = i / (3 * kBins), a = (i / kBins) % 3, q = i % kBins;
-    s_cnt[wi][a][q] = 0;
-    for (int c = 0; c < 6; ++c) s_box[wi][a][q][c] = c < 3 ? f2o(INFINITY) : f2o(-INFINITY);
-  }
-  __syncthreads();
-  for (uint32_t i = sb + tid; i < se; i += kWideThreads) {
-    const uint32_t k = idx_in[i];
-    const float4 lo = leaf_lo[k], hi = leaf_hi[k];
-    const float c[3] = {0.5f * (lo.x + hi.x), 0.5f * (lo.y + hi.y), 0.5f * (lo.z + hi.z)};
-    const float l3[3] = {lo.x, lo.y, lo.z}, h3[3] = {hi.x, hi.y, hi.z};
-    const uint32_t active = __activemask();
-    for (int a = 0; a < 3; ++a) {
-      if (!(cext[a] > 0.f)) continue;
-      const int bin = min(kBins - 1, (int)((c[a] - cmin[a]) * ((float)kBins / cext[a])));
-      const uint32_t grp = __match_any_sync(active, bin);
-      int v[6];
-      for (int q = 0; q < 3; ++q) {
-        v[q] = __reduce_min_sync(grp, f2o(l3[q]));
-        v[3 + q] = __reduce_max_sync(grp, f2o(h3[q]));
-      }
-      if ((uint32_t)(__ffs(grp) - 1) == (tid & 31)) {
-        const int wi = tid >> 5;
-        atomicAdd(&s_cnt[wi][a][bin], __popc(grp));
-        for (int q = 0; q < 3; ++q) {
-          atomicMin(&s_box[wi][a][bin][q], v[q]);
-          atomicMax(&s_box[wi][a][bin][3 + q], v[3 + q]);
+      int* to = words(t.bins) + i;
+      if (i < 64) {                              // whole warps
+        int sum = v;
+        for (int o = 1; o < kBins; o <<= 1) {
+          const int u = __shfl_up_sync(0xFFFFFFFFu, sum, o, kBins);
+          if ((i & (kBins - 1)) >= o) sum += u;
         }
+        if (op == 0) slice_cnt[(size_t)s * 3 * kBins + i] = sum;
       }
-    }
-  }
-  __syncthreads();
-  for (int i = tid; i < 3 * kBins * 7; i += kWideThreads) {
-    const int a = i / (kBins * 7), q = (i / 7) % kBins, f = i % 7;
-    if (f == 6) {
-      int t = 0;
-      for (int wi = 0; wi < kWarps; ++wi) t += s_cnt[wi][a][q];
-      if (t) atomicAdd(&w[j].cnt[a][q], t);
-    } else {
-      int v = s_box[0][a][q][f];
-      for (int wi = 1; wi < kWarps; ++wi) v = f < 3 ? min(v, s_box[wi][a][q][f]) : max(v, s_box[wi][a][q][f]);
-      if (f < 3) { if (v != f2o(INFINITY)) atomicMin(&w[j].box[a][q][f], v); }
-      else if (v != f2o(-INFINITY)) atomicMax(&w[j].box[a][q][f], v);
+      if (v == empty_word(i)) continue;
+      if (op == 0) atomicAdd(to, v); else if (op < 0) atomicMin(to, v); else atomicMax(to, v);
     }
   }
 }
 
-// the node's split from its merged bins (every block of the node the same)
-__device__ void wide_choice(const WideNode& v, const Job& job, float cmin[3], float cext[3],
-                            float* s_cost, int* s_choice) {
-  const uint32_t tid = threadIdx.x;
-  const bool median = wide_frame(v, job, cmin, cext);
-  if (!median && tid < 3 * (kBins - 1)) {
-    const int a = tid / (kBins - 1), s = tid % (kBins - 1);
-    s_cost[tid] = split_cost(v.cnt, v.box, cext[a], a, s);
-  }
-  __syncthreads();
-  if (tid == 0) {
-    if (median) { s_choice[0] = -1; s_choice[1] = 0; }
-    else pick_split(s_cost, s_choice);
-  }
-  __syncthreads();
-}
-
-__device__ __forceinline__ bool goes_left(const float4& lo, const float4& hi, int axis, int split_bin,
-                                          const float cmin[3], const float cext[3]) {
-  const float c = 0.5f * ((&lo.x)[axis] + (&hi.x)[axis]);
-  return min(kBins - 1, (int)((c - cmin[axis]) * ((float)kBins / cext[axis]))) <= split_bin;
-}
-
-// 3. the split, and the left count of each slice
-__global__ void __launch_bounds__(kWideThreads)
-k_wide_count(const float4* __restrict__ leaf_lo, const float4* __restrict__ leaf_hi,
-             const uint32_t* __restrict__ idx_in, const Job* __restrict__ jobs, uint32_t S,
-             WideNode* __restrict__ w, uint32_t* __restrict__ slice_left) {
-  __shared__ float s_cost[3 * (kBins - 1)];
-  __shared__ int s_choice[2];
-  __shared__ uint32_t s_sum;
-  const uint32_t j = blockIdx.x / S, sl = blockIdx.x % S, tid = threadIdx.x;
-  const Job job = jobs[j];
-  float cmin[3], cext[3];
-  wide_choice(w[j], job, cmin, cext, s_cost, s_choice);
-  const int axis = s_choice[0], split_bin = s_choice[1];
-  if (sl == 0 && tid == 0) { w[j].choice[0] = axis; w[j].choice[1] = split_bin; }
-  if (axis < 0) return;
-  uint32_t sb, se;
-  slice_range(job, sl, S, sb, se);
-  if (tid == 0) s_sum = 0;
-  __syncthreads();
-  uint32_t c = 0;
-  for (uint32_t i = sb + tid; i < se; i += kWideThreads) {
-    const uint32_t k = idx_in[i];
-    c += goes_left(leaf_lo[k], leaf_hi[k], axis, split_bin, cmin, cext) ? 1u : 0u;
-  }
-  c = __reduce_add_sync(0xFFFFFFFFu, c);
-  if ((tid & 31) == 0) atomicAdd(&s_sum, c);
-  __syncthreads();
-  if (tid == 0) slice_left[blockIdx.x] = s_sum;
-}
-
-// 4. stable scatter of each slice (lefts, then rights, in order) and the
-//    child boxes
-__global__ void __launch_bounds__(kWideThreads)
-k_wide_scatter(const float4* __restrict__ leaf_lo, const float4* __restrict__ leaf_hi,
-               const uint32_t* __restrict__ idx_in, uint32_t* __restrict__ idx_out,
-               const Job* __restrict__ jobs, uint32_t S, WideNode* __restrict__ w,
-               const uint32_t* __restrict__ slice_left) {
-  constexpr int kWarps = kWideThreads / 32;
-  __shared__ uint32_t s_scan[kWarps];
-  __shared__ int s_red[12];
-  const uint32_t j = blockIdx.x / S, sl = blockIdx.x % S, tid = threadIdx.x;
-  const uint32_t lane = tid & 31, warp = tid >> 5;
-  const Job job = jobs[j];
-  const uint32_t b = job.begin, m = job.end - job.begin;
-  float cmin[3], cext[3];
-  wide_frame(w[j], job, cmin, cext);
-  const int axis = w[j].choice[0], split_bin = w[j].choice[1];
-  uint32_t before = 0, n_left = 0;
-  if (axis >= 0)
-    for (uint32_t q = 0; q < S; ++q) {
-      const uint32_t v = slice_left[j * S + q];
-      if (q < sl) before += v;
-      n_left += v;
-    }
-  // an empty side cannot happen (the scatter repeats the binning
-  // arithmetic); the object median stands in, as in the one-block build
-  const bool median = axis < 0 || n_left == 0 || n_left == m;
-  if (median) n_left = m / 2;
-  if (sl == 0 && tid == 0) w[j].n_left = n_left;
-  uint32_t sb, se;
-  slice_range(job, sl, S, sb, se);
-  if (tid < 12) s_red[tid] = (tid % 6) < 3 ? f2o(INFINITY) : f2o(-INFINITY);
-  float l[2][3], h[2][3];
-  for (int c = 0; c < 2; ++c)
-    for (int x = 0; x < 3; ++x) { l[c][x] = INFINITY; h[c][x] = -INFINITY; }
-  uint32_t cnt_left = 0;
-  const uint32_t rights_before = (sb - b) - before;
-  for (uint32_t base = sb; base < se; base += kWideThreads) {
-    const uint32_t i = base + tid;
-    bool left = false;
-    uint32_t k = 0;
-    float4 lo = make_float4(0.f, 0.f, 0.f, 0.f), hi = lo;
-    if (i < se) {
-      k = idx_in[i];
-      lo = leaf_lo[k];
-      hi = leaf_hi[k];
-      left = median ? (i - b) < n_left : goes_left(lo, hi, axis, split_bin, cmin, cext);
-    }
-    const uint32_t ball = __ballot_sync(0xFFFFFFFFu, left);
-    __syncthreads();
-    if (lane == 0) s_scan[warp] = __popc(ball);
-    __syncthreads();
-    uint32_t wb = 0, chunk = 0;
-    for (uint32_t q = 0; q < (uint32_t)kWarps; ++q) {
-      if (q < warp) wb += s_scan[q];
-      chunk += s_scan[q];
-    }
-    const uint32_t rank = wb + __popc(ball & ((1u << lane) - 1u));   // lefts before i in the chunk
-    if (i < se) {
-      const uint32_t t = i - base;
-      if (median) idx_out[i] = k;
-      else if (left) idx_out[b + before + cnt_left + rank] = k;
-      else idx_out[b + n_left + rights_before + ((base - sb) - cnt_left) + (t - rank)] = k;
-      const int c = left ? 0 : 1;
-      l[c][0] = fminf(l[c][0], lo.x); l[c][1] = fminf(l[c][1], lo.y); l[c][2] = fminf(l[c][2], lo.z);
-      h[c][0] = fmaxf(h[c][0], hi.x); h[c][1] = fmaxf(h[c][1], hi.y); h[c][2] = fmaxf(h[c][2], hi.z);
-    }
-    cnt_left += chunk;
-  }
-  for (int c = 0; c < 2; ++c)
-    for (int x = 0; x < 3; ++x) {
-      atomicMin(&s_red[6 * c + x], f2o(l[c][x]));
-      atomicMax(&s_red[6 * c + 3 + x], f2o(h[c][x]));
-    }
-  __syncthreads();
+// 3. a node's record, and its children: top entries of the next level, mid
+// jobs or leaves (one block)
+struct NodeShared {
+  float box[2][6];
+  uint32_t at[2], slice0[2], id;
+};
+__device__ void top_node(const TopNode& t, uint32_t n_left, int axis, int bin, const uint32_t* idx_out,
+                         const Build& g, int cur, NodeShared& sh) {
+  const uint32_t tid = threadIdx.x, b = t.job.begin, e = t.job.end, split = b + n_left;
+  const uint32_t rb[2] = {b, split}, re[2] = {split, e};
+  Control* ctl = g.ctl;
   if (tid < 12) {
     const int c = tid / 6, f = tid % 6;
-    if (f < 3) { if (s_red[tid] != f2o(INFINITY)) atomicMin(&w[j].child[c][f], s_red[tid]); }
-    else if (s_red[tid] != f2o(-INFINITY)) atomicMax(&w[j].child[c][f], s_red[tid]);
-  }
-}
-
-// 5. the node records and the next jobs (one thread per node)
-__global__ void k_wide_nodes(const Job* __restrict__ jobs, uint32_t count, const WideNode* __restrict__ w,
-                             const uint32_t* __restrict__ idx_out, Job* __restrict__ next,
-                             uint32_t* __restrict__ next_count, Job* __restrict__ small,
-                             uint32_t* __restrict__ small_count, uint32_t out_buf, float4* __restrict__ out,
-                             uint32_t* __restrict__ root_split, uint32_t n, uint32_t* __restrict__ err) {
-  const uint32_t j = blockIdx.x * blockDim.x + threadIdx.x;
-  if (j >= count) return;
-  float cl[2][3], ch[2][3];
-  for (int c = 0; c < 2; ++c)
-    for (int x = 0; x < 3; ++x) { cl[c][x] = o2f(w[j].child[c][x]); ch[c][x] = o2f(w[j].child[c][3 + x]); }
-  write_node(jobs[j], w[j].n_left, cl, ch, idx_out, next, next_count, small, small_count, out_buf, out,
-             root_split, n, err);
-}
-
-// warp-wide inclusive scan of a box (lanes in order), forward or backward
-__device__ __forceinline__ void box_scan(float lo[3], float hi[3], bool backward) {
-  const uint32_t lane = threadIdx.x & 31;
-  for (int o = 1; o < 32; o <<= 1) {
-    float l[3], h[3];
-    for (int x = 0; x < 3; ++x) {
-      l[x] = backward ? __shfl_down_sync(0xFFFFFFFFu, lo[x], o) : __shfl_up_sync(0xFFFFFFFFu, lo[x], o);
-      h[x] = backward ? __shfl_down_sync(0xFFFFFFFFu, hi[x], o) : __shfl_up_sync(0xFFFFFFFFu, hi[x], o);
-    }
-    const bool ok = backward ? lane + o < 32 : lane >= (uint32_t)o;
-    if (ok)
-      for (int x = 0; x < 3; ++x) { lo[x] = fminf(lo[x], l[x]); hi[x] = fmaxf(hi[x], h[x]); }
-  }
-}
-
-// Subtrees of at most kSmallLeaves leaves, one warp each: every node takes
-// the split of least SAH cost over all positions of its leaves sorted by
-// centroid on each axis (a warp bitonic sort, ties by leaf order, then box
-// prefix and suffix scans), or the median of the current order when the
-// depth budget is short. Node ids follow the split positions as in
-// k_sah_level.
-constexpr int kSmallWarps = 4;
-__global__ void __launch_bounds__(32 * kSmallWarps)
-k_sah_small(const float4* __restrict__ leaf_lo, const float4* __restrict__ leaf_hi,
-            uint32_t* const* __restrict__ idx_bufs, const Job* __restrict__ jobs, uint32_t n_jobs,
-            float4* __restrict__ out, const uint32_t* __restrict__ root_split, uint32_t n,
-            uint32_t* __restrict__ err) {
-  __shared__ uint32_t s_slot[kSmallWarps][kSmallLeaves];     // leaf slots in the current order
-  __shared__ float s_box[kSmallWarps][kSmallLeaves][6];
-  __shared__ uint32_t s_tmp[kSmallWarps][kSmallLeaves];
-  __shared__ float s_tbox[kSmallWarps][kSmallLeaves][6];
-  __shared__ Job s_stack[kSmallWarps][kSmallLeaves];
-  const uint32_t warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const uint32_t j = blockIdx.x * kSmallWarps + warp;
-  if (j >= n_jobs) return;
-  const Job job = jobs[j];
-  const uint32_t base = job.begin, m = job.end - job.begin;
-  const uint32_t* idx = idx_bufs[job.depth >> 31];
-  if (m < 2 || m > (uint32_t)kSmallLeaves) { if (lane == 0) atomicOr(err, ERR_BUILD); return; }
-  const uint32_t rs = *root_split;
-  if (lane < m) {
-    const uint32_t k = idx[base + lane];
-    s_slot[warp][lane] = k;
-    const float4 lo = leaf_lo[k], hi = leaf_hi[k];
-    s_box[warp][lane][0] = lo.x; s_box[warp][lane][1] = lo.y; s_box[warp][lane][2] = lo.z;
-    s_box[warp][lane][3] = hi.x; s_box[warp][lane][4] = hi.y; s_box[warp][lane][5] = hi.z;
-  }
-  int sp = 0;
-  if (lane == 0) s_stack[warp][0] = Job{0, m, job.parent_slot, job.depth & 0x7FFFFFFFu};
-  sp = 1;
-  __syncwarp();
-  for (uint32_t guard = 0; sp > 0 && guard < 2 * kSmallLeaves; ++guard) {
-    const Job t = s_stack[warp][--sp];
-    __syncwarp();
-    const uint32_t b = t.begin, s = t.end - t.begin;
-    const bool in = lane < s;
-    float blo[3] = {INFINITY, INFINITY, INFINITY}, bhi[3] = {-INFINITY, -INFINITY, -INFINITY};
-    if (in)
-      for (int x = 0; x < 3; ++x) { blo[x] = s_box[warp][b + lane][x]; bhi[x] = s_box[warp][b + lane][3 + x]; }
-    uint32_t k_split = s / 2;                 // median of the current order unless the SAH wins
-    int best_axis = -1;
-    float best_cost = INFINITY;
-    if (t.depth + s - 1 <= (uint32_t)kMaxDepth) {
-      for (int axis = 0; axis < 3; ++axis) {
-        // sort (centroid, position) ascending over the lanes; out-of-range lanes last
-        float key = in ? 0.5f * (blo[axis] + bhi[axis]) : INFINITY;
-        uint32_t val = in ? lane : 0xFFFFFFFFu;
-        for (uint32_t kk = 2; kk <= 32; kk <<= 1)
-          for (uint32_t jj = kk >> 1; jj > 0; jj >>= 1) {
-            const float ok = __shfl_xor_sync(0xFFFFFFFFu, key, jj);
-            const uint32_t ov = __shfl_xor_sync(0xFFFFFFFFu, val, jj);
-            const bool up = (lane & kk) == 0, lower = (lane & jj) == 0;
-            const bool other_less = ok < key || (ok == key && ov < val);
-            const bool take = (lower == up) ? other_less : !other_less && !(ok == key && ov == val);
-            if (take) { key = ok; val = ov; }
-          }
-        // boxes in sorted order; prefix and suffix unions
-        float plo[3], phi[3], qlo[3], qhi[3];
-        for (int x = 0; x < 3; ++x) {
-          const float vlo = val < s ? s_box[warp][b + val][x] : INFINITY;
-          const float vhi = val < s ? s_box[warp][b + val][3 + x] : -INFINITY;
-          plo[x] = qlo[x] = vlo; phi[x] = qhi[x] = vhi;
-        }
-        box_scan(plo, phi, false);
-        box_scan(qlo, qhi, true);
-        // split after sorted position lane (left lane+1 leaves)
-        float q2lo[3], q2hi[3];
-        for (int x = 0; x < 3; ++x) {
-          q2lo[x] = __shfl_down_sync(0xFFFFFFFFu, qlo[x], 1);
-          q2hi[x] = __shfl_down_sync(0xFFFFFFFFu, qhi[x], 1);
-        }
-        float cost = INFINITY;
-        if (lane + 1 < s)
-          cost = half_area(plo, phi) * (float)(lane + 1) + half_area(q2lo, q2hi) * (float)(s - lane - 1);
-        // warp argmin, lowest position among equal costs
-        float bc = cost;
-        uint32_t bl = lane;
-        for (int o = 16; o > 0; o >>= 1) {
-          const float c2 = __shfl_xor_sync(0xFFFFFFFFu, bc, o);
-          const uint32_t l2 = __shfl_xor_sync(0xFFFFFFFFu, bl, o);
-          if (c2 < bc || (c2 == bc && l2 < bl)) { bc = c2; bl = l2; }
-        }
-        if (bc < best_cost) {               // warp-uniform
-          best_cost = bc;
-          best_axis = axis;
-          k_split = bl + 1;
-          // keep this axis's order
-          if (in) {
-            s_tmp[warp][lane] = s_slot[warp][b + val];
-            for (int x = 0; x < 6; ++x) s_tbox[warp][lane][x] = s_box[warp][b + val][x];
-          }
-        }
-        __syncwarp();
+    int v = empty6(f);
+    if (axis < 0) {
+      v = __ldcg(&t.child_box[c][f]);
+    } else {
+      for (int q = 0; q < kBins; ++q) {
+        const int x = t.bins.box[axis][q][f];        // an empty bin's box is empty
+        if ((q <= bin) == (c == 0)) v = f < 3 ? min(v, x) : max(v, x);
       }
-      if (best_axis >= 0 && in) {
-        s_slot[warp][b + lane] = s_tmp[warp][lane];
-        for (int x = 0; x < 6; ++x) s_box[warp][b + lane][x] = s_tbox[warp][lane][x];
+    }
+    sh.box[c][f] = o2f(v);
+  }
+  if (tid == 0) {
+    if (t.job.parent_slot == kRoot) ctl->root_split = split;
+    const uint32_t id = place_node(split, t.job.parent_slot, ctl->root_split, g.out, g.n, g.err);
+    sh.id = id;
+    for (int c = 0; c < 2; ++c) {
+      const uint32_t m = re[c] - rb[c];
+      sh.at[c] = kRoot;
+      if (m == 1) continue;
+      if (m <= kMidLeaves) {
+        const uint32_t at = atomicAdd(&ctl->n_mid, 1u);
+        if (at >= g.max_mid) { atomicOr(g.err, ERR_BUILD); continue; }
+        g.mid[at] = Job{rb[c], re[c], id << 1 | (uint32_t)c, (t.job.depth + 1) | ((uint32_t)(cur ^ 1) << 31)};
+      } else {
+        const uint32_t ns = (uint32_t)(((uint64_t)m + g.slice - 1) / g.slice);
+        const uint32_t at = atomicAdd(&ctl->n_nodes[cur ^ 1], 1u), s0 = atomicAdd(&ctl->n_slices[cur ^ 1], ns);
+        if (at >= g.max_nodes || s0 + ns > g.max_slices) { atomicOr(g.err, ERR_BUILD); continue; }
+        sh.at[c] = at;
+        sh.slice0[c] = s0;
+      }
+    }
+  }
+  __syncthreads();
+  const uint32_t id = sh.id;
+  if (tid == 0) {
+    float cl[2][3], ch[2][3];
+    for (int c = 0; c < 2; ++c)
+      for (int x = 0; x < 3; ++x) { cl[c][x] = sh.box[c][x]; ch[c][x] = sh.box[c][3 + x]; }
+    write_node(g.out, id, cl, ch, re[0] - rb[0] == 1 ? __ldcg(idx_out + rb[0]) : kRoot,
+               re[1] - rb[1] == 1 ? __ldcg(idx_out + rb[1]) : kRoot);
+  }
+  for (int c = 0; c < 2; ++c) {
+    if (sh.at[c] == kRoot) continue;
+    TopNode& u = g.nodes[1][sh.at[c]];
+    const uint32_t m = re[c] - rb[c], ns = (uint32_t)(((uint64_t)m + g.slice - 1) / g.slice);
+    for (int i = tid; i < kBinWords; i += kThreads) words(u.bins)[i] = empty_word(i);
+    if (tid < 6) u.bounds[tid] = __ldcg(&t.child_bounds[c][tid]);
+    if (tid < 12) {
+      u.child_bounds[tid / 6][tid % 6] = empty6(tid % 6);
+      u.child_box[tid / 6][tid % 6] = empty6(tid % 6);
+    }
+    if (tid == 0) {
+      u.job = Job{rb[c], re[c], id << 1 | (uint32_t)c, t.job.depth + 1};
+      u.slice0 = sh.slice0[c];
+      u.n_slices = ns;
+      u.done = 0;
+    }
+    for (uint32_t i = tid; i < ns; i += kThreads) g.slice_node[1][sh.slice0[c] + i] = sh.at[c];
+  }
+}
+
+// 2. the node's split (every slice computes it) and the stable partition of
+// the slice, with the centroid bounds (and for a median the boxes) of the sides;
+// then step 3 by the node's last slice
+__global__ void __launch_bounds__(kThreads, 4)
+k_top_scatter(const Build g, int cur) {
+  uint32_t* __restrict__ idx_out = g.idx[1];
+  const uint32_t* __restrict__ slice_node = g.slice_node[0];
+  const int* __restrict__ slice_cnt = g.slice_cnt;
+  TopNode* nodes = g.nodes[0];
+  const uint32_t slice = g.slice;
+  __shared__ NodeShared s_node;
+  __shared__ bool s_last;
+  __shared__ Bins s_bins;
+  __shared__ int s_choice[2];
+  __shared__ uint32_t s_sum[2], s_scan[kUnroll][kWarps];
+  __shared__ int s_bounds[2][6], s_box[2][6];
+  const uint32_t tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, n_slices = g.ctl->n_slices[cur];
+  for (uint32_t s = blockIdx.x; s < n_slices; s += gridDim.x) {
+    TopNode& t = nodes[slice_node[s]];
+    const uint32_t b = t.job.begin, m = t.job.end - b, q = s - t.slice0;
+    float cmin[3], cext[3];
+    bool median = node_frame(t.bounds, m, t.job.depth, cmin, cext);
+    __syncthreads();
+    for (int i = tid; i < kBinWords; i += kThreads) words(s_bins)[i] = words(t.bins)[i];
+    if (tid < 12) {
+      s_bounds[tid / 6][tid % 6] = empty6(tid % 6);
+      s_box[tid / 6][tid % 6] = empty6(tid % 6);
+    }
+    if (tid < 2) s_sum[tid] = 0;
+    __syncthreads();
+    if (!median && warp == 0) {
+      int axis, bin;
+      choose_split(s_bins, cext, axis, bin);
+      if (lane == 0) { s_choice[0] = axis; s_choice[1] = bin; }
+    }
+    __syncthreads();
+    int axis = median ? -1 : s_choice[0], bin = median ? 0 : s_choice[1];
+    // lefts of the slices before this one, and of the node
+    if (axis >= 0) {
+      uint32_t before = 0, all = 0;
+      for (uint32_t r = tid; r < t.n_slices; r += kThreads) {
+        const uint32_t left = (uint32_t)slice_cnt[(size_t)(t.slice0 + r) * 3 * kBins + axis * kBins + bin];
+        all += left;
+        if (r < q) before += left;
+      }
+      before = __reduce_add_sync(0xFFFFFFFFu, before);
+      all = __reduce_add_sync(0xFFFFFFFFu, all);
+      if (lane == 0 && all) { atomicAdd(&s_sum[0], before); atomicAdd(&s_sum[1], all); }
+    }
+    __syncthreads();
+    const uint32_t before = s_sum[0];
+    uint32_t n_left = s_sum[1];
+    // an empty side cannot happen with an axis (its cost is infinite)
+    if (axis < 0 || n_left == 0 || n_left == m) { axis = -1; n_left = m / 2; }
+    uint32_t sb, se;
+    slice_range(t, s, slice, sb, se);
+    const uint32_t rights_before = (sb - b) - before;
+    uint32_t cnt_left = 0;
+    int sides[2][6];                              // centroid bounds of the thread's lefts and rights
+    for (int c = 0; c < 2; ++c)
+      for (int f = 0; f < 6; ++f) sides[c][f] = empty6(f);
+    for (uint32_t base = sb; base < se; base += kUnroll * kThreads) {
+      float4 lo[kUnroll], hi[kUnroll];
+      uint32_t k[kUnroll], ball[kUnroll];
+      load_leaves(g, base, se, lo, hi, k);
+#pragma unroll
+      for (int u = 0; u < kUnroll; ++u) {
+        const uint32_t i = base + u * kThreads + tid;
+        float c[3];
+        centroid(lo[u], hi[u], c);
+        const bool left = i < se && (axis < 0 ? i - b < n_left
+                                              : bin_of(at3(c, axis), at3(cmin, axis), at3(cext, axis)) <= bin);
+        ball[u] = __ballot_sync(0xFFFFFFFFu, left);
+        if (lane == 0) s_scan[u][warp] = __popc(ball[u]);
+      }
+      __syncthreads();
+#pragma unroll
+      for (int u = 0; u < kUnroll; ++u) {
+        const uint32_t i = base + u * kThreads + tid;
+        uint32_t wb = 0, chunk = 0;
+#pragma unroll
+        for (uint32_t w = 0; w < (uint32_t)kWarps; ++w) {
+          const uint32_t x = s_scan[u][w];
+          if (w < warp) wb += x;
+          chunk += x;
+        }
+        const uint32_t rank = wb + __popc(ball[u] & ((1u << lane) - 1u));   // lefts before i among these
+        const uint32_t in = __ballot_sync(0xFFFFFFFFu, i < se);
+        if (i < se) {
+          const bool left = ball[u] >> lane & 1u;
+          if (axis < 0) idx_out[i] = k[u];
+          else if (left) idx_out[b + before + cnt_left + rank] = k[u];
+          else idx_out[b + n_left + rights_before + (i - sb) - cnt_left - rank] = k[u];
+          float c[3];
+          int v[6];
+          centroid(lo[u], hi[u], c);
+          centroid6(c, v);
+#pragma unroll
+          for (int f = 0; f < 3; ++f) {
+            sides[0][f] = min(sides[0][f], left ? v[f] : empty6(f));
+            sides[1][f] = min(sides[1][f], left ? empty6(f) : v[f]);
+            sides[0][3 + f] = max(sides[0][3 + f], left ? v[3 + f] : empty6(3));
+            sides[1][3 + f] = max(sides[1][3 + f], left ? empty6(3) : v[3 + f]);
+          }
+          if (axis < 0) {
+            box6(lo[u], hi[u], v);
+            combine6(left ? ball[u] : in & ~ball[u], v, s_box[left ? 0 : 1]);
+          }
+        }
+        cnt_left += chunk;
+      }
+      __syncthreads();
+    }
+    for (int c = 0; c < 2; ++c) combine6(0xFFFFFFFFu, sides[c], s_bounds[c]);
+    __syncthreads();
+    if (tid < 12) {
+      const int c = tid / 6, f = tid % 6, v = s_bounds[c][f], w = s_box[c][f];
+      if (v != empty6(f)) {
+        if (f < 3) atomicMin(&t.child_bounds[c][f], v); else atomicMax(&t.child_bounds[c][f], v);
+      }
+      if (axis < 0 && w != empty6(f)) {
+        if (f < 3) atomicMin(&t.child_box[c][f], w); else atomicMax(&t.child_box[c][f], w);
+      }
+    }
+    // the slice that finishes last writes the node
+    __threadfence();
+    __syncthreads();
+    if (tid == 0) s_last = atomicAdd(&t.done, 1u) + 1 == t.n_slices;
+    __syncthreads();
+    if (s_last) {
+      __threadfence();
+      top_node(t, n_left, axis, bin, idx_out, g, cur, s_node);
+    }
+  }
+}
+
+// ------------------------------------------------------------------ mid phase
+// The subtree over the m <= 32 leaves of a segment (one warp; lane < m: leaf
+// slot and box): every node takes the split of least SAH cost over all
+// positions of its leaves sorted by centroid on each axis (ties by the current
+// order, then by the lower axis), or the middle of the current order when the
+// depth budget is short. All nodes of a level at once: lane l belongs to the
+// segment [b, e) of lanes. Shuffles bound it (they share the one shared-memory
+// pipe of the SM), so ranks are counted and scans run only as far as the level's
+// longest segment, and only the winning position's child boxes are handed out.
+// key: the warp's scratch.
+__device__ void small_subtree(uint32_t m, uint32_t slot, float bx[6], uint32_t base, uint32_t parent_slot,
+                              uint32_t depth, uint32_t root_split, float4* __restrict__ out, uint32_t n,
+                              uint32_t* __restrict__ err, uint32_t* key) {
+  const uint32_t lane = threadIdx.x & 31;
+  uint32_t b = lane < m ? 0u : lane, e = lane < m ? m : lane + 1;
+  for (uint32_t guard = 0; guard < kSmallLeaves; ++guard) {
+    const uint32_t s = e - b;
+    const bool active = s >= 2;
+    const uint32_t longest = __reduce_max_sync(0xFFFFFFFFu, s);
+    if (longest < 2) return;
+    const bool sah = active && depth + s - 1 <= (uint32_t)kMaxDepth;
+    uint32_t order = lane, cut = b + s / 2 - 1;       // source lane of this position; last left position
+    float c0[6] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f}, c1[6] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f};   // child boxes
+    if (!__any_sync(0xFFFFFFFFu, s > 2 || (active && !sah))) {
+      // two leaves: every axis costs the same, so the first one's order (a
+      // cost past the largest float: the current order)
+      const uint32_t other = active ? (lane == b ? b + 1 : b) : lane;
+      const float mine = 0.5f * (bx[0] + bx[3]), area = half_area(bx, bx + 3);
+      const float theirs = __shfl_sync(0xFFFFFFFFu, mine, other), oa = __shfl_sync(0xFFFFFFFFu, area, other);
+      if (active) {
+        const bool swap = lane == b ? theirs < mine : mine < theirs;
+        if (swap && area + oa < INFINITY) order = other;
+        cut = b;
+      }
+      for (int x = 0; x < 6; ++x) {
+        const float v = __shfl_sync(0xFFFFFFFFu, bx[x], order);   // box at this position
+        c0[x] = __shfl_sync(0xFFFFFFFFu, v, b);
+        c1[x] = __shfl_sync(0xFFFFFFFFu, v, e - 1);
+      }
+    } else {
+      float best = INFINITY;
+      uint32_t at = 96, vals = 0;                    // axis << 5 | position of `best`; the three orders, 5 bits each
+      // rank by (centroid with -0 as 0, position) in the segment, all axes at once
+      int k3[3];
+      uint32_t rank[3] = {b, b, b};
+      for (int a = 0; a < 3; ++a) k3[a] = f2o(0.5f * (bx[a] + bx[3 + a]) + 0.f);
+      for (uint32_t j = 0; j < longest; ++j) {
+        const uint32_t src = b + j;
+        const bool in = src < e;
+#pragma unroll
+        for (int a = 0; a < 3; ++a) {
+          const int o = __shfl_sync(0xFFFFFFFFu, k3[a], src & 31u);
+          rank[a] += in && (src < lane ? o <= k3[a] : o < k3[a]) ? 1u : 0u;
+        }
       }
       __syncwarp();
-    }
-    // child boxes of the split at k_split in the current order
-    float c0lo[3], c0hi[3], c1lo[3], c1hi[3];
-    for (int x = 0; x < 3; ++x) {
-      const bool l0 = in && lane < k_split, l1 = in && lane >= k_split;
-      const float vlo = in ? s_box[warp][b + lane][x] : INFINITY, vhi = in ? s_box[warp][b + lane][3 + x] : -INFINITY;
-      float a0 = l0 ? vlo : INFINITY, a1 = l1 ? vlo : INFINITY, z0 = l0 ? vhi : -INFINITY, z1 = l1 ? vhi : -INFINITY;
-      for (int o = 16; o > 0; o >>= 1) {
-        a0 = fminf(a0, __shfl_xor_sync(0xFFFFFFFFu, a0, o));
-        a1 = fminf(a1, __shfl_xor_sync(0xFFFFFFFFu, a1, o));
-        z0 = fmaxf(z0, __shfl_xor_sync(0xFFFFFFFFu, z0, o));
-        z1 = fmaxf(z1, __shfl_xor_sync(0xFFFFFFFFu, z1, o));
+      for (int a = 0; a < 3; ++a) {
+        key[rank[a]] = lane;
+        __syncwarp();
+        vals |= key[lane] << (5 * a);
+        __syncwarp();
       }
-      c0lo[x] = a0; c1lo[x] = a1; c0hi[x] = z0; c1hi[x] = z1;
-    }
-    if (lane == 0) {
-      const uint32_t split = base + b + k_split;      // global split position
-      const uint32_t id = split == 1 ? rs - 1 : split - 1;
-      reinterpret_cast<int32_t*>(out + 4 * (size_t)(t.parent_slot >> 1) + 3)[t.parent_slot & 1u] = (int32_t)id;
-      if (id < n - 1) {
-        float4* o = out + 4 * (size_t)id;
-        o[0] = make_float4(c0lo[0], c0hi[0], c0lo[1], c0hi[1]);
-        o[1] = make_float4(c1lo[0], c1hi[0], c1lo[1], c1hi[1]);
-        o[2] = make_float4(c0lo[2], c0hi[2], c1lo[2], c1hi[2]);
-        const uint32_t rb[2] = {b, b + k_split}, re[2] = {b + k_split, b + s};
-        int32_t child[2];
-        for (int c = 0; c < 2; ++c) {
-          if (re[c] - rb[c] == 1) {
-            child[c] = ~(int32_t)s_slot[warp][rb[c]];
-          } else {
-            child[c] = 0;                       // filled in when the child is built
-            s_stack[warp][sp + c] = Job{rb[c], re[c], id << 1 | (uint32_t)c, t.depth + 1};
+      for (int axis = 0; axis < 3; ++axis) {
+        const uint32_t val = vals >> (5 * axis) & 31u;
+        float p[6], q[6];
+        for (int x = 0; x < 6; ++x) p[x] = q[x] = __shfl_sync(0xFFFFFFFFu, bx[x], val);
+        for (uint32_t o = 1; o < longest; o <<= 1) {
+          const bool up = lane >= b + o, dn = lane + o < e;
+#pragma unroll
+          for (int x = 0; x < 6; ++x) {
+            const float u = __shfl_up_sync(0xFFFFFFFFu, p[x], o), d = __shfl_down_sync(0xFFFFFFFFu, q[x], o);
+            if (up) p[x] = x < 3 ? fminf(p[x], u) : fmaxf(p[x], u);
+            if (dn) q[x] = x < 3 ? fminf(q[x], d) : fmaxf(q[x], d);
           }
         }
-        o[3] = make_float4(__int_as_float(child[0]), __int_as_float(child[1]), 0.f, 0.f);
-      } else {
-        atomicOr(err, ERR_BUILD);
+        for (int x = 0; x < 6; ++x) q[x] = __shfl_down_sync(0xFFFFFFFFu, q[x], 1);   // of the positions after this one
+        if (sah && lane + 1 < e) {
+          const float cost = half_area(p, p + 3) * (float)(lane - b + 1) + half_area(q, q + 3) * (float)(e - lane - 1);
+          if (cost < best) {
+            best = cost;
+            at = (uint32_t)axis << 5 | lane;
+            for (int x = 0; x < 6; ++x) { c0[x] = p[x]; c1[x] = q[x]; }
+          }
+        }
+      }
+      // the segment's least cost; among equals the lower axis, then position: its last lane's prefix
+      for (uint32_t o = 1; o < longest; o <<= 1) {
+        const float c = __shfl_up_sync(0xFFFFFFFFu, best, o);
+        const uint32_t i = __shfl_up_sync(0xFFFFFFFFu, at, o);
+        if (lane >= b + o && (c < best || (c == best && i < at))) { best = c; at = i; }
+      }
+      best = __shfl_sync(0xFFFFFFFFu, best, e - 1);
+      at = __shfl_sync(0xFFFFFFFFu, at, e - 1);
+      const bool found = active && best < INFINITY;
+      if (found) { cut = at & 31u; order = vals >> (5 * (at >> 5)) & 31u; }
+      for (int x = 0; x < 6; ++x) {
+        c0[x] = __shfl_sync(0xFFFFFFFFu, c0[x], cut & 31u);
+        c1[x] = __shfl_sync(0xFFFFFFFFu, c1[x], cut & 31u);
+      }
+      // no split by cost: the middle of the current order, its boxes by walking the segment
+      if (__any_sync(0xFFFFFFFFu, active && !found)) {
+        float m0[6], m1[6];
+        for (int x = 0; x < 6; ++x) m0[x] = m1[x] = x < 3 ? INFINITY : -INFINITY;
+        for (uint32_t j = 0; j < longest; ++j)
+          for (int x = 0; x < 6; ++x) {
+            const float v = __shfl_sync(0xFFFFFFFFu, bx[x], (b + j) & 31u);
+            if (b + j <= cut) m0[x] = x < 3 ? fminf(m0[x], v) : fmaxf(m0[x], v);
+            else if (b + j < e) m1[x] = x < 3 ? fminf(m1[x], v) : fmaxf(m1[x], v);
+          }
+        if (active && !found)
+          for (int x = 0; x < 6; ++x) { c0[x] = m0[x]; c1[x] = m1[x]; }
       }
     }
-    __syncwarp();
-    // the pushes lane 0 made (warp-uniform count)
-    sp += (k_split > 1 ? 1 : 0) + (s - k_split > 1 ? 1 : 0);
-    if (k_split == 1 && s - k_split > 1) {      // only the right child was pushed, at sp + 1
-      if (lane == 0) s_stack[warp][sp - 1] = s_stack[warp][sp];
+    slot = __shfl_sync(0xFFFFFFFFu, slot, order);
+    for (int x = 0; x < 6; ++x) bx[x] = __shfl_sync(0xFFFFFFFFu, bx[x], order);
+    const uint32_t mid = cut + 1;                    // first right position
+    const uint32_t right_slot = __shfl_sync(0xFFFFFFFFu, slot, active ? mid : lane);
+    uint32_t id = 0;
+    if (active && lane == b) {
+      id = place_node(base + mid, parent_slot, root_split, out, n, err);
+      const float cl[2][3] = {{c0[0], c0[1], c0[2]}, {c1[0], c1[1], c1[2]}};
+      const float ch[2][3] = {{c0[3], c0[4], c0[5]}, {c1[3], c1[4], c1[5]}};
+      write_node(out, id, cl, ch, mid - b == 1 ? slot : kRoot, e - mid == 1 ? right_slot : kRoot);
+    }
+    id = __shfl_sync(0xFFFFFFFFu, id, b);
+    if (active) {
+      const bool right = lane >= mid;
+      parent_slot = id << 1 | (right ? 1u : 0u);
+      ++depth;
+      if (right) b = mid; else e = mid;
     }
     __syncwarp();
   }
-  if (sp != 0 && lane == 0) atomicOr(err, ERR_BUILD);
+  if (lane == 0) atomicOr(err, ERR_BUILD);
 }
 
-}  // namespace
+// Subtrees of 2 to kMidLeaves leaves, one block each, one thread per leaf.
+constexpr int kMaxSeg = (int)(kMidLeaves / (kSmallLeaves + 1));   // segments of more than kSmallLeaves leaves (or the root)
+static_assert(kMaxSeg <= kWarps, "a warp per segment");
+__global__ void __launch_bounds__(kThreads, 4)
+k_sah_mid(const float4* __restrict__ leaf_lo, const float4* __restrict__ leaf_hi,
+          const uint32_t* __restrict__ idx0, const uint32_t* __restrict__ idx1, Control* ctl,
+          const Job* __restrict__ jobs, float4* __restrict__ out, uint32_t n, uint32_t* __restrict__ err) {
+  __shared__ uint32_t s_slot[kThreads];
+  __shared__ float s_box[6][kThreads];
+  __shared__ uint32_t s_begin[kThreads], s_end[kThreads];          // segment of each position
+  __shared__ uint32_t s_parent[kThreads], s_depth[kThreads];       // of the segment that begins here
+  __shared__ uint32_t s_scan[kWarps], s_seg[kThreads];
+  __shared__ Bins s_bins[kMaxSeg];
+  __shared__ int s_bounds[kMaxSeg][6], s_child[kMaxSeg][2][6];
+  __shared__ int s_choice[kMaxSeg][2];
+  __shared__ uint32_t s_at[kMaxSeg], s_nleft[kMaxSeg], s_root_split, s_total, s_key[kWarps][kSmallLeaves];
+  const uint32_t tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, n_jobs = ctl->n_mid;
+  for (uint32_t j = blockIdx.x; j < n_jobs; j += gridDim.x) {
+    const Job job = jobs[j];
+    const uint32_t base = job.begin, m = job.end - job.begin;
+    if (m < 2 || m > kMidLeaves) { if (tid == 0) atomicOr(err, ERR_BUILD); continue; }   // block-uniform
+    const uint32_t* idx = job.depth >> 31 ? idx1 : idx0;
+    __syncthreads();
+    if (tid == 0) s_root_split = ctl->root_split;
+    uint32_t slot = 0;
+    float bx[6] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+    if (tid < m) {
+      slot = idx[base + tid];
+      const float4 lo = leaf_lo[slot], hi = leaf_hi[slot];
+      bx[0] = lo.x; bx[1] = lo.y; bx[2] = lo.z; bx[3] = hi.x; bx[4] = hi.y; bx[5] = hi.z;
+    }
+    s_begin[tid] = tid < m ? 0u : tid;
+    s_end[tid] = tid < m ? m : tid + 1;
+    if (tid == 0) { s_parent[0] = job.parent_slot; s_depth[0] = job.depth & 0x7FFFFFFFu; }
+    __syncthreads();
+    for (int level = 0; level <= kMaxDepth; ++level) {
+      const uint32_t b = s_begin[tid], e = s_end[tid], sz = e - b;
+      const bool active = sz > kSmallLeaves || (sz >= 2 && s_parent[b] == kRoot);
+      // ordinals of the active segments
+      const bool head = active && tid == b;
+      const uint32_t hb = __ballot_sync(0xFFFFFFFFu, head);
+      if (lane == 0) s_scan[warp] = __popc(hb);
+      if (tid < kMaxSeg * 6) s_bounds[tid / 6][tid % 6] = empty6(tid % 6);
+      if (tid < kMaxSeg * 12) s_child[tid / 12][(tid / 6) % 2][tid % 6] = empty6(tid % 6);
+      __syncthreads();
+      uint32_t ord = 0, n_seg = 0;
+      for (uint32_t w = 0; w < (uint32_t)kWarps; ++w) {
+        if (w < warp) ord += s_scan[w];
+        n_seg += s_scan[w];
+      }
+      if (n_seg == 0) break;                                   // block-uniform
+      if (head) { ord += __popc(hb & ((1u << lane) - 1u)); s_seg[b] = ord; s_at[ord] = b; }
+      for (uint32_t i = tid; i < (uint32_t)kBinWords; i += kThreads) {
+        const int v = empty_word((int)i);
+        for (uint32_t w = 0; w < n_seg; ++w) words(s_bins[w])[i] = v;
+      }
+      __syncthreads();
+      const uint32_t g = active ? s_seg[b] : 0xFFu, members = __ballot_sync(0xFFFFFFFFu, active);
+      const float c[3] = {0.5f * (bx[0] + bx[3]), 0.5f * (bx[1] + bx[4]), 0.5f * (bx[2] + bx[5])};
+      const int v6[6] = {f2o(bx[0]), f2o(bx[1]), f2o(bx[2]), f2o(bx[3]), f2o(bx[4]), f2o(bx[5])};
+      if (active) {
+        int cv[6];
+        centroid6(c, cv);
+        combine6(__match_any_sync(members, g), cv, s_bounds[g]);
+      }
+      __syncthreads();
+      float cmin[3] = {0.f, 0.f, 0.f}, cext[3] = {0.f, 0.f, 0.f};
+      bool median = true;
+      if (active) median = node_frame(s_bounds[g], sz, s_depth[b], cmin, cext);
+      for (int a = 0; a < 3; ++a) {
+        if (median || !(cext[a] > 0.f)) continue;
+        const int bin = bin_of(c[a], cmin[a], cext[a]);
+        add_box(s_bins[g], a, bin, v6);
+      }
+      __syncthreads();
+      if (warp < n_seg) {
+        float ext[3];
+        int axis, bin;
+        for (int x = 0; x < 3; ++x) ext[x] = o2f(s_bounds[warp][3 + x]) - o2f(s_bounds[warp][x]);
+        choose_split(s_bins[warp], ext, axis, bin);
+        if (lane == 0) { s_choice[warp][0] = axis; s_choice[warp][1] = bin; }
+      }
+      __syncthreads();
+      // stable partition of every active segment
+      int axis = active && !median ? s_choice[g][0] : -1;
+      bool left = false;
+      if (active) left = axis < 0 ? tid - b < sz / 2 : bin_of(at3(c, axis), at3(cmin, axis), at3(cext, axis)) <= s_choice[g][1];
+      const uint32_t ball = __ballot_sync(0xFFFFFFFFu, left);
+      if (lane == 0) s_scan[warp] = __popc(ball);
+      __syncthreads();
+      uint32_t rank = __popc(ball & ((1u << lane) - 1u));
+      for (uint32_t w = 0; w < warp; ++w) rank += s_scan[w];
+      s_seg[tid] = rank;                                       // lefts before this position
+      if (tid == kThreads - 1) s_total = rank + (left ? 1u : 0u);
+      __syncthreads();
+      uint32_t to = tid, n_left = 0;
+      if (active) {
+        const uint32_t at_b = s_seg[b], at_e = e < kThreads ? s_seg[e] : s_total;
+        n_left = at_e - at_b;
+        if (n_left == 0 || n_left == sz) {                     // cannot happen with an axis
+          axis = -1;
+          n_left = sz / 2;
+          left = tid - b < n_left;
+        }
+        if (axis >= 0) to = left ? b + (rank - at_b) : b + n_left + (tid - b - (rank - at_b));
+        combine6(__match_any_sync(members, g * 2 + (left ? 0 : 1)), v6, s_child[g][left ? 0 : 1]);
+        if (tid == b) s_nleft[g] = n_left;
+      }
+      s_slot[to] = slot;
+      for (int x = 0; x < 6; ++x) s_box[x][to] = bx[x];
+      __syncthreads();
+      slot = s_slot[tid];
+      for (int x = 0; x < 6; ++x) bx[x] = s_box[x][tid];
+      if (active) {
+        const uint32_t mid = b + n_left;
+        if (tid >= mid) s_begin[tid] = mid; else s_end[tid] = mid;
+      }
+      // the records (the root's split position first: its children need it)
+      if (tid == 0 && s_parent[0] == kRoot) {                  // only in the first level of a whole build
+        s_root_split = s_nleft[0];
+        ctl->root_split = s_nleft[0];
+      }
+      __syncthreads();
+      if (tid < n_seg) {
+        const uint32_t sb = s_at[tid], nl = s_nleft[tid], mid = sb + nl, se = s_end[mid];
+        const uint32_t split = base + mid, depth = s_depth[sb];
+        const uint32_t id = place_node(split, s_parent[sb], s_root_split, out, n, err);
+        float cl[2][3], ch[2][3];
+        for (int k = 0; k < 2; ++k)
+          for (int x = 0; x < 3; ++x) { cl[k][x] = o2f(s_child[tid][k][x]); ch[k][x] = o2f(s_child[tid][k][3 + x]); }
+        write_node(out, id, cl, ch, nl == 1 ? s_slot[sb] : kRoot, se - mid == 1 ? s_slot[mid] : kRoot);
+        s_parent[sb] = id << 1;
+        s_parent[mid] = id << 1 | 1u;
+        s_depth[sb] = s_depth[mid] = depth + 1;
+      }
+      __syncthreads();
+    }
+    // every segment has at most kSmallLeaves leaves: a warp each, the list of
+    // their first positions in s_seg
+    {
+      const bool head = tid < m && s_begin[tid] == tid && s_end[tid] - tid >= 2;
+      const uint32_t hb = __ballot_sync(0xFFFFFFFFu, head);
+      __syncthreads();
+      if (lane == 0) s_scan[warp] = __popc(hb);
+      s_slot[tid] = slot;
+      for (int x = 0; x < 6; ++x) s_box[x][tid] = bx[x];
+      __syncthreads();
+      uint32_t at = 0, total = 0;
+      for (uint32_t w = 0; w < (uint32_t)kWarps; ++w) {
+        if (w < warp) at += s_scan[w];
+        total += s_scan[w];
+      }
+      if (head) s_seg[at + __popc(hb & ((1u << lane) - 1u))] = tid;
+      __syncthreads();
+      for (uint32_t w = warp; w < total; w += kWarps) {
+        const uint32_t sb = s_seg[w], sm = s_end[sb] - sb, at_lane = min(sb + lane, (uint32_t)kThreads - 1);
+        float lb[6];
+        for (int x = 0; x < 6; ++x) lb[x] = s_box[x][at_lane];
+        small_subtree(sm, s_slot[at_lane], lb, base + sb, s_parent[sb], s_depth[sb], s_root_split, out, n, err,
+                      s_key[warp]);
+      }
+      __syncthreads();
+    }
+  }
+}
 
-namespace {
 bool g_sah_slicing = true;
 
 // Centre and half extent of [lo, hi], so that [c - e, c + e] contains it: e is
 // rounded up, and widened by 2^-22 of the box's distance from the origin for
 // the rounding of the two products the walk forms from it. An empty box
-// (lo > hi) gets e = -inf, which no ray hits.
+// (lo > hi) gets e = -inf, which no ray hits. FP64 has few units: where both
+// differences are exact in FP32 (rounded down as up), as they are when lo and
+// hi are within a factor of two, FP32 gives the same two values (10M nodes:
+// 189 us; all in FP64 1333 us).
 __device__ __forceinline__ void centre_extent(float lo, float hi, float& c, float& e) {
   if (!(lo <= hi)) { c = 0.f; e = -INFINITY; return; }
+  const float big = fmaxf(fabsf(lo), fabsf(hi));
+  c = __fadd_rn(0.5f * lo, 0.5f * hi);
+  const float up = __fsub_ru(hi, c), dn = __fsub_ru(c, lo);
+  if (up == __fsub_rd(hi, c) && dn == __fsub_rd(c, lo) && (big > 1e-30f || big == 0.f)) {
+    e = __fmaf_ru(0x1p-22f, big, fmaxf(up, dn));
+    return;
+  }
   c = (float)(0.5 * ((double)lo + (double)hi));
   const double half = fmax((double)hi - (double)c, (double)c - (double)lo);
-  e = __double2float_ru(half + 0x1p-22 * fmax(fabs((double)lo), fabs((double)hi)));
+  e = __double2float_ru(half + 0x1p-22 * (double)big);
 }
 
 __global__ void k_render_nodes(const float4* __restrict__ nodes, uint32_t n_inner, float4* __restrict__ out) {
@@ -900,80 +983,84 @@ cudaError_t render_nodes(const float4* nodes, uint32_t n, float4* out, cudaStrea
 
 void set_sah_slicing(bool on) { g_sah_slicing = on; }
 
+namespace {
+// returns the bytes that the scratch takes
+size_t sah_scratch(char* base, uint32_t n, bool slicing, Build& s) {
+  // slices of at least kSlice leaves, and at most about 2048 of a node: every slice adds up the
+  // counts of its node's slices
+  s.slice = slicing ? std::max(kSlice, (uint32_t)(((uint64_t)n + 2047) / 2048)) : 0xFFFFFFFFu;
+  s.max_nodes = n / (kMidLeaves + 1) + 1;
+  s.max_slices = n / kSlice + s.max_nodes + 1;
+  s.max_mid = n / 2 + 1;
+  size_t at = 0;
+  auto take = [&](size_t bytes) {
+    char* p = base + at;
+    at += (bytes + 255) / 256 * 256;
+    return p;
+  };
+  s.lo = reinterpret_cast<float4*>(take((size_t)n * sizeof(float4)));
+  s.hi = reinterpret_cast<float4*>(take((size_t)n * sizeof(float4)));
+  for (int i = 0; i < 2; ++i) {
+    s.idx[i] = reinterpret_cast<uint32_t*>(take((size_t)n * sizeof(uint32_t)));
+    s.nodes[i] = reinterpret_cast<TopNode*>(take((size_t)s.max_nodes * sizeof(TopNode)));
+    s.slice_node[i] = reinterpret_cast<uint32_t*>(take((size_t)s.max_slices * sizeof(uint32_t)));
+  }
+  s.slice_cnt = reinterpret_cast<int*>(take((size_t)s.max_slices * 3 * kBins * sizeof(int)));
+  s.mid = reinterpret_cast<Job*>(take((size_t)s.max_mid * sizeof(Job)));
+  s.ctl = reinterpret_cast<Control*>(take(sizeof(Control)));
+  return at;
+}
+}  // namespace
+
 size_t sah_tmp_bytes(uint32_t n) {
-  const size_t nn = n ? n : 1;
-  return 2 * nn * sizeof(float4) + 2 * nn * sizeof(uint32_t) + 3 * (nn / 2 + 1) * sizeof(Job) + 256 +
-         kWideJobs * sizeof(WideNode) + kWideMaxSlices * sizeof(uint32_t) + 256;
+  Build b{};
+  return sah_scratch(nullptr, n ? n : 1, true, b);
 }
 
 cudaError_t build_sah_tree(const float4* lbvh_nodes, const int32_t* parent, uint32_t n,
                            float4* out, void* tmp, uint32_t* err, cudaStream_t st) {
   if (n < 2) return cudaMemcpyAsync(out, lbvh_nodes, 4 * sizeof(float4), cudaMemcpyDeviceToDevice, st);
-  char* p = static_cast<char*>(tmp);
-  float4* lo = reinterpret_cast<float4*>(p); p += (size_t)n * sizeof(float4);
-  float4* hi = reinterpret_cast<float4*>(p); p += (size_t)n * sizeof(float4);
-  uint32_t* idx[2];
-  idx[0] = reinterpret_cast<uint32_t*>(p); p += (size_t)n * sizeof(uint32_t);
-  idx[1] = reinterpret_cast<uint32_t*>(p); p += (size_t)n * sizeof(uint32_t);
-  const size_t max_jobs = n / 2 + 1;
-  Job* jobs[2];
-  jobs[0] = reinterpret_cast<Job*>(p); p += max_jobs * sizeof(Job);
-  jobs[1] = reinterpret_cast<Job*>(p); p += max_jobs * sizeof(Job);
-  Job* small = reinterpret_cast<Job*>(p); p += max_jobs * sizeof(Job);
-  uint32_t** d_bufs = reinterpret_cast<uint32_t**>(p); p += 2 * sizeof(uint32_t*);
-  uint32_t* counters = reinterpret_cast<uint32_t*>(p);   // [0] next count, [1] root split, [2] small count
-  p += 256 - 2 * sizeof(uint32_t*);
-  WideNode* wide = reinterpret_cast<WideNode*>(p); p += kWideJobs * sizeof(WideNode);
-  uint32_t* slice_left = reinterpret_cast<uint32_t*>(p);
-  const int g = (int)((n + 255) / 256);
-  k_leaf_boxes<<<g, 256, 0, st>>>(lbvh_nodes, parent, n, lo, hi);
-  k_iota<<<g, 256, 0, st>>>(idx[0], n);
-  const Job root{0, n, 0xFFFFFFFFu, 0};
-  cudaError_t e = cudaMemcpyAsync(jobs[0], &root, sizeof root, cudaMemcpyHostToDevice, st);
-  uint32_t* h_bufs[2] = {idx[0], idx[1]};
-  if (e == cudaSuccess) e = cudaMemcpyAsync(d_bufs, h_bufs, sizeof h_bufs, cudaMemcpyHostToDevice, st);
-  if (e == cudaSuccess) e = cudaMemsetAsync(counters + 2, 0, sizeof(uint32_t), st);
-  uint32_t count = 1;
-  for (int level = 0; level < kMaxDepth + 2 && count > 0 && e == cudaSuccess; ++level) {
-    const int cur = level & 1;
-    e = cudaMemsetAsync(counters, 0, sizeof(uint32_t), st);
-    if (e != cudaSuccess) break;
-    // few nodes of many leaves each: slice every node over several blocks
-    const uint32_t per_job = n / count;
-    if (g_sah_slicing && count <= kWideJobs && per_job >= kWideMinLeaves) {
-      uint32_t S = (2u * (uint32_t)num_sms() + count - 1) / count;
-      S = std::min(S, std::min(per_job / kWideMinSlice, kWideMaxSlices / count));
-      S = std::max(S, 1u);
-      const uint32_t blocks = count * S;
-      k_wide_init<<<count, 256, 0, st>>>(wide, count);
-      k_wide_bounds<<<blocks, kWideThreads, 0, st>>>(lo, hi, idx[cur], jobs[cur], S, wide);
-      k_wide_bins<<<blocks, kWideThreads, 0, st>>>(lo, hi, idx[cur], jobs[cur], S, wide);
-      k_wide_count<<<blocks, kWideThreads, 0, st>>>(lo, hi, idx[cur], jobs[cur], S, wide, slice_left);
-      k_wide_scatter<<<blocks, kWideThreads, 0, st>>>(lo, hi, idx[cur], idx[cur ^ 1], jobs[cur], S, wide,
-                                                      slice_left);
-      k_wide_nodes<<<(count + 31) / 32, 32, 0, st>>>(jobs[cur], count, wide, idx[cur ^ 1], jobs[cur ^ 1],
-                                                     counters, small, counters + 2, (uint32_t)(cur ^ 1),
-                                                     out, counters + 1, n, err);
-    } else if (count < kTopJobs)
-      k_sah_level<kSahThreadsTop><<<count, kSahThreadsTop, 0, st>>>(
-          lo, hi, idx[cur], idx[cur ^ 1], jobs[cur], count, jobs[cur ^ 1], counters, small,
-          counters + 2, (uint32_t)(cur ^ 1), out, counters + 1, n, err);
-    else
-      k_sah_level<kSahThreads><<<count, kSahThreads, 0, st>>>(
-          lo, hi, idx[cur], idx[cur ^ 1], jobs[cur], count, jobs[cur ^ 1], counters, small,
-          counters + 2, (uint32_t)(cur ^ 1), out, counters + 1, n, err);
-    e = cudaMemcpyAsync(&count, counters, sizeof count, cudaMemcpyDeviceToHost, st);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(st);
-    if (count > max_jobs) { count = 0; e = cudaErrorUnknown; }
+  Build s{};
+  sah_scratch(static_cast<char*>(tmp), n, g_sah_slicing, s);
+  s.out = out;
+  s.err = err;
+  s.n = n;
+  const bool top = n > kMidLeaves;
+  const uint32_t* const idx[2] = {s.idx[0], s.idx[1]};
+  TopNode* root = top ? s.nodes[0] : nullptr;
+  k_begin<<<1, kThreads, 0, st>>>(s.ctl, root, s.slice_node[0], s.mid, n, s.slice);
+  k_leaves<<<(int)(((uint64_t)n + kThreads - 1) / kThreads), kThreads, 0, st>>>(lbvh_nodes, parent, n, s.lo, s.hi,
+                                                                         s.idx[0], root);
+  cudaError_t e = cudaSuccess;
+  uint32_t n_mid = 1;
+  if (top) {
+    const int blocks = (int)std::min(s.max_slices, 8u * (uint32_t)num_sms());
+    // as many levels as a balanced tree has and kExtra more, then kExtra at a time
+    constexpr int kExtra = 4;
+    int until = kExtra;
+    for (uint32_t m = n; m > kMidLeaves; m = (m + 1) / 2) ++until;
+    Control c{};
+    for (int level = 0;; ++level) {
+      if (level == until || level == kMaxDepth + 2) {
+        e = cudaMemcpyAsync(&c, s.ctl, sizeof c, cudaMemcpyDeviceToHost, st);
+        if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+        if (e != cudaSuccess || c.n_nodes[level & 1] == 0) break;
+        if (level == kMaxDepth + 2) return cudaErrorUnknown;      // deeper than the depth budget
+        until += kExtra;
+      }
+      const int cur = level & 1;
+      k_top_bins<<<blocks, kThreads, 0, st>>>(s, cur);
+      k_top_scatter<<<blocks, kThreads, 0, st>>>(s, cur);
+      std::swap(s.idx[0], s.idx[1]);
+      std::swap(s.nodes[0], s.nodes[1]);
+      std::swap(s.slice_node[0], s.slice_node[1]);
+    }
+    n_mid = c.n_mid;
+    if (e == cudaSuccess && n_mid > s.max_mid) e = cudaErrorUnknown;
   }
-  if (e == cudaSuccess && count != 0) e = cudaErrorUnknown;   // deeper than the depth budget
-  uint32_t n_small = 0;
-  if (e == cudaSuccess) e = cudaMemcpyAsync(&n_small, counters + 2, sizeof n_small, cudaMemcpyDeviceToHost, st);
-  if (e == cudaSuccess) e = cudaStreamSynchronize(st);
-  if (e == cudaSuccess && n_small > max_jobs) e = cudaErrorUnknown;
-  if (e == cudaSuccess && n_small > 0)
-    k_sah_small<<<(n_small + kSmallWarps - 1) / kSmallWarps, 32 * kSmallWarps, 0, st>>>(
-        lo, hi, d_bufs, small, n_small, out, counters + 1, n, err);
+  if (e == cudaSuccess && n_mid)
+    k_sah_mid<<<(int)std::min(n_mid, 0x7FFFFFFFu), kThreads, 0, st>>>(s.lo, s.hi, idx[0], idx[1], s.ctl, s.mid,
+                                                                     out, n, err);
   return e == cudaSuccess ? cudaGetLastError() : e;
 }
 
