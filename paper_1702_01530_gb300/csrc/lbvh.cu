@@ -472,7 +472,36 @@ k_refit(const float* sph, const float* tri, uint32_t ns, uint32_t n, bool wide, 
   atomicOr(err, ERR_BUILD);
 }
 
+// Raw primitive records word by word: spheres of 5 (centre, radius, material),
+// triangles of 10 (vertices, material). Bound by the read.
+__global__ void __launch_bounds__(256)
+k_check_prims(const uint32_t* __restrict__ sph, const uint32_t* __restrict__ tri, uint64_t sph_words,
+              uint64_t tri_words, uint32_t n_mats, uint32_t* __restrict__ bad) {
+  const uint64_t step = (uint64_t)gridDim.x * blockDim.x, first = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  bool wrong = false;
+  for (uint64_t i = first; i < sph_words; i += step) {
+    const uint32_t v = sph[i], f = (uint32_t)(i % 5);
+    if (f == 4) wrong |= v >= n_mats;
+    else wrong |= (v & 0x7F800000u) == 0x7F800000u || (f == 3 && !(__uint_as_float(v) > 0.f));
+  }
+  for (uint64_t i = first; i < tri_words; i += step) {
+    const uint32_t v = tri[i];
+    wrong |= i % 10 == 9 ? v >= n_mats : (v & 0x7F800000u) == 0x7F800000u;
+  }
+  if (__any_sync(0xFFFFFFFFu, wrong) && (threadIdx.x & 31) == 0) *bad = 1;
+}
+
 }  // namespace
+
+cudaError_t check_prims(const float4* d_sph_in, const float* d_tri_in, uint32_t ns, uint32_t nt, uint32_t n_mats,
+                        uint32_t* bad, cudaStream_t st) {
+  const uint64_t sph_words = 5ull * ns, tri_words = 10ull * nt;
+  const uint64_t blocks = (std::max(sph_words, tri_words) + 255) / 256;
+  k_check_prims<<<(int)std::min<uint64_t>(blocks, 8ull * (uint64_t)num_sms()), 256, 0, st>>>(
+      reinterpret_cast<const uint32_t*>(d_sph_in), reinterpret_cast<const uint32_t*>(d_tri_in), sph_words,
+      tri_words, n_mats, bad);
+  return cudaGetLastError();
+}
 
 size_t lbvh_tmp_bytes(uint32_t n) {
   size_t nblocks = (n + kTile - 1) / kTile;

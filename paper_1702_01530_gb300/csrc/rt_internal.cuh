@@ -186,6 +186,10 @@ cudaError_t build_lbvh(const float4* d_sph_in, const float* d_tri_in, uint32_t n
                        float4* d_nodes, float4* d_prims, uint64_t* d_keys, int32_t* d_parent,
                        void* d_tmp, size_t tmp_bytes, uint32_t* d_err, cudaStream_t st);
 size_t lbvh_tmp_bytes(uint32_t n);
+// *bad = 1 if a record is invalid: a value that is not finite, a radius not
+// above 0, a material not below n_mats (raw records; *bad is 0 before)
+cudaError_t check_prims(const float4* d_sph_in, const float* d_tri_in, uint32_t ns, uint32_t nt, uint32_t n_mats,
+                        uint32_t* bad, cudaStream_t st);
 size_t sah_tmp_bytes(uint32_t n);
 // binned-SAH binary tree over the leaves of the LBVH (nodes, parent): same
 // node layout and leaf slots, root 0; synchronises st about once
