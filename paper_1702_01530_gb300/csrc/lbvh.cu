@@ -4,8 +4,7 @@
 // structure; this is the linear BVH over Morton codes:
 //   1. k_centroid_bounds : FP64 centroids (triangle ((v0+v1)+v2)/3, every
 //      operation correctly rounded, no FMA), their per-axis min/max per block.
-//      FP64 units are few, so triangles are compared by their sums (division
-//      by 3 is monotonic) and as integers.
+//      Triangles are compared by their sums (division by 3 is monotonic).
 //   2. k_reduce_bounds     : the bounds of all blocks.
 //   3. k_keys              : q_a = min(1023, floor((c_a - min_a) /
 //      (max_a - min_a) * 1024)) (0 when the extent is 0), morton30 with x at
@@ -16,22 +15,22 @@
 //      digits; per pass a histogram of every 2048-key tile (k_keys makes the
 //      first), a scan of each digit's tile counts, a scatter). Keys start in
 //      id order, so the result is sorted by the whole 64-bit key.
-//   5. k_karras            : binary radix tree over the sorted keys, one
-//      thread per internal node (direction, range end, split by binary
-//      search on delta(i, j) = clz(key_i ^ key_j)).
-//   6. k_refit             : leaf boxes (triangle min/max; sphere c -/+ r in
-//      FP64 rounded outward to FP32) and bottom-up refit: the second thread to
-//      arrive at a node merges both children and climbs on. A node whose
-//      leaves all belong to one block (all but a few per block) is met in
-//      shared memory; only the others pay for global arrival counters and
-//      fences.
+//   5. k_tree              : primitives in sorted order with their boxes
+//      (triangle min/max; sphere c -/+ r in FP64 rounded outward to FP32) and
+//      the binary radix tree with its boxes over every 256 of them, bottom-up in
+//      shared memory.
+//   6. k_tree_up           : the same over what 16 such blocks leave over, and so
+//      on until one block is left.
 //
 // Measured (GB300, 1,000,000 primitives in random order, the whole device-side
-// build): 0.359 ms; 1.110 before, when one block scanned the tile counts
-// (0.40), one thread reduced the bounds (0.12), every key was divided twice in
-// FP64 (0.27 with the bounds) and every node had a global arrival counter
-// (0.18). The kernels' shares now (alone, cold caches): refit 125 us, scatter
-// 4 x 14, karras 38, bounds 38, keys 22, histograms 3 x 7, scans 4 x 4.
+// build): 0.299 ms; 1.110 when one block scanned the tile counts (0.40),
+// one thread reduced the bounds (0.12), every key was divided twice in FP64
+// (0.27 with the bounds) and every node had a global arrival counter (0.18);
+// 0.359 with a search per node (38 us) and a refit that read its parents,
+// children and ranges from memory at every step (125 us). Its kernels' shares
+// now: tree 77 us, upper levels 15 each, scatter 4 x 13, bounds 25, keys 23,
+// histograms 3 x 5, scans 4 x 3. What is left in k_tree is the chain of a
+// block's climb, seven to ten levels of shared-memory exchanges.
 #include <cuda_runtime.h>
 #include <stdint.h>
 
@@ -45,7 +44,7 @@ namespace {
 constexpr int kSortThreads = 256;
 constexpr int kSortItems = 8;                       // items per thread per tile
 constexpr int kTile = kSortThreads * kSortItems;    // 2048 keys per block
-constexpr int kRedThreads = 256;
+constexpr int kRedThreads = 512;
 constexpr int kRedBlocks = 256;
 
 struct Bounds6 { double lo[3], hi[3]; };
@@ -82,53 +81,98 @@ __device__ __forceinline__ double o2d(long long o) {
   return __longlong_as_double(o >= 0 ? o : o ^ 0x7FFFFFFFFFFFFFFFll);
 }
 
-// per-block partial min/max of the centroids; spheres by their centres,
-// triangles by the sums of their vertices, divided by 3 at the end
-__global__ void k_centroid_bounds(const float* sph, const float* tri, uint32_t ns, uint32_t n, bool wide,
-                                  Bounds6* partial) {
-  __shared__ long long s[12][kRedThreads / 32];
+// Per-block partial min/max of the centroids; spheres by their centres,
+// triangles by the sums of their vertices, divided by 3 at the end. FP64 has few
+// units, so FP32 sums with a bound of their error (two roundings, each at most
+// 2^-24 of the vertices' magnitudes) first find which triangles can hold an
+// extreme of the block's range; only their sums are formed in FP64 (1M triangles:
+// 25 us; 38 with every sum in FP64).
+__device__ __forceinline__ void sum_range(const float v[9], int k, float& least, float& most) {
+  const float f = (v[k] + v[3 + k]) + v[6 + k];
+  const float e = 0x1p-22f * (fabsf(v[k]) + fabsf(v[3 + k]) + fabsf(v[6 + k])) + 1e-44f;
+  least = f - e;
+  most = f + e;
+}
+
+__global__ void __launch_bounds__(kRedThreads)
+k_centroid_bounds(const float* sph, const float* tri, uint32_t ns, uint32_t n, bool wide, Bounds6* partial) {
+  __shared__ float s_f[12][kRedThreads / 32];      // sphere min, -max; triangle: upper bound of the min, of -max
+  __shared__ long long s_d[6][kRedThreads / 32];   // triangle min, ~max
   const long long kMost = 0x7FFFFFFFFFFFFFFFll;
-  long long v[12];                 // sphere min, triangle min, sphere -max, triangle -max (x, y, z each)
+  const uint32_t first = blockIdx.x * kRedThreads + threadIdx.x, step = gridDim.x * kRedThreads;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  float f[12];
 #pragma unroll
-  for (int k = 0; k < 12; ++k) v[k] = kMost;
-  for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
-    if (i < ns) {
+  for (int k = 0; k < 12; ++k) f[k] = INFINITY;
+  uint32_t i = first;
+  for (; i < ns && i < n; i += step)
 #pragma unroll
-      for (int k = 0; k < 3; ++k) {
-        const long long o = d2o((double)__ldg(sph + 5ull * i + k));
-        v[k] = min(v[k], o);
-        v[6 + k] = min(v[6 + k], ~o);
-      }
-    } else {
-      float t[9];
-      load_tri(tri, i - ns, wide, t);
+    for (int k = 0; k < 3; ++k) {
+      const float c = __ldg(sph + 5ull * i + k);
+      f[k] = fminf(f[k], c);
+      f[3 + k] = fminf(f[3 + k], -c);
+    }
+  const uint32_t first_tri = i;
+  for (; i < n; i += step) {
+    float t[9];
+    load_tri(tri, i - ns, wide, t);
 #pragma unroll
-      for (int k = 0; k < 3; ++k) {
+    for (int k = 0; k < 3; ++k) {
+      float least, most;
+      sum_range(t, k, least, most);
+      f[6 + k] = fminf(f[6 + k], most);
+      f[9 + k] = fminf(f[9 + k], -least);
+    }
+  }
+#pragma unroll
+  for (int k = 0; k < 12; ++k) {
+    for (int off = 16; off > 0; off >>= 1) f[k] = fminf(f[k], __shfl_xor_sync(0xFFFFFFFFu, f[k], off));
+    if (lane == 0) s_f[k][warp] = f[k];
+  }
+  __syncthreads();
+#pragma unroll
+  for (int k = 0; k < 12; ++k)
+    for (int w = 0; w < kRedThreads / 32; ++w) f[k] = fminf(f[k], s_f[k][w]);
+  long long v[6];
+#pragma unroll
+  for (int k = 0; k < 6; ++k) v[k] = kMost;
+  for (i = first_tri; i < n; i += step) {
+    float t[9];
+    load_tri(tri, i - ns, wide, t);
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+      float least, most;
+      sum_range(t, k, least, most);
+      if (!(least > f[6 + k]) || !(-most > f[9 + k])) {      // also what overflows FP32
         const long long o = d2o(sum3(t, k));
-        v[3 + k] = min(v[3 + k], o);
-        v[9 + k] = min(v[9 + k], ~o);
+        v[k] = min(v[k], o);
+        v[3 + k] = min(v[3 + k], ~o);
       }
     }
   }
 #pragma unroll
-  for (int k = 0; k < 12; ++k)
+  for (int k = 0; k < 6; ++k) {
     for (int off = 16; off > 0; off >>= 1) v[k] = min(v[k], __shfl_xor_sync(0xFFFFFFFFu, v[k], off));
-  if ((threadIdx.x & 31) == 0)
-#pragma unroll
-    for (int k = 0; k < 12; ++k) s[k][threadIdx.x >> 5] = v[k];
+    if (lane == 0) s_d[k][warp] = v[k];
+  }
   __syncthreads();
   if (threadIdx.x >= 3) return;
-  long long m[4] = {kMost, kMost, kMost, kMost};
-  for (int q = 0; q < 4; ++q)
-    for (int w = 0; w < kRedThreads / 32; ++w) m[q] = min(m[q], s[3 * q + threadIdx.x][w]);
-  double lo = INFINITY, hi = -INFINITY;
-  if (m[0] != kMost) { lo = o2d(m[0]); hi = o2d(~m[2]); }
-  if (m[1] != kMost) {
-    lo = fmin(lo, __ddiv_rn(o2d(m[1]), 3.0));
-    hi = fmax(hi, __ddiv_rn(o2d(~m[3]), 3.0));
+  const int a = threadIdx.x;
+  long long least = kMost, most = kMost;
+  float c0 = INFINITY, c1 = INFINITY;
+  for (int w = 0; w < kRedThreads / 32; ++w) {
+    least = min(least, s_d[a][w]);
+    most = min(most, s_d[3 + a][w]);
+    c0 = fminf(c0, s_f[a][w]);
+    c1 = fminf(c1, s_f[3 + a][w]);
   }
-  partial[blockIdx.x].lo[threadIdx.x] = lo;
-  partial[blockIdx.x].hi[threadIdx.x] = hi;
+  double lo = (double)c0, hi = -(double)c1;
+  if (least != kMost) {
+    lo = fmin(lo, __ddiv_rn(o2d(least), 3.0));
+    hi = fmax(hi, __ddiv_rn(o2d(~most), 3.0));
+  }
+  partial[blockIdx.x].lo[a] = lo;
+  partial[blockIdx.x].hi[a] = hi;
 }
 
 // bounds of all blocks: warp q takes value q (lo x, y, z, hi x, y, z)
@@ -342,34 +386,6 @@ __device__ __forceinline__ int delta(const uint64_t* k, int64_t n, int64_t i, in
   return __clzll(k[i] ^ k[j]);
 }
 
-// also writes each node's range of leaves, [first, last]
-__global__ void k_karras(const uint64_t* keys, uint32_t n, float4* nodes, int32_t* parent, uint2* range) {
-  int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= (int64_t)n - 1) return;
-  int d = (delta(keys, n, i, i + 1) - delta(keys, n, i, i - 1)) > 0 ? 1 : -1;
-  int dmin = delta(keys, n, i, i - d);
-  int64_t lmax = 2;
-  while (delta(keys, n, i, i + lmax * d) > dmin) lmax <<= 1;
-  int64_t l = 0;
-  for (int64_t t = lmax >> 1; t >= 1; t >>= 1)
-    if (delta(keys, n, i, i + (l + t) * d) > dmin) l += t;
-  int64_t j = i + l * d;
-  int dnode = delta(keys, n, i, j);
-  int64_t s = 0, t = l;
-  do {
-    t = (t + 1) >> 1;
-    if (delta(keys, n, i, i + (s + t) * d) > dnode) s += t;
-  } while (t > 1);
-  int64_t g = i + s * d + min(d, 0);
-  int32_t left = (min(i, j) == g) ? ~(int32_t)g : (int32_t)g;
-  int32_t right = (max(i, j) == g + 1) ? ~(int32_t)(g + 1) : (int32_t)(g + 1);
-  nodes[4 * i + 3] = make_float4(__int_as_float(left), __int_as_float(right), 0.f, 0.f);
-  parent[left >= 0 ? left : (int64_t)n - 1 + ~left] = (int32_t)i;
-  parent[right >= 0 ? right : (int64_t)n - 1 + ~right] = (int32_t)i;
-  range[i] = make_uint2((uint32_t)min(i, j), (uint32_t)max(i, j));
-  if (i == 0) parent[0] = -1;
-}
-
 // write box (lo, hi) into the child slot `slot` (0 left, 1 right) of node p
 __device__ __forceinline__ void store_child_box(float4* nodes, int32_t p, int slot,
                                                 const float lo[3], const float hi[3]) {
@@ -383,93 +399,285 @@ __device__ __forceinline__ void store_child_box(float4* nodes, int32_t p, int sl
   }
 }
 
-constexpr int kRefitThreads = 256;
-
-__global__ void __launch_bounds__(kRefitThreads)
-k_refit(const float* sph, const float* tri, uint32_t ns, uint32_t n, bool wide, const uint64_t* keys,
-        float4* nodes, float4* prims, const int32_t* parent, const uint2* range, uint32_t* arrivals,
-        uint32_t* err) {
-  // a block's own nodes (all leaves in this block; node i lies in its own
-  // range, so i - first leaf is a slot): arrival count and both children's boxes
-  __shared__ uint32_t s_arrived[kRefitThreads];
-  __shared__ float s_box[2][6][kRefitThreads];
-  const uint32_t b0 = blockIdx.x * kRefitThreads, b1 = min(n, b0 + kRefitThreads) - 1;
-  s_arrived[threadIdx.x] = 0;
-  __syncthreads();
-  const uint32_t k = b0 + threadIdx.x;
-  if (k >= n) return;
-  const uint32_t id = (uint32_t)(keys[k] & 0xFFFFFFFFull);
-  float lo[3], hi[3];
+// box of the primitive with raw index id
+__device__ __forceinline__ void prim_box(const float* sph, const float v[9], uint32_t ns, uint32_t id, float lo[3],
+                                         float hi[3]) {
   if (id < ns) {
     const float* p = sph + 5ull * id;
-    float r = p[3];
-    uint32_t mat = __float_as_uint(p[4]);
+    const float r = p[3];
     for (int a = 0; a < 3; ++a) {
       lo[a] = __double2float_rd(__dsub_rd((double)p[a], (double)r));
       hi[a] = __double2float_ru(__dadd_ru((double)p[a], (double)r));
     }
-    prims[3ull * k + 0] = make_float4(p[0], p[1], p[2], __uint_as_float(id));
-    prims[3ull * k + 1] = make_float4(r, 0.f, 0.f, __uint_as_float(mat));
-    prims[3ull * k + 2] = make_float4(0.f, 0.f, 0.f, 0.f);
   } else {
-    float v[9];
-    load_tri(tri, id - ns, wide, v);
-    uint32_t mat = __float_as_uint(tri[10ull * (id - ns) + 9]);
     for (int a = 0; a < 3; ++a) {
       lo[a] = fminf(v[a], fminf(v[3 + a], v[6 + a]));
       hi[a] = fmaxf(v[a], fmaxf(v[3 + a], v[6 + a]));
     }
-    prims[3ull * k + 0] = make_float4(v[0], v[1], v[2], __uint_as_float(id));
-    prims[3ull * k + 1] = make_float4(v[3] - v[0], v[4] - v[1], v[5] - v[2], __uint_as_float(mat));
-    prims[3ull * k + 2] = make_float4(v[6] - v[0], v[7] - v[1], v[8] - v[2], 0.f);
   }
-  if (n == 1) {  // no internal node: keep the leaf box in the spare slot 0
-    store_child_box(nodes, 0, 0, lo, hi);
+}
+
+// The tree is found bottom-up, without searches (Apetrei 2014): of a range's two
+// neighbours the one with the longer common prefix is its sibling's side; the
+// second of two siblings to arrive at their split makes the parent, whose number
+// is the end of its range that faces its own sibling (Karras' numbering; the root
+// is 0). A block does this in shared memory for a run of items, which cover a
+// range of leaves: first 256 leaves, then the subtrees that kUpGroup such runs
+// leave over, and so on until one run is left. Prefix and suffix minima of the
+// run's deltas tell whether a sibling's range ends inside the run; a subtree whose
+// sibling's does not is left over. What a run leaves over hangs off the two paths
+// of nodes that contain one of its ends, which are at most one per bit of the
+// keys: at most 128.
+template <int N>
+struct Run {
+  int delta[N + 1];                    // [j]: of the leaves on either side of boundary j, before item j
+  int pre[N + 1], suf[N + 2];          // minima up to and from j
+  uint32_t arrived[N + 1], far[2][N + 1];   // at a split: arrivals, and the sides' other ends
+  float box[2][6][N + 1];              // and their boxes
+};
+
+// minima of r.delta[0 .. m] from either end, by the whole block
+template <int N, int THREADS>
+__device__ __forceinline__ void run_minima(Run<N>& r, int m, int (*s_warp)[THREADS / 32]) {
+  constexpr int kPer = (N + 1 + THREADS - 1) / THREADS;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, j0 = tid * kPer;
+  int pre = 64, suf = 64;
+  for (int j = j0; j < j0 + kPer && j <= m; ++j) pre = min(pre, r.delta[j]);
+  suf = pre;
+  for (int o = 1; o < 32; o <<= 1) {
+    const int x = __shfl_up_sync(0xFFFFFFFFu, pre, o), y = __shfl_down_sync(0xFFFFFFFFu, suf, o);
+    if (lane >= o) pre = min(pre, x);
+    if (lane + o < 32) suf = min(suf, y);
+  }
+  if (lane == 31) s_warp[0][warp] = pre;
+  if (lane == 0) s_warp[1][warp] = suf;
+  // of the threads before (after) this one alone
+  pre = __shfl_up_sync(0xFFFFFFFFu, pre, 1);
+  suf = __shfl_down_sync(0xFFFFFFFFu, suf, 1);
+  if (lane == 0) pre = 64;
+  if (lane == 31) suf = 64;
+  __syncthreads();
+  for (int w = 0; w < THREADS / 32; ++w) {
+    if (w < warp) pre = min(pre, s_warp[0][w]);
+    if (w > warp) suf = min(suf, s_warp[1][w]);
+  }
+  for (int j = j0; j < j0 + kPer && j <= m; ++j) r.pre[j] = pre = min(pre, r.delta[j]);
+  for (int j = j0 + kPer - 1; j >= j0; --j)
+    if (j <= m) r.suf[j] = suf = min(suf, r.delta[j]);
+  if (tid == 0) r.suf[m + 1] = 64;     // past the last boundary: above every delta
+}
+
+// Climb from item i of a run of m items with box (lo, hi). first(j) is the
+// first leaf of item j (first(m): past the run). Returns whether the climb ended
+// at a subtree that is left over: then l is its first item and child its number.
+template <int N, typename First>
+__device__ __forceinline__ bool run_climb(Run<N>& run, const First& first, int i, int m, int32_t item, float lo[3],
+                                          float hi[3], float4* nodes, int32_t* parent, uint32_t n, int& l,
+                                          int32_t& child) {
+  int r = i;
+  l = i;
+  child = item;
+  for (int step = 0; step <= m; ++step) {
+    const int dl = run.delta[l], dr = run.delta[r + 1];
+    if (dl < 0 && dr < 0) {                            // all leaves: the root
+      parent[0] = -1;
+      return false;
+    }
+    const bool is_left = dr > dl;
+    const int q = is_left ? r + 1 : l;                 // the split: a boundary inside the run if the parent is
+    if (!(is_left ? run.suf[q + 1] < dr : q > 0 && run.pre[q - 1] < dl)) return true;
+    const int side = is_left ? 0 : 1;
+    for (int a = 0; a < 3; ++a) { run.box[side][a][q] = lo[a]; run.box[side][3 + a][q] = hi[a]; }
+    run.far[side][q] = (uint32_t)(is_left ? l : r);
+    __threadfence_block();
+    if (atomicAdd(&run.arrived[q], 1u) == 0u) return false;   // sibling not done yet
+    __threadfence_block();
+    float sl[3], sh[3];
+    for (int a = 0; a < 3; ++a) { sl[a] = run.box[side ^ 1][a][q]; sh[a] = run.box[side ^ 1][3 + a][q]; }
+    if (is_left) r = (int)run.far[1][q]; else l = (int)run.far[0][q];
+    const uint32_t begin = first(l), split = first(q), end = first(r + 1);   // leaves [begin, split) and [split, end)
+    const int32_t left = split - begin == 1 ? ~(int32_t)begin : (int32_t)(split - 1);
+    const int32_t right = end - split == 1 ? ~(int32_t)split : (int32_t)split;
+    child = (int32_t)(run.delta[r + 1] > run.delta[l] ? end - 1 : begin);
+    float4* o = nodes + 4 * (int64_t)child;
+    o[0] = is_left ? make_float4(lo[0], hi[0], lo[1], hi[1]) : make_float4(sl[0], sh[0], sl[1], sh[1]);
+    o[1] = is_left ? make_float4(sl[0], sh[0], sl[1], sh[1]) : make_float4(lo[0], hi[0], lo[1], hi[1]);
+    o[2] = is_left ? make_float4(lo[2], hi[2], sl[2], sh[2]) : make_float4(sl[2], sh[2], lo[2], hi[2]);
+    o[3] = make_float4(__int_as_float(left), __int_as_float(right), 0.f, 0.f);
+    parent[left >= 0 ? left : (int64_t)n - 1 + ~left] = child;
+    parent[right >= 0 ? right : (int64_t)n - 1 + ~right] = child;
+    for (int a = 0; a < 3; ++a) { lo[a] = fminf(lo[a], sl[a]); hi[a] = fmaxf(hi[a], sh[a]); }
+  }
+  return false;
+}
+
+// the primitives in sorted order, and the trees over every 256 of them
+constexpr int kTreeThreads = 256;
+__global__ void __launch_bounds__(kTreeThreads, 6)
+k_tree(const float* sph, const float* tri, uint32_t ns, uint32_t n, bool wide, const uint64_t* __restrict__ keys,
+       float4* nodes, float4* prims, int32_t* parent, uint2* left_over, uint32_t* counts) {
+  __shared__ union {
+    float4 prim[3 * kTreeThreads];
+    Run<kTreeThreads> run;
+  } u;
+  __shared__ int s_warp[2][kTreeThreads / 32];
+  __shared__ int32_t s_left[kTreeThreads];             // by first leaf: what is left over
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const uint32_t b0 = blockIdx.x * kTreeThreads, m = min((uint32_t)kTreeThreads, n - b0), k = b0 + tid;
+  const bool leaf = (uint32_t)tid < m;
+  constexpr int32_t kNone = 0x7FFFFFFF;
+
+  // primitives: gathered, then written whole lines at a time
+  float lo[3] = {0.f, 0.f, 0.f}, hi[3] = {0.f, 0.f, 0.f};
+  if (leaf) {
+    const uint32_t id = (uint32_t)(keys[k] & 0xFFFFFFFFull);
+    float v[9];
+    if (id < ns) {
+      const float* p = sph + 5ull * id;
+      u.prim[3 * tid] = make_float4(p[0], p[1], p[2], __uint_as_float(id));
+      u.prim[3 * tid + 1] = make_float4(p[3], 0.f, 0.f, p[4]);
+      u.prim[3 * tid + 2] = make_float4(0.f, 0.f, 0.f, 0.f);
+    } else {
+      load_tri(tri, id - ns, wide, v);
+      const float mat = tri[10ull * (id - ns) + 9];
+      u.prim[3 * tid] = make_float4(v[0], v[1], v[2], __uint_as_float(id));
+      u.prim[3 * tid + 1] = make_float4(v[3] - v[0], v[4] - v[1], v[5] - v[2], mat);
+      u.prim[3 * tid + 2] = make_float4(v[6] - v[0], v[7] - v[1], v[8] - v[2], 0.f);
+    }
+    prim_box(sph, v, ns, id, lo, hi);
+  }
+  const int d = leaf ? delta(keys, n, (int64_t)k, (int64_t)k - 1) : -1;
+  __syncthreads();
+  for (uint32_t i = tid; i < 3 * m; i += kTreeThreads) prims[3ull * b0 + i] = u.prim[i];
+  if (n == 1) {                                        // no internal node: keep the leaf box in the spare slot 0
+    if (tid == 0) store_child_box(nodes, 0, 0, lo, hi);
     return;
   }
-  int32_t child = ~(int32_t)k;
-  int32_t p = parent[n - 1 + k];
-  for (int step = 0; step < 130; ++step) {
-    const float4 cd = __ldg(nodes + 4 * (int64_t)p + 3);      // written by k_karras
-    const int slot = (__float_as_int(cd.x) == child) ? 0 : 1;
-    const uint2 rg = __ldg(range + p);
-    if (rg.x >= b0 && rg.y <= b1) {                  // this block's node
-      const uint32_t s = (uint32_t)p - b0;
-      for (int a = 0; a < 3; ++a) { s_box[slot][a][s] = lo[a]; s_box[slot][3 + a][s] = hi[a]; }
-      __threadfence_block();
-      if (atomicAdd(&s_arrived[s], 1u) == 0u) return;  // sibling not done yet
-      __threadfence_block();
-      float sl[3], sh[3];
-      for (int a = 0; a < 3; ++a) { sl[a] = s_box[slot ^ 1][a][s]; sh[a] = s_box[slot ^ 1][3 + a][s]; }
-      float4* o = nodes + 4 * (int64_t)p;
-      if (slot == 0) {
-        o[0] = make_float4(lo[0], hi[0], lo[1], hi[1]);
-        o[1] = make_float4(sl[0], sh[0], sl[1], sh[1]);
-        o[2] = make_float4(lo[2], hi[2], sl[2], sh[2]);
-      } else {
-        o[0] = make_float4(sl[0], sh[0], sl[1], sh[1]);
-        o[1] = make_float4(lo[0], hi[0], lo[1], hi[1]);
-        o[2] = make_float4(sl[2], sh[2], lo[2], hi[2]);
-      }
-      for (int a = 0; a < 3; ++a) { lo[a] = fminf(lo[a], sl[a]); hi[a] = fmaxf(hi[a], sh[a]); }
+  __syncthreads();
+  s_left[tid] = kNone;
+  u.run.arrived[tid] = 0;
+  if (leaf) u.run.delta[tid] = d;
+  if (tid == 0) {
+    u.run.arrived[kTreeThreads] = 0;
+    u.run.delta[m] = delta(keys, n, (int64_t)b0 + m - 1, (int64_t)b0 + m);
+  }
+  __syncthreads();
+  run_minima<kTreeThreads, kTreeThreads>(u.run, (int)m, s_warp);
+  __syncthreads();
+  if (leaf) {
+    int l;
+    int32_t child;
+    if (run_climb(u.run, [&](int j) { return b0 + (uint32_t)j; }, tid, (int)m, ~(int32_t)k, lo, hi, nodes, parent, n,
+                  l, child))
+      s_left[l] = child;
+  }
+  __syncthreads();
+  const int32_t mine = s_left[tid];
+  const uint32_t ball = __ballot_sync(0xFFFFFFFFu, mine != kNone);
+  if (lane == 0) s_warp[0][warp] = __popc(ball);
+  __syncthreads();
+  uint32_t at = __popc(ball & ((1u << lane) - 1u)), total = 0;
+  for (int w = 0; w < kTreeThreads / 32; ++w) {
+    if (w < warp) at += s_warp[0][w];
+    total += s_warp[0][w];
+  }
+  if (mine != kNone) left_over[b0 + at] = make_uint2((uint32_t)mine, k);
+  if (tid == 0) counts[blockIdx.x] = total;
+}
+
+// The trees over what kUpGroup runs left over (runs of `span` leaves each; run
+// j's list begins at left_over[j span]); what these leave over begins at their
+// first run's list.
+constexpr int kUpThreads = 512, kUpGroup = 16, kUpItems = kUpGroup * 128;
+struct UpShared {
+  Run<kUpItems> run;
+  uint32_t first[kUpItems + 1];
+  int32_t num[kUpItems], left[kUpItems];   // items; by first item: what is left over
+  int warp[2][kUpThreads / 32];
+  uint32_t base[kUpGroup + 1];
+};
+__global__ void __launch_bounds__(kUpThreads)
+k_tree_up(const float* sph, const float* tri, uint32_t ns, uint32_t n, bool wide, const uint64_t* __restrict__ keys,
+          float4* nodes, int32_t* parent, uint2* left_over, const uint32_t* __restrict__ counts, uint32_t runs,
+          uint64_t span, uint32_t* counts_out, uint32_t* err) {
+  extern __shared__ __align__(16) unsigned char up_smem[];
+  UpShared& s = *reinterpret_cast<UpShared*>(up_smem);
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const uint32_t r0 = blockIdx.x * kUpGroup, r1 = min(runs, r0 + kUpGroup);
+  constexpr int32_t kNone = 0x7FFFFFFF;
+  if (warp == 0) {
+    const uint32_t c = r0 + lane < r1 ? counts[r0 + lane] : 0u;
+    uint32_t sum = c;
+    for (int o = 1; o < 32; o <<= 1) {
+      const uint32_t x = __shfl_up_sync(0xFFFFFFFFu, sum, o);
+      if (lane >= o) sum += x;
+    }
+    if (lane <= kUpGroup) s.base[lane] = sum - c;
+  }
+  __syncthreads();
+  const uint32_t m = s.base[kUpGroup];
+  if (m > (uint32_t)kUpItems || m == 0) {              // cannot happen (see above)
+    if (tid == 0) { atomicOr(err, ERR_BUILD); counts_out[blockIdx.x] = 0; }
+    return;
+  }
+  const uint64_t begin = r0 * span, end = min((uint64_t)n, begin + kUpGroup * span);
+  auto item = [&](uint32_t i) {                        // (number, first leaf) of item i
+    uint32_t g = 0;
+    while (g + 1 < kUpGroup && s.base[g + 1] <= i) ++g;
+    return left_over[(r0 + g) * span + (i - s.base[g])];
+  };
+  for (uint32_t i = tid; i < m; i += kUpThreads) {
+    const uint2 x = item(i);
+    s.first[i] = x.y;
+    s.num[i] = (int32_t)x.x;
+    s.left[i] = kNone;
+    s.run.delta[i] = delta(keys, n, (int64_t)x.y, (int64_t)x.y - 1);
+    s.run.arrived[i] = 0;
+  }
+  if (tid == 0) {
+    s.first[m] = (uint32_t)end;
+    s.run.delta[m] = delta(keys, n, (int64_t)end - 1, (int64_t)end);
+    s.run.arrived[m] = 0;
+  }
+  __syncthreads();
+  run_minima<kUpItems, kUpThreads>(s.run, (int)m, s.warp);
+  __syncthreads();
+  for (uint32_t i = tid; i < m; i += kUpThreads) {
+    const int32_t num = s.num[i];
+    float lo[3], hi[3];
+    if (num < 0) {
+      const uint32_t id = (uint32_t)(keys[~num] & 0xFFFFFFFFull);
+      float v[9];
+      if (id >= ns) load_tri(tri, id - ns, wide, v);
+      prim_box(sph, v, ns, id, lo, hi);
     } else {
-      store_child_box(nodes, p, slot, lo, hi);
-      __threadfence();
-      if (atomicAdd(&arrivals[p], 1u) == 0u) return;   // sibling not done yet
-      __threadfence();
-      // both children are in: merge them into the box of p
-      const float4 a = __ldcg(nodes + 4 * (int64_t)p + 0);
-      const float4 b = __ldcg(nodes + 4 * (int64_t)p + 1);
-      const float4 c = __ldcg(nodes + 4 * (int64_t)p + 2);
+      const float4 a = nodes[4 * (int64_t)num], b = nodes[4 * (int64_t)num + 1], c = nodes[4 * (int64_t)num + 2];
       lo[0] = fminf(a.x, b.x); hi[0] = fmaxf(a.y, b.y);
       lo[1] = fminf(a.z, b.z); hi[1] = fmaxf(a.w, b.w);
       lo[2] = fminf(c.x, c.z); hi[2] = fmaxf(c.y, c.w);
     }
-    if (p == 0) return;                                // root reached
-    child = p;
-    p = parent[p];
+    int l;
+    int32_t child;
+    if (run_climb(s.run, [&](int j) { return s.first[j]; }, (int)i, (int)m, num, lo, hi, nodes, parent, n, l, child))
+      s.left[l] = child;
   }
-  atomicOr(err, ERR_BUILD);
+  __syncthreads();
+  uint32_t total = 0;
+  for (uint32_t base = 0; base < m; base += kUpThreads) {
+    const uint32_t i = base + tid;
+    const int32_t mine = i < m ? s.left[i] : kNone;
+    const uint32_t ball = __ballot_sync(0xFFFFFFFFu, mine != kNone);
+    if (lane == 0) s.warp[0][warp] = __popc(ball);
+    __syncthreads();
+    uint32_t at = total + __popc(ball & ((1u << lane) - 1u));
+    for (int w = 0; w < kUpThreads / 32; ++w) {
+      if (w < warp) at += s.warp[0][w];
+      total += s.warp[0][w];
+    }
+    if (mine != kNone) left_over[begin + at] = make_uint2((uint32_t)mine, s.first[i]);
+    __syncthreads();
+  }
+  if (tid == 0) counts_out[blockIdx.x] = total;
 }
 
 // Raw primitive records word by word: spheres of 5 (centre, radius, material),
@@ -507,10 +715,9 @@ size_t lbvh_tmp_bytes(uint32_t n) {
   size_t nblocks = (n + kTile - 1) / kTile;
   size_t b = 0;
   b += kRedBlocks * sizeof(Bounds6);                         // bounds
-  b += (size_t)n * 8 + 256;                                  // ping-pong keys, then the nodes' leaf ranges
+  b += (size_t)n * 8 + 256;                                  // ping-pong keys, then what the runs leave over
   b += 256 * nblocks * 4 + 256;                              // histogram
   b += 256 * 4;                                              // digit totals
-  b += (size_t)n * 4 + 256;                                  // arrival counters
   return b + 1024;
 }
 
@@ -527,7 +734,6 @@ cudaError_t build_lbvh(const float4* d_sph_in, const float* d_tri_in, uint32_t n
   uint64_t* keys_b = reinterpret_cast<uint64_t*>(take((size_t)n * 8));
   uint32_t* hist = reinterpret_cast<uint32_t*>(take(256ull * nblocks * 4));
   uint32_t* totals = reinterpret_cast<uint32_t*>(take(256 * 4));
-  uint32_t* arrivals = reinterpret_cast<uint32_t*>(take((size_t)n * 4));
   const bool wide = (reinterpret_cast<uintptr_t>(d_tri_in) & 7u) == 0;
 
   int red_grid = (int)std::min<uint32_t>((uint32_t)kRedBlocks, (n + kRedThreads - 1) / kRedThreads);
@@ -542,16 +748,25 @@ cudaError_t build_lbvh(const float4* d_sph_in, const float* d_tri_in, uint32_t n
     k_scatter<<<nblocks, kSortThreads, 0, st>>>(a, b, n, shift, hist, nblocks, totals);
     uint64_t* x = a; a = b; b = x;
   }
-  // four passes: the sorted keys are back in d_keys, and keys_b is free
-  uint2* range = reinterpret_cast<uint2*>(keys_b);
-  if (n > 1) {
-    k_karras<<<(n - 1 + 255) / 256, 256, 0, st>>>(d_keys, n, d_nodes, d_parent, range);
-    cudaMemsetAsync(arrivals, 0, (size_t)n * 4, st);
-  } else {
-    cudaMemsetAsync(d_parent, 0xFF, 4, st);
+  // four passes: the sorted keys are back in d_keys; keys_b holds what the runs leave over, the
+  // histograms their counts
+  uint2* left_over = reinterpret_cast<uint2*>(keys_b);
+  if (n == 1) cudaMemsetAsync(d_parent, 0xFF, 4, st);
+  uint32_t runs = (uint32_t)(((uint64_t)n + kTreeThreads - 1) / kTreeThreads);
+  k_tree<<<runs, kTreeThreads, 0, st>>>(sph, d_tri_in, ns, n, wide, d_keys, d_nodes, d_prims, d_parent, left_over, hist);
+  if (runs > 1) {
+    // an attribute of the current device: set on every call
+    const cudaError_t e = cudaFuncSetAttribute(k_tree_up, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(UpShared));
+    if (e != cudaSuccess) return e;
   }
-  k_refit<<<(n + kRefitThreads - 1) / kRefitThreads, kRefitThreads, 0, st>>>(
-      sph, d_tri_in, ns, n, wide, d_keys, d_nodes, d_prims, d_parent, range, arrivals, d_err);
+  uint32_t* counts = hist;
+  for (uint64_t span = kTreeThreads; runs > 1; span *= kUpGroup) {
+    const uint32_t groups = (runs + kUpGroup - 1) / kUpGroup;
+    k_tree_up<<<groups, kUpThreads, sizeof(UpShared), st>>>(sph, d_tri_in, ns, n, wide, d_keys, d_nodes, d_parent, left_over,
+                                                       counts, runs, span, counts + runs, d_err);
+    counts += runs;
+    runs = groups;
+  }
   return cudaGetLastError();
 }
 

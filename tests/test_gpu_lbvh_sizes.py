@@ -71,3 +71,32 @@ def test_device_records_of_any_alignment():
         got.append(out)
     for a, b in zip(*got):
         assert torch.equal(a, b)
+
+
+@pytest.mark.parametrize("n", [512, 4095, 4096, 4097, 65536, 65793])
+def test_levels_of_runs(n):
+    """Trees over runs of 256 leaves, over 16 of those, and over 256 of those."""
+    _check(_scene(n // 2, n - n // 2, n))
+
+
+def test_runs_that_leave_much_over():
+    """Points at powers of two towards one corner: prefixes shorten by a bit from
+    leaf to leaf, so that most subtrees hang off the path to one end of a run."""
+    s = _scene(0, 6000, 1)
+    tr = s.triangles.copy()
+    p = np.float32(2.0) ** -np.random.default_rng(2).uniform(0, 12, (6000, 3)).astype(np.float32)
+    for v in ("v0", "v1", "v2"):
+        tr[v] = p
+    _check(s.with_view(triangles=tr))
+
+
+@pytest.mark.parametrize("scale", [1e-40, 1e37, 3e38])
+def test_bounds_of_extreme_coordinates(scale):
+    """Sums of vertices past the range of FP32, and denormal ones."""
+    s = _scene(40, 3000, 9)
+    tr, sp = s.triangles.copy(), s.spheres.copy()
+    rng = np.random.default_rng(4)
+    for v in ("v0", "v1", "v2"):
+        tr[v] = (rng.uniform(-1, 1, (3000, 3)) * scale).astype(np.float32)
+    sp["center"] = (rng.uniform(-1, 1, (40, 3)) * min(scale, 1e37)).astype(np.float32)
+    _check(s.with_view(spheres=sp, triangles=tr))
