@@ -23,14 +23,15 @@
 //      on until one block is left.
 //
 // Measured (GB300, 1,000,000 primitives in random order, the whole device-side
-// build): 0.299 ms; 1.110 when one block scanned the tile counts (0.40),
-// one thread reduced the bounds (0.12), every key was divided twice in FP64
-// (0.27 with the bounds) and every node had a global arrival counter (0.18);
-// 0.359 with a search per node (38 us) and a refit that read its parents,
-// children and ranges from memory at every step (125 us). Its kernels' shares
-// now: tree 77 us, upper levels 15 each, scatter 4 x 13, bounds 25, keys 23,
-// histograms 3 x 5, scans 4 x 3. What is left in k_tree is the chain of a
-// block's climb, seven to ten levels of shared-memory exchanges.
+// build): 0.267 ms (0.30 when each launch waited for the kernel before it to
+// end). 1.110 when one block scanned the tile counts (0.40), one thread reduced
+// the bounds (0.12), every key was divided twice in FP64 (0.27 with the bounds)
+// and every node had a global arrival counter (0.18); 0.359 with a search per
+// node (38 us) and a refit that read its parents, children and ranges from
+// memory at every step (125 us). Its kernels' shares now: tree 77 us, upper
+// levels 15 each, scatter 4 x 13, bounds 25, keys 23, histograms 3 x 5, scans
+// 4 x 3. What is left in k_tree is the chain of a block's climb, seven to ten
+// levels of shared-memory exchanges.
 #include <cuda_runtime.h>
 #include <stdint.h>
 
@@ -96,6 +97,7 @@ __device__ __forceinline__ void sum_range(const float v[9], int k, float& least,
 
 __global__ void __launch_bounds__(kRedThreads)
 k_centroid_bounds(const float* sph, const float* tri, uint32_t ns, uint32_t n, bool wide, Bounds6* partial) {
+  after_previous();
   __shared__ float s_f[12][kRedThreads / 32];      // sphere min, -max; triangle: upper bound of the min, of -max
   __shared__ long long s_d[6][kRedThreads / 32];   // triangle min, ~max
   const long long kMost = 0x7FFFFFFFFFFFFFFFll;
@@ -177,6 +179,7 @@ k_centroid_bounds(const float* sph, const float* tri, uint32_t ns, uint32_t n, b
 
 // bounds of all blocks: warp q takes value q (lo x, y, z, hi x, y, z)
 __global__ void k_reduce_bounds(Bounds6* partial, int nparts) {
+  after_previous();
   const int q = threadIdx.x >> 5, lane = threadIdx.x & 31;
   double m = q < 3 ? INFINITY : -INFINITY;
   for (int p = lane; p < nparts; p += 32) {
@@ -229,6 +232,7 @@ __device__ __forceinline__ AxisEstimate axis_estimate(double lo, double hi) {
 __global__ void __launch_bounds__(kSortThreads)
 k_keys(const float* sph, const float* tri, uint32_t ns, uint32_t n, bool wide, const Bounds6* b,
        uint64_t* keys, uint32_t* ghist, int nblocks) {
+  after_previous();
   __shared__ uint32_t h[256];
   __shared__ AxisEstimate est[3];
   h[threadIdx.x] = 0;
@@ -268,6 +272,7 @@ k_keys(const float* sph, const float* tri, uint32_t ns, uint32_t n, bool wide, c
 
 // ---------------------------------------------------------------- radix sort
 __global__ void k_hist(const uint64_t* keys, uint32_t n, int shift, uint32_t* ghist, int nblocks) {
+  after_previous();
   __shared__ uint32_t h[256];
   h[threadIdx.x] = 0;
   __syncthreads();
@@ -283,6 +288,7 @@ __global__ void k_hist(const uint64_t* keys, uint32_t n, int shift, uint32_t* gh
 // exclusive scan of each digit's tile counts (block d: row d of ghist), and
 // the digit's total
 __global__ void __launch_bounds__(256) k_scan(uint32_t* ghist, int nblocks, uint32_t* totals) {
+  after_previous();
   __shared__ uint32_t part[8];
   uint32_t* a = ghist + (size_t)blockIdx.x * nblocks;
   const uint32_t lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -317,6 +323,7 @@ __global__ void __launch_bounds__(256) k_scan(uint32_t* ghist, int nblocks, uint
 __global__ void __launch_bounds__(kSortThreads)
 k_scatter(const uint64_t* in, uint64_t* out, uint32_t n, int shift, const uint32_t* gscan, int nblocks,
           const uint32_t* totals) {
+  after_previous();
   constexpr int kWarps = kSortThreads / 32;
   __shared__ uint32_t wcnt[kWarps][256];
   __shared__ uint32_t to_global[256];          // global position of a digit's run minus its local one
@@ -516,6 +523,7 @@ constexpr int kTreeThreads = 256;
 __global__ void __launch_bounds__(kTreeThreads, 6)
 k_tree(const float* sph, const float* tri, uint32_t ns, uint32_t n, bool wide, const uint64_t* __restrict__ keys,
        float4* nodes, float4* prims, int32_t* parent, uint2* left_over, uint32_t* counts) {
+  after_previous();
   __shared__ union {
     float4 prim[3 * kTreeThreads];
     Run<kTreeThreads> run;
@@ -600,6 +608,7 @@ __global__ void __launch_bounds__(kUpThreads)
 k_tree_up(const float* sph, const float* tri, uint32_t ns, uint32_t n, bool wide, const uint64_t* __restrict__ keys,
           float4* nodes, int32_t* parent, uint2* left_over, const uint32_t* __restrict__ counts, uint32_t runs,
           uint64_t span, uint32_t* counts_out, uint32_t* err) {
+  after_previous();
   extern __shared__ __align__(16) unsigned char up_smem[];
   UpShared& s = *reinterpret_cast<UpShared*>(up_smem);
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -737,15 +746,15 @@ cudaError_t build_lbvh(const float4* d_sph_in, const float* d_tri_in, uint32_t n
   const bool wide = (reinterpret_cast<uintptr_t>(d_tri_in) & 7u) == 0;
 
   int red_grid = (int)std::min<uint32_t>((uint32_t)kRedBlocks, (n + kRedThreads - 1) / kRedThreads);
-  k_centroid_bounds<<<red_grid, kRedThreads, 0, st>>>(sph, d_tri_in, ns, n, wide, partial);
-  k_reduce_bounds<<<1, 192, 0, st>>>(partial, red_grid);
-  k_keys<<<nblocks, kSortThreads, 0, st>>>(sph, d_tri_in, ns, n, wide, partial, d_keys, hist, nblocks);
+  launch_after(k_centroid_bounds, red_grid, kRedThreads, 0, st, sph, d_tri_in, ns, n, wide, partial);
+  launch_after(k_reduce_bounds, 1, 192, 0, st, partial, red_grid);
+  launch_after(k_keys, nblocks, kSortThreads, 0, st, sph, d_tri_in, ns, n, wide, partial, d_keys, hist, nblocks);
   uint64_t* a = d_keys;
   uint64_t* b = keys_b;
   for (int shift = 32; shift < 64; shift += 8) {
-    if (shift > 32) k_hist<<<nblocks, kSortThreads, 0, st>>>(a, n, shift, hist, nblocks);
-    k_scan<<<256, 256, 0, st>>>(hist, nblocks, totals);
-    k_scatter<<<nblocks, kSortThreads, 0, st>>>(a, b, n, shift, hist, nblocks, totals);
+    if (shift > 32) launch_after(k_hist, nblocks, kSortThreads, 0, st, a, n, shift, hist, nblocks);
+    launch_after(k_scan, 256, 256, 0, st, hist, nblocks, totals);
+    launch_after(k_scatter, nblocks, kSortThreads, 0, st, a, b, n, shift, hist, nblocks, totals);
     uint64_t* x = a; a = b; b = x;
   }
   // four passes: the sorted keys are back in d_keys; keys_b holds what the runs leave over, the
@@ -753,7 +762,7 @@ cudaError_t build_lbvh(const float4* d_sph_in, const float* d_tri_in, uint32_t n
   uint2* left_over = reinterpret_cast<uint2*>(keys_b);
   if (n == 1) cudaMemsetAsync(d_parent, 0xFF, 4, st);
   uint32_t runs = (uint32_t)(((uint64_t)n + kTreeThreads - 1) / kTreeThreads);
-  k_tree<<<runs, kTreeThreads, 0, st>>>(sph, d_tri_in, ns, n, wide, d_keys, d_nodes, d_prims, d_parent, left_over, hist);
+  launch_after(k_tree, runs, kTreeThreads, 0, st, sph, d_tri_in, ns, n, wide, d_keys, d_nodes, d_prims, d_parent, left_over, hist);
   if (runs > 1) {
     // an attribute of the current device: set on every call
     const cudaError_t e = cudaFuncSetAttribute(k_tree_up, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(UpShared));
@@ -762,8 +771,7 @@ cudaError_t build_lbvh(const float4* d_sph_in, const float* d_tri_in, uint32_t n
   uint32_t* counts = hist;
   for (uint64_t span = kTreeThreads; runs > 1; span *= kUpGroup) {
     const uint32_t groups = (runs + kUpGroup - 1) / kUpGroup;
-    k_tree_up<<<groups, kUpThreads, sizeof(UpShared), st>>>(sph, d_tri_in, ns, n, wide, d_keys, d_nodes, d_parent, left_over,
-                                                       counts, runs, span, counts + runs, d_err);
+    launch_after(k_tree_up, groups, kUpThreads, sizeof(UpShared), st, sph, d_tri_in, ns, n, wide, d_keys, d_nodes, d_parent, left_over, counts, runs, span, counts + runs, d_err);
     counts += runs;
     runs = groups;
   }

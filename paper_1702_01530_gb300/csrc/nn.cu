@@ -394,6 +394,7 @@ __global__ void __launch_bounds__(kConvTmaThreads, 1)
     k_conv_tma(const __grid_constant__ CUtensorMap tmap, const void* __restrict__ wpk,
                const __nv_bfloat16* __restrict__ mask16, __nv_bfloat16* __restrict__ out, uint32_t W,
                uint32_t H, uint32_t* err) {
+  after_previous();
   using Lt = ConvTmaLayout<CIN>;
   static_assert(CIN % 16 == 0, "shape");
   extern __shared__ __align__(1024) unsigned char smem[];
@@ -928,6 +929,7 @@ __device__ __forceinline__ float bce_gradient(float p, float y, uint4& g8) {
 template <bool FP8, bool STORE>
 __global__ void __launch_bounds__(kFuThreads, 1)
     k_net_fused(const __grid_constant__ CUtensorMap tmap, const __grid_constant__ FusedArgs a) {
+  after_previous();
   using Lt = FusedLayout<FP8>;
   extern __shared__ __align__(1024) unsigned char smem[];
   uint64_t* bars = reinterpret_cast<uint64_t*>(smem + Lt::kOffB);
@@ -1514,6 +1516,7 @@ __device__ __forceinline__ void wgrad_body(const WgradArgs& args, const int laye
 
 template <int CHAIN>
 __global__ void __launch_bounds__(kWgThreads, 1) k_wgrad(const __grid_constant__ WgradArgs args) {
+  after_previous();
   extern __shared__ __align__(1024) unsigned char smem[];
   if (blockIdx.x < args.share[1].blk0) wgrad_body<2, 4, CHAIN>(args, 0, smem);
   else if (blockIdx.x < args.share[2].blk0) wgrad_body<4, 4, CHAIN>(args, 1, smem);
@@ -1551,6 +1554,7 @@ struct UpdateArgs {
 };
 
 __global__ void __launch_bounds__(256) k_update(const __grid_constant__ UpdateArgs a) {
+  after_previous();
   __shared__ float s[8][32], sc[8][32];
   const uint32_t lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   int l = 3;
@@ -1737,7 +1741,7 @@ cudaError_t launch_conv(const void* in, uint32_t chunks, const void* wpk, const 
   const cudaError_t e = make_halo_map(&map, in, W, H, chunks);
   if (e != cudaSuccess) return e;
   const uint32_t grid = std::min<uint32_t>((uint32_t)num_sms(), tiles);
-  k_conv_tma<CIN><<<grid, kConvTmaThreads, smem, st>>>(map, wpk, mask16, out, W, H, err);
+  launch_after(k_conv_tma<CIN>, grid, kConvTmaThreads, smem, st, map, wpk, mask16, out, W, H, err);
   return cudaGetLastError();
 }
 }  // namespace
@@ -1817,7 +1821,7 @@ cudaError_t launch_fused(const __nv_bfloat16* feat16, FusedArgs& a, uint32_t W, 
   const uint64_t items = strips * a.segs;
   const int grid = (int)std::min(items, sms);
   if (grid_out) *grid_out = grid;
-  k_net_fused<FP8, STORE><<<grid, kFuThreads, smem, st>>>(map, a);
+  launch_after(k_net_fused<FP8, STORE>, grid, kFuThreads, smem, st, map, a);
   return cudaGetLastError();
 }
 }  // namespace
@@ -1933,8 +1937,8 @@ cudaError_t train_step(const __nv_bfloat16* feat16, const float* label, const Tr
     configured = true;
   }
   const uint32_t grid = g.share[3].blk0 + g.share[3].nblk;
-  if (wgrad_tiles(W, H) <= (uint64_t)kWgFewTiles * g.share[1].nblk) k_wgrad<2><<<grid, kWgThreads, smem, st>>>(g);
-  else k_wgrad<4><<<grid, kWgThreads, smem, st>>>(g);
+  if (wgrad_tiles(W, H) <= (uint64_t)kWgFewTiles * g.share[1].nblk) launch_after(k_wgrad<2>, grid, kWgThreads, smem, st, g);
+  else launch_after(k_wgrad<4>, grid, kWgThreads, smem, st, g);
 
   UpdateArgs u = {};
   uint32_t block = 0;
@@ -1956,7 +1960,7 @@ cudaError_t train_step(const __nv_bfloat16* feat16, const float* label, const Tr
   u.loss_part = t.loss_part;
   u.n_loss = 4u * (uint32_t)fwd_grid;
   u.loss = t.loss;
-  k_update<<<block, 256, 0, st>>>(u);
+  launch_after(k_update, block, 256, 0, st, u);
   return cudaGetLastError();
 }
 

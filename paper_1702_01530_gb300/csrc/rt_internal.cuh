@@ -206,6 +206,32 @@ cudaError_t render(const RenderArgs& a, Workspace& ws, cudaStream_t st);
 // stage timing: start a profiled call (resets the event list) / mark the end of a stage
 void profile_begin(Workspace& ws, cudaStream_t st);
 void profile_mark(Workspace& ws, int stage, cudaStream_t st);
+// Launch of a kernel that begins with after_previous(): it is put on the SMs as
+// the kernel before it in the stream drains instead of after that has ended and
+// waits there (programmatic dependent launch), which hides its launch: 1 to 2 us
+// a kernel in the training step and the builds. It reads and writes nothing
+// before that wait, which covers all earlier work of the stream.
+template <typename... P, typename... A>
+cudaError_t launch_after(void (*kernel)(P...), unsigned grid, unsigned block, size_t smem, cudaStream_t st, A&&... args) {
+  cudaLaunchAttribute attr = {};
+  attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr.val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t c = {};
+  c.gridDim = dim3(grid);
+  c.blockDim = dim3(block);
+  c.dynamicSmemBytes = smem;
+  c.stream = st;
+  c.attrs = &attr;
+  c.numAttrs = 1;
+  return cudaLaunchKernelEx(&c, kernel, static_cast<P>(args)...);
+}
+#ifdef __CUDACC__
+// waits for all earlier work of the stream; lets the next kernel be put in place
+__device__ __forceinline__ void after_previous() {
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+#endif
 int num_sms();
 int render_grid();      // persistent blocks of the render kernel
 int render_threads();   // threads per block of the render kernel

@@ -261,6 +261,7 @@ __device__ __forceinline__ void combine6(uint32_t grp, const int v[6], int* dst)
 __global__ void __launch_bounds__(kThreads)
 k_leaves(const float4* __restrict__ nodes, const int32_t* __restrict__ parent, uint32_t n,
          float4* __restrict__ lo, float4* __restrict__ hi, uint32_t* __restrict__ idx, TopNode* root) {
+  after_previous();
   const uint32_t k = blockIdx.x * blockDim.x + threadIdx.x;
   __shared__ int s_bounds[6];
   if (threadIdx.x < 6) s_bounds[threadIdx.x] = empty6(threadIdx.x);
@@ -291,6 +292,7 @@ k_leaves(const float4* __restrict__ nodes, const int32_t* __restrict__ parent, u
 // the build's control words and, in a build with a top phase, its root entry;
 // else the whole build is one mid job
 __global__ void k_begin(Control* c, TopNode* root, uint32_t* slice_node, Job* mid, uint32_t n, uint32_t slice) {
+  after_previous();
   const uint32_t slices = (uint32_t)(((uint64_t)n + slice - 1) / slice);
   if (root) {
     for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < slices; i += gridDim.x * blockDim.x)
@@ -348,6 +350,7 @@ __device__ __forceinline__ void load_leaves(const Build& g, uint32_t base, uint3
 // 1. bins of a slice, added to its node's; the slice's own counts are kept
 __global__ void __launch_bounds__(kThreads)
 k_top_bins(const Build g, int cur) {
+  after_previous();
   const uint32_t* __restrict__ slice_node = g.slice_node[0];
   int* __restrict__ slice_cnt = g.slice_cnt;
   TopNode* nodes = g.nodes[0];
@@ -500,6 +503,7 @@ __device__ void top_node(const TopNode& t, uint32_t n_left, int axis, int bin, c
 // then step 3 by the node's last slice
 __global__ void __launch_bounds__(kThreads, 4)
 k_top_scatter(const Build g, int cur) {
+  after_previous();
   uint32_t* __restrict__ idx_out = g.idx[1];
   const uint32_t* __restrict__ slice_node = g.slice_node[0];
   const int* __restrict__ slice_cnt = g.slice_cnt;
@@ -774,6 +778,7 @@ __global__ void __launch_bounds__(kThreads, 4)
 k_sah_mid(const float4* __restrict__ leaf_lo, const float4* __restrict__ leaf_hi,
           const uint32_t* __restrict__ idx0, const uint32_t* __restrict__ idx1, Control* ctl,
           const Job* __restrict__ jobs, float4* __restrict__ out, uint32_t n, uint32_t* __restrict__ err) {
+  after_previous();
   __shared__ uint32_t s_slot[kThreads];
   __shared__ float s_box[6][kThreads];
   __shared__ uint32_t s_begin[kThreads], s_end[kThreads];          // segment of each position
@@ -957,6 +962,7 @@ __device__ __forceinline__ void centre_extent(float lo, float hi, float& c, floa
 }
 
 __global__ void k_render_nodes(const float4* __restrict__ nodes, uint32_t n_inner, float4* __restrict__ out) {
+  after_previous();
   const uint32_t i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= n_inner) return;
   const float4 a = nodes[4 * (size_t)i], b = nodes[4 * (size_t)i + 1], c = nodes[4 * (size_t)i + 2];
@@ -977,7 +983,7 @@ __global__ void k_render_nodes(const float4* __restrict__ nodes, uint32_t n_inne
 
 cudaError_t render_nodes(const float4* nodes, uint32_t n, float4* out, cudaStream_t st) {
   if (n < 2) return cudaSuccess;      // no inner node
-  k_render_nodes<<<(n - 1 + 255) / 256, 256, 0, st>>>(nodes, n - 1, out);
+  launch_after(k_render_nodes, (n - 1 + 255) / 256, 256, 0, st, nodes, n - 1, out);
   return cudaGetLastError();
 }
 
@@ -1028,9 +1034,8 @@ cudaError_t build_sah_tree(const float4* lbvh_nodes, const int32_t* parent, uint
   const bool top = n > kMidLeaves;
   const uint32_t* const idx[2] = {s.idx[0], s.idx[1]};
   TopNode* root = top ? s.nodes[0] : nullptr;
-  k_begin<<<1, kThreads, 0, st>>>(s.ctl, root, s.slice_node[0], s.mid, n, s.slice);
-  k_leaves<<<(int)(((uint64_t)n + kThreads - 1) / kThreads), kThreads, 0, st>>>(lbvh_nodes, parent, n, s.lo, s.hi,
-                                                                         s.idx[0], root);
+  launch_after(k_begin, 1, kThreads, 0, st, s.ctl, root, s.slice_node[0], s.mid, n, s.slice);
+  launch_after(k_leaves, (int)(((uint64_t)n + kThreads - 1) / kThreads), kThreads, 0, st, lbvh_nodes, parent, n, s.lo, s.hi, s.idx[0], root);
   cudaError_t e = cudaSuccess;
   uint32_t n_mid = 1;
   if (top) {
@@ -1049,8 +1054,8 @@ cudaError_t build_sah_tree(const float4* lbvh_nodes, const int32_t* parent, uint
         until += kExtra;
       }
       const int cur = level & 1;
-      k_top_bins<<<blocks, kThreads, 0, st>>>(s, cur);
-      k_top_scatter<<<blocks, kThreads, 0, st>>>(s, cur);
+      launch_after(k_top_bins, blocks, kThreads, 0, st, s, cur);
+      launch_after(k_top_scatter, blocks, kThreads, 0, st, s, cur);
       std::swap(s.idx[0], s.idx[1]);
       std::swap(s.nodes[0], s.nodes[1]);
       std::swap(s.slice_node[0], s.slice_node[1]);
@@ -1059,8 +1064,7 @@ cudaError_t build_sah_tree(const float4* lbvh_nodes, const int32_t* parent, uint
     if (e == cudaSuccess && n_mid > s.max_mid) e = cudaErrorUnknown;
   }
   if (e == cudaSuccess && n_mid)
-    k_sah_mid<<<(int)std::min(n_mid, 0x7FFFFFFFu), kThreads, 0, st>>>(s.lo, s.hi, idx[0], idx[1], s.ctl, s.mid,
-                                                                     out, n, err);
+    launch_after(k_sah_mid, (int)std::min(n_mid, 0x7FFFFFFFu), kThreads, 0, st, s.lo, s.hi, idx[0], idx[1], s.ctl, s.mid, out, n, err);
   return e == cudaSuccess ? cudaGetLastError() : e;
 }
 
