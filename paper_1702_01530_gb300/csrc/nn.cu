@@ -7,43 +7,20 @@
 // written only where training or calibration asks for them.
 //
 // Backward pass: data gradients are convolutions with the 3x3 taps flipped and
-// Cin/Cout swapped (k_conv_tma, below); weight gradients are contractions over
-// the pixels (k_wgrad); BCE on the sigmoid output; Adam on FP32 master
-// weights.
+// Cin/Cout swapped (k_bwd_fused, all three in one kernel); weight gradients are
+// contractions over the pixels (k_wgrad); BCE on the sigmoid output; Adam on FP32
+// master weights.
 //
-// Convolution as implicit GEMM on tcgen05 (k_conv_tma):
-//   a persistent CTA computes tiles of R rows x 126 consecutive pixels:
-//   output row ry is D_ry[128 pixels, 32] = sum over the 9 taps (dy, dx) of
-//   A(ry+dy, dx)[128, Cin] x B(dy, dx)[Cin, 32], where A(h, dx) is halo row h
-//   shifted by dx pixels. The input halo (R+2 rows of Cin channels) sits in
-//   shared memory as 16-byte channel chunks ordered [chunk][halo pixel], so
-//   every A(h, dx) is the same matrix shifted by h*128 + dx rows: the
-//   K-major, non-swizzled operand layout with 8-row core matrices 128 B apart
-//   (SBO) and chunk planes (R+2)*128*16 B apart (LBO). The chunk planes are
-//   loaded as 2 KB box rows of 128 pixels (the MMA lanes 126 and 127 read the
-//   next row and are not stored).
-//   Stacked taps: an MMA of N = Cout costs the tensor core as much as one of
-//   N = 64 (about 45 cycles on GB300, measured; N = 96 about 56, N = 256 about
-//   128, the full rate), so the three vertical taps of a kernel column are
-//   multiplied in one MMA of N = 3 Cout: B(dx) = [B(2, dx) | B(1, dx) |
-//   B(0, dx)], and A(h, dx) x B(dx) lands in TMEM at column h*Cout of the
-//   tile's accumulators, where output row ry keeps its sum at column
-//   (ry+2)*Cout: block j of the product (tap dy = 2 - j) adds into row h - dy.
-//   Consecutive MMAs thus accumulate into overlapping column ranges (exact,
-//   measured), (R+2) * 3 MMAs per K step and tile instead of R * 9; rows -2,
-//   -1, R, R+1 of the accumulators take the products that fall outside the
-//   tile and are never read. Every MMA accumulates; the epilogue zeroes the
-//   columns it has read (and the four outside rows) before handing the
-//   accumulators back. Weights are pre-packed in this stacked core-matrix
-//   layout, [dx][chunk][3 Cout][chunk elements].
-//   The CTA is warp-specialised: a TMA warp loads each tile's halo
-//   (cp.async.bulk.tensor, zeros outside the image) into a ring of halo
-//   buffers; an MMA warp issues the tile's MMAs into one of two TMEM
-//   accumulator sets; the epilogue warps read their TMEM lanes (tcgen05.ld
-//   32x32b), hand the set back and apply the ReLU mask, so loads, MMAs and
-//   epilogues of consecutive tiles overlap.
-//   Every mbarrier wait has an iteration bound; on expiry the kernel sets the
-//   error word, waits (bounded) for what it has in flight and frees its TMEM.
+// Convolution as implicit GEMM on tcgen05: 128 pixels of a row are the M of an
+// MMA. A row's input sits in shared memory as 16-byte channel chunks ordered
+// [chunk][pixel], so kernel column dx is the same K-major, non-swizzled operand
+// (8-row core matrices 128 B apart, SBO; chunk planes apart by LBO) moved by dx
+// pixels. An MMA of N = Cout costs the tensor core as much as one of N = 64 (about
+// 45 cycles on GB300, measured; N = 96 about 56, N = 256 about 128, the full rate),
+// so the three vertical taps of a kernel column are stacked along N; weights are
+// packed in this stacked core-matrix layout, [dx][chunk][3 Cout][chunk elements].
+// Every mbarrier wait has an iteration bound; on expiry the kernel sets the error
+// word, waits (bounded) for what it has in flight and frees its TMEM.
 //
 // Layouts in HBM: the network input features are interleaved [P][16]; the BCE
 // gradient is one chunk per pixel [P][8]; the 32-channel activations and data
@@ -64,35 +41,7 @@
 namespace rt {
 namespace nn {
 
-// Tuning knobs of k_conv_tma: RT_CONV_ROWS = image rows per tile (R accumulators
-// of 128 pixels share one halo of R+2 rows; with the stacked taps each
-// accumulator set takes (R+4) * 32 TMEM columns, so R <= 4); RT_CONV_STAGES =
-// the most halo buffers a CTA keeps (as many as fit in ~220 KB of shared
-// memory, up to this; the loads run that many tiles ahead of the MMAs; deeper
-// rings were slower); RT_CONV_EPI_WG = epilogue warpgroups (4 warps each; group
-// g takes the rows ry with ry % RT_CONV_EPI_WG == g of every tile; 4 groups were
-// slower than 2).
-#ifndef RT_CONV_ROWS
-#define RT_CONV_ROWS 4
-#endif
-#ifndef RT_CONV_STAGES
-#define RT_CONV_STAGES 4
-#endif
-#ifndef RT_CONV_EPI_WG
-#define RT_CONV_EPI_WG 2
-#endif
-constexpr int kMaxStages = RT_CONV_STAGES;
-static_assert(kMaxStages >= 2 && kMaxStages <= 8, "halo stages");
 constexpr uint32_t kSmemBudget = 220u * 1024u;
-constexpr int kEpiWarps = 4 * RT_CONV_EPI_WG;
-constexpr int kConvTmaThreads = 32 * (kEpiWarps + 2);   // + the MMA warp and the TMA warp
-constexpr int kRows = RT_CONV_ROWS;
-constexpr int kTileM = 128;          // pixels per row tile (one MMA M block)
-// An input is loaded as one TMA box per chunk whose rows are 128 pixels x 16
-// bytes (256 8-byte elements, the largest box row), so tiles are 126 output
-// pixels wide. Boxes with rows of one 16-byte chunk make one 16-byte request
-// per pixel that moves a whole 32-byte sector from L2 (measured slower).
-constexpr int kHaloW = kTileM;
 constexpr uint32_t kWaitBound = 1u << 26;
 
 // ------------------------------------------------------------ PTX helpers
@@ -271,6 +220,13 @@ __device__ __forceinline__ uint32_t pack_bf16(float a, float b) {
   return *reinterpret_cast<uint32_t*>(&h);
 }
 
+// BF16 of (a, b), each zero where its half of `mask` is not above zero
+__device__ __forceinline__ uint32_t masked_pair(uint32_t mask, uint32_t a, uint32_t b) {
+  const __nv_bfloat162 zero = __float2bfloat162_rn(0.f);
+  return pack_bf16(__uint_as_float(a), __uint_as_float(b)) &
+         __hgt2_mask(*reinterpret_cast<const __nv_bfloat162*>(&mask), zero);
+}
+
 // (a0, a1) += (b0, b1) in one instruction, each sum rounded to nearest
 __device__ __forceinline__ void add2(float& a0, float& a1, float b0, float b1) {
   asm("{\n\t.reg .b64 x, y;\n\t"
@@ -313,35 +269,6 @@ __device__ __forceinline__ uint32_t relu_e4m3x4(float x0, float x1, float x2, fl
   return d;
 }
 
-// All MMAs of one tile: for halo row h, kernel column dx and 32-byte K step
-// ks (16 channels), the halo shifted by h*128 + dx pixels times the stacked
-// weights B(dx) (N = 96) accumulate into TMEM columns dtmem + h*32 .. + 95
-// (output rows h-2 .. h). kChunks = 16-byte channel chunks per pixel,
-// kPlaneBytes = the distance between chunk planes of the halo. The
-// accumulators start at zero (cleared by the epilogue).
-template <int kChunks, uint32_t kPlaneBytes>
-__device__ __forceinline__ void issue_tile_mmas(uint32_t hbase, uint32_t wbase, uint32_t dtmem) {
-  constexpr int kN = 96;
-  constexpr uint32_t idesc = make_idesc(kTileM, kN);
-  // A: LBO = the distance from an even chunk's core matrix to the odd one's;
-  // B: chunk c + 1 of a weight row sits kN * 16 bytes after chunk c
-  const uint32_t a_lo = desc_lo(hbase, kPlaneBytes), b_lo = desc_lo(wbase, kN * 16);
-  constexpr uint32_t hi = desc_hi(128u);
-#pragma unroll
-  for (int h = 0; h < kRows + 2; ++h) {
-#pragma unroll
-    for (int dx = 0; dx < 3; ++dx) {
-#pragma unroll
-      for (int ks = 0; ks < kChunks / 2; ++ks) {
-        const uint32_t a_off = (2u * ks) * kPlaneBytes + (uint32_t)(h * kHaloW + dx) * 16u;
-        const uint32_t b_off = (uint32_t)((dx * kChunks + 2 * ks) * kN) * 16u;
-        mma_bf16(dtmem + (uint32_t)(h * 32), desc_join(a_lo + (a_off >> 4), hi),
-                 desc_join(b_lo + (b_off >> 4), hi), idesc, 1u);
-      }
-    }
-  }
-}
-
 // zeroes 16 consecutive TMEM columns of this warp's 32 lanes
 __device__ __forceinline__ void tmem_zero16(uint32_t taddr) {
   asm volatile(
@@ -351,234 +278,6 @@ __device__ __forceinline__ void tmem_zero16(uint32_t taddr) {
       : "memory");
 }
 __device__ __forceinline__ void tmem_wait_st() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
-
-// ------------------------------------------------------- data gradients
-// in:  CIN / 8 chunk planes of BF16 ([P][8] each); a map with fewer planes (the
-//      BCE gradient's one) reads zeros for the others
-// wpk: packed weights, [dx][16-byte chunk][96: dy = 2, 1, 0][8]
-// out: BF16 planar [4][P][8] = acc where the layer's activation (mask16, same
-//      layout) is positive, else 0
-//
-// Three roles. The last warp loads each tile's halo (one TMA box per 16-byte
-// channel chunk, zeros outside the image) into a ring of RT_CONV_STAGES halo
-// buffers, as far ahead as the ring allows; the warp before it issues the
-// tile's MMAs into one of two TMEM accumulator sets as soon as its halo has
-// landed and the epilogue has drained that set; the epilogue warps
-// (RT_CONV_EPI_WG warpgroups; warp w reads TMEM lanes 32 (w % 4) .. +31) run
-// the epilogue of tile i while the tensor cores work on tile i+1 and the TMA
-// engine fetches the next tiles.
-//   halo_full[b]:  TMA bytes of halo buffer b arrived (expect_tx by the loader)
-//   halo_empty[b]: the MMAs that read buffer b completed (tcgen05.commit)
-//   acc_full[s]:   MMAs of accumulator set s done (tcgen05.commit)
-//   acc_empty[s]:  every epilogue thread has read and zeroed set s
-// Every wait is bounded; a wait that gives up sets the error word, and before
-// the CTA frees TMEM and exits, the TMA warp waits (bounded) for the last copy
-// into each buffer and the MMA warp for the MMAs it has issued.
-template <int CIN>
-struct ConvTmaLayout {
-  static constexpr int kChunks = CIN / 8;                                // 16-byte chunks per pixel
-  static constexpr int kOutW = kHaloW - 2;                               // output pixels per row
-  static constexpr uint32_t kPlane = (uint32_t)(kRows + 2) * kHaloW * 16u;   // one TMA box
-  static constexpr uint32_t kHalo = kChunks * kPlane;
-  static constexpr uint32_t kW = 9u * 32 * CIN * 2;
-  static constexpr uint32_t kSet = (kRows + 4) * 32;                     // rows -2 .. R+1
-  static constexpr uint32_t kTmemCols = 512;
-  static constexpr uint32_t kFit = (kSmemBudget - kW - 1024u) / kHalo;   // halo buffers that fit
-  static constexpr int kSt = kFit < 2u ? 2 : (kFit > (uint32_t)kMaxStages ? kMaxStages : (int)kFit);
-  static constexpr size_t kSmem = kSt * (size_t)kHalo + kW + 20 * 8 + 16;
-  static_assert(2 * kSet <= kTmemCols, "two accumulator sets must fit in TMEM");
-};
-
-template <int CIN>
-__global__ void __launch_bounds__(kConvTmaThreads, 1)
-    k_conv_tma(const __grid_constant__ CUtensorMap tmap, const void* __restrict__ wpk,
-               const __nv_bfloat16* __restrict__ mask16, __nv_bfloat16* __restrict__ out, uint32_t W,
-               uint32_t H, uint32_t* err) {
-  after_previous();
-  using Lt = ConvTmaLayout<CIN>;
-  static_assert(CIN % 16 == 0, "shape");
-  extern __shared__ __align__(1024) unsigned char smem[];
-  unsigned char* halo0 = smem;
-  unsigned char* wsm = smem + Lt::kSt * Lt::kHalo;
-  uint64_t* bars = reinterpret_cast<uint64_t*>(wsm + Lt::kW);
-  uint64_t* halo_full = bars;        // [kSt]
-  uint64_t* halo_empty = bars + 8;   // [kSt]
-  uint64_t* acc_full = bars + 16;    // [2]
-  uint64_t* acc_empty = bars + 18;   // [2]
-  uint32_t* tslot = reinterpret_cast<uint32_t*>(bars + 20);
-
-  const int tid = threadIdx.x, lane = tid & 31;
-  const int warp = __shfl_sync(0xFFFFFFFFu, tid >> 5, 0);   // known to be uniform
-  const uint32_t tiles_x = (W + Lt::kOutW - 1) / Lt::kOutW;
-  const uint32_t n_tiles = tiles_x * ((H + kRows - 1) / kRows);
-  {
-    const uint4* src = reinterpret_cast<const uint4*>(wpk);
-    uint4* dst = reinterpret_cast<uint4*>(wsm);
-    for (uint32_t i = tid; i < Lt::kW / 16u; i += blockDim.x) dst[i] = src[i];
-  }
-  if (tid == 0) {
-    for (int b = 0; b < Lt::kSt; ++b) {
-      mbar_init(halo_full + b, 1);
-      mbar_init(halo_empty + b, 1);
-    }
-    for (int b = 0; b < 2; ++b) {
-      mbar_init(acc_full + b, 1);
-      mbar_init(acc_empty + b, 32 * kEpiWarps);
-    }
-    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-    asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&tmap)) : "memory");
-  }
-  if (warp == 0) tmem_alloc(tslot, Lt::kTmemCols);
-  fence_async_smem();
-  fence_before();
-  __syncthreads();
-  fence_after();
-  const uint32_t tmem = __shfl_sync(0xFFFFFFFFu, *tslot, 0);
-  // the MMAs only accumulate: clear both accumulator sets once (warp w % 4
-  // may address TMEM lanes 32 (w % 4) .. +31)
-  if (warp < 4) {
-    for (uint32_t c = 0; c < Lt::kTmemCols; c += 16) tmem_zero16(tmem + ((uint32_t)(warp * 32) << 16) + c);
-    tmem_wait_st();
-  }
-  fence_before();
-  __syncthreads();
-  fence_after();
-
-  const uint32_t my_tiles = blockIdx.x < n_tiles ? (n_tiles - 1 - blockIdx.x) / gridDim.x + 1 : 0;
-  if (warp == kEpiWarps) {
-    // ---- MMA issue: tile it of this CTA's sequence reads halo buffer it % kSt.
-    // The whole warp walks the loop and one elected lane issues, so that the
-    // compiler keeps the descriptors in uniform registers (in a loop of one
-    // lane every MMA paid for moving them there).
-    const uint32_t wbase = smem_u32(wsm);
-    uint32_t n_mma = 0;
-    bool ok = true;
-    for (uint32_t it = 0; it < my_tiles; ++it) {
-      const uint32_t b = it % Lt::kSt, sa = it & 1u;
-      ok = mbar_wait(halo_full + b, (it / Lt::kSt) & 1u) &&
-           (it < 2 || mbar_wait(acc_empty + sa, ((it >> 1) - 1) & 1u));
-      ok = __all_sync(0xFFFFFFFFu, ok);
-      if (!ok) break;
-      fence_after();
-      if (elect_one()) {
-        issue_tile_mmas<Lt::kChunks, Lt::kPlane>(smem_u32(halo0) + b * Lt::kHalo, wbase, tmem + sa * Lt::kSet);
-        mma_commit(halo_empty + b);   // the buffer may be reloaded once these MMAs completed
-        mma_commit(acc_full + sa);
-      }
-      __syncwarp();
-      n_mma = it + 1;
-    }
-    if (!ok && lane == 0) atomicOr(err, ERR_ITER);
-    // drain: the MMAs issued here complete (and signal) before TMEM is freed
-    for (uint32_t it = n_mma > 2 ? n_mma - 2 : 0; it < n_mma; ++it)
-      mbar_wait(acc_full + (it & 1u), (it >> 1) & 1u);
-    for (uint32_t it = n_mma > (uint32_t)Lt::kSt ? n_mma - Lt::kSt : 0; it < n_mma; ++it)
-      mbar_wait(halo_empty + it % Lt::kSt, (it / Lt::kSt) & 1u);
-  } else if (warp == kEpiWarps + 1) {
-    // ---- TMA loads: tile j into buffer j % kSt once the MMAs of tile
-    // j - kSt (the buffer's previous tile) completed
-    if (lane == 0) {
-      bool ok = true;
-      uint32_t n_loaded = 0;
-      for (uint32_t j = 0; j < my_tiles; ++j) {
-        const int b = (int)(j % Lt::kSt);
-        if (j >= (uint32_t)Lt::kSt && !mbar_wait(halo_empty + b, ((j / Lt::kSt) - 1) & 1u)) { ok = false; break; }
-        const uint32_t tile = blockIdx.x + j * gridDim.x;
-        const int ty = (int)(tile / tiles_x);
-        const int y = ty * kRows, x0 = (int)(tile - (uint32_t)ty * tiles_x) * Lt::kOutW;
-        mbar_arrive_expect_tx(halo_full + b, (uint32_t)Lt::kChunks * Lt::kPlane);
-#pragma unroll
-        for (int c = 0; c < Lt::kChunks; ++c)   // tensor {8-byte halves of pixels (2 W), H, chunks}
-          tma_load_3d(halo0 + (size_t)b * Lt::kHalo + (size_t)c * Lt::kPlane, &tmap, 2 * (x0 - 1), y - 1, c,
-                      halo_full + b);
-        n_loaded = j + 1;
-      }
-      if (!ok) atomicOr(err, ERR_ITER);
-      // drain: the last copy into each buffer has landed before the CTA exits
-      for (uint32_t j = n_loaded > (uint32_t)Lt::kSt ? n_loaded - Lt::kSt : 0; j < n_loaded; ++j)
-        mbar_wait(halo_full + (j % Lt::kSt), (j / Lt::kSt) & 1u);
-    }
-    __syncwarp();
-  } else {
-    // Each epilogue warp first copies its rows of the accumulator set into
-    // registers, zeroes them (and group 0 the rows outside the tile) and hands
-    // the set back, so the next tile's MMAs start while it converts and
-    // stores: the tensor core then waits only for the TMEM reads, not for the
-    // whole epilogue.
-    constexpr int kMine = kRows / RT_CONV_EPI_WG;   // rows per epilogue warp
-    static_assert(kRows % RT_CONV_EPI_WG == 0, "rows per tile must split evenly over the epilogue groups");
-    const int quarter = warp & 3, group = warp >> 2;   // TMEM lanes 32*quarter .. +31
-    const size_t P = (size_t)W * H;                    // pixels of a channel plane
-    uint32_t it = 0;
-    for (uint32_t tile = blockIdx.x; tile < n_tiles; tile += gridDim.x, ++it) {
-      const int s = (int)(it & 1u);
-      // warp-uniform outcome: tcgen05.ld below is a warp-collective instruction
-      if (!__all_sync(0xFFFFFFFFu, mbar_wait(acc_full + s, (it >> 1) & 1u))) {
-        if (lane == 0) atomicOr(err, ERR_ITER);
-        break;
-      }
-      fence_after();
-      // output row ry's sums sit in columns (ry + 2) * 32 of the set
-      const uint32_t set_addr = tmem + ((uint32_t)(quarter * 32) << 16) + (uint32_t)s * Lt::kSet;
-      uint32_t r[kMine][2][16];
-#pragma unroll
-      for (int k = 0; k < kMine; ++k)
-#pragma unroll
-        for (int half = 0; half < 2; ++half)
-          tmem_ld16_nowait(set_addr + (uint32_t)((group + k * RT_CONV_EPI_WG + 2) * 32 + half * 16), r[k][half]);
-      tmem_wait_ld();
-#pragma unroll
-      for (int k = 0; k < kMine; ++k)
-#pragma unroll
-        for (int half = 0; half < 2; ++half)
-          tmem_zero16(set_addr + (uint32_t)((group + k * RT_CONV_EPI_WG + 2) * 32 + half * 16));
-      if (group == 0) {   // rows -2, -1, R, R+1
-#pragma unroll
-        for (int c = 0; c < 64; c += 16) {
-          tmem_zero16(set_addr + (uint32_t)c);
-          tmem_zero16(set_addr + (uint32_t)((kRows + 2) * 32 + c));
-        }
-      }
-      tmem_wait_st();
-      fence_before();
-      mbar_arrive(acc_empty + s);
-
-      const int ty = (int)(tile / tiles_x);
-      const int y = ty * kRows;
-      const int x0 = (int)(tile - (uint32_t)ty * tiles_x) * Lt::kOutW;
-      const int x = x0 + quarter * 32 + lane;
-      const bool lane_ok = quarter * 32 + lane < Lt::kOutW;
-#pragma unroll
-      for (int k = 0; k < kMine; ++k) {
-        const int yy = y + group + k * RT_CONV_EPI_WG;
-        if (!(lane_ok && x < (int)W && yy < (int)H)) continue;
-        const size_t p = (size_t)yy * W + x;
-#pragma unroll
-        for (int half = 0; half < 2; ++half) {
-          // channels 16 half + 0..7 and + 8..15 sit in planes 2 half, 2 half + 1
-          const uint4 ma = *reinterpret_cast<const uint4*>(mask16 + ((2 * half) * P + p) * 8);
-          const uint4 mb = *reinterpret_cast<const uint4*>(mask16 + ((2 * half + 1) * P + p) * 8);
-          const uint32_t mw[8] = {ma.x, ma.y, ma.z, ma.w, mb.x, mb.y, mb.z, mb.w};
-          uint32_t packed[8];
-#pragma unroll
-          for (int i = 0; i < 8; ++i) {
-            const __nv_bfloat162 mm = *reinterpret_cast<const __nv_bfloat162*>(&mw[i]);
-            packed[i] = pack_bf16(__bfloat162float(mm.x) > 0.f ? __uint_as_float(r[k][half][2 * i]) : 0.f,
-                                  __bfloat162float(mm.y) > 0.f ? __uint_as_float(r[k][half][2 * i + 1]) : 0.f);
-          }
-          *reinterpret_cast<uint4*>(out + ((2 * half) * P + p) * 8) =
-              make_uint4(packed[0], packed[1], packed[2], packed[3]);
-          *reinterpret_cast<uint4*>(out + ((2 * half + 1) * P + p) * 8) =
-              make_uint4(packed[4], packed[5], packed[6], packed[7]);
-        }
-      }
-    }
-  }
-  fence_before();
-  __syncthreads();
-  fence_after();
-  if (warp == 0) tmem_dealloc(tmem, Lt::kTmemCols);
-}
 
 // ------------------------------------------------------------ fused forward
 // The whole network in one kernel: a strip of 122 output pixels streams down
@@ -629,7 +328,6 @@ __global__ void __launch_bounds__(kConvTmaThreads, 1)
 //                   refilled, and the accumulators are up to date
 //   acc_empty[k]    layer k's epilogue has read and zeroed its slot (k < 3)
 //   acc4_empty[b]   layer 4's epilogue has read TMEM buffer b
-// Every wait is bounded, as in k_conv_tma.
 constexpr int kFuW = 122;                     // output pixels of a strip
 constexpr int kFuPx = 130;                    // pixels of a row buffer
 constexpr uint32_t kFuPitch = kFuPx * 16u;    // one chunk of a row buffer
@@ -656,6 +354,7 @@ struct FusedArgs {
   const float* inv[4];           // E4M3 inputs: inverse scale per output channel (null: 1)
   float out_scale[4];            // E4M3 outputs (1 otherwise)
   __nv_bfloat16* act[3];         // hidden activations to keep, BF16 planar [4][P][8] (null: none)
+  __nv_bfloat16* dz[3];          // (data gradients) of layers 3, 2, 1, BF16 planar
   float* prob;                   // output (null: none)
   // training: labels in, the BCE's gradient out and the loss' partial sums,
   // one per warp of layer 4's epilogue (see "BCE and d(logit)")
@@ -668,13 +367,18 @@ struct FusedArgs {
 
 // a unit of work: `rows` output rows (fewer at the bottom) of one strip
 struct FusedItem {
-  int img, x0, y0, rows;         // x0: image column of layer 1's lane 0
+  int img, x0, y0, rows;         // x0: image column of the first layer's lane 0
 };
+// LAYERS convolutions in a row: every one but the last loses a pixel at either
+// end of the strip
+template <int LAYERS>
+__host__ __device__ constexpr int strip_width() { return 128 - 2 * (LAYERS - 1); }
+template <int LAYERS>
 __device__ __forceinline__ FusedItem fused_item(const FusedArgs& a, uint32_t item) {
   const uint32_t strip = item % a.strips, q = item / a.strips, seg = q % a.segs;
   FusedItem it;
   it.img = (int)(q / a.segs);
-  it.x0 = (int)strip * kFuW - 3;
+  it.x0 = (int)strip * strip_width<LAYERS>() - (LAYERS - 1);
   it.y0 = (int)(seg * a.rows);
   it.rows = (int)min(a.rows, a.H - seg * a.rows);
   return it;
@@ -708,6 +412,7 @@ struct Ring {
 
 // The feature rows of a CTA's items in order: one TMA box per row into the
 // ring, zeros outside the image.
+template <int LAYERS>
 struct FeatureLoader {
   uint32_t item, n_loaded;
   int i;
@@ -715,14 +420,14 @@ struct FeatureLoader {
   __device__ __forceinline__ void load(const FusedArgs& a, const CUtensorMap* map, unsigned char* smem,
                                        uint32_t row_bytes, uint64_t* full, uint32_t n_items) {
     if (item >= n_items) return;
-    if (i == 0) it = fused_item(a, item);
+    if (i == 0) it = fused_item<LAYERS>(a, item);
     const uint32_t d = n_loaded % kFuF;
     if (elect_one()) {
       mbar_arrive_expect_tx(full + d, 2 * kFuPitch);
-      tma_load_5d(smem + d * row_bytes, map, 0, it.x0 - 1, 0, it.y0 - 4 + i, it.img, full + d);
+      tma_load_5d(smem + d * row_bytes, map, 0, it.x0 - 1, 0, it.y0 - LAYERS + i, it.img, full + d);
     }
     ++n_loaded;
-    if (++i == it.rows + 8) { i = 0; item += gridDim.x; }
+    if (++i == it.rows + 2 * LAYERS) { i = 0; item += gridDim.x; }
   }
 };
 
@@ -731,7 +436,7 @@ struct FeatureLoader {
 // also loads the feature rows: when the epilogue has read row r - 1's sums,
 // that row's MMAs are done and its slot takes row r - 1 + kFuF.
 // KIND: 0 layer 1, 1 layers 2 and 3 (K = 1, 2), 2 layer 4.
-template <int KIND, bool FP8>
+template <int KIND, bool FP8, int LAYERS>
 __device__ __forceinline__ bool fused_mmas(const int K, const FusedArgs& a, const CUtensorMap* map,
                                            unsigned char* smem, uint64_t* full, uint64_t* done,
                                            uint64_t* empty, uint32_t tmem) {
@@ -747,11 +452,11 @@ __device__ __forceinline__ bool fused_mmas(const int K, const FusedArgs& a, cons
   Ring ring;
   uint32_t row3 = 0, n_row = 0;
   bool ok = true;
-  FeatureLoader ld = {blockIdx.x, 0u, 0, {}};
+  FeatureLoader<LAYERS> ld = {blockIdx.x, 0u, 0, {}};
   if (KIND == 0)
     for (int i = 0; i < kFuF - 1; ++i) ld.load(a, map, smem, Lt::kRowF, full, n_items);
   for (uint32_t item = blockIdx.x; ok && item < n_items; item += gridDim.x) {
-    const int n = fused_item(a, item).rows + 8 - 2 * K;
+    const int n = fused_item<LAYERS>(a, item).rows + 2 * (LAYERS - K);
     for (int i = 0; i < n; ++i) {
       if (KIND < 2)
         ok = n_row == 0 ? mbar_wait(full_k + ring.slot, ring.par)
@@ -829,7 +534,7 @@ __device__ __forceinline__ bool fused_epilogue(const int KR, const FusedArgs& a,
   bool out_wrapped = false;
   uint32_t fin = 1;                   // slot of the finished row: (row - 2) % 3
   for (uint32_t item = blockIdx.x; item < n_items; item += gridDim.x) {
-    const FusedItem it = fused_item(a, item);
+    const FusedItem it = fused_item<4>(a, item);
     const int n = it.rows + 8 - 2 * K;
     const int x = it.x0 + K + m;
     const bool col_in = x >= 0 && x < (int)a.W;
@@ -1001,9 +706,9 @@ __global__ void __launch_bounds__(kFuThreads, 1)
   if (warp >= 16) {
     // ---- MMA issue, one thread per layer
     asm volatile("setmaxnreg.dec.sync.aligned.u32 40;");
-    const bool ok = warp == 16  ? fused_mmas<0, FP8>(0, a, &tmap, smem, full, done, acc_empty, tmem)
-                    : warp < 19 ? fused_mmas<1, FP8>(warp - 16, a, &tmap, smem, full, done, acc_empty, tmem)
-                                : fused_mmas<2, FP8>(3, a, &tmap, smem, full, done, acc4_empty, tmem);
+    const bool ok = warp == 16  ? fused_mmas<0, FP8, 4>(0, a, &tmap, smem, full, done, acc_empty, tmem)
+                    : warp < 19 ? fused_mmas<1, FP8, 4>(warp - 16, a, &tmap, smem, full, done, acc_empty, tmem)
+                                : fused_mmas<2, FP8, 4>(3, a, &tmap, smem, full, done, acc4_empty, tmem);
     if (!ok && lane == 0) atomicOr(a.err, ERR_ITER);
   } else if (warp < 12) {
     asm volatile("setmaxnreg.inc.sync.aligned.u32 120;");
@@ -1027,7 +732,7 @@ __global__ void __launch_bounds__(kFuThreads, 1)
     float s1[3] = {0.f, 0.f, 0.f}, s2[3] = {0.f, 0.f, 0.f};      // rows with one and with two taps added
     bool ok = true;
     for (uint32_t item = blockIdx.x; ok && item < n_items; item += gridDim.x) {
-      const FusedItem it = fused_item(a, item);
+      const FusedItem it = fused_item<4>(a, item);
       const int x = it.x0 + 2 + m;
       for (int i = 0; i < it.rows + 2; ++i, ++n_row) {
         if (!__all_sync(0xFFFFFFFFu, mbar_wait(done + 3 * kFuF + in.slot, in.par))) { ok = false; break; }
@@ -1076,9 +781,163 @@ __global__ void __launch_bounds__(kFuThreads, 1)
   if (warp == 0) tmem_dealloc(tmem, 512);
 }
 
+// ------------------------------------------------------- data gradients
+// The three data-gradient convolutions (weights flipped, channels swapped, each
+// followed by the ReLU mask of the layer's activations) in one kernel, streamed
+// like the forward pass: BCE gradient in, the gradients of layers 3, 2 and 1
+// stay on the SM on their way to the next one and go to memory once, for the
+// weight gradients. Same MMAs in the same order as one launch per layer: same
+// bits. A strip is 124 pixels wide. Bound by memory: 64 bytes of mask and 64 of
+// gradient per pixel and layer; the mask of a row is loaded before the wait for
+// its sums. Measured: 960x540 three
+// launches 21 + 26 + 26 us -> 54; training step 180 -> 169 us, 251x143 49.3 -> 44.1.
+constexpr int kBwThreads = 32 * (12 + 4);
+
+// Epilogue of gradient K (one warpgroup, lane = pixel)
+__device__ __forceinline__ bool bwd_epilogue(const int K, const FusedArgs& a, unsigned char* smem, uint64_t* full,
+                                             uint64_t* done, uint64_t* acc_empty, uint32_t tmem) {
+  using Lt = FusedLayout<false>;
+  constexpr int kLayers = 3;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int quarter = warp & 3, m = quarter * 32 + lane;
+  const uint32_t slots = tmem + ((uint32_t)(quarter * 32) << 16) + 96u * K;
+  unsigned char* ring = smem + Lt::kOffA + (uint32_t)K * kFuD * Lt::kRowA + (uint32_t)m * 16u;
+  const uint32_t n_items = a.strips * a.segs;
+  const uint32_t depth = K == 0 ? kFuF : kFuD;
+  const bool to_next = K + 1 < kLayers;
+  uint64_t* full_n = full + (K + 1) * kFuF;
+  uint64_t* done_k = done + K * kFuF;
+  uint64_t* done_n = done + (K + 1) * kFuF;
+  const uint4* const mask = reinterpret_cast<const uint4*>(a.act[2 - K]);
+  uint4* const out = reinterpret_cast<uint4*>(a.dz[K]);
+  const size_t P = (size_t)a.W * a.H;
+  Ring in, next;
+  bool wrapped = false;
+  uint32_t fin = 1;
+  for (uint32_t item = blockIdx.x; item < n_items; item += gridDim.x) {
+    const FusedItem it = fused_item<kLayers>(a, item);
+    const int n = it.rows + 2 * (kLayers - K);
+    const int x = it.x0 + K + m;
+    const bool col_in = x >= 0 && x < (int)a.W, col_own = m + K - 2 >= 0 && m + K - 2 < strip_width<kLayers>();
+    for (int i = 0; i < n; ++i) {
+      const int y = it.y0 - 2 + K + (i - 2);
+      const bool inside = i >= 2 && col_in && y >= 0 && y < (int)a.H;
+      const size_t p = inside ? (size_t)y * a.W + x : 0;
+      uint4 mk[4];
+#pragma unroll
+      for (int c = 0; c < 4; ++c) mk[c] = inside ? __ldg(mask + c * P + p) : make_uint4(0u, 0u, 0u, 0u);
+      const bool ok = i >= 2 && to_next && wrapped
+                          ? mbar_wait2<false>(done_n + next.slot, next.par ^ 1u, done_k + in.slot, in.par)
+                          : mbar_wait(done_k + in.slot, in.par);
+      if (!__all_sync(0xFFFFFFFFu, ok)) return false;
+      in.next(depth);
+      fence_after();
+      uint32_t r[2][16];
+      const uint32_t at = slots + fin * 32u;
+      tmem_ld16_nowait(at, r[0]);
+      tmem_ld16_nowait(at + 16u, r[1]);
+      tmem_wait_ld();
+      tmem_zero16(at);
+      tmem_zero16(at + 16u);
+      tmem_wait_st();
+      fence_before();
+      __syncwarp();
+      if (lane == 0) mbar_arrive(acc_empty + K);
+      fin = fin == 2u ? 0u : fin + 1u;
+      if (i < 2) continue;
+      uint4 v[4];                       // a zero mask (outside the image too) gives zeros
+#pragma unroll
+      for (int c = 0; c < 4; ++c) {
+        const uint32_t* q = &r[c >> 1][(c & 1) * 8];
+        v[c].x = masked_pair(mk[c].x, q[0], q[1]);
+        v[c].y = masked_pair(mk[c].y, q[2], q[3]);
+        v[c].z = masked_pair(mk[c].z, q[4], q[5]);
+        v[c].w = masked_pair(mk[c].w, q[6], q[7]);
+      }
+      if (to_next) {
+        unsigned char* dst = ring + next.slot * Lt::kRowA;
+#pragma unroll
+        for (int c = 0; c < 4; ++c) *reinterpret_cast<uint4*>(dst + (uint32_t)c * kFuPitch) = v[c];
+        fence_async_smem();
+        __syncwarp();
+        if (lane == 0) mbar_arrive(full_n + next.slot);
+        next.next(kFuD);
+        if (next.slot == 0) wrapped = true;
+      }
+      if (inside && col_own && y >= it.y0 && y < it.y0 + it.rows)
+#pragma unroll
+        for (int c = 0; c < 4; ++c) out[c * P + p] = v[c];
+    }
+  }
+  return true;
+}
+
+__global__ void __launch_bounds__(kBwThreads, 1)
+    k_bwd_fused(const __grid_constant__ CUtensorMap tmap, const __grid_constant__ FusedArgs a) {
+  after_previous();
+  using Lt = FusedLayout<false>;
+  extern __shared__ __align__(1024) unsigned char smem[];
+  uint64_t* bars = reinterpret_cast<uint64_t*>(smem + Lt::kOffB);
+  uint64_t* full = bars;                         // [4][kFuF]
+  uint64_t* done = bars + 4 * kFuF;              // [4][kFuF]
+  uint64_t* acc_empty = bars + 8 * kFuF;         // [3]
+  uint32_t* tslot = reinterpret_cast<uint32_t*>(acc_empty + 3);
+  const int tid = threadIdx.x, lane = tid & 31;
+  const int warp = __shfl_sync(0xFFFFFFFFu, tid >> 5, 0);   // known to be uniform
+#pragma unroll
+  for (int k = 0; k < 3; ++k) {
+    const uint32_t groups = 3u * (k == 0 ? 2u : 4u);
+    const uint4* src = static_cast<const uint4*>(a.w[k]);
+    uint4* dst = reinterpret_cast<uint4*>(smem + Lt::kOffW + (k > 0 ? Lt::kW1 : 0u) + (k > 1 ? Lt::kWk : 0u));
+    for (uint32_t i = tid; i < groups * 160u; i += kBwThreads) {
+      const uint32_t g = i / 160u, r = i - g * 160u;
+      dst[i] = src[g * 96u + (r >= 96u ? r - 96u : r)];
+    }
+  }
+  // the two pixels past every gradient row feed unused lanes only: finite
+  for (uint32_t i = tid; i < 2u * kFuD * Lt::kRowA / 16u; i += kBwThreads)
+    reinterpret_cast<uint4*>(smem + Lt::kOffA)[i] = make_uint4(0u, 0u, 0u, 0u);
+  if (tid == 0) {
+    for (int k = 0; k < 3; ++k) {
+      for (int d = 0; d < kFuF; ++d) {
+        mbar_init(full + k * kFuF + d, k == 0 ? 1 : 4);
+        mbar_init(done + k * kFuF + d, 1);
+      }
+      mbar_init(acc_empty + k, 4);
+    }
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&tmap)) : "memory");
+  }
+  if (warp == 0) tmem_alloc(tslot, 512);
+  fence_async_smem();
+  fence_before();
+  __syncthreads();
+  fence_after();
+  const uint32_t tmem = __shfl_sync(0xFFFFFFFFu, *tslot, 0);
+  if (warp < 4) {
+    for (uint32_t c = 0; c < 288u; c += 16) tmem_zero16(tmem + ((uint32_t)(warp * 32) << 16) + c);
+    tmem_wait_st();
+  }
+  fence_before();
+  __syncthreads();
+  fence_after();
+  bool ok = true;
+  if (warp < 12)
+    ok = bwd_epilogue(warp >> 2, a, smem, full, done, acc_empty, tmem);
+  else if (warp == 12)
+    ok = fused_mmas<0, false, 3>(0, a, &tmap, smem, full, done, acc_empty, tmem);
+  else if (warp < 15)
+    ok = fused_mmas<1, false, 3>(warp - 12, a, &tmap, smem, full, done, acc_empty, tmem);
+  if (!ok && lane == 0) atomicOr(a.err, ERR_ITER);
+  fence_before();
+  __syncthreads();
+  fence_after();
+  if (warp == 0) tmem_dealloc(tmem, 512);
+}
+
 // ------------------------------------------------ weight packing (FP32 -> BF16)
 // Canonical parameter layout of a layer: W[Cout][Cin][3][3] then b[Cout].
-// Packed (k_conv_tma's stacked taps): element i of a conv with output
+// Packed (stacked taps): element i of a conv with output
 // channels cout_p and input channels cin_p, chunks of `per` elements, is
 // [dx][ci / per][j * cout_p + co][ci % per] with tap (dy = 2 - j, dx).
 struct StackedIndex {
@@ -1267,8 +1126,9 @@ struct WgradArgs {
 
 // One CTA's tiles of one layer. Barriers: full[b] TMA bytes of stage b;
 // empty[b] its MMAs (commit) and the bias warps' sums are done;
-// acc_full[s] / acc_empty[s] as in k_conv_tma. A partial row is kOuts + kCo
-// floats, [tap][co][ci] then [co].
+// acc_full[s]: the sums are complete (commit); acc_empty[s]: the epilogue has
+// read and zeroed them. A partial row is kOuts + kCo floats, [tap][co][ci] then
+// [co].
 template <int AC, int ZC, int CHAIN>
 __device__ __forceinline__ void wgrad_body(const WgradArgs& args, const int layer, unsigned char* smem) {
   using Lt = WgradLayout<AC, ZC>;
@@ -1641,23 +1501,6 @@ EncodeTiledFn encode_tiled() {
   return fn;
 }
 
-// Tensor map of `chunks` BF16 chunk planes for the halo boxes of k_conv_tma:
-// 8-byte elements {2 W, H, chunks}, one box {256 (128 pixels), R+2, 1} per
-// chunk. A map may hold fewer chunks than the kernel's CIN: the boxes of the
-// others lie outside the tensor and read zeros.
-cudaError_t make_halo_map(CUtensorMap* map, const void* in, uint32_t W, uint32_t H, uint32_t chunks) {
-  const EncodeTiledFn fn = encode_tiled();
-  if (!fn) return cudaErrorNotSupported;
-  if (reinterpret_cast<uintptr_t>(in) & 15u) return cudaErrorInvalidValue;
-  const cuuint32_t estr[3] = {1, 1, 1};
-  const cuuint64_t d[3] = {2ull * W, H, chunks}, st[2] = {16ull * W, 16ull * W * H};
-  const cuuint32_t bx[3] = {2u * kHaloW, (cuuint32_t)(kRows + 2), 1};
-  const CUresult r = fn(map, CU_TENSOR_MAP_DATA_TYPE_UINT64, 3, const_cast<void*>(in), d, st, bx, estr,
-                        CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE,
-                        CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
-  return r == CUDA_SUCCESS ? cudaSuccess : cudaErrorInvalidValue;
-}
-
 // One map of W x H pixels for k_wgrad: `chunks` 16-byte channel chunks per
 // pixel, interleaved ([P][16], 2 chunks) as {8 channels, W, chunks, H} or
 // planar ([chunks][P][8]) as 8-byte elements {2 W, chunks, H}; the box is
@@ -1721,29 +1564,6 @@ void wgrad_shares(uint32_t W, uint32_t H, WgradShare share[4], uint64_t* part_fl
   *part_floats = at;
 }
 
-// data gradient of a layer: `in` holds `chunks` planes (CIN / 8 at most)
-template <int CIN>
-cudaError_t launch_conv(const void* in, uint32_t chunks, const void* wpk, const __nv_bfloat16* mask16,
-                        __nv_bfloat16* out, uint32_t W, uint32_t H, uint32_t* err, cudaStream_t st) {
-  using Lt = ConvTmaLayout<CIN>;
-  const uint32_t tiles = ((W + Lt::kOutW - 1) / Lt::kOutW) * ((H + kRows - 1) / kRows);
-  // a CTA that takes all 512 TMEM columns must be alone on its SM: ask for
-  // more than half of the SM's shared memory so a second one cannot be placed
-  constexpr size_t smem = Lt::kSmem < 116u * 1024u ? 116u * 1024u : Lt::kSmem;
-  static bool configured = false;
-  if (!configured) {
-    const cudaError_t e = cudaFuncSetAttribute(k_conv_tma<CIN>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                               (int)smem);
-    if (e != cudaSuccess) return e;
-    configured = true;
-  }
-  CUtensorMap map;
-  const cudaError_t e = make_halo_map(&map, in, W, H, chunks);
-  if (e != cudaSuccess) return e;
-  const uint32_t grid = std::min<uint32_t>((uint32_t)num_sms(), tiles);
-  launch_after(k_conv_tma<CIN>, grid, kConvTmaThreads, smem, st, map, wpk, mask16, out, W, H, err);
-  return cudaGetLastError();
-}
 }  // namespace
 
 // parameter offsets (canonical layout W[Cout][Cin][3][3], b[Cout] per layer)
@@ -1772,19 +1592,41 @@ cudaError_t pack_weights(const float* params, __nv_bfloat16* const wf[4], __nv_b
 }
 
 namespace {
-// feature maps [n_img][H][W][16] BF16 as {8 channels, W, chunks, H, images}:
-// one box is one row of a strip, in shared memory [chunk][130 pixels]
-cudaError_t make_feature_map(CUtensorMap* map, const void* in, uint32_t W, uint32_t H, uint32_t n_img) {
+// feature maps [n_img][H][W][8 chunks] BF16, chunks = 2, or the BCE gradient with
+// one (the second is zero fill), as {8 channels, W, chunks, H, images}: one box is
+// one row of a strip, in shared memory [chunk][130 pixels]
+cudaError_t make_feature_map(CUtensorMap* map, const void* in, uint32_t chunks, uint32_t W, uint32_t H,
+                             uint32_t n_img) {
   const EncodeTiledFn fn = encode_tiled();
   if (!fn) return cudaErrorNotSupported;
   if (reinterpret_cast<uintptr_t>(in) & 15u) return cudaErrorInvalidValue;
   const cuuint32_t estr[5] = {1, 1, 1, 1, 1};
-  const cuuint64_t d[5] = {8, W, 2, H, n_img}, st[4] = {32, 16, 32ull * W, 32ull * W * H};
+  const cuuint64_t px = 16ull * chunks;
+  const cuuint64_t d[5] = {8, W, chunks, H, n_img}, st[4] = {px, 16, px * W, px * W * H};
   const cuuint32_t bx[5] = {8, (cuuint32_t)kFuPx, 2, 1, 1};
   const CUresult r = fn(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 5, const_cast<void*>(in), d, st, bx, estr,
                         CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE,
                         CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
   return r == CUDA_SUCCESS ? cudaSuccess : cudaErrorInvalidValue;
+}
+
+// Segments per strip: a segment of R rows costs R + 2 LAYERS steps (the rows above
+// and below it that its first layers recompute), and the CTAs take the segments in
+// whole rounds, so the fewest steps over all rounds. Returns the grid.
+template <int LAYERS>
+int choose_segments(FusedArgs& a, uint32_t W, uint32_t H, uint32_t n_img) {
+  a.W = W; a.H = H; a.n_img = n_img;
+  a.strips = (W + strip_width<LAYERS>() - 1) / strip_width<LAYERS>();
+  uint64_t best = ~0ull;
+  const uint64_t strips = (uint64_t)a.strips * n_img, sms = (uint64_t)num_sms();
+  for (uint32_t rows = H;;) {
+    const uint32_t segs = (H + rows - 1) / rows;
+    const uint64_t cost = (strips * segs + sms - 1) / sms * (rows + 2u * LAYERS);
+    if (cost < best) { best = cost; a.segs = segs; a.rows = rows; }
+    if (rows == 1) break;
+    rows = std::min(rows - 1, (H + segs) / (segs + 1));   // one more segment, shorter by a row at least
+  }
+  return (int)std::min(strips * a.segs, sms);
 }
 
 template <bool FP8, bool STORE>
@@ -1802,27 +1644,37 @@ cudaError_t launch_fused(const __nv_bfloat16* feat16, FusedArgs& a, uint32_t W, 
     configured = true;
   }
   CUtensorMap map;
-  const cudaError_t e = make_feature_map(&map, feat16, W, H, n_img);
+  const cudaError_t e = make_feature_map(&map, feat16, 2, W, H, n_img);
   if (e != cudaSuccess) return e;
-  // Segments per strip: a segment of R rows costs R + 8 steps (the rows above
-  // and below it that its first layers recompute), and the CTAs take the
-  // segments in whole rounds, so the fewest steps over all rounds.
-  a.W = W; a.H = H; a.n_img = n_img;
-  a.strips = (W + kFuW - 1) / kFuW;
-  uint64_t best = ~0ull;
-  const uint64_t strips = (uint64_t)a.strips * n_img, sms = (uint64_t)num_sms();
-  for (uint32_t rows = H;;) {
-    const uint32_t segs = (H + rows - 1) / rows;
-    const uint64_t cost = (strips * segs + sms - 1) / sms * (rows + 8u);
-    if (cost < best) { best = cost; a.segs = segs; a.rows = rows; }
-    if (rows == 1) break;
-    rows = std::min(rows - 1, (H + segs) / (segs + 1));   // one more segment, shorter by a row at least
-  }
-  const uint64_t items = strips * a.segs;
-  const int grid = (int)std::min(items, sms);
+  const int grid = choose_segments<4>(a, W, H, n_img);
   if (grid_out) *grid_out = grid;
   launch_after(k_net_fused<FP8, STORE>, grid, kFuThreads, smem, st, map, a);
   return cudaGetLastError();
+}
+
+// gradients of layers 3, 2, 1 (dz[0..2]) from the BCE gradient g8
+cudaError_t launch_bwd(const void* g8, __nv_bfloat16* const wb[4], __nv_bfloat16* const act[3],
+                       __nv_bfloat16* const dz[3], uint32_t W, uint32_t H, uint32_t* err, cudaStream_t st) {
+  constexpr uint32_t smem = FusedLayout<false>::kSmem;
+  static_assert(smem > 116u * 1024u, "a CTA takes all TMEM columns: one on an SM");
+  static bool configured = false;
+  if (!configured) {
+    const cudaError_t e = cudaFuncSetAttribute(k_bwd_fused, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e != cudaSuccess) return e;
+    configured = true;
+  }
+  CUtensorMap map;
+  const cudaError_t e = make_feature_map(&map, g8, 1, W, H, 1);
+  if (e != cudaSuccess) return e;
+  FusedArgs a = {};
+  for (int k = 0; k < 3; ++k) {
+    a.w[k] = wb[3 - k];
+    a.act[k] = act[k];
+    a.dz[k] = dz[k];
+  }
+  a.err = err;
+  const int grid = choose_segments<3>(a, W, H, 1);
+  return launch_after(k_bwd_fused, grid, kBwThreads, smem, st, map, a);
 }
 }  // namespace
 
@@ -1905,9 +1757,7 @@ cudaError_t train_step(const __nv_bfloat16* feat16, const float* label, const Tr
   f.err = err;
   int fwd_grid = 0;
   cudaError_t e = launch_fused<false, true>(feat16, f, W, H, 1, st, &fwd_grid);
-  if (e == cudaSuccess) e = launch_conv<16>(t.g8, 1, t.wb[3], t.act[2], t.dz[0], W, H, err, st);
-  if (e == cudaSuccess) e = launch_conv<32>(t.dz[0], 4, t.wb[2], t.act[1], t.dz[1], W, H, err, st);
-  if (e == cudaSuccess) e = launch_conv<32>(t.dz[1], 4, t.wb[1], t.act[0], t.dz[2], W, H, err, st);
+  if (e == cudaSuccess) e = launch_bwd(t.g8, t.wb, t.act, t.dz, W, H, err, st);
   if (e != cudaSuccess) return e;
 
   // weight gradients: layer l + 1 from its input and its data gradient

@@ -45,3 +45,10 @@ def test_weight_gradients_at_tile_edges(W, H):
             a, b = g[k:k + n], emu[k:k + n]
             assert np.linalg.norm(a - b) <= bound * np.linalg.norm(b) + 1e-12, (k, n)
             k += n
+
+
+@pytest.mark.parametrize("W,H", [(2, 1), (123, 2), (124, 1), (125, 3), (128, 6), (248, 7), (249, 2), (372, 29)])
+def test_data_gradients_at_strip_edges(W, H):
+    """The data gradients stream through strips of 124 pixels and segments of
+    rows; every layer's weight gradient but the last is a product of one."""
+    test_weight_gradients_at_tile_edges(W, H)
