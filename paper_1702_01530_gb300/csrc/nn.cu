@@ -220,11 +220,17 @@ __device__ __forceinline__ uint32_t pack_bf16(float a, float b) {
   return *reinterpret_cast<uint32_t*>(&h);
 }
 
-// BF16 of (a, b), each zero where its half of `mask` is not above zero
-__device__ __forceinline__ uint32_t masked_pair(uint32_t mask, uint32_t a, uint32_t b) {
+// A pixel's ReLU mask of 32 channels in one word: pair j of channels (2 j, 2 j + 1)
+// has bits j and 16 + j. Adds pair j of BF16 values.
+__device__ __forceinline__ uint32_t mask_bits(uint32_t word, uint32_t pair, int j) {
   const __nv_bfloat162 zero = __float2bfloat162_rn(0.f);
-  return pack_bf16(__uint_as_float(a), __uint_as_float(b)) &
-         __hgt2_mask(*reinterpret_cast<const __nv_bfloat162*>(&mask), zero);
+  return word | (__hgt2_mask(*reinterpret_cast<const __nv_bfloat162*>(&pair), zero) & (0x00010001u << j));
+}
+// BF16 of (a, b), each zero where its bit of pair j is not set
+__device__ __forceinline__ uint32_t masked_pair(uint32_t word, int j, uint32_t a, uint32_t b) {
+  uint32_t m;                          // bits 15 and 31 after the shift: signs of bytes 1 and 3, over their halves
+  asm("prmt.b32 %0, %1, 0, 0xBB99;" : "=r"(m) : "r"(word << (15 - j)));
+  return pack_bf16(__uint_as_float(a), __uint_as_float(b)) & m;
 }
 
 // (a0, a1) += (b0, b1) in one instruction, each sum rounded to nearest
@@ -354,6 +360,7 @@ struct FusedArgs {
   const float* inv[4];           // E4M3 inputs: inverse scale per output channel (null: 1)
   float out_scale[4];            // E4M3 outputs (1 otherwise)
   __nv_bfloat16* act[3];         // hidden activations to keep, BF16 planar [4][P][8] (null: none)
+  uint32_t* mask;                // training: ReLU masks of the hidden layers, [3][P] words
   __nv_bfloat16* dz[3];          // (data gradients) of layers 3, 2, 1, BF16 planar
   float* prob;                   // output (null: none)
   // training: labels in, the BCE's gradient out and the loss' partial sums,
@@ -608,6 +615,17 @@ __device__ __forceinline__ bool fused_epilogue(const int KR, const FusedArgs& a,
           const size_t P = (size_t)a.W * a.H * a.n_img, p = ((size_t)it.img * a.H + y) * a.W + x;
 #pragma unroll
           for (int c = 0; c < Lt::kCh; ++c) *reinterpret_cast<uint4*>(a.act[K] + ((size_t)c * P + p) * 8) = v[c];
+          if (a.mask) {
+            uint32_t word = 0u;
+#pragma unroll
+            for (int c = 0; c < Lt::kCh; ++c) {
+              word = mask_bits(word, v[c].x, 4 * c);
+              word = mask_bits(word, v[c].y, 4 * c + 1);
+              word = mask_bits(word, v[c].z, 4 * c + 2);
+              word = mask_bits(word, v[c].w, 4 * c + 3);
+            }
+            a.mask[K * P + p] = word;
+          }
         }
       }
     }
@@ -787,10 +805,11 @@ __global__ void __launch_bounds__(kFuThreads, 1)
 // like the forward pass: BCE gradient in, the gradients of layers 3, 2 and 1
 // stay on the SM on their way to the next one and go to memory once, for the
 // weight gradients. Same MMAs in the same order as one launch per layer: same
-// bits. A strip is 124 pixels wide. Bound by memory: 64 bytes of mask and 64 of
-// gradient per pixel and layer; the mask of a row is loaded before the wait for
-// its sums. Measured: 960x540 three
-// launches 21 + 26 + 26 us -> 54; training step 180 -> 169 us, 251x143 49.3 -> 44.1.
+// bits. A strip is 124 pixels wide. Bound by memory: 64 bytes of gradient per
+// pixel and layer, and 4 of mask (one bit a channel, written by the forward pass;
+// loaded before the wait for the row's sums). Measured at 960x540: three launches
+// 21 + 26 + 26 us; one with the activations themselves as masks (64 bytes) 54, with
+// bits 42. Training step 180 -> 169 -> 153 us, 251x143 49.3 -> 44.1 -> 43.5.
 constexpr int kBwThreads = 32 * (12 + 4);
 
 // Epilogue of gradient K (one warpgroup, lane = pixel)
@@ -808,9 +827,9 @@ __device__ __forceinline__ bool bwd_epilogue(const int K, const FusedArgs& a, un
   uint64_t* full_n = full + (K + 1) * kFuF;
   uint64_t* done_k = done + K * kFuF;
   uint64_t* done_n = done + (K + 1) * kFuF;
-  const uint4* const mask = reinterpret_cast<const uint4*>(a.act[2 - K]);
   uint4* const out = reinterpret_cast<uint4*>(a.dz[K]);
   const size_t P = (size_t)a.W * a.H;
+  const uint32_t* const mask = a.mask + (2 - K) * P;
   Ring in, next;
   bool wrapped = false;
   uint32_t fin = 1;
@@ -823,9 +842,7 @@ __device__ __forceinline__ bool bwd_epilogue(const int K, const FusedArgs& a, un
       const int y = it.y0 - 2 + K + (i - 2);
       const bool inside = i >= 2 && col_in && y >= 0 && y < (int)a.H;
       const size_t p = inside ? (size_t)y * a.W + x : 0;
-      uint4 mk[4];
-#pragma unroll
-      for (int c = 0; c < 4; ++c) mk[c] = inside ? __ldg(mask + c * P + p) : make_uint4(0u, 0u, 0u, 0u);
+      const uint32_t mk = inside ? __ldg(mask + p) : 0u;
       const bool ok = i >= 2 && to_next && wrapped
                           ? mbar_wait2<false>(done_n + next.slot, next.par ^ 1u, done_k + in.slot, in.par)
                           : mbar_wait(done_k + in.slot, in.par);
@@ -849,10 +866,10 @@ __device__ __forceinline__ bool bwd_epilogue(const int K, const FusedArgs& a, un
 #pragma unroll
       for (int c = 0; c < 4; ++c) {
         const uint32_t* q = &r[c >> 1][(c & 1) * 8];
-        v[c].x = masked_pair(mk[c].x, q[0], q[1]);
-        v[c].y = masked_pair(mk[c].y, q[2], q[3]);
-        v[c].z = masked_pair(mk[c].z, q[4], q[5]);
-        v[c].w = masked_pair(mk[c].w, q[6], q[7]);
+        v[c].x = masked_pair(mk, 4 * c + 0, q[0], q[1]);
+        v[c].y = masked_pair(mk, 4 * c + 1, q[2], q[3]);
+        v[c].z = masked_pair(mk, 4 * c + 2, q[4], q[5]);
+        v[c].w = masked_pair(mk, 4 * c + 3, q[6], q[7]);
       }
       if (to_next) {
         unsigned char* dst = ring + next.slot * Lt::kRowA;
@@ -1653,8 +1670,7 @@ cudaError_t launch_fused(const __nv_bfloat16* feat16, FusedArgs& a, uint32_t W, 
 }
 
 // gradients of layers 3, 2, 1 (dz[0..2]) from the BCE gradient g8
-cudaError_t launch_bwd(const void* g8, __nv_bfloat16* const wb[4], __nv_bfloat16* const act[3],
-                       __nv_bfloat16* const dz[3], uint32_t W, uint32_t H, uint32_t* err, cudaStream_t st) {
+cudaError_t launch_bwd(const void* g8, __nv_bfloat16* const wb[4], uint32_t* mask, __nv_bfloat16* const dz[3], uint32_t W, uint32_t H, uint32_t* err, cudaStream_t st) {
   constexpr uint32_t smem = FusedLayout<false>::kSmem;
   static_assert(smem > 116u * 1024u, "a CTA takes all TMEM columns: one on an SM");
   static bool configured = false;
@@ -1669,9 +1685,9 @@ cudaError_t launch_bwd(const void* g8, __nv_bfloat16* const wb[4], __nv_bfloat16
   FusedArgs a = {};
   for (int k = 0; k < 3; ++k) {
     a.w[k] = wb[3 - k];
-    a.act[k] = act[k];
     a.dz[k] = dz[k];
   }
+  a.mask = mask;
   a.err = err;
   const int grid = choose_segments<3>(a, W, H, 1);
   return launch_after(k_bwd_fused, grid, kBwThreads, smem, st, map, a);
@@ -1751,13 +1767,14 @@ cudaError_t train_step(const __nv_bfloat16* feat16, const float* label, const Tr
     f.out_scale[l] = 1.f;
   }
   for (int l = 0; l < 3; ++l) f.act[l] = t.act[l];
+  f.mask = t.mask;
   f.label = label;
   f.g8 = reinterpret_cast<uint4*>(t.g8);
   f.loss_part = t.loss_part;
   f.err = err;
   int fwd_grid = 0;
   cudaError_t e = launch_fused<false, true>(feat16, f, W, H, 1, st, &fwd_grid);
-  if (e == cudaSuccess) e = launch_bwd(t.g8, t.wb, t.act, t.dz, W, H, err, st);
+  if (e == cudaSuccess) e = launch_bwd(t.g8, t.wb, t.mask, t.dz, W, H, err, st);
   if (e != cudaSuccess) return e;
 
   // weight gradients: layer l + 1 from its input and its data gradient

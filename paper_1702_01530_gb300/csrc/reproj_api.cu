@@ -35,6 +35,7 @@ struct rt_net {
   __nv_bfloat16* act[3] = {};
   float* prob = nullptr;
   __nv_bfloat16* g8 = nullptr;  // BCE gradient, 8 channels
+  uint32_t* mask = nullptr;      // ReLU masks of the hidden layers
   __nv_bfloat16* dz[3] = {};
   float* loss_part = nullptr;   // partial sums of the loss
   uint64_t part_floats = 0;     // size of wpart
@@ -68,10 +69,10 @@ int net_buffers(rt_net* net, uint32_t W, uint32_t H) {
   const uint64_t P = (uint64_t)W * H, floats = rt::nn::wgrad_part_floats(W, H);
   if (net->tb && net->tcap >= P && net->part_floats >= floats) return RT_OK;
   const uint64_t cap = std::max(net->tcap, P), part = std::max(net->part_floats, floats);
-  const size_t b_act = a256(cap * 32 * 2), b_prob = a256(cap * 4), b_g8 = a256(cap * 8 * 2),
+  const size_t b_act = a256(cap * 32 * 2), b_prob = a256(cap * 4), b_g8 = a256(cap * 8 * 2), b_mask = a256(cap * 3 * 4),
                b_part = a256(part * 4), b_loss = a256((size_t)rt::nn::loss_parts() * 4);
   void* base = nullptr;
-  cudaError_t e = cudaMalloc(&base, 6 * b_act + b_prob + b_g8 + b_part + b_loss);
+  cudaError_t e = cudaMalloc(&base, 6 * b_act + b_prob + b_g8 + b_mask + b_part + b_loss);
   if (e != cudaSuccess) { cudaGetLastError(); return cuda_fail(e, "network activations"); }
   if (net->tb) cudaFree(net->tb);
   net->tb = base;
@@ -82,6 +83,7 @@ int net_buffers(rt_net* net, uint32_t W, uint32_t H) {
   net->prob = reinterpret_cast<float*>(p); p += b_prob;
   net->g8 = reinterpret_cast<__nv_bfloat16*>(p); p += b_g8;
   for (int i = 0; i < 3; ++i) { net->dz[i] = reinterpret_cast<__nv_bfloat16*>(p); p += b_act; }
+  net->mask = reinterpret_cast<uint32_t*>(p); p += b_mask;
   net->wpart = reinterpret_cast<float*>(p); p += b_part;
   net->loss_part = reinterpret_cast<float*>(p);
   return RT_OK;
@@ -421,6 +423,7 @@ int rt_net_train_step(rt_net* net, const uint16_t* d_feat16, const float* d_labe
   for (int l = 0; l < 4; ++l) { t.wf[l] = net->wf[l]; t.wb[l] = net->wb[l]; }
   for (int i = 0; i < 3; ++i) { t.act[i] = net->act[i]; t.dz[i] = net->dz[i]; }
   t.g8 = net->g8;
+  t.mask = net->mask;
   t.wpart = net->wpart;
   t.loss_part = net->loss_part;
   t.loss = net->loss;

@@ -270,6 +270,7 @@ struct TrainBuffers {
   __nv_bfloat16* act[3];             // hidden activations, planar
   __nv_bfloat16* dz[3];              // data gradients of layers 3, 2, 1, planar
   __nv_bfloat16* g8;                 // BCE gradient, 8 channels per pixel
+  uint32_t* mask;                    // ReLU masks of the hidden layers, a word per pixel each
   float* wpart;                      // wgrad_part_floats partial sums
   float* loss_part;                  // loss_parts partial sums of the loss
   float* loss;                       // sum of the pixels' losses
