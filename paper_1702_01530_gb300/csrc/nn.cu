@@ -652,7 +652,6 @@ __device__ __forceinline__ float bce_gradient(float p, float y, uint4& g8) {
 template <bool FP8, bool STORE>
 __global__ void __launch_bounds__(kFuThreads, 1)
     k_net_fused(const __grid_constant__ CUtensorMap tmap, const __grid_constant__ FusedArgs a) {
-  after_previous();
   using Lt = FusedLayout<FP8>;
   extern __shared__ __align__(1024) unsigned char smem[];
   uint64_t* bars = reinterpret_cast<uint64_t*>(smem + Lt::kOffB);
@@ -666,29 +665,6 @@ __global__ void __launch_bounds__(kFuThreads, 1)
   const int warp = __shfl_sync(0xFFFFFFFFu, tid >> 5, 0);   // known to be uniform
   const uint32_t n_items = a.strips * a.segs * a.n_img;
 
-  // weights: three stacked blocks per (dx, chunk) become five
-  uint32_t off_w[4] = {Lt::kOffW, Lt::kOffW + Lt::kW1, Lt::kOffW + Lt::kW1 + Lt::kWk,
-                       Lt::kOffW + Lt::kW1 + 2 * Lt::kWk};
-#pragma unroll
-  for (int k = 0; k < 3; ++k) {
-    const uint32_t groups = 3u * (k == 0 ? 2u : (uint32_t)Lt::kCh);
-    const uint4* src = static_cast<const uint4*>(a.w[k]);
-    uint4* dst = reinterpret_cast<uint4*>(smem + off_w[k]);
-    for (uint32_t i = tid; i < groups * 160u; i += kFuThreads) {
-      const uint32_t g = i / 160u, r = i - g * 160u;
-      dst[i] = src[g * 96u + (r >= 96u ? r - 96u : r)];
-    }
-  }
-  for (uint32_t i = tid; i < Lt::kW4 / 16u; i += kFuThreads)
-    reinterpret_cast<uint4*>(smem + off_w[3])[i] = static_cast<const uint4*>(a.w[3])[i];
-  float* cst = reinterpret_cast<float*>(smem + Lt::kOffC);
-  for (uint32_t i = tid; i < 4u * 32u; i += kFuThreads) {
-    const uint32_t k = i / 32u, c = i % 32u;
-    const bool real = k < 3u || c == 0u;
-    // powers of two: the folded form rounds like scaling the rounded sum
-    cst[i] = real ? (a.inv[k] ? a.inv[k][c] : 1.f) * a.out_scale[k] : 0.f;
-    cst[4 * 32 + i] = real ? a.bias[k][c] * a.out_scale[k] : 0.f;
-  }
   // the two pixels past every activation row feed unused lanes only: finite
   for (uint32_t i = tid; i < 3u * kFuD * Lt::kRowA / 16u; i += kFuThreads)
     reinterpret_cast<uint4*>(smem + Lt::kOffA)[i] = make_uint4(0u, 0u, 0u, 0u);
@@ -716,6 +692,32 @@ __global__ void __launch_bounds__(kFuThreads, 1)
     for (uint32_t c = 0; c < 288u; c += 16) tmem_zero16(tmem + ((uint32_t)(warp * 32) << 16) + c);
     tmem_wait_st();
   }
+  after_previous();              // the weights may come from the kernel before
+
+  // weights: three stacked blocks per (dx, chunk) become five
+  uint32_t off_w[4] = {Lt::kOffW, Lt::kOffW + Lt::kW1, Lt::kOffW + Lt::kW1 + Lt::kWk,
+                       Lt::kOffW + Lt::kW1 + 2 * Lt::kWk};
+#pragma unroll
+  for (int k = 0; k < 3; ++k) {
+    const uint32_t groups = 3u * (k == 0 ? 2u : (uint32_t)Lt::kCh);
+    const uint4* src = static_cast<const uint4*>(a.w[k]);
+    uint4* dst = reinterpret_cast<uint4*>(smem + off_w[k]);
+    for (uint32_t i = tid; i < groups * 160u; i += kFuThreads) {
+      const uint32_t g = i / 160u, r = i - g * 160u;
+      dst[i] = src[g * 96u + (r >= 96u ? r - 96u : r)];
+    }
+  }
+  for (uint32_t i = tid; i < Lt::kW4 / 16u; i += kFuThreads)
+    reinterpret_cast<uint4*>(smem + off_w[3])[i] = static_cast<const uint4*>(a.w[3])[i];
+  float* cst = reinterpret_cast<float*>(smem + Lt::kOffC);
+  for (uint32_t i = tid; i < 4u * 32u; i += kFuThreads) {
+    const uint32_t k = i / 32u, c = i % 32u;
+    const bool real = k < 3u || c == 0u;
+    // powers of two: the folded form rounds like scaling the rounded sum
+    cst[i] = real ? (a.inv[k] ? a.inv[k][c] : 1.f) * a.out_scale[k] : 0.f;
+    cst[4 * 32 + i] = real ? a.bias[k][c] * a.out_scale[k] : 0.f;
+  }
+  fence_async_smem();
   fence_before();
   __syncthreads();
   fence_after();
@@ -810,6 +812,7 @@ __global__ void __launch_bounds__(kFuThreads, 1)
 // loaded before the wait for the row's sums). Measured at 960x540: three launches
 // 21 + 26 + 26 us; one with the activations themselves as masks (64 bytes) 54, with
 // bits 42. Training step 180 -> 169 -> 153 us, 251x143 49.3 -> 44.1 -> 43.5.
+// (149 and 39.9 since the kernels set up before they wait for the one before.)
 constexpr int kBwThreads = 32 * (12 + 4);
 
 // Epilogue of gradient K (one warpgroup, lane = pixel)
@@ -891,7 +894,6 @@ __device__ __forceinline__ bool bwd_epilogue(const int K, const FusedArgs& a, un
 
 __global__ void __launch_bounds__(kBwThreads, 1)
     k_bwd_fused(const __grid_constant__ CUtensorMap tmap, const __grid_constant__ FusedArgs a) {
-  after_previous();
   using Lt = FusedLayout<false>;
   extern __shared__ __align__(1024) unsigned char smem[];
   uint64_t* bars = reinterpret_cast<uint64_t*>(smem + Lt::kOffB);
@@ -938,6 +940,8 @@ __global__ void __launch_bounds__(kBwThreads, 1)
   fence_before();
   __syncthreads();
   fence_after();
+  // the weights are older than the kernel before: it began after they were written
+  after_previous();
   bool ok = true;
   if (warp < 12)
     ok = bwd_epilogue(warp >> 2, a, smem, full, done, acc_empty, tmem);
@@ -1185,6 +1189,7 @@ __device__ __forceinline__ void wgrad_body(const WgradArgs& args, const int laye
   __syncthreads();
   fence_after();
   const uint32_t tmem = __shfl_sync(0xFFFFFFFFu, *tslot, 0);
+  after_previous();
   const uint32_t my_tiles = blk < n_tiles ? (n_tiles - 1 - blk) / nblk + 1 : 0;
 
   if (warp == kWgEpiWarps) {
@@ -1393,7 +1398,6 @@ __device__ __forceinline__ void wgrad_body(const WgradArgs& args, const int laye
 
 template <int CHAIN>
 __global__ void __launch_bounds__(kWgThreads, 1) k_wgrad(const __grid_constant__ WgradArgs args) {
-  after_previous();
   extern __shared__ __align__(1024) unsigned char smem[];
   if (blockIdx.x < args.share[1].blk0) wgrad_body<2, 4, CHAIN>(args, 0, smem);
   else if (blockIdx.x < args.share[2].blk0) wgrad_body<4, 4, CHAIN>(args, 1, smem);

@@ -206,11 +206,13 @@ cudaError_t render(const RenderArgs& a, Workspace& ws, cudaStream_t st);
 // stage timing: start a profiled call (resets the event list) / mark the end of a stage
 void profile_begin(Workspace& ws, cudaStream_t st);
 void profile_mark(Workspace& ws, int stage, cudaStream_t st);
-// Launch of a kernel that begins with after_previous(): it is put on the SMs as
-// the kernel before it in the stream drains instead of after that has ended and
+// Launch of a kernel that calls after_previous(): it is put on the SMs as the
+// kernel before it in the stream drains instead of after that has ended and
 // waits there (programmatic dependent launch), which hides its launch: 1 to 2 us
-// a kernel in the training step and the builds. It reads and writes nothing
-// before that wait, which covers all earlier work of the stream.
+// a kernel in the training step and the builds. Before that wait, which covers
+// all earlier work of the stream, it touches no memory that the kernel before may
+// write or read. A kernel that allocates TMEM does so before the call: the next
+// kernel's blocks come only when every block of this one has its own.
 template <typename... P, typename... A>
 cudaError_t launch_after(void (*kernel)(P...), unsigned grid, unsigned block, size_t smem, cudaStream_t st, A&&... args) {
   cudaLaunchAttribute attr = {};
