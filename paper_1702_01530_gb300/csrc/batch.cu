@@ -283,14 +283,32 @@ __global__ void __launch_bounds__(kThreads, RT_BATCH_MIN_BLOCKS) k_render_batch(
   }
 }
 
-// fixed-point sums -> float RGB; blockIdx.y = request (launch order)
+// fixed-point sums -> float RGB; blockIdx.y = request (launch order). Bound by
+// memory: 4 values per thread with 16-byte accesses where the request's sums and
+// images are aligned (16 requests, 12.7 M stereo pixels: 91 us, 6.7 TB/s; 149 us
+// with 4-byte ones).
 __global__ void k_resolve_batch(const BatchReq* __restrict__ req, const uint32_t* __restrict__ acc) {
   const BatchReq& rq = req[blockIdx.y];
   const uint32_t n3 = 3u * rq.cam.W * rq.cam.H;
   const uint32_t* a = acc + 3 * (size_t)rq.pix_base;
-  for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < 2 * n3; i += gridDim.x * blockDim.x) {
-    const float v = fminf(1.f, (float)a[i] * rq.inv_scale);
-    if (i < n3) rq.out_L[i] = v; else rq.out_R[i - n3] = v;
+  const float scale = rq.inv_scale;
+  float* const out_L = rq.out_L;
+  float* const out_R = rq.out_R;
+  const uint32_t first = blockIdx.x * blockDim.x + threadIdx.x, step = gridDim.x * blockDim.x;
+  if (n3 % 4 == 0 && (((uintptr_t)a | (uintptr_t)out_L | (uintptr_t)out_R) & 15u) == 0) {
+    const uint4* a4 = reinterpret_cast<const uint4*>(a);
+    for (uint32_t i = first; i < n3 / 2; i += step) {
+      const uint4 s = __ldcs(a4 + i);
+      const float4 v = make_float4(fminf(1.f, (float)s.x * scale), fminf(1.f, (float)s.y * scale),
+                                   fminf(1.f, (float)s.z * scale), fminf(1.f, (float)s.w * scale));
+      if (i < n3 / 4) reinterpret_cast<float4*>(out_L)[i] = v;
+      else reinterpret_cast<float4*>(out_R)[i - n3 / 4] = v;
+    }
+    return;
+  }
+  for (uint32_t i = first; i < 2 * n3; i += step) {
+    const float v = fminf(1.f, (float)a[i] * scale);
+    if (i < n3) out_L[i] = v; else out_R[i - n3] = v;
   }
 }
 
