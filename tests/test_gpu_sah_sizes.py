@@ -1,5 +1,5 @@
 """The SAH build at the edges of its phases: warps of 32 leaves, blocks of 256,
-slices of 1024, degenerate centroids and the depth budget.
+slices of 512, degenerate centroids and the depth budget.
 
 The tree has to hold every leaf and node once, no deeper than the traversal
 stack allows, with boxes that are exactly the unions of their leaves', the same
