@@ -50,21 +50,30 @@ constexpr int kRedBlocks = 256;
 
 struct Bounds6 { double lo[3], hi[3]; };
 
+// Words of the raw records. FIRST: the first kernel of a build, which may overlap
+// the one that writes them, so ordinary loads; complete for the later ones.
+template <bool FIRST, typename T>
+__device__ __forceinline__ T raw(const T* p) {
+  if (FIRST) return *p;
+  return __ldg(p);
+}
+
 // triangle i of 10-word records; `wide`: the array is 8-byte aligned
+template <bool FIRST = false>
 __device__ __forceinline__ void load_tri(const float* t, uint32_t i, bool wide, float v[9]) {
   const float* p = t + 10ull * i;
   if (wide) {
     const float2* q = reinterpret_cast<const float2*>(p);
 #pragma unroll
     for (int k = 0; k < 4; ++k) {
-      const float2 x = __ldg(q + k);
+      const float2 x = raw<FIRST>(q + k);
       v[2 * k] = x.x;
       v[2 * k + 1] = x.y;
     }
-    v[8] = __ldg(p + 8);
+    v[8] = raw<FIRST>(p + 8);
   } else {
 #pragma unroll
-    for (int k = 0; k < 9; ++k) v[k] = __ldg(p + k);
+    for (int k = 0; k < 9; ++k) v[k] = raw<FIRST>(p + k);
   }
 }
 
@@ -110,14 +119,14 @@ k_centroid_bounds(const float* sph, const float* tri, uint32_t ns, uint32_t n, b
   for (; i < ns && i < n; i += step)
 #pragma unroll
     for (int k = 0; k < 3; ++k) {
-      const float c = __ldg(sph + 5ull * i + k);
+      const float c = raw<true>(sph + 5ull * i + k);
       f[k] = fminf(f[k], c);
       f[3 + k] = fminf(f[3 + k], -c);
     }
   const uint32_t first_tri = i;
   for (; i < n; i += step) {
     float t[9];
-    load_tri(tri, i - ns, wide, t);
+    load_tri<true>(tri, i - ns, wide, t);
 #pragma unroll
     for (int k = 0; k < 3; ++k) {
       float least, most;
@@ -140,7 +149,7 @@ k_centroid_bounds(const float* sph, const float* tri, uint32_t ns, uint32_t n, b
   for (int k = 0; k < 6; ++k) v[k] = kMost;
   for (i = first_tri; i < n; i += step) {
     float t[9];
-    load_tri(tri, i - ns, wide, t);
+    load_tri<true>(tri, i - ns, wide, t);
 #pragma unroll
     for (int k = 0; k < 3; ++k) {
       float least, most;
@@ -246,7 +255,7 @@ k_keys(const float* sph, const float* tri, uint32_t ns, uint32_t n, bool wide, c
     float v[9];
     const bool is_sphere = i < ns;
     if (is_sphere)
-      for (int k = 0; k < 3; ++k) v[k] = v[3 + k] = v[6 + k] = __ldg(sph + 5ull * i + k);
+      for (int k = 0; k < 3; ++k) v[k] = v[3 + k] = v[6 + k] = raw<false>(sph + 5ull * i + k);
     else
       load_tri(tri, i - ns, wide, v);
     uint32_t q[3];
@@ -521,7 +530,7 @@ __device__ __forceinline__ bool run_climb(Run<N>& run, const First& first, int i
 // the primitives in sorted order, and the trees over every 256 of them
 constexpr int kTreeThreads = 256;
 __global__ void __launch_bounds__(kTreeThreads, 6)
-k_tree(const float* sph, const float* tri, uint32_t ns, uint32_t n, bool wide, const uint64_t* __restrict__ keys,
+k_tree(const float* sph, const float* tri, uint32_t ns, uint32_t n, bool wide, const uint64_t* keys,
        float4* nodes, float4* prims, int32_t* parent, uint2* left_over, uint32_t* counts) {
   after_previous();
   __shared__ union {
@@ -605,8 +614,8 @@ struct UpShared {
   uint32_t base[kUpGroup + 1];
 };
 __global__ void __launch_bounds__(kUpThreads)
-k_tree_up(const float* sph, const float* tri, uint32_t ns, uint32_t n, bool wide, const uint64_t* __restrict__ keys,
-          float4* nodes, int32_t* parent, uint2* left_over, const uint32_t* __restrict__ counts, uint32_t runs,
+k_tree_up(const float* sph, const float* tri, uint32_t ns, uint32_t n, bool wide, const uint64_t* keys,
+          float4* nodes, int32_t* parent, uint2* left_over, const uint32_t* counts, uint32_t runs,
           uint64_t span, uint32_t* counts_out, uint32_t* err) {
   after_previous();
   extern __shared__ __align__(16) unsigned char up_smem[];

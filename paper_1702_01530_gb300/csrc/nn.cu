@@ -845,7 +845,7 @@ __device__ __forceinline__ bool bwd_epilogue(const int K, const FusedArgs& a, un
       const int y = it.y0 - 2 + K + (i - 2);
       const bool inside = i >= 2 && col_in && y >= 0 && y < (int)a.H;
       const size_t p = inside ? (size_t)y * a.W + x : 0;
-      const uint32_t mk = inside ? __ldg(mask + p) : 0u;
+      const uint32_t mk = inside ? __ldcg(mask + p) : 0u;   // written by the kernel before
       const bool ok = i >= 2 && to_next && wrapped
                           ? mbar_wait2<false>(done_n + next.slot, next.par ^ 1u, done_k + in.slot, in.par)
                           : mbar_wait(done_k + in.slot, in.par);

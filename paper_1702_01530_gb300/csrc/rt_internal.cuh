@@ -213,6 +213,14 @@ void profile_mark(Workspace& ws, int stage, cudaStream_t st);
 // all earlier work of the stream, it touches no memory that the kernel before may
 // write or read. A kernel that allocates TMEM does so before the call: the next
 // kernel's blocks come only when every block of this one has its own.
+// It overlaps the kernel before it and no earlier one. What an earlier kernel of
+// its chain writes is therefore no constant of its run: it is read with ordinary
+// (or ld.cg) loads through pointers without __restrict__, which stay behind the
+// wait, never with __ldg or through const __restrict__, which promise a value that
+// nobody writes while the kernel is resident and need not stay behind the wait.
+// The first kernel of a chain reads the caller's data so too. The read-only path
+// is for what was complete before the chain: a scene's trees and primitives in a
+// render, the raw records from a build's second kernel on.
 template <typename... P, typename... A>
 cudaError_t launch_after(void (*kernel)(P...), unsigned grid, unsigned block, size_t smem, cudaStream_t st, A&&... args) {
   cudaLaunchAttribute attr = {};

@@ -208,7 +208,7 @@ __device__ __forceinline__ void choose_split(const Bins& bins, const float cext[
 
 // the id of a node from its split position; it goes into the parent's record
 __device__ __forceinline__ uint32_t place_node(uint32_t split, uint32_t parent_slot, uint32_t root_split,
-                                               float4* __restrict__ out, uint32_t n, uint32_t* __restrict__ err) {
+                                               float4* out, uint32_t n, uint32_t* err) {
   if (parent_slot == kRoot) return 0u;
   uint32_t id = split == 1 ? root_split - 1 : split - 1;
   if (id >= n - 1) { atomicOr(err, ERR_BUILD); id = n - 2; }   // splits lie in [1, n-1]: cannot happen
@@ -218,7 +218,7 @@ __device__ __forceinline__ uint32_t place_node(uint32_t split, uint32_t parent_s
 
 // a node's boxes, and its leaf children (slots; kRoot: an inner child, which
 // writes itself)
-__device__ __forceinline__ void write_node(float4* __restrict__ out, uint32_t id, const float cl[2][3],
+__device__ __forceinline__ void write_node(float4* out, uint32_t id, const float cl[2][3],
                                            const float ch[2][3], uint32_t leaf0, uint32_t leaf1) {
   float4* o = out + 4 * (size_t)id;
   o[0] = make_float4(cl[0][0], ch[0][0], cl[0][1], ch[0][1]);
@@ -260,8 +260,8 @@ __device__ __forceinline__ void combine6(uint32_t grp, const int v[6], int* dst)
 // leaf box of slot k: the child box of k's parent that holds leaf ~k; the
 // identity order; and the centroid bounds of all leaves
 __global__ void __launch_bounds__(kThreads)
-k_leaves(const float4* __restrict__ nodes, const int32_t* __restrict__ parent, uint32_t n,
-         float4* __restrict__ lo, float4* __restrict__ hi, uint32_t* __restrict__ idx, TopNode* root) {
+k_leaves(const float4* nodes, const int32_t* parent, uint32_t n,
+         float4* lo, float4* hi, uint32_t* idx, TopNode* root) {
   after_previous();
   const uint32_t k = blockIdx.x * blockDim.x + threadIdx.x;
   __shared__ int s_bounds[6];
@@ -352,8 +352,8 @@ __device__ __forceinline__ void load_leaves(const Build& g, uint32_t base, uint3
 __global__ void __launch_bounds__(kThreads)
 k_top_bins(const Build g, int cur) {
   after_previous();
-  const uint32_t* __restrict__ slice_node = g.slice_node[0];
-  int* __restrict__ slice_cnt = g.slice_cnt;
+  const uint32_t* slice_node = g.slice_node[0];
+  int* slice_cnt = g.slice_cnt;
   TopNode* nodes = g.nodes[0];
   Control* ctl = g.ctl;
   const uint32_t slice = g.slice;
@@ -511,9 +511,9 @@ __device__ void top_node(const TopNode& t, uint32_t n_left, int axis, int bin, c
 __global__ void __launch_bounds__(kThreads, 4)
 k_top_scatter(const Build g, int cur) {
   after_previous();
-  uint32_t* __restrict__ idx_out = g.idx[1];
-  const uint32_t* __restrict__ slice_node = g.slice_node[0];
-  const int* __restrict__ slice_cnt = g.slice_cnt;
+  uint32_t* idx_out = g.idx[1];
+  const uint32_t* slice_node = g.slice_node[0];
+  const int* slice_cnt = g.slice_cnt;
   TopNode* nodes = g.nodes[0];
   const uint32_t slice = g.slice;
   __shared__ NodeShared s_node;
@@ -653,8 +653,8 @@ k_top_scatter(const Build g, int cur) {
 // longest segment, and only the winning position's child boxes are handed out.
 // key: the warp's scratch.
 __device__ void small_subtree(uint32_t m, uint32_t slot, float bx[6], uint32_t base, uint32_t parent_slot,
-                              uint32_t depth, uint32_t root_split, float4* __restrict__ out, uint32_t n,
-                              uint32_t* __restrict__ err, uint32_t* key) {
+                              uint32_t depth, uint32_t root_split, float4* out, uint32_t n,
+                              uint32_t* err, uint32_t* key) {
   const uint32_t lane = threadIdx.x & 31;
   uint32_t b = lane < m ? 0u : lane, e = lane < m ? m : lane + 1;
   for (uint32_t guard = 0; guard < kSmallLeaves; ++guard) {
@@ -782,9 +782,9 @@ __device__ void small_subtree(uint32_t m, uint32_t slot, float bx[6], uint32_t b
 constexpr int kMaxSeg = (int)(kMidLeaves / (kSmallLeaves + 1));   // segments of more than kSmallLeaves leaves (or the root)
 static_assert(kMaxSeg <= kWarps, "a warp per segment");
 __global__ void __launch_bounds__(kThreads, 4)
-k_sah_mid(const float4* __restrict__ leaf_lo, const float4* __restrict__ leaf_hi,
-          const uint32_t* __restrict__ idx0, const uint32_t* __restrict__ idx1, Control* ctl,
-          const Job* __restrict__ jobs, float4* __restrict__ out, uint32_t n, uint32_t* __restrict__ err) {
+k_sah_mid(const float4* leaf_lo, const float4* leaf_hi,
+          const uint32_t* idx0, const uint32_t* idx1, Control* ctl,
+          const Job* jobs, float4* out, uint32_t n, uint32_t* err) {
   after_previous();
   __shared__ uint32_t s_slot[kThreads];
   __shared__ float s_box[6][kThreads];
@@ -968,7 +968,7 @@ __device__ __forceinline__ void centre_extent(float lo, float hi, float& c, floa
   e = __double2float_ru(half + 0x1p-22 * (double)big);
 }
 
-__global__ void k_render_nodes(const float4* __restrict__ nodes, uint32_t n_inner, float4* __restrict__ out) {
+__global__ void k_render_nodes(const float4* nodes, uint32_t n_inner, float4* out) {
   after_previous();
   const uint32_t i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= n_inner) return;

@@ -490,8 +490,7 @@ k_render(KParams kp) {
   }
 }
 
-__global__ void k_resolve(const uint32_t* __restrict__ acc, float* __restrict__ out_L,
-                          float* __restrict__ out_R, uint32_t n3, float inv_scale) {
+__global__ void k_resolve(const uint32_t* acc, float* out_L, float* out_R, uint32_t n3, float inv_scale) {
   after_previous();
   const uint32_t total = out_R ? 2 * n3 : n3;      // no right image: the left eye only
   for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < total; i += gridDim.x * blockDim.x) {
@@ -504,8 +503,7 @@ __global__ void k_resolve(const uint32_t* __restrict__ acc, float* __restrict__ 
 // multiple of 4 and both images are 16-byte aligned: the images may be
 // pinned host memory mapped into the device (the host-output render), where
 // wide stores make fuller transfers over the CPU-GPU link.
-__global__ void k_resolve4(const uint4* __restrict__ acc, float4* __restrict__ out_L,
-                           float4* __restrict__ out_R, uint32_t n3_4, float inv_scale) {
+__global__ void k_resolve4(const uint4* acc, float4* out_L, float4* out_R, uint32_t n3_4, float inv_scale) {
   after_previous();
   const uint32_t total = out_R ? 2 * n3_4 : n3_4;  // no right image: the left eye only
   for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < total; i += gridDim.x * blockDim.x) {
