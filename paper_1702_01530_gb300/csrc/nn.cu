@@ -1694,7 +1694,8 @@ cudaError_t launch_bwd(const void* g8, __nv_bfloat16* const wb[4], uint32_t* mas
   a.mask = mask;
   a.err = err;
   const int grid = choose_segments<3>(a, W, H, 1);
-  return launch_after(k_bwd_fused, grid, kBwThreads, smem, st, map, a);
+  launch_after(k_bwd_fused, grid, kBwThreads, smem, st, map, a);
+  return cudaGetLastError();
 }
 }  // namespace
 
@@ -1808,8 +1809,11 @@ cudaError_t train_step(const __nv_bfloat16* feat16, const float* label, const Tr
     configured = true;
   }
   const uint32_t grid = g.share[3].blk0 + g.share[3].nblk;
-  if (wgrad_tiles(W, H) <= (uint64_t)kWgFewTiles * g.share[1].nblk) launch_after(k_wgrad<2>, grid, kWgThreads, smem, st, g);
-  else launch_after(k_wgrad<4>, grid, kWgThreads, smem, st, g);
+  const bool few = wgrad_tiles(W, H) <= (uint64_t)kWgFewTiles * g.share[1].nblk;
+  launch_after(few ? k_wgrad<2> : k_wgrad<4>, grid, kWgThreads, smem, st, g);
+  // no update from partial sums that were not made
+  e = cudaGetLastError();
+  if (e != cudaSuccess) return e;
 
   UpdateArgs u = {};
   uint32_t block = 0;
