@@ -1650,6 +1650,13 @@ int choose_segments(FusedArgs& a, uint32_t W, uint32_t H, uint32_t n_img) {
   return (int)std::min(strips * a.segs, sms);
 }
 
+// Dynamic shared memory of a kernel. An attribute of the current device, so set
+// before every launch (0.2 us), not once in a process.
+template <typename Kernel>
+cudaError_t allow_smem(Kernel* kernel, size_t bytes) {
+  return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+}
+
 template <bool FP8, bool STORE>
 cudaError_t launch_fused(const __nv_bfloat16* feat16, FusedArgs& a, uint32_t W, uint32_t H,
                          uint32_t n_img, cudaStream_t st, int* grid_out = nullptr) {
@@ -1657,15 +1664,9 @@ cudaError_t launch_fused(const __nv_bfloat16* feat16, FusedArgs& a, uint32_t W, 
   // a CTA takes all TMEM columns: more than half of an SM's shared memory, so
   // that no second one can be placed beside it
   constexpr uint32_t smem = Lt::kSmem < 116u * 1024u ? 116u * 1024u : Lt::kSmem;
-  static bool configured = false;
-  if (!configured) {
-    const cudaError_t e = cudaFuncSetAttribute(k_net_fused<FP8, STORE>,
-                                               cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-    configured = true;
-  }
   CUtensorMap map;
-  const cudaError_t e = make_feature_map(&map, feat16, 2, W, H, n_img);
+  cudaError_t e = allow_smem(k_net_fused<FP8, STORE>, smem);
+  if (e == cudaSuccess) e = make_feature_map(&map, feat16, 2, W, H, n_img);
   if (e != cudaSuccess) return e;
   const int grid = choose_segments<4>(a, W, H, n_img);
   if (grid_out) *grid_out = grid;
@@ -1677,14 +1678,9 @@ cudaError_t launch_fused(const __nv_bfloat16* feat16, FusedArgs& a, uint32_t W, 
 cudaError_t launch_bwd(const void* g8, __nv_bfloat16* const wb[4], uint32_t* mask, __nv_bfloat16* const dz[3], uint32_t W, uint32_t H, uint32_t* err, cudaStream_t st) {
   constexpr uint32_t smem = FusedLayout<false>::kSmem;
   static_assert(smem > 116u * 1024u, "a CTA takes all TMEM columns: one on an SM");
-  static bool configured = false;
-  if (!configured) {
-    const cudaError_t e = cudaFuncSetAttribute(k_bwd_fused, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-    configured = true;
-  }
   CUtensorMap map;
-  const cudaError_t e = make_feature_map(&map, g8, 1, W, H, 1);
+  cudaError_t e = allow_smem(k_bwd_fused, smem);
+  if (e == cudaSuccess) e = make_feature_map(&map, g8, 1, W, H, 1);
   if (e != cudaSuccess) return e;
   FusedArgs a = {};
   for (int k = 0; k < 3; ++k) {
@@ -1801,16 +1797,12 @@ cudaError_t train_step(const __nv_bfloat16* feat16, const float* label, const Tr
   // the largest layer's stages; one CTA (and its TMEM) per SM
   constexpr size_t smem = std::max(std::max(WgradLayout<2, 4>::kSmem, WgradLayout<4, 4>::kSmem),
                                    std::max(WgradLayout<4, 1>::kSmem, (size_t)116 * 1024));
-  static bool configured = false;
-  if (!configured) {
-    e = cudaFuncSetAttribute(k_wgrad<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(k_wgrad<4>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-    configured = true;
-  }
   const uint32_t grid = g.share[3].blk0 + g.share[3].nblk;
   const bool few = wgrad_tiles(W, H) <= (uint64_t)kWgFewTiles * g.share[1].nblk;
-  launch_after(few ? k_wgrad<2> : k_wgrad<4>, grid, kWgThreads, smem, st, g);
+  const auto wgrad = few ? k_wgrad<2> : k_wgrad<4>;
+  e = allow_smem(wgrad, smem);
+  if (e != cudaSuccess) return e;
+  launch_after(wgrad, grid, kWgThreads, smem, st, g);
   // no update from partial sums that were not made
   e = cudaGetLastError();
   if (e != cudaSuccess) return e;

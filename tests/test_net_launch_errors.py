@@ -121,3 +121,12 @@ def test_a_step_ends_at_its_first_failed_launch(fake, W, H):
         assert fake.fake_launches() == at + 1, "a kernel was launched on what the failed one did not make"
         fake.fake_begin(0, -1)
         assert fake.fake_train(W, H) == 0, "the failure is reported once"
+
+
+@pytest.mark.parametrize("W,H", [(960, 540), (33, 9)])     # either weight-gradient kernel
+def test_a_second_device_allows_the_shared_memory_too(fake, W, H):
+    for device in (0, 1, 0, 2):
+        fake.fake_begin(device, -1)
+        assert fake.fake_forward(0, W, H) == 0, device
+        assert fake.fake_forward(1, W, H) == 0, device
+        assert fake.fake_train(W, H) == 0, device
