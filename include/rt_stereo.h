@@ -95,6 +95,9 @@ typedef struct rt_scene rt_scene;  /* opaque */
  *     before returning.
  *   out_scene: receives the new scene; owned by the caller, released with
  *     rt_scene_destroy.
+ * A scene holds 256 bytes of device memory per primitive (the two trees, the
+ * render form of the one renders walk, the records), in one allocation that also
+ * serves as the build's scratch; renders add their own scratch.
  * Errors: RT_ERR_INVALID_ARG (validation), RT_ERR_OOM, RT_ERR_CUDA.
  */
 int rt_scene_create(const rt_sphere* spheres, uint32_t n_spheres,
@@ -303,12 +306,13 @@ int rt_debug_set_pool_capacity(rt_scene* scene, uint32_t entries);
  *   RT_TREE_LBVH (2) the Morton-code binary radix tree itself, the tree
  *                rt_scene_get_bvh returns and rt_debug_set_node edits.
  * The instrumented work counts of rt_render_stereo_aux follow the binary
- * tree in use (the SAH tree for RT_TREE_WIDE). The 4-wide tree is built the
- * first time it is chosen (synchronous: the device is synchronised and a
- * scratch buffer of ~21 bytes per primitive is allocated and freed; errors
- * RT_ERR_CUDA); choosing the LBVH for the first time converts its nodes to the
- * form renders walk (synchronous too, no allocation); choosing a tree is
- * otherwise host-only and takes effect with the next render. Other values: RT_ERR_INVALID_ARG.
+ * tree in use (the SAH tree for RT_TREE_WIDE). The 4-wide tree (112 bytes per
+ * primitive, and ~21 of scratch that is freed again) and the form of the LBVH
+ * that renders walk (64 bytes per primitive) are made the first time they are
+ * chosen: the device is synchronised and the memory allocated, which the scene
+ * then keeps; errors RT_ERR_OOM and RT_ERR_CUDA leave the choice as it was.
+ * Choosing a tree is otherwise host-only and takes effect with the next render.
+ * Other values: RT_ERR_INVALID_ARG.
  */
 #define RT_TREE_SAH 0
 #define RT_TREE_WIDE 1

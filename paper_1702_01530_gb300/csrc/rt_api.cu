@@ -268,16 +268,16 @@ int rt_scene_create(const rt_sphere* spheres, uint32_t n_spheres, const rt_trian
   const size_t b_lights = align256((size_t)n_lights * sizeof(float4));
   const size_t b_keys = align256(n * sizeof(uint64_t));
   const size_t b_parent = align256((2 * n - 1) * sizeof(int32_t));
-  const size_t b_nodes4 = align256((n > 1 ? n - 1 : 1) * 7 * sizeof(float4));
   const size_t b_err = 256;
-  // the build's scratch (raw input records, then the two builds' own) lies
-  // where the trees of the other traversals go when a render first asks for
-  // them: an allocation of its own costs 0.15 ms
+  // the builds' scratch lies where the render nodes go, which are made last: an
+  // allocation of its own costs 0.15 ms, and one that stayed would hold memory for
+  // the scene's whole life. The raw records and the LBVH build's scratch (49
+  // bytes a primitive) come first, then the SAH build's (61); the nodes take 64.
   const size_t b_sph = align256((size_t)n_spheres * sizeof(rt_sphere) + 16);
   const size_t b_tri = align256((size_t)n_tris * sizeof(rt_triangle) + 16);
-  const size_t b_tmp = align256(std::max(rt::lbvh_tmp_bytes((uint32_t)n), rt::sah_tmp_bytes((uint32_t)n)));
-  const size_t b_late = std::max(b_nodes4 + b_nodes, b_sph + b_tri + b_tmp);
-  const size_t total = 3 * b_nodes + b_prims + b_mats + b_lights + b_keys + b_parent + b_late + b_err;
+  const size_t b_lbvh = align256(rt::lbvh_tmp_bytes((uint32_t)n));
+  const size_t b_last = std::max({b_nodes, b_sph + b_tri + b_lbvh, align256(rt::sah_tmp_bytes((uint32_t)n))});
+  const size_t total = 2 * b_nodes + b_prims + b_mats + b_lights + b_keys + b_parent + b_last + b_err;
   cudaError_t e = cudaMalloc(&sc->block, total);
   if (e != cudaSuccess) {
     cudaGetLastError();
@@ -293,10 +293,8 @@ int rt_scene_create(const rt_sphere* spheres, uint32_t n_spheres, const rt_trian
   sc->keys = reinterpret_cast<uint64_t*>(p); p += b_keys;
   sc->parent = reinterpret_cast<int32_t*>(p); p += b_parent;
   sc->nodes_sah = reinterpret_cast<float4*>(p); p += b_nodes;
-  sc->render_sah = reinterpret_cast<float4*>(p); p += b_nodes;
   char* const tp = p;
-  sc->nodes4 = reinterpret_cast<float4*>(p);
-  sc->render_lbvh = reinterpret_cast<float4*>(p + b_nodes4); p += b_late;
+  sc->render_sah = reinterpret_cast<float4*>(p); p += b_last;
   sc->err = reinterpret_cast<uint32_t*>(p);
   e = cudaMallocHost(&sc->h_err, sizeof(uint32_t));
   if (e != cudaSuccess) {
@@ -330,12 +328,12 @@ int rt_scene_create(const rt_sphere* spheres, uint32_t n_spheres, const rt_trian
     }
   }
   e = rt::build_lbvh(d_sph, d_tri, n_spheres, n_tris, sc->nodes, sc->prims, sc->keys, sc->parent,
-                     d_lbvh, b_tmp, sc->err, st);
+                     d_lbvh, b_lbvh, sc->err, st);
   // the render tree: SAH splits over the LBVH's leaves
   if (e == cudaSuccess)
-    e = rt::build_sah_tree(sc->nodes, sc->parent, (uint32_t)n, sc->nodes_sah, d_lbvh, sc->err, st);
+    e = rt::build_sah_tree(sc->nodes, sc->parent, (uint32_t)n, sc->nodes_sah, tp, sc->err, st);
   if (e == cudaSuccess) e = rt::render_nodes(sc->nodes_sah, (uint32_t)n, sc->render_sah, st);
-  // (the 4-wide tree is built when a render first asks for it:
+  // (the other traversals' nodes are made when first chosen:
   // rt_scene_set_traversal)
   if (e == cudaSuccess) e = cudaMemcpyAsync(sc->h_err, sc->err, sizeof(uint32_t), cudaMemcpyDeviceToHost, st);
   if (e == cudaSuccess) e = cudaStreamSynchronize(st);
@@ -353,6 +351,8 @@ void rt_scene_destroy(rt_scene* scene) {
   if (!scene) return;
   free_workspace(scene->ws);
   if (scene->block) cudaFree(scene->block);
+  if (scene->nodes4) cudaFree(scene->nodes4);
+  if (scene->render_lbvh) cudaFree(scene->render_lbvh);
   if (scene->h_err) cudaFreeHost(scene->h_err);
   delete scene;
 }
@@ -607,7 +607,7 @@ int rt_debug_set_node(rt_scene* scene, uint32_t node, int32_t left, int32_t righ
     nd[2].w = -1.f;
   }
   e = cudaMemcpy(scene->nodes + 4 * (size_t)node, nd, sizeof nd, cudaMemcpyHostToDevice);
-  if (e == cudaSuccess && scene->lbvh_ready) {
+  if (e == cudaSuccess && scene->render_lbvh) {
     e = rt::render_nodes(scene->nodes, scene->n, scene->render_lbvh, 0);
     if (e == cudaSuccess) e = cudaDeviceSynchronize();
   }
@@ -641,17 +641,18 @@ int rt_scene_set_traversal(rt_scene* scene, int tree) {
   if (!scene) return fail(RT_ERR_INVALID_ARG, "scene is NULL");
   if (tree != RT_TREE_SAH && tree != RT_TREE_WIDE && tree != RT_TREE_LBVH)
     return fail(RT_ERR_INVALID_ARG, "tree must be RT_TREE_SAH, RT_TREE_WIDE or RT_TREE_LBVH");
-  if (tree == RT_TREE_WIDE && !scene->wide_built && scene->n > 1) {
+  const uint32_t n = scene->n;
+  if (tree == RT_TREE_WIDE && !scene->nodes4 && n > 1) {
     // the 4-wide tree, collapsed from the SAH tree (1.28 against 1.40 ms on
     // the 1080p blob pair when collapsed from the LBVH); scratch: the build's
     // own, then the SAH tree's inner parents, then two counts
-    const uint32_t n = scene->n;
     const size_t b4 = align256(rt::bvh4_tmp_bytes(n)), bp = align256(4 * (size_t)n);
-    void* tmp = nullptr;
+    void *tmp = nullptr, *nodes4 = nullptr;
     cudaError_t e = cudaSetDevice(scene->device);
     if (e == cudaSuccess) e = cudaDeviceSynchronize();
     if (e == cudaSuccess) e = cudaMalloc(&tmp, b4 + bp + 256);
-    if (e != cudaSuccess) { cudaGetLastError(); return cuda_fail(e, "4-wide tree scratch"); }
+    if (e == cudaSuccess) e = cudaMalloc(&nodes4, (size_t)(n - 1) * 7 * sizeof(float4));
+    if (e != cudaSuccess) { cudaGetLastError(); cudaFree(tmp); return cuda_fail(e, "4-wide tree allocation"); }
     char* t = static_cast<char*>(tmp);
     int32_t* sah_parent = reinterpret_cast<int32_t*>(t + b4);
     uint32_t* d_counts = reinterpret_cast<uint32_t*>(t + b4 + bp);
@@ -659,22 +660,25 @@ int rt_scene_set_traversal(rt_scene* scene, int tree) {
     e = cudaMemset(d_counts, 0, 2 * sizeof(uint32_t));
     if (e == cudaSuccess) e = rt::inner_parents(scene->nodes_sah, n, sah_parent, 0);
     if (e == cudaSuccess)
-      e = rt::build_bvh4(scene->render_sah, sah_parent, n, rt::treelet_depth(), scene->nodes4, d_counts,
-                         tmp, 0);
+      e = rt::build_bvh4(scene->render_sah, sah_parent, n, rt::treelet_depth(),
+                         static_cast<float4*>(nodes4), d_counts, tmp, 0);
     if (e == cudaSuccess) e = cudaMemcpy(counts, d_counts, sizeof counts, cudaMemcpyDeviceToHost);
     cudaFree(tmp);
-    if (e != cudaSuccess) return cuda_fail(e, "4-wide tree build");
+    if (e != cudaSuccess) { cudaFree(nodes4); return cuda_fail(e, "4-wide tree build"); }
+    scene->nodes4 = static_cast<float4*>(nodes4);
     scene->n_top = counts[0];
     scene->n4 = counts[1];
-    scene->wide_built = true;
   }
-  if (tree == RT_TREE_LBVH && !scene->lbvh_ready) {
+  if (tree == RT_TREE_LBVH && !scene->render_lbvh && n > 1) {
     // the render nodes of the LBVH (the SAH tree's are made with the scene)
+    void* nodes = nullptr;
     cudaError_t e = cudaSetDevice(scene->device);
-    if (e == cudaSuccess) e = rt::render_nodes(scene->nodes, scene->n, scene->render_lbvh, 0);
+    if (e == cudaSuccess) e = cudaMalloc(&nodes, (size_t)(n - 1) * 4 * sizeof(float4));
+    if (e != cudaSuccess) { cudaGetLastError(); return cuda_fail(e, "LBVH render nodes allocation"); }
+    e = rt::render_nodes(scene->nodes, n, static_cast<float4*>(nodes), 0);
     if (e == cudaSuccess) e = cudaDeviceSynchronize();
-    if (e != cudaSuccess) return cuda_fail(e, "LBVH render nodes");
-    scene->lbvh_ready = true;
+    if (e != cudaSuccess) { cudaFree(nodes); return cuda_fail(e, "LBVH render nodes"); }
+    scene->render_lbvh = static_cast<float4*>(nodes);
   }
   scene->tree = tree;
   return RT_OK;

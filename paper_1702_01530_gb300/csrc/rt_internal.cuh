@@ -310,13 +310,12 @@ struct rt_scene {
   uint32_t ns = 0, nt = 0, n = 0, nm = 0, nl = 0;
   void* block = nullptr;       // persistent device allocation
   float4* nodes = nullptr;
-  float4* nodes4 = nullptr;
   float4* nodes_sah = nullptr; // binary tree rebuilt with the SAH over the same leaves (sah.cu)
   float4* render_sah = nullptr;   // render nodes of the SAH tree
-  float4* render_lbvh = nullptr;  // render nodes of the LBVH (made on first use)
-  bool lbvh_ready = false;     // render_lbvh holds them
+  // allocated and made when first chosen (rt_scene_set_traversal):
+  float4* render_lbvh = nullptr;  // render nodes of the LBVH
+  float4* nodes4 = nullptr;       // the 4-wide tree
   uint32_t n4 = 0, n_top = 0;
-  bool wide_built = false;     // nodes4 holds the 4-wide tree (built on first use)
   int tree = RT_TREE_SAH;      // the tree renders walk (rt_scene_set_traversal)
   float4* prims = nullptr;
   float4* mats = nullptr;
