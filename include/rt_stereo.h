@@ -291,6 +291,15 @@ int rt_debug_set_sah_slicing(int enable);
 int rt_debug_set_pool_capacity(rt_scene* scene, uint32_t entries);
 
 /*
+ * rt_debug_render_state -- TEST HOOK. *warps: warps of the render kernel's launch.
+ * *tiles_out: 1 if a warp of the scene's last render has found every primary tile
+ * handed out (from then on the others hand their queues to the drain pools), 0 if
+ * none has, or before the first render. Both are HOST words. Synchronises the
+ * device. RT_ERR_INVALID_ARG for a NULL argument.
+ */
+int rt_debug_render_state(const rt_scene* scene, uint32_t* warps, uint32_t* tiles_out);
+
+/*
  * rt_scene_set_traversal -- choose the tree renders of this scene walk
  * (Table 1 of the paper: BVH trees). Every scene holds three over the same
  * leaves (one primitive each) and the same conservative leaf boxes, so all

@@ -57,6 +57,7 @@ _SIGS = {
     "rt_scene_get_bvh": (ctypes.c_int, [_vp, _vp, _vp, _vp, _vp, _vp, _vp]),
     "rt_scene_num_prims": (_u32, [_vp]),
     "rt_debug_set_pool_capacity": (ctypes.c_int, [_vp, _u32]),
+    "rt_debug_render_state": (ctypes.c_int, [_vp, _vp, _vp]),
     "rt_debug_get_sah_tree": (ctypes.c_int, [_vp, _vp]),
     "rt_debug_set_sah_slicing": (ctypes.c_int, [ctypes.c_int]),
     "rt_debug_set_node": (ctypes.c_int, [_vp, _u32, ctypes.c_int32, ctypes.c_int32,
@@ -259,6 +260,13 @@ def rt_debug_set_node(scene, node, left, right, empty_right=False):
 
 def rt_debug_set_pool_capacity(scene, entries):
     _check(lib().rt_debug_set_pool_capacity(scene, entries))
+
+
+def rt_debug_render_state(scene) -> tuple:
+    """(warps of the render kernel's launch, whether the last render found every tile handed out)."""
+    warps, out = ctypes.c_uint32(), ctypes.c_uint32()
+    _check(lib().rt_debug_render_state(scene, ctypes.byref(warps), ctypes.byref(out)))
+    return warps.value, bool(out.value)
 
 
 def rt_debug_get_sah_tree(scene) -> np.ndarray:

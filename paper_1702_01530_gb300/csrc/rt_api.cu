@@ -631,6 +631,18 @@ int rt_debug_set_sah_slicing(int enable) {
   return RT_OK;
 }
 
+int rt_debug_render_state(const rt_scene* scene, uint32_t* warps, uint32_t* tiles_out) {
+  if (!scene || !warps || !tiles_out) return fail(RT_ERR_INVALID_ARG, "scene or output is NULL");
+  *warps = (uint32_t)rt::render_grid() * (uint32_t)rt::render_threads() / 32u;
+  *tiles_out = 0;
+  if (!scene->ws.counters) return RT_OK;       // nothing rendered yet
+  cudaError_t e = cudaDeviceSynchronize();
+  if (e == cudaSuccess)
+    e = cudaMemcpy(tiles_out, scene->ws.counters + rt::C_TILES_OUT, sizeof *tiles_out, cudaMemcpyDeviceToHost);
+  if (e != cudaSuccess) return cuda_fail(e, "render state download");
+  return RT_OK;
+}
+
 int rt_debug_set_pool_capacity(rt_scene* scene, uint32_t entries) {
   if (!scene) return fail(RT_ERR_INVALID_ARG, "scene is NULL");
   scene->ws.cap_p_limit = entries;
