@@ -228,13 +228,14 @@ k_render(KParams kp) {
         const uint32_t n_warps = gridDim.x * (kThreads / 32);
         t = (uint32_t)gwarp;
         if (round > 0) {
-          // every tile went out in round 0: warp 0 says so too, since of as many
-          // tiles as warps no warp finds one gone (304x288 pair of 26k primitives,
-          // 5472 of both: 149 us; 188 with no word of it, so queues not shared)
-          t = n_tiles + (gwarp != 0 ? 1u : 0u);
           if (n_tiles > n_warps) {
             if (lane == 0) t = n_warps + atomicAdd(&cnt[C_TILE], 1u);
             t = __shfl_sync(0xFFFFFFFFu, t, 0);
+          } else {
+            // every tile went out in round 0: warp 0 says so too, since of as many
+            // tiles as warps no warp finds one gone (304x288 pair of 26k primitives,
+            // 5472 of both: 160 us; 179 with no word of it, so queues not shared)
+            t = n_tiles + (gwarp != 0 ? 1u : 0u);
           }
         }
       } else {
