@@ -268,9 +268,8 @@ int rt_debug_get_sah_tree(const rt_scene* scene, float* nodes);
 
 /*
  * rt_debug_set_sah_slicing -- TEST HOOK. Process-wide: with enable != 0 (the
- * default) scene creation builds the top levels of the SAH tree (levels of at
- * most 32 nodes averaging at least 16384 leaves) with every node sliced over
- * many blocks; with 0 every level runs one block per node. Both give the same
+ * default) scene creation cuts every node of more than 256 leaves into slices of
+ * at least 512, a block each; with 0 such a node is one slice. Both give the same
  * tree; the switch lets a test compare them. Host-only; affects scenes
  * created afterwards. Returns RT_OK.
  */
@@ -367,7 +366,7 @@ int rt_profile_read(const rt_scene* scene, float* ms);
  *     d_keys:   n sorted keys; d_parent: 2n-1 parent indices (as in
  *               rt_scene_get_bvh).
  *   The call synchronises cuda_stream and returns RT_ERR_DEVICE_CHECK if the
- *   device-side refit check trips. Every call uses the same scratch array:
+ *   device-side check of the tree's item counts trips. Every call uses the same scratch array:
  *   calls whose GPU work overlaps (other streams or host threads) race and
  *   must be serialised by the caller. Each call looks up the array's device
  *   address in the current context (cudaGetSymbolAddress), so the address
@@ -487,8 +486,8 @@ int rt_net_load(const char* path, rt_net** out);
  *             16-byte aligned (it is read by the tensor-memory-access engine;
  *             a misaligned pointer gives RT_ERR_CUDA).
  *   d_prob:   DEVICE, W*H float32 output in (0, 1).
- * Asynchronous on cuda_stream; the network's activation buffers are grown
- * on demand (allocation on the first call at a size).
+ * Asynchronous on cuda_stream; one launch, which keeps the activations on the
+ * chip: nothing is allocated.
  */
 int rt_net_forward(rt_net* net, const uint16_t* d_feat16, uint32_t W, uint32_t H, float* d_prob,
                    void* cuda_stream);
@@ -496,7 +495,7 @@ int rt_net_forward(rt_net* net, const uint16_t* d_feat16, uint32_t W, uint32_t H
 /*
  * rt_net_forward_images -- rt_net_forward of n_img feature maps of W x H
  * pixels stored one after the other (d_feat16: n_img*W*H*16 BF16; d_prob:
- * n_img*W*H floats), one launch per layer for all of them. Each image is
+ * n_img*W*H floats), one launch for all of them. Each image is
  * convolved on its own (zero padding at its borders), so image i's output
  * equals rt_net_forward on image i alone bit for bit. The paper has no
  * network; this serves the multi-frame reprojection below.
@@ -507,8 +506,11 @@ int rt_net_forward_images(rt_net* net, const uint16_t* d_feat16, uint32_t n_img,
 /*
  * rt_net_train_step -- one step on the mean binary cross-entropy of the
  * network's output against d_label (DEVICE, W*H floats in {0,1}): forward,
- * backward (data gradients on the tensor cores, weight gradients in FP32),
- * then Adam (beta 0.9 / 0.999, eps 1e-8, step size lr) when lr > 0.
+ * backward (data and weight gradients on the tensor cores, BF16 operands; the
+ * weight gradients' sums in FP32, compensated across blocks), then Adam (beta 0.9 /
+ * 0.999, eps 1e-8, step size lr) when lr > 0. The network keeps 416 bytes of
+ * scratch per pixel of its largest training or calibration map, and partial sums of
+ * at most 90 MB; they are allocated on the first call at a size.
  *   host_loss: if non-NULL receives the loss before the update (synchronises).
  *   d_grads:   if non-NULL, DEVICE RT_NET_PARAMS floats receive the gradient.
  */

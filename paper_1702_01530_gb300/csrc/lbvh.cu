@@ -757,7 +757,8 @@ cudaError_t build_lbvh(const float4* d_sph_in, const float* d_tri_in, uint32_t n
   int red_grid = (int)std::min<uint32_t>((uint32_t)kRedBlocks, (n + kRedThreads - 1) / kRedThreads);
   launch_after(k_centroid_bounds, red_grid, kRedThreads, 0, st, sph, d_tri_in, ns, n, wide, partial);
   launch_after(k_reduce_bounds, 1, 192, 0, st, partial, red_grid);
-  launch_after(k_keys, nblocks, kSortThreads, 0, st, sph, d_tri_in, ns, n, wide, partial, d_keys, hist, nblocks);
+  launch_after(k_keys, nblocks, kSortThreads, 0, st, sph, d_tri_in, ns, n, wide, partial, d_keys, hist,
+               nblocks);
   uint64_t* a = d_keys;
   uint64_t* b = keys_b;
   for (int shift = 32; shift < 64; shift += 8) {
@@ -771,16 +772,19 @@ cudaError_t build_lbvh(const float4* d_sph_in, const float* d_tri_in, uint32_t n
   uint2* left_over = reinterpret_cast<uint2*>(keys_b);
   if (n == 1) cudaMemsetAsync(d_parent, 0xFF, 4, st);
   uint32_t runs = (uint32_t)(((uint64_t)n + kTreeThreads - 1) / kTreeThreads);
-  launch_after(k_tree, runs, kTreeThreads, 0, st, sph, d_tri_in, ns, n, wide, d_keys, d_nodes, d_prims, d_parent, left_over, hist);
+  launch_after(k_tree, runs, kTreeThreads, 0, st, sph, d_tri_in, ns, n, wide, d_keys, d_nodes, d_prims,
+               d_parent, left_over, hist);
   if (runs > 1) {
     // an attribute of the current device: set on every call
-    const cudaError_t e = cudaFuncSetAttribute(k_tree_up, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(UpShared));
+    const cudaError_t e = cudaFuncSetAttribute(k_tree_up, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                               (int)sizeof(UpShared));
     if (e != cudaSuccess) return e;
   }
   uint32_t* counts = hist;
   for (uint64_t span = kTreeThreads; runs > 1; span *= kUpGroup) {
     const uint32_t groups = (runs + kUpGroup - 1) / kUpGroup;
-    launch_after(k_tree_up, groups, kUpThreads, sizeof(UpShared), st, sph, d_tri_in, ns, n, wide, d_keys, d_nodes, d_parent, left_over, counts, runs, span, counts + runs, d_err);
+    launch_after(k_tree_up, groups, kUpThreads, sizeof(UpShared), st, sph, d_tri_in, ns, n, wide, d_keys,
+                 d_nodes, d_parent, left_over, counts, runs, span, counts + runs, d_err);
     counts += runs;
     runs = groups;
   }

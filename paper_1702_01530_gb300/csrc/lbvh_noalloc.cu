@@ -14,9 +14,8 @@
 // library, held until the process exits; it bounds a build to
 // kNoAllocMaxPrims primitives. Every call shares the array, so calls whose
 // GPU work overlaps (different streams, or different host threads) race on
-// it; calls issued one after another on one stream are fine. Whatever must
-// start at zero (the refit arrival counters, the error word) is cleared by
-// each call.
+// it; calls issued one after another on one stream are fine. The error word is
+// cleared by each call; the kernels write the rest of the array before they read it.
 #include <cuda_runtime.h>
 #include <stdint.h>
 

@@ -591,8 +591,8 @@ int rt_render_stereo_reproj_frames(const rt_scene* scene, const rt_camera* cams,
                         eye_sep, convergence, rp.zbuf, net ? rp.feat16 : nullptr, nullptr, rp.hole,
                         rp.warped, st);
   rt::profile_mark(sc->ws, rt::ST_WARP, st);
-  // 3. the network over all frames, one launch per layer (a 3x3 window never
-  //    crosses from one frame into the next)
+  // 3. the network over all frames in one launch (a 3x3 window never crosses
+  //    from one frame into the next)
   if (e == cudaSuccess && net) {
     e = net_forward(net, rp.feat16, rp.prob, W, H, st, n_frames);
     rt::profile_mark(sc->ws, rt::ST_NET, st);

@@ -222,7 +222,8 @@ void profile_mark(Workspace& ws, int stage, cudaStream_t st);
 // is for what was complete before the chain: a scene's trees and primitives in a
 // render, the raw records from a build's second kernel on.
 template <typename... P, typename... A>
-cudaError_t launch_after(void (*kernel)(P...), unsigned grid, unsigned block, size_t smem, cudaStream_t st, A&&... args) {
+cudaError_t launch_after(void (*kernel)(P...), unsigned grid, unsigned block, size_t smem, cudaStream_t st,
+                         A&&... args) {
   cudaLaunchAttribute attr = {};
   attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
   attr.val.programmaticStreamSerializationAllowed = 1;

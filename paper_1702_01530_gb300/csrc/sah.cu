@@ -779,7 +779,8 @@ __device__ void small_subtree(uint32_t m, uint32_t slot, float bx[6], uint32_t b
 }
 
 // Subtrees of 2 to kMidLeaves leaves, one block each, one thread per leaf.
-constexpr int kMaxSeg = (int)(kMidLeaves / (kSmallLeaves + 1));   // segments of more than kSmallLeaves leaves (or the root)
+// segments of more than kSmallLeaves leaves (or the root)
+constexpr int kMaxSeg = (int)(kMidLeaves / (kSmallLeaves + 1));
 static_assert(kMaxSeg <= kWarps, "a warp per segment");
 __global__ void __launch_bounds__(kThreads, 4)
 k_sah_mid(const float4* leaf_lo, const float4* leaf_hi,
@@ -865,7 +866,9 @@ k_sah_mid(const float4* leaf_lo, const float4* leaf_hi,
       // stable partition of every active segment
       int axis = active && !median ? s_choice[g][0] : -1;
       bool left = false;
-      if (active) left = axis < 0 ? tid - b < sz / 2 : bin_of(at3(c, axis), at3(cmin, axis), at3(cext, axis)) <= s_choice[g][1];
+      if (active)
+        left = axis < 0 ? tid - b < sz / 2
+                        : bin_of(at3(c, axis), at3(cmin, axis), at3(cext, axis)) <= s_choice[g][1];
       const uint32_t ball = __ballot_sync(0xFFFFFFFFu, left);
       if (lane == 0) s_scan[warp] = __popc(ball);
       __syncthreads();
@@ -1042,7 +1045,8 @@ cudaError_t build_sah_tree(const float4* lbvh_nodes, const int32_t* parent, uint
   const uint32_t* const idx[2] = {s.idx[0], s.idx[1]};
   TopNode* root = top ? s.nodes[0] : nullptr;
   launch_after(k_begin, 1, kThreads, 0, st, s.ctl, root, s.slice_node[0], s.mid, n, s.slice);
-  launch_after(k_leaves, (int)(((uint64_t)n + kThreads - 1) / kThreads), kThreads, 0, st, lbvh_nodes, parent, n, s.lo, s.hi, s.idx[0], root);
+  launch_after(k_leaves, (int)(((uint64_t)n + kThreads - 1) / kThreads), kThreads, 0, st, lbvh_nodes, parent,
+               n, s.lo, s.hi, s.idx[0], root);
   cudaError_t e = cudaSuccess;
   uint32_t n_mid = 1;
   if (top) {
@@ -1071,7 +1075,8 @@ cudaError_t build_sah_tree(const float4* lbvh_nodes, const int32_t* parent, uint
     if (e == cudaSuccess && n_mid > s.max_mid) e = cudaErrorUnknown;
   }
   if (e == cudaSuccess && n_mid)
-    launch_after(k_sah_mid, (int)std::min(n_mid, 0x7FFFFFFFu), kThreads, 0, st, s.lo, s.hi, idx[0], idx[1], s.ctl, s.mid, out, n, err);
+    launch_after(k_sah_mid, (int)std::min(n_mid, 0x7FFFFFFFu), kThreads, 0, st, s.lo, s.hi, idx[0], idx[1],
+                 s.ctl, s.mid, out, n, err);
   return e == cudaSuccess ? cudaGetLastError() : e;
 }
 

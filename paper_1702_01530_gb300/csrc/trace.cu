@@ -167,10 +167,11 @@ enum Mode : int { M_SHADOW = 0, M_PRIMARY = 1, M_MIRROR = 2 };
 // Mirror queue entry: (origin | pixel) (direction | depth) (weight | 0)
 // SHORT: a warp's first tile is its own number, without the atomic on the tile
 // counter that all warps share, and a frame of no more tiles than warps needs none
-// at all (320x240 pair, 4800 tiles for 5472 warps: 39.9 -> 31.4 us; 1920x251, 30k
-// tiles: 226.7 -> 223.3). Frames of 130k tiles gain nothing, and one of 518k took 0.3 %
-// longer with the changed loop, so frames of more than 16 tiles a warp keep the
-// other.
+// at all (320x240 pair, 4800 tiles for 5472 warps: 39.9 -> 31.4 us). The gain fades
+// with the tiles a warp takes: 257k blob primitives at 4 / 8 / 12 / 16 / 20 / 24 / 48
+// of them 359 / 503 / 650 / 768 / 899 / 1008 / 1695 us without it, 355 / 502 / 648 /
+// 767 / 899 / 1011 / 1702 with it (10 primitives gain 2.5 us at each), so frames of
+// more than 16 tiles a warp keep the other loop.
 constexpr uint32_t kShortTiles = 16;
 template <bool COUNT, int TREE, bool SHORT>
 __global__ void
@@ -593,9 +594,12 @@ cudaError_t render_impl(const RenderArgs& a, Workspace& ws, cudaStream_t st) {
   if (a.resolve) {
     const bool wide = n3 % 4 == 0 && ((uintptr_t)a.out_L % 16) == 0 && ((uintptr_t)a.out_R % 16) == 0;
     if (wide)
-      launch_after(k_resolve4, num_sms() * 8, 256, 0, st, reinterpret_cast<const uint4*>(ws.accum), reinterpret_cast<float4*>(a.out_L), reinterpret_cast<float4*>(a.out_R), n3 / 4, 1.f / a.color_scale);
+      launch_after(k_resolve4, num_sms() * 8, 256, 0, st, reinterpret_cast<const uint4*>(ws.accum),
+                   reinterpret_cast<float4*>(a.out_L), reinterpret_cast<float4*>(a.out_R), n3 / 4,
+                   1.f / a.color_scale);
     else
-      launch_after(k_resolve, num_sms() * 8, 256, 0, st, ws.accum, a.out_L, a.out_R, n3, 1.f / a.color_scale);
+      launch_after(k_resolve, num_sms() * 8, 256, 0, st, ws.accum, a.out_L, a.out_R, n3,
+                   1.f / a.color_scale);
     profile_mark(ws, ST_RESOLVE, st);
   }
   const uint64_t primary = a.plist ? a.plist_n : (a.eyes == 3u ? 2 * P : P);

@@ -13,16 +13,15 @@
 namespace rt {
 namespace {
 
-// Tuning knobs (compile-time; times are means of 100 1080p blob pairs on
-// GB300, SAH tree, both eyes of a 4x4-pixel tile per warp: 1.042 ms by
-// default, 0.221 ms for a 10-primitive scene):
+// Tuning knobs (compile-time; GB300, SAH tree, each knob's times from one run, so
+// they compare with one another and not with another knob's):
 // RT_MIN_BLOCKS = minimum resident blocks per SM requested from the register
-// allocator (0 = no request; 9 measured best: the default walk fits 56
-// registers with 8 bytes spilled outside its loop, 36 warps per SM; against 8 blocks (64 registers,
-// 32 warps) 1.005 against 1.014 ms per 1080p blob pair and 13.94 against
-// 14.05 ms per 4K terrain frame; 6 blocks: 1.051 / 0.216 ms; 7 blocks: 1.048
-// ms; 10 blocks (48 registers, spills in the shading code): 1.047 / 0.242 ms
-// in earlier builds).
+// allocator (0 = no request). 9 measured best: the default walk fits 56 registers
+// with 8 bytes spilled outside its loop, 36 warps per SM. Pair of 257k blob
+// primitives at 1080p / of 10 primitives at 1080p / of a terrain of 2.1 M triangles
+// at 4K, ms, with 6, 7, 8, 9, 10 blocks (48 registers, spills in the shading code):
+// 1.057, 1.041, 1.036, 1.015, 1.045 / 0.175, 0.174, 0.174, 0.174, 0.199 / 14.67,
+// 14.31, 14.19, 13.49, 13.91.
 #ifndef RT_MIN_BLOCKS
 #define RT_MIN_BLOCKS 9
 #endif
