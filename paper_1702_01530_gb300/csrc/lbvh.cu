@@ -755,40 +755,40 @@ cudaError_t build_lbvh(const float4* d_sph_in, const float* d_tri_in, uint32_t n
   const bool wide = (reinterpret_cast<uintptr_t>(d_tri_in) & 7u) == 0;
 
   int red_grid = (int)std::min<uint32_t>((uint32_t)kRedBlocks, (n + kRedThreads - 1) / kRedThreads);
-  launch_after(k_centroid_bounds, red_grid, kRedThreads, 0, st, sph, d_tri_in, ns, n, wide, partial);
-  launch_after(k_reduce_bounds, 1, 192, 0, st, partial, red_grid);
-  launch_after(k_keys, nblocks, kSortThreads, 0, st, sph, d_tri_in, ns, n, wide, partial, d_keys, hist,
-               nblocks);
+  Chain chain{st};
+  chain.then(k_centroid_bounds, red_grid, kRedThreads, 0, sph, d_tri_in, ns, n, wide, partial);
+  chain.then(k_reduce_bounds, 1, 192, 0, partial, red_grid);
+  chain.then(k_keys, nblocks, kSortThreads, 0, sph, d_tri_in, ns, n, wide, partial, d_keys, hist, nblocks);
   uint64_t* a = d_keys;
   uint64_t* b = keys_b;
   for (int shift = 32; shift < 64; shift += 8) {
-    if (shift > 32) launch_after(k_hist, nblocks, kSortThreads, 0, st, a, n, shift, hist, nblocks);
-    launch_after(k_scan, 256, 256, 0, st, hist, nblocks, totals);
-    launch_after(k_scatter, nblocks, kSortThreads, 0, st, a, b, n, shift, hist, nblocks, totals);
+    if (shift > 32) chain.then(k_hist, nblocks, kSortThreads, 0, a, n, shift, hist, nblocks);
+    chain.then(k_scan, 256, 256, 0, hist, nblocks, totals);
+    chain.then(k_scatter, nblocks, kSortThreads, 0, a, b, n, shift, hist, nblocks, totals);
     uint64_t* x = a; a = b; b = x;
   }
   // four passes: the sorted keys are back in d_keys; keys_b holds what the runs leave over, the
   // histograms their counts
   uint2* left_over = reinterpret_cast<uint2*>(keys_b);
-  if (n == 1) cudaMemsetAsync(d_parent, 0xFF, 4, st);
+  if (n == 1 && chain.error == cudaSuccess) chain.error = cudaMemsetAsync(d_parent, 0xFF, 4, st);
   uint32_t runs = (uint32_t)(((uint64_t)n + kTreeThreads - 1) / kTreeThreads);
-  launch_after(k_tree, runs, kTreeThreads, 0, st, sph, d_tri_in, ns, n, wide, d_keys, d_nodes, d_prims,
-               d_parent, left_over, hist);
+  chain.then(k_tree, runs, kTreeThreads, 0, sph, d_tri_in, ns, n, wide, d_keys, d_nodes, d_prims, d_parent,
+             left_over, hist);
   if (runs > 1) {
     // an attribute of the current device: set on every call
     const cudaError_t e = cudaFuncSetAttribute(k_tree_up, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                                (int)sizeof(UpShared));
-    if (e != cudaSuccess) return e;
+    if (chain.error == cudaSuccess) chain.error = e;
   }
   uint32_t* counts = hist;
   for (uint64_t span = kTreeThreads; runs > 1; span *= kUpGroup) {
     const uint32_t groups = (runs + kUpGroup - 1) / kUpGroup;
-    launch_after(k_tree_up, groups, kUpThreads, sizeof(UpShared), st, sph, d_tri_in, ns, n, wide, d_keys,
-                 d_nodes, d_parent, left_over, counts, runs, span, counts + runs, d_err);
+    chain.then(k_tree_up, groups, kUpThreads, sizeof(UpShared), sph, d_tri_in, ns, n, wide, d_keys, d_nodes,
+               d_parent, left_over, counts, runs, span, counts + runs, d_err);
     counts += runs;
     runs = groups;
   }
-  return cudaGetLastError();
+  return chain.end();
 }
 
 }  // namespace rt

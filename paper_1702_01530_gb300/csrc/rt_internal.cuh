@@ -25,6 +25,7 @@
 #include <stdint.h>
 
 #include <string>
+#include <utility>
 
 #include "../../include/rt_stereo.h"
 
@@ -236,6 +237,21 @@ cudaError_t launch_after(void (*kernel)(P...), unsigned grid, unsigned block, si
   c.numAttrs = 1;
   return cudaLaunchKernelEx(&c, kernel, static_cast<P>(args)...);
 }
+// Launches of launch_after one after another, none after one that failed: a later
+// kernel would index by what the failed one did not write (its keys, jobs, counts).
+struct Chain {
+  cudaStream_t st;
+  cudaError_t error = cudaSuccess;
+  template <typename... P, typename... A>
+  void then(void (*kernel)(P...), unsigned grid, unsigned block, size_t smem, A&&... args) {
+    if (error == cudaSuccess) error = launch_after(kernel, grid, block, smem, st, std::forward<A>(args)...);
+  }
+  // the first error, which the runtime then no longer reports
+  cudaError_t end() const {
+    const cudaError_t last = cudaGetLastError();
+    return error != cudaSuccess ? error : last;
+  }
+};
 #ifdef __CUDACC__
 // waits for all earlier work of the stream; lets the next kernel be put in place
 __device__ __forceinline__ void after_previous() {

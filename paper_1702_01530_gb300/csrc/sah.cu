@@ -1044,10 +1044,10 @@ cudaError_t build_sah_tree(const float4* lbvh_nodes, const int32_t* parent, uint
   const bool top = n > kMidLeaves;
   const uint32_t* const idx[2] = {s.idx[0], s.idx[1]};
   TopNode* root = top ? s.nodes[0] : nullptr;
-  launch_after(k_begin, 1, kThreads, 0, st, s.ctl, root, s.slice_node[0], s.mid, n, s.slice);
-  launch_after(k_leaves, (int)(((uint64_t)n + kThreads - 1) / kThreads), kThreads, 0, st, lbvh_nodes, parent,
-               n, s.lo, s.hi, s.idx[0], root);
-  cudaError_t e = cudaSuccess;
+  Chain chain{st};
+  chain.then(k_begin, 1, kThreads, 0, s.ctl, root, s.slice_node[0], s.mid, n, s.slice);
+  chain.then(k_leaves, (int)(((uint64_t)n + kThreads - 1) / kThreads), kThreads, 0, lbvh_nodes, parent, n, s.lo,
+             s.hi, s.idx[0], root);
   uint32_t n_mid = 1;
   if (top) {
     const int blocks = (int)std::min(s.max_slices, 8u * (uint32_t)num_sms());
@@ -1056,28 +1056,28 @@ cudaError_t build_sah_tree(const float4* lbvh_nodes, const int32_t* parent, uint
     int until = kExtra;
     for (uint32_t m = n; m > kMidLeaves; m = (m + 1) / 2) ++until;
     Control c{};
-    for (int level = 0;; ++level) {
+    for (int level = 0; chain.error == cudaSuccess; ++level) {
       if (level == until || level == kMaxDepth + 2) {
-        e = cudaMemcpyAsync(&c, s.ctl, sizeof c, cudaMemcpyDeviceToHost, st);
-        if (e == cudaSuccess) e = cudaStreamSynchronize(st);
-        if (e != cudaSuccess || c.n_nodes[level & 1] == 0) break;
+        chain.error = cudaMemcpyAsync(&c, s.ctl, sizeof c, cudaMemcpyDeviceToHost, st);
+        if (chain.error == cudaSuccess) chain.error = cudaStreamSynchronize(st);
+        if (chain.error != cudaSuccess || c.n_nodes[level & 1] == 0) break;
         if (level == kMaxDepth + 2) return cudaErrorUnknown;      // deeper than the depth budget
         until += kExtra;
       }
       const int cur = level & 1;
-      launch_after(k_top_bins, blocks, kThreads, 0, st, s, cur);
-      launch_after(k_top_scatter, blocks, kThreads, 0, st, s, cur);
+      chain.then(k_top_bins, blocks, kThreads, 0, s, cur);
+      chain.then(k_top_scatter, blocks, kThreads, 0, s, cur);
       std::swap(s.idx[0], s.idx[1]);
       std::swap(s.nodes[0], s.nodes[1]);
       std::swap(s.slice_node[0], s.slice_node[1]);
     }
     n_mid = c.n_mid;
-    if (e == cudaSuccess && n_mid > s.max_mid) e = cudaErrorUnknown;
+    if (chain.error == cudaSuccess && n_mid > s.max_mid) chain.error = cudaErrorUnknown;
   }
-  if (e == cudaSuccess && n_mid)
-    launch_after(k_sah_mid, (int)std::min(n_mid, 0x7FFFFFFFu), kThreads, 0, st, s.lo, s.hi, idx[0], idx[1],
-                 s.ctl, s.mid, out, n, err);
-  return e == cudaSuccess ? cudaGetLastError() : e;
+  if (n_mid)
+    chain.then(k_sah_mid, (int)std::min(n_mid, 0x7FFFFFFFu), kThreads, 0, s.lo, s.hi, idx[0], idx[1], s.ctl, s.mid,
+               out, n, err);
+  return chain.end();
 }
 
 }  // namespace rt

@@ -574,7 +574,9 @@ cudaError_t render_impl(const RenderArgs& a, Workspace& ws, cudaStream_t st) {
     ws.epoch = 1;
   }
   kp.epoch = ws.epoch;
-  launch_after(k_clear, 1, C_TOTAL, 0, st, ws.counters);
+  Chain chain{st};
+  chain.then(k_clear, 1, C_TOTAL, 0, ws.counters);
+  if (chain.error != cudaSuccess) return chain.end();
   // the colour sums of the traced pixels start at their primary ray's store;
   // with atomic adds only, clear the sums of the eyes this render traces
   if (!RT_PRIMARY_STORE) {
@@ -587,24 +589,22 @@ cudaError_t render_impl(const RenderArgs& a, Workspace& ws, cudaStream_t st) {
   profile_mark(ws, ST_CLEAR, st);
   const size_t top_bytes = (TREE == kTreeWide4 && !COUNT) ? 7 * sizeof(float4) * a.sc.n_top : 0;
   const bool is_short = !COUNT && !a.plist && kp.n_tiles <= kShortTiles * (uint32_t)grid * (kThreads / 32);
-  if (is_short) launch_after(k_render<COUNT, TREE, !COUNT>, grid, kThreads, top_bytes, st, kp);
-  else launch_after(k_render<COUNT, TREE, false>, grid, kThreads, top_bytes, st, kp);
+  chain.then(is_short ? k_render<COUNT, TREE, !COUNT> : k_render<COUNT, TREE, false>, grid, kThreads, top_bytes, kp);
   profile_mark(ws, a.trace_stage, st);
   const uint32_t n3 = (uint32_t)(P * 3);
   if (a.resolve) {
     const bool wide = n3 % 4 == 0 && ((uintptr_t)a.out_L % 16) == 0 && ((uintptr_t)a.out_R % 16) == 0;
     if (wide)
-      launch_after(k_resolve4, num_sms() * 8, 256, 0, st, reinterpret_cast<const uint4*>(ws.accum),
-                   reinterpret_cast<float4*>(a.out_L), reinterpret_cast<float4*>(a.out_R), n3 / 4,
-                   1.f / a.color_scale);
+      chain.then(k_resolve4, num_sms() * 8, 256, 0, reinterpret_cast<const uint4*>(ws.accum),
+                 reinterpret_cast<float4*>(a.out_L), reinterpret_cast<float4*>(a.out_R), n3 / 4, 1.f / a.color_scale);
     else
-      launch_after(k_resolve, num_sms() * 8, 256, 0, st, ws.accum, a.out_L, a.out_R, n3,
-                   1.f / a.color_scale);
+      chain.then(k_resolve, num_sms() * 8, 256, 0, ws.accum, a.out_L, a.out_R, n3, 1.f / a.color_scale);
     profile_mark(ws, ST_RESOLVE, st);
   }
   const uint64_t primary = a.plist ? a.plist_n : (a.eyes == 3u ? 2 * P : P);
-  if (a.ray_counts && !a.plist_n_dev) k_counts<<<1, 32, 0, st>>>(ws.counters, primary, a.ray_counts);
-  return cudaGetLastError();
+  if (chain.error == cudaSuccess && a.ray_counts && !a.plist_n_dev)
+    k_counts<<<1, 32, 0, st>>>(ws.counters, primary, a.ray_counts);
+  return chain.end();
 }
 
 }  // namespace
